@@ -216,18 +216,13 @@ __device__ __forceinline__ void side_flux(T qxA, T qyA, T cA, T hA, T hsA, T qxB
 // r = 2); r = 3 carries all six directions per lane and keeps more
 template <int R, typename Pix, int MODE>
 __global__ void __maxnreg__(R == 3 ? 232 : 160)
-    k_residual_vjp(const __grid_constant__ Dev d, const __grid_constant__ Tables tb_g,
+    k_residual_vjp(const __grid_constant__ Dev d,
                    const double* __restrict__ u, const uint8_t* __restrict__ cmask,
                    const double* __restrict__ rbar, double* __restrict__ ubar,
                    double* __restrict__ nbar, double* __restrict__ dbar, int accumulate) {
     // the basis tables in shared memory, as in the forward residual (lane-indexed reads)
     __shared__ Tables s_tb;
-    {
-        const unsigned* src = (const unsigned*)&tb_g;
-        unsigned* dst = (unsigned*)&s_tb;
-        for (int i = threadIdx.x; i < (int)(sizeof(Tables) / 4); i += blockDim.x) dst[i] = src[i];
-        __syncthreads();
-    }
+    copy_table(s_tb, d.tabs);
     const Tables& tb = s_tb;
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE>;
@@ -711,15 +706,10 @@ constexpr int stage_vjp_smem() {
 
 template <int R, typename Pix, int MODE>
 __global__ void __maxnreg__(128)
-    k_stage_vjp(const __grid_constant__ Dev d, const __grid_constant__ Tables tb_g,
+    k_stage_vjp(const __grid_constant__ Dev d,
                 const __grid_constant__ StageVjpArgs a) {
     __shared__ Tables s_tb; // basis tables in shared memory (lane-indexed reads)
-    {
-        const unsigned* src = (const unsigned*)&tb_g;
-        unsigned* dst = (unsigned*)&s_tb;
-        for (int i = threadIdx.x; i < (int)(sizeof(Tables) / 4); i += blockDim.x) dst[i] = src[i];
-        __syncthreads();
-    }
+    copy_table(s_tb, d.tabs);
     const Tables& tb = s_tb;
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE>;
@@ -831,13 +821,13 @@ __global__ void __maxnreg__(128)
             }
             allfull = __all_sync(tm, allfull);
             __syncwarp(tm);
-            // the forward's mixed-precision solve (FP32 factor, FP64 refinement to
-            // 1e-15, FP64 Cholesky fallback); its FP32 arrays overlay M and Y, its
-            // iterate and residual take x and Tb, its points pw (all idle here)
+            // the forward's mixed-precision solve (FP32 factor, refinement to 1e-15,
+            // FP64 Cholesky fallback); its FP32 arrays overlay M and Y, its digit
+            // pairs take x, pw and tmp (all idle here)
             for (int i = lane; i < ND; i += TL) rcb[i] = vb[3 * ND + i];
             __syncwarp(tm);
-            solve_mass_mixed<ND1, NM, TL>(tb, pV, rcb, (float*)M, (float*)Y, x, Tb, pw, tmp, M, Y,
-                                          inv, lane, tm);
+            solve_mass_mixed<ND1, NM, TL>(tb, tb.fs, pV, rcb, (float*)M, (float*)Y, (int2*)x, (int2*)pw,
+                                          (int2*)tmp, M, Y, inv, lane, tm);
             // dH_c/dzeta: zeta_bar(p) -= J w A rcb(p) c(p); the same for delta
             tens_interp<ND1, NM, double, TL>(tb.Bm, rcb, tmp, pw, lane, tm);
             for (int p = lane; p < NMP; p += TL) {
@@ -1035,15 +1025,10 @@ constexpr int begin_vjp_smem() {
 
 template <int R, typename Pix, int MODE>
 __global__ void __maxnreg__(96)
-    k_begin_vjp(const __grid_constant__ Dev d, const __grid_constant__ Tables tb_g,
+    k_begin_vjp(const __grid_constant__ Dev d,
                 const __grid_constant__ BeginVjpArgs a) {
     __shared__ Tables s_tb; // basis tables in shared memory (lane-indexed reads)
-    {
-        const unsigned* src = (const unsigned*)&tb_g;
-        unsigned* dst = (unsigned*)&s_tb;
-        for (int i = threadIdx.x; i < (int)(sizeof(Tables) / 4); i += blockDim.x) dst[i] = src[i];
-        __syncthreads();
-    }
+    copy_table(s_tb, d.tabs);
     const Tables& tb = s_tb;
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE>;

@@ -272,6 +272,80 @@ static void breakpoints(const double* w, int n, double* sb) {
     sb[n] = 1.0;
 }
 
+// digit pairs of the tables T[m][no][ni] (swdg_fixed.cuh), all m at one scale:
+// the smallest power of two 2^t that bounds every row's sum of |T| (or t_min,
+// if larger); writes out[m][no][ld]
+static int fx_tables(const double* T, int m, int no, int ni, int ld, int2* out, int stride,
+                     int t_min = -64) {
+    double big = 0.0;
+    for (int r = 0; r < m * no; ++r) {
+        double s = 0.0;
+        for (int i = 0; i < ni; ++i) s += std::fabs(T[r * ni + i]);
+        big = std::max(big, s);
+    }
+    int t = t_min;
+    while (std::ldexp(1.0, t) < big) ++t;
+    for (int q = 0; q < m; ++q)
+        for (int r = 0; r < no; ++r)
+            for (int i = 0; i < ni; ++i)
+                out[q * stride + r * ld + i] =
+                    fx::split(std::llrint(std::ldexp(T[(q * no + r) * ni + i], fx::FB - t)));
+    return t;
+}
+
+static void build_fx_tables(int R, Tables& tb) {
+    const int n1 = R + 1, nv = (3 * R) / 2 + 1, nm = R + 2;
+    FxTables& x = tb.fx;
+    double B[MXP * MXN], D[MXP * MXN], WB[MXP * MXN], WD[MXP * MXN], F[3 * MXP * MXN];
+    for (int q = 0; q < nv; ++q)
+        for (int a = 0; a < n1; ++a) {
+            B[q * n1 + a] = tb.Bv[q][a];
+            D[q * n1 + a] = tb.Dv[q][a];
+            WB[a * nv + q] = tb.wv[q] * tb.Bv[q][a];
+            WD[a * nv + q] = tb.wv[q] * tb.Dv[q][a];
+        }
+    x.tBv = fx_tables(B, 1, nv, n1, MXN, &x.Bv[0][0], 0);
+    x.tDv = fx_tables(D, 1, nv, n1, MXN, &x.Dv[0][0], 0);
+    x.tWB = fx_tables(WB, 1, n1, nv, MXP, &x.WB[0][0], 0);
+    x.tWD = fx_tables(WD, 1, n1, nv, MXP, &x.WD[0][0], 0);
+    fx_tables(WB, 1, n1, nv, MXP, &x.WDB[0][0], 0, x.tWD);
+    for (int m = 0; m < 3; ++m)
+        for (int a = 0; a < n1; ++a)
+            for (int q = 0; q < nm; ++q)
+                F[(m * n1 + a) * nm + q] = m == 0 ? tb.Bm[q][a] : tb.BmH[m - 1][q][a];
+    static_assert(offsetof(FxTables, BmHT) - offsetof(FxTables, BmT) == sizeof(x.BmT), "layout");
+    x.tBmT = fx_tables(F, 3, n1, nm, MXP, &x.BmT[0][0], MXN * MXP);
+    FxStage& y = tb.fs;
+    // T[no][ni] = M[r][i] or, transposed, M[i][r], M of leading dimension ld
+    auto put = [](const double* M, int ld, bool tr, int no, int ni, int2* out, int old) {
+        double T[MXP * MXP];
+        for (int r = 0; r < no; ++r)
+            for (int i = 0; i < ni; ++i) T[r * ni + i] = tr ? M[i * ld + r] : M[r * ld + i];
+        return fx_tables(T, 1, no, ni, old, out, 0);
+    };
+    y.tBm = put(&tb.Bm[0][0], MXN, false, nm, n1, &y.Bm[0][0], MXN);
+    y.tBmT = put(&tb.Bm[0][0], MXN, true, n1, nm, &y.BmT[0][0], MXP);
+    y.tBg = put(&tb.Bg[0][0], MXN, false, n1, n1, &y.Bg[0][0], MXN);
+    y.tBgT = put(&tb.Bg[0][0], MXN, true, n1, n1, &y.BgT[0][0], MXN);
+    y.tGi = put(&tb.Bginv[0][0], MXP, false, n1, n1, &y.Gi[0][0], MXN);
+    y.tGiT = put(&tb.Bginv[0][0], MXP, true, n1, n1, &y.GiT[0][0], MXN);
+    y.tM1i = put(&tb.M1inv[0][0], MXN, false, n1, n1, &y.M1i[0][0], MXN);
+    memcpy(y.wm, tb.wm, sizeof y.wm);
+    memcpy(y.wg, tb.wg, sizeof y.wg);
+    memcpy(y.BmF, tb.BmF, sizeof y.BmF);
+    memcpy(y.wgF, tb.wgF, sizeof y.wgF);
+    memcpy(tb.ft.Bm, tb.Bm, sizeof tb.Bm);
+    memcpy(tb.ft.BmH, tb.BmH, sizeof tb.BmH);
+    memcpy(tb.ft.wm, tb.wm, sizeof tb.wm);
+    memcpy(tb.ft.BmF, tb.BmF, sizeof tb.BmF);
+    memcpy(tb.ft.BmHF, tb.BmHF, sizeof tb.BmHF);
+    for (int a = 0; a < n1; ++a)
+        for (int q = 0; q < n1; ++q) {
+            y.BgF[q][a] = y.BgTF[a][q] = tb.BgF[q][a];
+            y.GiF[a][q] = y.GiTF[q][a] = tb.BginvF[a][q];
+        }
+}
+
 static bool build_tables(int R, Tables& tb) {
     const int nd1 = R + 1, nv = (3 * R) / 2 + 1, nm = R + 2, ng = R + 1;
     double w[MXP];
@@ -333,6 +407,7 @@ static bool build_tables(int R, Tables& tb) {
         tb.wvF[q] = (float)tb.wv[q];
         tb.wgF[q] = (float)tb.wg[q];
     }
+    build_fx_tables(R, tb);
     return true;
 }
 
@@ -365,6 +440,14 @@ static bool build_overlaps(int R, int P, const Tables& tb, OvTab& ov) {
             memcpy(ov.frac[SET_HALF][h * nm + a], tmp.frac[SET_HALF][a], sizeof(ov.frac[0][0]));
         }
     }
+    for (int s = 0; s < NSET; ++s)
+        for (int a = 0; a < MXI; ++a) {
+            const int c = ov.cnt[s][a];
+            const double e[3] = {c > 0 ? ov.frac[s][a][0] : 0.0, c > 2 ? ov.frac[s][a][1] : 0.0,
+                                 c > 1 ? ov.frac[s][a][c - 1] : 0.0};
+            for (int i = 0; i < 3; ++i)
+                ov.ed[s][a][i] = fx::split(std::llrint(std::ldexp(e[i], fx::FB)));
+        }
     return true;
 }
 
@@ -711,6 +794,7 @@ int swdg_create(const swdg_config* cfg, swdg_ctx** out) {
     Dev& d = ctx->d;
     d.mode = ctx->mode;
     d.g = cfg->g;
+    d.sg = std::sqrt(cfg->g);
     d.eps = cfg->eps_vel;
     d.hlim = cfg->h_lim;
     d.eps0 = cfg->eps0;
@@ -724,7 +808,13 @@ int swdg_create(const swdg_config* cfg, swdg_ctx** out) {
         d.bc_per[i] = 1.0;
         d.bc_ph[i] = 0.0;
     }
-    cudaError_t e = cudaMalloc(&ctx->sc, sizeof(Scalars));
+    // the step scalars, and behind them the tables for the kernels' copies
+    constexpr size_t sc_bytes = (sizeof(Scalars) + 255) / 256 * 256;
+    cudaError_t e = cudaMalloc(&ctx->sc, sc_bytes + sizeof(Tables));
+    d.tabs = (const Tables*)((const char*)ctx->sc + sc_bytes);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync((char*)ctx->sc + sc_bytes, &ctx->tb, sizeof(Tables),
+                            cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess) e = cudaMallocHost(&ctx->sc_host, sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMallocHost(&ctx->pin, 64 * sizeof(double));
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->sc, 0, sizeof(Scalars), ctx->st);
@@ -2695,8 +2785,9 @@ extern "C" int swdg_probe_roots(const double* h, int64_t n, double* z, double* r
 // modules eagerly)
 // ---------------------------------------------------------------------------
 constexpr size_t NOALLOC_OV_BYTES = ((sizeof(OvTab) + 255) / 256) * 256;
+constexpr size_t NOALLOC_TAB_BYTES = ((sizeof(Tables) + 255) / 256) * 256;
 static __device__ __align__(256) unsigned char
-    g_noalloc_scratch[256 + NOALLOC_OV_BYTES + SWDG_NOALLOC_MAX_CELLS];
+    g_noalloc_scratch[256 + NOALLOC_OV_BYTES + NOALLOC_TAB_BYTES + SWDG_NOALLOC_MAX_CELLS];
 static void* g_noalloc_addr[256];   // device address of the array, per device ordinal
 static bool g_noalloc_ready[256];
 
@@ -2776,7 +2867,8 @@ extern "C" int swdg_residual_noalloc(const swdg_config* cfg, int64_t n, const do
     unsigned char* scratch = (unsigned char*)g_noalloc_addr[dev];
     Scalars* sc = (Scalars*)scratch;
     OvTab* ovd = (OvTab*)(scratch + 256);
-    uint8_t* cmask = (uint8_t*)(scratch + 256 + NOALLOC_OV_BYTES);
+    Tables* tabd = (Tables*)(scratch + 256 + NOALLOC_OV_BYTES);
+    uint8_t* cmask = (uint8_t*)(scratch + 256 + NOALLOC_OV_BYTES + NOALLOC_TAB_BYTES);
     cudaStream_t st = (cudaStream_t)cfg->stream;
 
     Tables tb;
@@ -2791,6 +2883,7 @@ extern "C" int swdg_residual_noalloc(const swdg_config* cfg, int64_t n, const do
     d.hxhy = hxhy;
     d.nbr = nbr;
     d.tiles = tiles;
+    d.tabs = tabd;
     d.ov = ovd; // one pixel count; tile k starts at k P^2; conforming faces only
     d.manning = manning;
     d.U = const_cast<double*>(state); // read only: buffer 0 of the kernels' state layout
@@ -2801,6 +2894,7 @@ extern "C" int swdg_residual_noalloc(const swdg_config* cfg, int64_t n, const do
     d.nmemb = 1;
     d.mode = 0;
     d.g = cfg->g;
+    d.sg = std::sqrt(cfg->g);
     d.eps = cfg->eps_vel;
     d.cfl = cfg->cfl;
     for (int i = 0; i < MXTAG; ++i) {
@@ -2814,6 +2908,8 @@ extern "C" int swdg_residual_noalloc(const swdg_config* cfg, int64_t n, const do
             return noalloc_fail(err, err_len, SWDG_EINVAL, "residual_noalloc: tide period <= 0");
     }
     cudaError_t ec = cudaMemcpyAsync(ovd, &ovh, sizeof(OvTab), cudaMemcpyHostToDevice, st);
+    if (ec == cudaSuccess)
+        ec = cudaMemcpyAsync(tabd, &tb, sizeof(Tables), cudaMemcpyHostToDevice, st);
     if (ec != cudaSuccess) return noalloc_fail(err, err_len, SWDG_ECUDA, cudaGetErrorString(ec));
     k_noalloc_begin<<<1, 1, 0, st>>>(sc, t);
     k_noalloc_check_mesh<<<(int)std::min<int64_t>(152 * 8, (n + 255) / 256), 256, 0, st>>>(hxhy, nbr,

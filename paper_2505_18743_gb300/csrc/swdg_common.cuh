@@ -17,6 +17,8 @@
 
 #include <type_traits>
 
+#include "swdg_fixed.cuh"
+
 namespace swdg {
 
 constexpr int MXP = 6;    // max quadrature points per direction (GL 5 for r = 3)
@@ -48,6 +50,9 @@ struct OvTab {
     int P;
     int lo[NSET][MXI], cnt[NSET][MXI];
     double frac[NSET][MXI][MXPIX + 1];
+    // the fractions of the first, the inner (all equal) and the last pixel as
+    // digit pairs (swdg_fixed.cuh), exponent 0
+    int2 ed[NSET][MXI][3];
 };
 
 // status bits
@@ -60,6 +65,37 @@ struct Sz {
     static constexpr int NM = R + 2, NMP = NM * NM;
     static constexpr int NG = R + 1, NGP = NG * NG;
     static constexpr int NZP = NVP + NMP + NGP; // mode P samples per cell
+};
+
+// the basis tables as digit pairs (swdg_fixed.cuh), each with the exponent t*
+// that bounds its rows' absolute sums; test tables are stored by node, and the
+// volume ones carry the quadrature weight
+struct FxTables {
+    int2 Bv[MXP][MXN], Dv[MXP][MXN];                 // nodal -> volume (value, d/dxi)
+    int2 WB[MXN][MXP], WD[MXN][MXP], WDB[MXN][MXP];  // wv Bv, wv Dv; wv Bv at the scale of wv Dv
+    int2 BmT[MXN][MXP], BmHT[2][MXN][MXP];           // face test tables, one scale
+    int tBv, tDv, tWB, tWD, tBmT;
+};
+
+// what the stage update and its adjoint take from the tables: digit pairs of
+// the mass- and momentum-point contractions and of the inverse 1D matrices,
+// with the plain weights and the FP32 basis
+struct FxStage {
+    int2 Bm[MXP][MXN], BmT[MXN][MXP]; // nodal -> mass points, its transpose
+    int2 Bg[MXN][MXN], BgT[MXN][MXN]; // nodal -> momentum points, its transpose
+    int2 Gi[MXN][MXN], GiT[MXN][MXN]; // inverse of Bg, its transpose
+    int2 M1i[MXN][MXN];               // inverse 1D mass matrix
+    double wm[MXP], wg[MXP];
+    float BmF[MXP][MXN], wgF[MXP];
+    float BgF[MXN][MXN], BgTF[MXN][MXN], GiF[MXN][MXN], GiTF[MXN][MXN];
+    int tBm, tBmT, tBg, tBgT, tGi, tGiT, tM1i, pad_;
+};
+
+// the face points' basis: nodal -> face GLL points, and those of half h of a
+// 2:1 face (FP64 and FP32)
+struct FaceTables {
+    double Bm[MXP][MXN], BmH[2][MXP][MXN], wm[MXP];
+    float BmF[MXP][MXN], BmHF[2][MXP][MXN];
 };
 
 struct Tables {
@@ -76,6 +112,9 @@ struct Tables {
     float wgF[MXP];                             // momentum GL weights (FP32-bulk stage update)
     double xs[MXN];                             // support nodes on [0, 1]
     double xq[3][MXP];                          // nodes of the three point sets on [0, 1]
+    FxTables fx;
+    FxStage fs;
+    FaceTables ft;
 };
 
 // clock of one ensemble member (a plain context is an ensemble of one)
@@ -100,6 +139,7 @@ struct Scalars {
 
 struct Dev {
     int64_t n;
+    const Tables* tabs; // the tables in device memory (the kernels' copies to shared memory)
     const double* x0y0;
     const double* hxhy;
     const double* ihxhy; // 1/hx, 1/hy per cell (null: computed in the kernel)
@@ -147,6 +187,7 @@ struct Dev {
     int mode; // 0 S, 1 P
     int s;    // stages
     double g, eps, hlim, eps0, cfl, newton_tol;
+    double sg; // sqrt(g)
     int newton_max;
     int any_friction;
     int bc_kind[MXTAG];
@@ -256,6 +297,16 @@ __device__ __forceinline__ double* rfield(const Dev& d, int stage, int f, int nd
     return d.res + ((size_t)stage * 6 + f) * (size_t)d.n * nd;
 }
 
+// a block's copy of a table (or part of one) in shared memory, from device
+// memory: the kernel's parameter bank would serialise the lanes' reads
+template <typename T>
+__device__ __forceinline__ void copy_table(T& dst, const T* __restrict__ src) {
+    static_assert(sizeof(T) % 8 == 0, "8-byte words");
+    for (int i = threadIdx.x; i < (int)(sizeof(T) / 8); i += blockDim.x)
+        ((unsigned long long*)&dst)[i] = ((const unsigned long long*)src)[i];
+    __syncthreads();
+}
+
 __device__ __forceinline__ int member_of(const Dev& d, int64_t k) {
     return d.memb ? d.memb[k] : 0;
 }
@@ -266,14 +317,49 @@ __device__ __forceinline__ double get_dt(const Dev& d, int m) {
     return d.sc->fixed_dt >= 0.0 ? d.sc->fixed_dt : d.cfl / __longlong_as_double(d.mb[m].rmax);
 }
 
+// FP32 value of a positive double in the FP32 normal range and the double of a
+// positive FP32 normal, by bit patterns on the integer pipe (conversions run
+// on the FP64 pipe: 9 and 17 clocks per warp against 1-2); the first truncates
+__device__ __forceinline__ bool f32_range(double x) {
+    const unsigned h = (unsigned)__double2hiint(x);
+    return h - 0x39e00000u < 0x46000000u - 0x39e00000u; // 2^-97 <= x < 2^97
+}
+__device__ __forceinline__ float f32_trunc(double x) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    return __uint_as_float(((h - 0x38000000u) << 3) | (l >> 29));
+}
+// the nearest FP32 value of any double (ties to even, as a conversion rounds)
+// and the double of any FP32 value, the same way; outside the FP32 normal
+// range by conversion
+__device__ __forceinline__ float f32_of(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned h = (unsigned)(b >> 32) & 0x7fffffffu;
+    if (h - 0x38100000u < 0x47e00000u - 0x38100000u) {
+        const unsigned m = (unsigned)(((b & 0x7fffffffffffffffull) + 0xfffffffull +
+                                       ((b >> 29) & 1ull)) >> 29);
+        return __uint_as_float((m - 0xc0000000u) | ((unsigned)(b >> 32) & 0x80000000u));
+    }
+    return b << 1 ? (float)x : 0.0f;
+}
+__device__ __forceinline__ double f64_any(float v) {
+    const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xffu;
+    if (e - 1u < 254u)
+        return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)),
+                                (int)(b << 29));
+    return b << 1 ? (double)v : 0.0;
+}
+__device__ __forceinline__ double f64_of(float v) {
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
 // x^(-1/3) of a positive double: an FP32 reciprocal-cube-root seed refined by
 // two Newton-Raphson steps for z^-3 = x in FP64, z <- z + z (1 - x z^3) / 3
 // (quadratic convergence, no division: ~1e-7 -> ~1e-14 -> rounding).  Values
 // outside the FP32 seed's comfortable range take 1 / cbrt(x).
 __device__ __forceinline__ double inv_cbrt(double x) {
-    const float xf = (float)x;
-    if (!(xf > 1e-30f && xf < 1e30f)) return 1.0 / cbrt(x);
-    double z = (double)rcbrtf(xf);
+    if (!f32_range(x)) return 1.0 / cbrt(x);
+    double z = f64_of(rcbrtf(f32_trunc(x)));
     constexpr double third = 1.0 / 3.0;
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
@@ -281,6 +367,39 @@ __device__ __forceinline__ double inv_cbrt(double x) {
         z = fma(z * third, e, z);
     }
     return z;
+}
+
+// sqrt(x), x >= 0, in six FP64 instructions (CUDA's takes nine): Goldschmidt's
+// coupled iteration for sqrt(x) and 1 / (2 sqrt(x)) from an FP32 seed, then one
+// Newton correction of the root (within 1 ulp).  Values outside the FP32
+// seed's comfortable range, 0 and NaN among them, take sqrt itself.
+__device__ __forceinline__ double sqrt_fast(double x) {
+    if (!f32_range(x)) return sqrt(x);
+    const double y = f64_of(rsqrtf(f32_trunc(x)));
+    double s = x * y;
+    double h = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y)); // y / 2
+    const double r = fma(-s, h, 0.5);
+    s = fma(s, r, s);
+    h = fma(h, r, h);
+    return fma(fma(-s, s, x), h, s);
+}
+
+// 1/h and sqrt(g h) of a wet depth (h >= eps) from one root y = h^(-1/2): an
+// FP32 seed (~2^-22) and one third-order (Halley) step y (1 + e/2 + 3/8 e^2),
+// e = 1 - h y^2; then 1/h = y^2 with one Newton correction.  Ten FP64
+// instructions where a division and a square root take fifteen.
+__device__ __forceinline__ void inv_and_wave(double h, double g, double sg, double& rh, double& cw) {
+    if (!f32_range(h)) {
+        rh = 1.0 / h;
+        cw = sqrt(g * h);
+        return;
+    }
+    const double y0 = f64_of(rsqrtf(f32_trunc(h)));
+    const double e = fma(-(h * y0), y0, 1.0);
+    const double y = fma(fma(e, 0.375, 0.5), y0 * e, y0);
+    const double y2 = y * y;
+    rh = fma(fma(-h, y2, 1.0), y2, y2);
+    cw = sg * (h * y);
 }
 
 // desingularised velocity factor u = f q, Eq. velocity (T = double or float)
@@ -316,9 +435,11 @@ __device__ __forceinline__ T gamma_manning(T n, T h, T qx, T qy, T g, T eps) {
 // cbrt(1/h); below eps as vel_factor and gamma_manning
 template <typename T>
 __device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& fv, T& gam) {
-    if (h >= eps && h > T(0)) {
-        if constexpr (std::is_same<T, double>::value) {
-            if (n == 0.0) {
+    if constexpr (std::is_same<T, double>::value) {
+        // h >= eps on the bit patterns (h is not negative, eps > 0; a NaN depth
+        // stays on this branch), off the FP64 pipe
+        if (__double_as_longlong(h) >= __double_as_longlong(eps)) {
+            if (zero_bits(n)) {
                 fv = 1.0 / h;
                 gam = 0.0;
             } else {
@@ -326,10 +447,12 @@ __device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& f
                 // rounded quotient, no FP64 division); gamma ~ z^7
                 const double z = inv_cbrt(h), rh = z * z * z;
                 fv = rh;
-                gam = g * n * n * sqrt(qx * qx + qy * qy) * (rh * rh) * z;
+                gam = g * n * n * sqrt_fast(qx * qx + qy * qy) * (rh * rh) * z;
             }
             return;
         }
+    }
+    if (h >= eps && h > T(0)) {
         const T rh = T(1) / h;
         fv = rh;
         const T c3 = cbrt(rh); // h^(-1/3)
@@ -340,37 +463,71 @@ __device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& f
     }
 }
 
-// sub-grid wet depth V and wet area A of sub-cell (ia, ib) of point set `set`
-// (mode S): V = sum_k w_k max(eta + z_k, 0), A = sum_k w_k [eta + z_k > 0]
+// sub-grid wet depth V and wet area A of sub-cell (ia, ib) of point sets setx,
+// sety (mode S): V = sum_k w_k max(eta + z_k, 0), A = sum_k w_k [eta + z_k > 0].
+// The pixels are summed as integers (swdg_fixed.cuh): in FP64 a pixel costs five
+// instructions of the FP64 pipe (80 clocks per warp), here about 15 of the
+// integer pipe, and the weights enter once per row, since w_k = fy fx with fx
+// equal for all but the first and last pixel of a row.  The block exponent is
+// that of eta and the cell's largest depth (zmag: its high word; 0: found
+// here), with six bits of room for a row's sum: 2^-54 of the larger of the two,
+// half the last place of eta + z.  Not inlined: most cells never get here, and
+// the callers' code stays small.
+struct SubV {
+    double V, A;
+    bool full;
+};
+__device__ __forceinline__ long long fx_pixel(float z, int e) { return fx::from_float(z, e); }
+__device__ __forceinline__ long long fx_pixel(double z, int e) { return fx::from_double(z, e); }
 template <typename Pix>
-__device__ __forceinline__ void subgrid_S(const Pix* __restrict__ tile, const OvTab& ov, int setx,
-                                          int ia, int sety, int ib, double eta, double& V,
-                                          double& A, bool& full) {
-    const int P = ov.P;
-    const int lox = ov.lo[setx][ia], cx = ov.cnt[setx][ia];
-    const int loy = ov.lo[sety][ib], cy = ov.cnt[sety][ib];
-    double v = 0.0, a = 0.0;
-    bool f = true;
-    for (int j = 0; j < cy; ++j) {
-        const Pix* row = tile + (size_t)(loy + j) * P + lox;
-        double vr = 0.0, ar = 0.0;
-        for (int i = 0; i < cx; ++i) {
-            double dd = eta + (double)row[i];
-            if (dd > 0.0) {
-                double fx = ov.frac[setx][ia][i];
-                vr += fx * dd;
-                ar += fx;
-            } else {
-                f = false;
-            }
-        }
-        double fy = ov.frac[sety][ib][j];
-        v += fy * vr;
-        a += fy * ar;
+__device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab* __restrict__ ov,
+                                       int setx, int ia, int sety, int ib, double eta, unsigned zmag) {
+    const int P = ov->P;
+    const int lox = ov->lo[setx][ia], cx = ov->cnt[setx][ia];
+    const int loy = ov->lo[sety][ib], cy = ov->cnt[sety][ib];
+    if (fx::mag(eta) >= 0x7ff00000u) { // an infinity or a NaN reads as entirely wet or dry
+        const bool wet = eta > 0.0;
+        return {wet ? eta : 0.0, wet ? 1.0 : 0.0, wet};
     }
-    V = v;
-    A = a;
-    full = f;
+    if (zmag == 0) {
+        for (int j = 0; j < cy; ++j)
+            for (int i = 0; i < cx; ++i)
+                zmag = max(zmag, fx::mag((double)tile[(loy + j) * P + lox + i]));
+    }
+    const int es = fx::block_exp(max(zmag, fx::mag(eta))) + 6;
+    const long long E = fx::from_double(eta, es);
+    fx::Acc v, a;
+    int wet = 0;
+#pragma unroll 1
+    for (int j = 0; j < cy; ++j) {
+        const Pix* row = tile + (loy + j) * P + lox;
+        long long T = 0, first = 0, last = 0; // sums over the row, its first and last pixel
+        int c = 0, cf = 0, cl = 0;
+        for (int i = 0; i < cx; ++i) {
+            const long long D = E + fx_pixel(row[i], es);
+            const int w = D > 0;
+            const long long Dp = w ? D : 0;
+            T += Dp;
+            c += w;
+            if (i == 0) { first = Dp; cf = w; }
+            if (i == cx - 1 && i > 0) { last = Dp; cl = w; }
+        }
+        wet += c;
+        const int2 f0 = ov->ed[setx][ia][0], f1 = ov->ed[setx][ia][1], f2 = ov->ed[setx][ia][2];
+        const int2 fy = ov->ed[sety][ib][j == 0 ? 0 : j == cy - 1 ? 2 : 1];
+        fx::Acc r, q;
+        r.mac(f0, fx::split(first));
+        r.mac(f1, fx::split(T - first - last));
+        r.mac(f2, fx::split(last));
+        v.mac(fy, fx::split(r.get()));
+        constexpr long long ONE = 1ll << (fx::FB - 6); // a count of one, at exponent 1028
+        q.mac(f0, fx::split(cf * ONE));
+        q.mac(f1, fx::split((c - cf - cl) * ONE));
+        q.mac(f2, fx::split(cl * ONE));
+        a.mac(fy, fx::split(q.get()));
+    }
+    const bool full = wet == cx * cy;
+    return {fx::to_double(v.get(), es), full ? 1.0 : wet ? fx::to_double(a.get(), 1028) : 0.0, full};
 }
 
 __device__ __forceinline__ void subgrid_P(double z, double eta, double& V, double& A) {

@@ -11,10 +11,16 @@ namespace swdg {
 template <int R, typename Pix, int MODE, typename B>
 struct Launchers {
     using S = Sz<R>;
-    static constexpr size_t res_b = sizeof(double) * res_smem<R, B>();   // per warp
+    static constexpr bool F64 = sizeof(B) == sizeof(double);
+    static constexpr size_t res_b =
+        sizeof(double) * (F64 ? ResFx<R>::words * (32 / ResFx<R>::TL) : res_smem<R, B>()); // per warp
+    static auto residual_kernel() {
+        if constexpr (F64) return k_residual<R, Pix, MODE>;
+        else return k_residual_bulk<R, Pix, MODE, B>;
+    }
     static constexpr size_t begin_b = sizeof(double) * begin_smem<R>();
     // k_stage runs two cells per warp (a team of 16 lanes each)
-    static constexpr size_t stage_b = 2 * sizeof(double) * stage_smem<R>();
+    static constexpr size_t stage_b = 2 * sizeof(double) * StageFx<R>::words;
     static constexpr size_t diag_b = sizeof(double) * (2 * S::ND + 2 * S::NMP + 2 * S::NM * S::NM);
     static constexpr size_t vjp_b = sizeof(double) * vjp_smem<R>();
     static constexpr size_t svjp_b = 2 * sizeof(double) * stage_vjp_smem<R>(); // two cells per warp
@@ -24,14 +30,25 @@ struct Launchers {
 
     static void residual(const Dev& d, const Tables& tb, int buf, int stage, double c_stage,
                          int want_dt, Shape s, cudaStream_t st) {
-        k_residual<R, Pix, MODE, B><<<s.grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, tb, buf, stage,
-                                                                              c_stage, want_dt);
+        if constexpr (F64) {
+            // 32 / TL cells per warp: no more blocks than their cells
+            const int cpb = s.wpb * 32 / ResFx<R>::TL;
+            const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
+            k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage, c_stage,
+                                                                              want_dt);
+        } else {
+            k_residual_bulk<R, Pix, MODE, B><<<s.grid, 32 * s.wpb, res_b * s.wpb, st>>>(
+                d, buf, stage, c_stage, want_dt);
+        }
     }
     static void faces(const Dev& d, const Tables& tb, int buf, double c_stage, int want_dt,
                       cudaStream_t st) {
         if (d.njobs <= 0) return;
         const int64_t blocks = std::min<int64_t>((d.njobs + 255) / 256, 152 * 16);
-        k_faces<R, Pix, MODE, B><<<(int)blocks, 256, 0, st>>>(d, tb, buf, c_stage, want_dt);
+        if constexpr (F64)
+            k_faces<R, Pix, MODE><<<(int)blocks, 256, 0, st>>>(d, buf, c_stage, want_dt);
+        else
+            k_faces_bulk<R, Pix, MODE, B><<<(int)blocks, 256, 0, st>>>(d, buf, c_stage, want_dt);
     }
     static void step_begin(const Dev& d, const Tables& tb, int do_switch, Shape s, cudaStream_t st) {
         k_step_begin<R, Pix, MODE><<<s.grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, tb, do_switch);
@@ -60,17 +77,17 @@ struct Launchers {
                              const double* rbar, double* ubar, double* nbar, double* dbar,
                              int accumulate, Shape s, cudaStream_t st) {
         k_residual_vjp<R, Pix, MODE><<<s.grid, 32 * s.wpb, vjp_b * s.wpb, st>>>(
-            d, tb, u, cm, rbar, ubar, nbar, dbar, accumulate);
+            d, u, cm, rbar, ubar, nbar, dbar, accumulate);
     }
     static void stage_vjp(const Dev& d, const Tables& tb, const StageVjpArgs& a, Shape s,
                           cudaStream_t st) {
         const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
-        k_stage_vjp<R, Pix, MODE><<<grid, 32 * s.wpb, svjp_b * s.wpb, st>>>(d, tb, a);
+        k_stage_vjp<R, Pix, MODE><<<grid, 32 * s.wpb, svjp_b * s.wpb, st>>>(d, a);
     }
     static void begin_vjp(const Dev& d, const Tables& tb, const BeginVjpArgs& a, Shape s,
                           cudaStream_t st) {
-        k_begin_vjp<R, Pix, MODE><<<s.grid, 32 * s.wpb, bvjp_b * s.wpb, st>>>(d, tb, a);
+        k_begin_vjp<R, Pix, MODE><<<s.grid, 32 * s.wpb, bvjp_b * s.wpb, st>>>(d, a);
     }
     static void indicator(const Dev& d, const Tables& tb, int kind, double* eta, Shape s,
                           cudaStream_t st) {
@@ -85,7 +102,7 @@ struct Launchers {
                                     (int)(per_warp * MAXWPB)) == cudaSuccess;
     }
     static bool prepare() {
-        return opt_in(k_residual<R, Pix, MODE, B>, res_b) &&
+        return opt_in(residual_kernel(), res_b) &&
                opt_in(k_step_begin<R, Pix, MODE>, begin_b) &&
                opt_in(k_stage<R, Pix, MODE, B>, stage_b) &&
                opt_in(k_cell_diag<R, Pix, MODE>, diag_b) &&
@@ -105,7 +122,7 @@ struct Launchers {
         if (wpb < 1 || wpb > MAXWPB) return 0;
         switch (kind) {
         case KK_BEGIN: return occ(k_step_begin<R, Pix, MODE>, wpb, begin_b);
-        case KK_RESIDUAL: return occ(k_residual<R, Pix, MODE, B>, wpb, res_b);
+        case KK_RESIDUAL: return occ(residual_kernel(), wpb, res_b);
         case KK_STAGE: return occ(k_stage<R, Pix, MODE, B>, wpb, stage_b);
         default: return occ(k_cell_diag<R, Pix, MODE>, wpb, diag_b);
         }

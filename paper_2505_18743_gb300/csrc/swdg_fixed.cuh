@@ -1,0 +1,193 @@
+// swdg_fixed.cuh -- block fixed-point arithmetic of the 1D contractions.
+//
+// GB300 issues one FP64 warp instruction per SM every 16 clocks, and one
+// 32 x 32 -> 64-bit integer multiply-add (mad.wide) every 0.55 (measured:
+// 64 lanes per clock).  A contraction with a constant table is a sum of
+// products of numbers of one size, so it needs no floating point: the values
+// of one field on one cell share an exponent (the block's), each is a 61-bit
+// integer, and the sum is formed exactly by integer multiply-adds, three per
+// term.
+//
+// Format: value = X 2^(eb - 1022 - FB), |X| <= 2^FB, eb the block's biased
+// exponent (the largest IEEE exponent field among its values, so that
+// |value| < 2^(eb - 1022)).  X = hi 2^LB + lo with lo in [-2^(LB-1), 2^(LB-1)):
+// the digit pair that the multiply-adds take.  Tables are held the same way,
+// T = Tint 2^(tb - FB), where 2^tb bounds every row's sum of |T|, so a
+// contraction of |X| <= 2^FB gives |X| <= 2^FB again, with exponent eb + tb:
+// nothing overflows and no step renormalises.
+//
+// Rounding: a conversion truncates 2^-60 of the block's largest value, a
+// contraction leaves out lo lo (at most a quarter of a unit of 2^-60 per term)
+// and rounds the table to 2^-61 of its row bound: together about a unit of
+// 2^-60 of the bound of the result, against 2^-53 of each partial sum in FP64
+// arithmetic (the row bounds of two or four contractions in a row exceed the
+// values by a few bits, so the room is used).  What this gives up is relative
+// accuracy of a value far below the largest of its block, which the FP64 sum
+// of the block does not have either.
+//
+// Room: the sums hold up to 13 terms of tables whose rows together are bounded
+// by two row bounds (hi Tlo and lo Thi are below 2^59 each).
+//
+// A block that holds an infinity or a NaN takes the exponent POISON; every
+// value converted back from it is NaN.  Blocks below 2^-958 count as zero.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace swdg {
+namespace fx {
+
+constexpr int FB = 60;
+constexpr int LB = 30;
+constexpr int EMIN = 64;       // smallest block exponent: values below it shift out to 0
+constexpr int POISON = 4096;   // block exponent of a block with an infinity or a NaN
+constexpr int POISON_MIN = 3072; // any exponent derived from POISON by table exponents is above
+
+__host__ __device__ __forceinline__ int clz64(unsigned long long a) {
+#ifdef __CUDA_ARCH__
+    const unsigned h = (unsigned)(a >> 32);
+    return h ? __clz((int)h) : 32 + __clz((int)(unsigned)a);
+#else
+    return a ? __builtin_clzll(a) : 64;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned long long dbits(double v) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long b;
+    __builtin_memcpy(&b, &v, 8);
+    return b;
+#endif
+}
+__host__ __device__ __forceinline__ double bitsd(unsigned long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double v;
+    __builtin_memcpy(&v, &b, 8);
+    return v;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned fbits(float v) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(v);
+#else
+    unsigned b;
+    __builtin_memcpy(&b, &v, 4);
+    return b;
+#endif
+}
+__host__ __device__ __forceinline__ float bitsf(unsigned b) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float v;
+    __builtin_memcpy(&v, &b, 4);
+    return v;
+#endif
+}
+
+// digit pair {hi, lo} of X, |X| < 2^60.9
+__host__ __device__ __forceinline__ int2 split(long long X) {
+    int2 d;
+    d.y = (int)((unsigned)X << (32 - LB)) >> (32 - LB);
+    d.x = (int)((X + (1ll << (LB - 1))) >> LB);
+    return d;
+}
+__host__ __device__ __forceinline__ long long join(int2 d) {
+    return (long long)d.x * (1ll << LB) + d.y;
+}
+
+// exact sum of table x value products, without lo x lo
+struct Acc {
+    long long a1, a2;
+    // a2 starts at half a unit of the final shift (round to nearest)
+    __host__ __device__ __forceinline__ Acc() : a1(0), a2(1ll << (FB - LB - 1)) {}
+    __host__ __device__ __forceinline__ void mac(int2 t, int2 v) {
+        a1 += (long long)t.x * v.x;
+        a2 += (long long)t.x * v.y;
+        a2 += (long long)t.y * v.x;
+    }
+    // X of the sum: (a1 2^(2 LB) + a2 2^LB) 2^-FB
+    __host__ __device__ __forceinline__ long long get() const {
+        return (a1 << (2 * LB - FB)) + (a2 >> (FB - LB));
+    }
+};
+static_assert(2 * LB >= FB, "scale of a1");
+
+// the exponent that a double contributes to its block's (from its high word),
+// and the block's exponent from the largest of them
+__host__ __device__ __forceinline__ unsigned mag(double v) {
+    return (unsigned)(dbits(v) >> 32) & 0x7fffffffu;
+}
+__host__ __device__ __forceinline__ int block_exp(unsigned maxmag) {
+    const int e = (int)(maxmag >> 20);
+    return e == 0x7ff ? POISON : (e < EMIN ? EMIN : e);
+}
+// X of v in a block of exponent eb (truncated toward zero).  On the integer
+// pipe: the conversion instructions take 17 clocks of the FP64 pipe (measured
+// in the residual: 10 % slower with them).
+__host__ __device__ __forceinline__ long long from_double(double v, int eb) {
+    const unsigned long long b = dbits(v);
+    const int ev = (int)(b >> 52) & 0x7ff;
+    int d = eb - ev;
+    d = d < 63 ? d : 63;
+    const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << (FB - 53);
+    const long long X = (long long)(m >> d);
+    return (long long)b < 0 ? -X : X;
+}
+// the value of X in a block of exponent eb, rounded to nearest (ties away
+// from zero); below the normal range 0, above it infinity
+__host__ __device__ __forceinline__ double to_double(long long X, int eb) {
+    const unsigned long long sign = (unsigned long long)X & 0x8000000000000000ull;
+    const unsigned long long a = (unsigned long long)(X < 0 ? -X : X);
+    const int lz = clz64(a);
+    const unsigned long long m = a << (lz & 63); // leading bit at 63
+    const int E = eb + (64 - FB) - lz;           // biased exponent of the result
+    unsigned long long r = ((unsigned long long)(unsigned)(E - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    if ((unsigned)(eb - 128) < 1792u) // every result is in the normal range
+        return bitsd(a == 0 ? 0ull : r | sign);
+    if (a == 0 || E <= 0) r = 0ull;
+    if (E >= 2047) r = 0x7ff0000000000000ull;
+    if (eb >= POISON_MIN) r = 0x7ff8000000000000ull;
+    return bitsd(r | sign);
+}
+// product of two block values: X of exponent product_exp(e1, e2)
+__host__ __device__ __forceinline__ long long product(int2 a, int2 b) {
+    Acc s;
+    s.mac(a, b);
+    return s.get();
+}
+__host__ __device__ __forceinline__ int product_exp(int e1, int e2) { return e1 + e2 - 1022; }
+
+// the same for FP32 values: the block exponent (in the double's bias) from the
+// largest bit pattern of the magnitudes, X of a value, the value of an X
+// (FP32 subnormals count as zero)
+__host__ __device__ __forceinline__ int block_exp_f(unsigned maxbits) {
+    const int e = (int)(maxbits >> 23);
+    return e == 0xff ? POISON : e + 896;
+}
+__host__ __device__ __forceinline__ long long from_float(float v, int eb) {
+    const unsigned b = fbits(v);
+    const int ef = (int)(b >> 23) & 0xff;
+    int d = eb - (ef + 896);
+    d = ef == 0 ? 63 : (d < 63 ? d : 63);
+    const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (FB - 24);
+    const long long X = (long long)(m >> d);
+    return (int)b < 0 ? -X : X;
+}
+__host__ __device__ __forceinline__ float to_float(long long X, int eb) {
+    const unsigned long long a = (unsigned long long)(X < 0 ? -X : X);
+    const int lz = clz64(a);
+    const unsigned long long m = a << (lz & 63);
+    const int E = eb + (64 - FB) - lz - 896;
+    unsigned r = ((unsigned)(E - 1) << 23) + (unsigned)(m >> 40) + ((unsigned)(m >> 39) & 1u);
+    if (a == 0 || E <= 0) r = 0u;
+    if (E >= 255) r = 0x7f800000u;
+    if (eb >= POISON_MIN) r = 0x7fc00000u;
+    return bitsf(r | ((unsigned)((unsigned long long)X >> 32) & 0x80000000u));
+}
+
+} // namespace fx
+} // namespace swdg

@@ -167,6 +167,41 @@ __device__ __forceinline__ void kron_apply2(const E (*M)[LD], const E* in0, cons
     __syncwarp(tm);
 }
 
+// The same contractions in block fixed point (swdg_fixed.cuh): T (NO x NI, by
+// rows) applied along both directions of NI x NI digit pairs; f(it, i, X) takes
+// the result at output i = q1 NO + q0 = lane + it TL, whose exponent is the
+// input's plus twice the table's.  tmp: NI NO digit pairs.
+template <int NI, int NO, int TL, int LD, typename F>
+__device__ __forceinline__ void fx_tens(const int2 (*T)[LD], const int2* in, int2* tmp, int lane,
+                                        unsigned tm, F f) {
+    constexpr int M1 = NI * NO, M2 = NO * NO;
+#pragma unroll
+    for (int it = 0; it < (M1 + TL - 1) / TL; ++it) {
+        const int i = lane + it * TL, b = i / NO, q0 = i % NO;
+        if (i < M1) {
+            fx::Acc s;
+#pragma unroll
+            for (int a = 0; a < NI; ++a) s.mac(T[q0][a], in[b * NI + a]);
+            tmp[i] = fx::split(s.get());
+        }
+    }
+    __syncwarp(tm);
+#pragma unroll
+    for (int it = 0; it < (M2 + TL - 1) / TL; ++it) {
+        const int i = lane + it * TL, q1 = i / NO, q0 = i % NO;
+        if (i < M2) {
+            fx::Acc s;
+#pragma unroll
+            for (int b = 0; b < NI; ++b) s.mac(T[q1][b], tmp[b * NO + q0]);
+            f(it, i, s.get());
+        }
+    }
+}
+// the block exponent of one value per lane of a team
+__device__ __forceinline__ int team_exp(double v, unsigned tm) {
+    return fx::block_exp(__reduce_max_sync(tm, fx::mag(v)));
+}
+
 // ---------------------------------------------------------------------------
 // bathymetry sampling sites
 // ---------------------------------------------------------------------------
@@ -184,6 +219,10 @@ struct Site {
     }
     static __device__ __forceinline__ const Pix* tile(const Dev& d, const OvTab& o, int64_t k) {
         return (const Pix*)d.tiles + (d.tile_off ? d.tile_off[k] : (int64_t)k * o.P * o.P);
+    }
+    // high word of the cell's largest depth magnitude (0: unknown)
+    static __device__ __forceinline__ unsigned zmag(const Dev& d, int64_t k) {
+        return d.zabs ? fx::mag(d.zabs[k]) : 0u;
     }
     // mode S: a cell entirely wet (eta > -min z_b) gives V = eta + the sub-cell
     // mean depth and A = 1; entirely dry (eta <= -max z_b) gives V = A = 0;
@@ -236,7 +275,10 @@ struct Site {
                 }
             }
             const OvTab& o = tab(d, k);
-            subgrid_S<Pix>(tile(d, o, k), o, set, ia, set, ib, eta, V, A, full);
+            const SubV r = subgrid_S<Pix>(tile(d, o, k), &o, set, ia, set, ib, eta, zmag(d, k));
+            V = r.V;
+            A = r.A;
+            full = r.full;
         } else {
             subgrid_P(d.zpts[(size_t)k * S::NZP + offset(set) + ia + count(set) * ib], eta, V, A);
             full = A > 0.0;
@@ -257,13 +299,11 @@ struct Site {
             bool full;
             if (shortcut(d, k, eta, zh, V, A, full)) return;
             const OvTab& o = tab(d, k);
-            const int m = (f == 0 || f == 2) ? 0 : S::NM - 1;
-            if (f < 2)
-                subgrid_S<Pix>(tile(d, o, k), o, SET_MASS, m, SET_HALF, h * S::NM + al, eta, V, A,
-                               full);
-            else
-                subgrid_S<Pix>(tile(d, o, k), o, SET_HALF, h * S::NM + al, SET_MASS, m, eta, V, A,
-                               full);
+            const int m = (f == 0 || f == 2) ? 0 : S::NM - 1, t = h * S::NM + al;
+            const SubV r = subgrid_S<Pix>(tile(d, o, k), &o, f < 2 ? SET_MASS : SET_HALF, f < 2 ? m : t,
+                                          f < 2 ? SET_HALF : SET_MASS, f < 2 ? t : m, eta, zmag(d, k));
+            V = r.V;
+            A = r.A;
         } else {
             subgrid_P(zh, eta, V, A);
         }
@@ -432,7 +472,7 @@ __device__ __forceinline__ const B (*tab_or(const double (*d)[MXN], const float 
 // boundary point returns k's final flux in raw (bnd = true, nb = -1).  lam is
 // the wave speed bound of the point.
 template <int R, typename Pix, int MODE, typename B>
-__device__ __forceinline__ void face_point(const Dev& d, const Tables& tb, int64_t k, const double* uk,
+__device__ __forceinline__ void face_point(const Dev& d, const FaceTables& tb, int64_t k, const double* uk,
                                            const float* ukF, size_t ustride, unsigned cm, int buf,
                                            int f, int h, int al,
                                            unsigned info, double hx, double hy, int mem, double t,
@@ -457,7 +497,7 @@ __device__ __forceinline__ void face_point(const Dev& d, const Tables& tb, int64
     auto own_V = [&](double eta) {
         double V, A;
         if (coarse) ST::VA_half(d, k, f, h, al, eta, V, A);
-        else ST::VA(d, tb, k, SET_MASS, ia, ib, eta, V, A);
+        else ST::VA(d, *d.tabs, k, SET_MASS, ia, ib, eta, V, A);
         return V;
     };
     const int32_t s0 = d.nbr[k * 8 + f * 2];
@@ -476,7 +516,7 @@ __device__ __forceinline__ void face_point(const Dev& d, const Tables& tb, int64
         auto nb_V = [&](double eta) {
             double V, A;
             if (fine) ST::VA_half(d, nb, fo, half, al, eta, V, A);
-            else ST::VA(d, tb, nb, SET_MASS, ja, jb, eta, V, A);
+            else ST::VA(d, *d.tabs, nb, SET_MASS, ja, jb, eta, V, A);
             return V;
         };
         hp = nb_V(zp);
@@ -519,6 +559,150 @@ __device__ __forceinline__ void face_point(const Dev& d, const Tables& tb, int64
     }
 }
 
+// One face point in FP64 (Sec. 3.2), as face_point below evaluates it for the
+// FP32-bulk path, in the face's own frame: faces are axis-aligned, so the
+// fluxes have an axis and a tangential component, normals are signs (applied to
+// the sign bit) and one evaluation serves interior and boundary points.  flux =
+// {F, G axis, G tangential, R} outward from side A (the lower cell index), pr
+// the pressure vector's axis component g {{h*}} (h*A - h*B)/2 n_A, lam the wave
+// speed bound.  uk: the cell's fields, ustride apart; Bm, BmH: the face basis.
+__device__ __forceinline__ double flip(double v, unsigned sign) { // sign: 0 or 0x80000000
+    return __hiloint2double(__double2hiint(v) ^ (int)sign, __double2loint(v));
+}
+// the smaller of two depths, on the bit patterns (they are not negative)
+__device__ __forceinline__ double min_nonneg(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
+// velocity factor and wave speed sqrt(g h) of a depth, as vel_factor below eps
+__device__ __forceinline__ void vel_wave(double h, double g, double sg, double eps, double& f, double& w) {
+    if (__double_as_longlong(h) >= __double_as_longlong(eps)) {
+        inv_and_wave(h, g, sg, f, w);
+    } else {
+        f = vel_factor<double>(h, eps);
+        w = h > 0.0 ? sqrt(g * h) : 0.0;
+    }
+}
+struct FaceFlux {
+    double flux[4], pr, lam;
+    bool own_first, bnd;
+    int64_t nb;
+};
+template <int ND1>
+__device__ __forceinline__ void face_trace_axis(const double* u, size_t fstride, unsigned cm, int f,
+                                                const double* B, double t[4]) {
+    const int base = f == 1 ? ND1 - 1 : f == 3 ? ND1 * (ND1 - 1) : 0, st = f < 2 ? ND1 : 1;
+    double b[ND1];
+#pragma unroll
+    for (int j = 0; j < ND1; ++j) b[j] = B[j];
+#pragma unroll
+    for (int fl = 0; fl < 4; ++fl) {
+        const double* uf = u + fl * fstride + base;
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < ND1; ++j) s += b[j] * uf[j * st];
+        t[fl] = (cm & (1u << fl)) ? uf[0] : s;
+    }
+}
+template <int R, typename Pix, int MODE>
+__device__ __forceinline__ FaceFlux face_flux(const Dev& d, const FaceTables& ft, int64_t k,
+                                              const double* uk, size_t ustride, unsigned cm, int buf,
+                                              int f, int h, int al, unsigned info, int mem,
+                                              double c_stage) {
+    using S = Sz<R>;
+    using ST = Site<R, Pix, MODE>;
+    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM;
+    const int64_t n = d.n;
+    const bool coarse = (info & 3) == FI_COARSE, fine = (info & 3) == FI_FINE;
+    const int half = (int)(info >> 2), ax = f >> 1;
+    FaceFlux out;
+    const int32_t s0 = d.nbr[k * 8 + f * 2];
+    out.bnd = s0 < 0;
+    // a boundary's ghost takes the own cell's sub-grid operator
+    const int64_t nb = out.bnd ? k : coarse && h ? (int64_t)d.nbr[k * 8 + f * 2 + 1] : (int64_t)s0;
+    const int fo = out.bnd ? f : f ^ 1;
+    out.nb = out.bnd ? -1 : nb;
+    out.own_first = out.bnd || k < nb;
+    double tm[4], tp[4];
+    face_trace_axis<ND1>(uk, ustride, cm, f, coarse ? ft.BmH[h][al] : ft.Bm[al], tm);
+    if (!out.bnd) {
+        face_trace_axis<ND1>(ufield(d, buf, 0, ND) + nb * ND, (size_t)n * ND,
+                             d.cmask[(size_t)buf * n + nb], fo, fine ? ft.BmH[half][al] : ft.Bm[al], tp);
+    } else {
+        const int tag = -1 - s0;
+#pragma unroll
+        for (int fl = 0; fl < 4; ++fl) tp[fl] = tm[fl];
+        const bool tide = d.mbc ? d.mbc[mem].kind[tag] == 1 : d.bc_kind[tag] == 1;
+        if (tide) {
+            const double t = (c_stage == 0.0) ? d.mb[mem].t : d.mb[mem].t + c_stage * get_dt(d, mem);
+            const double amp = d.mbc ? d.mbc[mem].amp[tag] : d.bc_amp[tag];
+            const double per = d.mbc ? d.mbc[mem].per[tag] : d.bc_per[tag];
+            const double ph = d.mbc ? d.mbc[mem].ph[tag] : d.bc_ph[tag];
+            tp[0] = amp * sin(2.0 * M_PI * t / per + ph);
+        } else { // mirrored: the normal discharge changes sign
+            if (ax == 0) tp[1] = -tm[1];
+            else tp[2] = -tm[2];
+        }
+    }
+    // the sub-grid depths of both sides at both elevations, side by side in a loop
+    // (one copy of the sampling code): hm, hp each side's own, hx V+(zeta-),
+    // hy V-(zeta+)
+    double hm = 0.0, hp = 0.0, hx = 0.0, hy = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < (out.bnd ? 1 : 2); ++s) {
+        const int64_t kc = s ? nb : k;
+        const int fc = s ? fo : f;
+        double Vm, Vp, A;
+        if (s ? fine : coarse) {
+            ST::VA_half(d, kc, fc, s ? half : h, al, tm[0], Vm, A);
+            ST::VA_half(d, kc, fc, s ? half : h, al, tp[0], Vp, A);
+        } else {
+            int ia, ib;
+            face_site_index<NM>(fc, al, ia, ib);
+            ST::VA(d, *d.tabs, kc, SET_MASS, ia, ib, tm[0], Vm, A);
+            ST::VA(d, *d.tabs, kc, SET_MASS, ia, ib, tp[0], Vp, A);
+        }
+        if (s == 0) { hm = Vm; hy = Vp; }
+        else { hx = Vm; hp = Vp; }
+    }
+    // h*- = min(V-(zeta-), V+(zeta-)), h*+ = min(V+(zeta+), V-(zeta+)); a boundary's
+    // ghost has the own operator
+    double hsm, hsp;
+    if (out.bnd) { hp = hy; hsm = hm; hsp = hp; }
+    else { hsm = min_nonneg(hm, hx); hsp = min_nonneg(hp, hy); }
+    const bool of = out.own_first;
+    const double qnm = ax ? tm[2] : tm[1], qtm = ax ? tm[1] : tm[2];
+    const double qnp = ax ? tp[2] : tp[1], qtp = ax ? tp[1] : tp[2];
+    const double hA = of ? hm : hp, hB = of ? hp : hm, hsA = of ? hsm : hsp, hsB = of ? hsp : hsm;
+    const double cA = of ? tm[3] : tp[3], cB = of ? tp[3] : tm[3];
+    const unsigned sA = ((f & 1) != 0) == of ? 0u : 0x80000000u; // sign of A's outward normal
+    double fA, fB, wA, wB;
+    vel_wave(hA, d.g, d.sg, d.eps, fA, wA);
+    vel_wave(hB, d.g, d.sg, d.eps, fB, wB);
+    const double vA = fA * (of ? qnm : qnp), uA = fA * (of ? qtm : qtp);
+    const double vB = fB * (of ? qnp : qnm), uB = fB * (of ? qtp : qtm);
+    const double lA = fabs(vA) + wA, lB = fabs(vB) + wB;
+    const double lam = __double_as_longlong(lA) > __double_as_longlong(lB) ? lA : lB;
+    const double hl = 0.5 * lam, dh = hsA - hsB;
+    const double qsA = hsA * vA, qsB = hsB * vB, rsA = hsA * uA, rsB = hsB * uB;
+    out.flux[0] = fma(hl, dh, flip(0.5 * (qsA + qsB), sA));
+    out.flux[1] = fma(hl, qsA - qsB, flip(0.5 * fma(qsA, vA, qsB * vB), sA));
+    out.flux[2] = fma(hl, rsA - rsB, flip(0.5 * fma(rsA, vA, rsB * vB), sA));
+    out.flux[3] = fma(hl, fma(dh, cA, hsB * (cA - cB)), flip(0.5 * fma(qsA, cA, qsB * cB), sA));
+    out.pr = flip(0.25 * d.g * (hsA + hsB) * dh, sA);
+    out.lam = lam;
+    return out;
+}
+// the four flux components (F, G_x, G_y, R) of a face flux seen from its own
+// cell or (other) from the neighbour, times the weight w
+__device__ __forceinline__ void side_values(const FaceFlux& q, int f, bool other, double w, double (&o)[4]) {
+    const unsigned sg = q.own_first != other ? 0u : 0x80000000u;
+    const double a = w * (flip(q.flux[1], sg) - q.pr), t = w * flip(q.flux[2], sg);
+    o[0] = w * flip(q.flux[0], sg);
+    o[1] = f < 2 ? a : t;
+    o[2] = f < 2 ? t : a;
+    o[3] = w * flip(q.flux[3], sg);
+}
+
 // the flux of an interior face point as seen from the cell whose face f it
 // is: the canonical flux with the sign of that side, and the pressure vector
 // g {{h*}} (h*A - h*B)/2 n_A, which is the same for both sides
@@ -535,23 +719,334 @@ __device__ __forceinline__ void side_flux(const B raw[4], B pres, bool own_first
     out[3] = raw[3] * sg;
 }
 
+// The FP64 residual.  What bounds it is the FP64 pipe (one warp instruction
+// per SM and 16 clocks, however few lanes are active), so only the pointwise
+// physics runs there: every contraction is block fixed-point on the integer
+// pipe (swdg_fixed.cuh), nodal values and point values being converted on the
+// integer pipe too.  A team of TL lanes takes a cell, one volume point per
+// lane: 32 lanes at r = 3 (25 points), 16 at r = 2 (16 points), 8 at r = 1
+// (4 points), so that the FP64 instructions of the points serve 1, 2 or 4
+// cells at once.  The per-point values carry the geometric factors of their
+// test integral (h_y for d/dxi, h_x for d/deta, J for values), the test tables
+// the quadrature weights, so the parts of one residual component share a block
+// exponent and are summed as integers.
+template <int R>
+struct ResFx {
+    using S = Sz<R>;
+    static constexpr int TL = R == 3 ? 32 : (R == 2 ? 16 : 8);
+    static constexpr int SUB = R == 1 ? 4 : 16; // lanes that load one field
+    static constexpr int FPP = TL / SUB;        // fields loaded at once
+    static constexpr int NE = S::ND1 * S::NV;
+    // 8-byte words per team, two regions: nodal digits and x-contractions, then
+    // the y-test sums; point values, then the face values (with the nodal values
+    // where the faces are integrated inline)
+    static constexpr int UD = 4 * S::ND, TX = 6 * NE, XP = 12 * S::NVP, SY = 10 * NE,
+                         FD = 32 * S::NM;
+    static constexpr int RA = UD + TX > SY ? UD + TX : SY, RB = XP > FD + UD ? XP : FD + UD;
+    static constexpr int words = RA + RB + 4;
+    static_assert(S::NVP <= TL && S::ND <= SUB, "one point per lane");
+};
+
+template <int R, typename Pix, int MODE>
+#ifndef RES_REGS
+#define RES_REGS 80
+#endif
+__global__ void __maxnreg__(RES_REGS)
+    k_residual(const __grid_constant__ Dev d, int buf, int stage, double c_stage, int want_dt) {
+    // the tables in shared memory: the contractions index them by lane, which
+    // the constant cache would serialise
+    __shared__ FxTables tx;
+    copy_table(tx, &d.tabs->fx);
+    const Tables& tb = *d.tabs;
+    using S = Sz<R>;
+    using L = ResFx<R>;
+    using ST = Site<R, Pix, MODE>;
+    constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP, NM = S::NM, NE = L::NE;
+    constexpr int TL = L::TL;
+    extern __shared__ double smem[];
+    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
+    const unsigned tm =
+        TL == 32 ? 0xffffffffu : ((1u << (TL & 31)) - 1u) << (threadIdx.x & 31 & ~(TL - 1));
+    int2* ud = (int2*)(smem + team * L::words); // [4][ND]
+    int2* sx = ud + L::UD;                      // [6][ND1][NV]: zeta (Bv, Dv), qx, qy, c (Bv), c (Dv)
+    int2* sy = ud;                              // [10][NV][ND1]
+    int2* xp = ud + L::RA;                      // [12][NVP]
+    int2* fd = xp;                              // [4 fields][2 halves][4 faces][NM]
+    double* c0 = (double*)(xp + L::RB);         // [4] first nodal value of each field
+    double* fh = (double*)fd;                   // the face values before their conversion
+    double* su = fh + L::FD;                    // [4][ND] (inline faces only)
+    const double g = d.g, eps = d.eps;
+    const int64_t n = d.n;
+    const int tBB = 2 * tx.tBv, tBD = tx.tBv + tx.tDv, tW = tx.tWB + tx.tWD;
+    // the lane's volume point (idle lanes take point 0 and store nothing)
+    const bool pt = lane < NVP;
+    const int pl = pt ? lane : 0, pal = pl % NV, pbe = pl / NV;
+
+    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
+        const unsigned cm = d.cmask[(size_t)buf * n + k];
+        const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1];
+        int eu[4]; // block exponents of the nodal fields
+#pragma unroll
+        for (int ps = 0; ps < 4 / L::FPP; ++ps) {
+            const int sub = lane / L::SUB, f = ps * L::FPP + sub, node = lane % L::SUB;
+            const double v = node < ND ? ufield(d, buf, f, ND)[k * ND + node] : 0.0;
+            int e = 0;
+#pragma unroll
+            for (int s = 0; s < L::FPP; ++s) {
+                const int eb = fx::block_exp(__reduce_max_sync(tm, sub == s ? fx::mag(v) : 0u));
+                eu[ps * L::FPP + s] = eb;
+                e = sub == s ? eb : e;
+            }
+            if (node < ND) {
+                ud[f * ND + node] = fx::split(fx::from_double(v, e));
+                if (node == 0) c0[f] = v;
+            }
+        }
+        unsigned fi[4]; // indexed by constants only (registers)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) fi[f] = d.finfo ? d.finfo[k * 4 + f] : 0;
+        const bool c_f[4] = {(fi[0] & 3) == FI_COARSE, (fi[1] & 3) == FI_COARSE,
+                             (fi[2] & 3) == FI_COARSE, (fi[3] & 3) == FI_COARSE};
+        const int nslot = (c_f[0] || c_f[1] || c_f[2] || c_f[3]) ? 8 * NM : 4 * NM;
+        __syncwarp(tm);
+        // x-contractions: zeta (value, d/dxi), qx, qy, c, and c's d/dxi for the
+        // tracer numerical diffusion (Eq. numdiff)
+        const double nu = d.nu_c ? d.nu_c[k] : 0.0;
+        for (int i = lane; i < (nu != 0.0 ? 6 : 5) * NE; i += TL) {
+            const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
+            const int2* T = (f == 1 || f == 5) ? tx.Dv[al] : tx.Bv[al];
+            const int2* u = ud + (f < 2 ? 0 : f < 5 ? f - 1 : 3) * ND + ND1 * b;
+            fx::Acc s;
+#pragma unroll
+            for (int a = 0; a < ND1; ++a) s.mac(T[a], u[a]);
+            sx[i] = fx::split(s.get());
+        }
+        __syncwarp(tm);
+        // y-contraction and pointwise physics, one volume point per lane
+        int ex[5]; // block exponents of F, R, Gx, Gy, L
+        {
+            double X[12];
+            {
+                fx::Acc az, azx, azy, aqx, aqy, ac;
+#pragma unroll
+                for (int b = 0; b < ND1; ++b) {
+                    const int2 Tb = tx.Bv[pbe][b], Td = tx.Dv[pbe][b];
+                    const int2* s = sx + b * NV + pal;
+                    az.mac(Tb, s[0]);
+                    azy.mac(Td, s[0]);
+                    azx.mac(Tb, s[NE]);
+                    aqx.mac(Tb, s[2 * NE]);
+                    aqy.mac(Tb, s[3 * NE]);
+                    ac.mac(Tb, s[4 * NE]);
+                }
+                // a constant field is that constant exactly
+                const double z = (cm & 1u) ? c0[0] : fx::to_double(az.get(), eu[0] + tBB);
+                const double zx = (cm & 1u) ? 0.0 : fx::to_double(azx.get(), eu[0] + tBD);
+                const double zy = (cm & 1u) ? 0.0 : fx::to_double(azy.get(), eu[0] + tBD);
+                const double qx = (cm & 2u) ? c0[1] : fx::to_double(aqx.get(), eu[1] + tBB);
+                const double qy = (cm & 4u) ? c0[2] : fx::to_double(aqy.get(), eu[2] + tBB);
+                const double c = (cm & 8u) ? c0[3] : fx::to_double(ac.get(), eu[3] + tBB);
+                double h = 0.0, A;
+                if (pt) ST::VA(d, tb, k, SET_VOL, pal, pbe, z, h, A);
+                double fv, gam;
+                vel_gamma<double>(d.manning[k], h, qx, qy, g, eps, fv, gam);
+                const double ux = fv * qx, uy = fv * qy;
+                X[0] = hy * qx;
+                X[1] = hx * qy;
+                X[2] = c * X[0];
+                X[3] = c * X[1];
+                if (nu != 0.0 && !(cm & 8u)) {
+                    // -nu h grad c . grad psi: the reference derivatives of c at the point
+                    fx::Acc acx, acy;
+#pragma unroll
+                    for (int b = 0; b < ND1; ++b) {
+                        acx.mac(tx.Bv[pbe][b], sx[(5 * ND1 + b) * NV + pal]);
+                        acy.mac(tx.Dv[pbe][b], sx[(4 * ND1 + b) * NV + pal]);
+                    }
+                    X[2] -= nu * h * fx::to_double(acx.get(), eu[3] + tBD) * (hy / hx);
+                    X[3] -= nu * h * fx::to_double(acy.get(), eu[3] + tBD) * (hx / hy);
+                }
+                const double gh = g * h, gJ = gam * (hx * hy);
+                X[4] = X[0] * ux; // Gx: h_y qx ux, h_x qx uy (= qy ux), -J g h zeta_x
+                X[5] = X[1] * ux;
+                X[6] = -(gh * hy) * zx;
+                X[7] = X[0] * uy; // Gy
+                X[8] = X[1] * uy;
+                X[9] = -(gh * hx) * zy;
+                X[10] = -gJ * qx; // Lx, Ly
+                X[11] = -gJ * qy;
+            }
+            unsigned m[5];
+            m[0] = max(fx::mag(X[0]), fx::mag(X[1]));
+            m[1] = max(fx::mag(X[2]), fx::mag(X[3]));
+            m[2] = max(max(fx::mag(X[4]), fx::mag(X[5])), fx::mag(X[6]));
+            m[3] = max(max(fx::mag(X[7]), fx::mag(X[8])), fx::mag(X[9]));
+            m[4] = max(fx::mag(X[10]), fx::mag(X[11]));
+#pragma unroll
+            for (int j = 0; j < 5; ++j) ex[j] = fx::block_exp(__reduce_max_sync(tm, pt ? m[j] : 0u));
+            if (pt) {
+#pragma unroll
+                for (int j = 0; j < 12; ++j)
+                    xp[j * NVP + pl] = fx::split(
+                        fx::from_double(X[j], ex[j < 2 ? 0 : j < 4 ? 1 : j < 7 ? 2 : j < 10 ? 3 : 4]));
+            }
+        }
+        __syncwarp(tm);
+        // the face fluxes of k_faces, loaded here (the first halves) so that the
+        // y-contraction hides the latency; slot i = (half, face, point), 0 where a
+        // face has no second half
+        constexpr int SL = (4 * NM + TL - 1) / TL;
+        auto slot = [&](int cf, int i) -> double {
+            const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
+            const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
+            if (i >= nslot || !own) return 0.0;
+            return d.fflux ? d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al]
+                           : fh[cf * 8 * NM + i];
+        };
+        double fv[SL][4];
+        if (d.fflux) {
+#pragma unroll
+            for (int j = 0; j < SL; ++j)
+#pragma unroll
+                for (int cf = 0; cf < 4; ++cf) fv[j][cf] = slot(cf, lane + j * TL);
+        }
+        // test integration, y-contraction: jobs 0, 1 the x-parts of F and R, 2, 3
+        // their y-parts, 4, 5 the x-parts of Gx and Gy, 6, 7 Lx and Ly; then 8, 9
+        // the y- and value parts of Gx and Gy
+        for (int i = lane; i < 8 * NE; i += TL) {
+            const int job = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
+            const int2* T = (job == 2 || job == 3) ? tx.WD[b] : tx.WB[b];
+            const int2* X = xp + ((0xBA743120u >> (4 * job)) & 15u) * NVP + al;
+            fx::Acc s;
+#pragma unroll
+            for (int be = 0; be < NV; ++be) s.mac(T[be], X[NV * be]);
+            sy[i] = fx::split(s.get());
+        }
+        for (int i = lane; i < 2 * NE; i += TL) {
+            const int cg = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
+            const int2* X = xp + (5 + 3 * cg) * NVP + al;
+            fx::Acc s;
+#pragma unroll
+            for (int be = 0; be < NV; ++be) {
+                s.mac(tx.WD[b][be], X[NV * be]);
+                s.mac(tx.WDB[b][be], X[NVP + NV * be]);
+            }
+            sy[8 * NE + i] = fx::split(s.get());
+        }
+        __syncwarp(tm);
+        if (!d.fflux) {
+            // the allocation-free entry: the cell's faces here, one (sub)face
+            // point per lane; the face points of faces 0..3 start at 0, b1, b2,
+            // b3 (2 NM points on a coarse 2:1 face, else NM)
+            const int mem = member_of(d, k);
+            const double ihx = d.ihxhy ? d.ihxhy[2 * k] : 1.0 / hx;
+            const double ihy = d.ihxhy ? d.ihxhy[2 * k + 1] : 1.0 / hy;
+            for (int i = lane; i < 4 * ND; i += TL)
+                su[i] = ufield(d, buf, i / ND, ND)[k * ND + (i % ND)];
+            __syncwarp(tm);
+            double dtl = 0.0;
+            const int b1 = c_f[0] ? 2 * NM : NM, b2 = b1 + (c_f[1] ? 2 * NM : NM),
+                      b3 = b2 + (c_f[2] ? 2 * NM : NM), b4 = b3 + (c_f[3] ? 2 * NM : NM);
+            for (int it = lane; it < b4; it += TL) {
+                const int f = (it >= b1) + (it >= b2) + (it >= b3);
+                const int r_ = it - (f == 0 ? 0 : f == 1 ? b1 : f == 2 ? b2 : b3), h = r_ / NM,
+                          al = r_ % NM;
+                const unsigned info = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
+                const bool coarse = (info & 3) == FI_COARSE;
+                const FaceFlux q = face_flux<R, Pix, MODE>(d, d.tabs->ft, k, su, ND, cm, buf, f, h, al,
+                                                           info, mem, c_stage);
+                double out[4];
+                side_values(q, f, false, ((f < 2) ? hy : hx) * (coarse ? 0.5 : 1.0) * d.tabs->ft.wm[al],
+                            out);
+#pragma unroll
+                for (int cf = 0; cf < 4; ++cf) fh[((cf * 2 + h) * 4 + f) * NM + al] = out[cf];
+                // lambda l / J for the positivity step (l = L, J = hx hy)
+                dtl = fmax(dtl, fmax(q.lam, 1e-12) * ((f < 2) ? ihx : ihy) * (coarse ? 0.5 : 1.0));
+            }
+            if (want_dt) {
+                const double m = team_max_nonneg(dtl, tm);
+                if (lane == 0) atomic_max_pos(&d.mb[mem].rmax, m);
+            }
+            __syncwarp(tm);
+        }
+        // the face fluxes (of k_faces, or from above) to digits, field by field
+        int ef[4];
+#pragma unroll
+        for (int cf = 0; cf < 4; ++cf) {
+            unsigned m = 0;
+#pragma unroll
+            for (int j = 0; j < SL; ++j) {
+                if (!d.fflux) fv[j][cf] = slot(cf, lane + j * TL);
+                m = max(m, fx::mag(fv[j][cf]));
+            }
+            for (int i = lane + SL * TL; i < nslot; i += TL) m = max(m, fx::mag(slot(cf, i)));
+            ef[cf] = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll
+            for (int j = 0; j < SL; ++j)
+                if (lane + j * TL < nslot)
+                    fd[cf * 8 * NM + lane + j * TL] = fx::split(fx::from_double(fv[j][cf], ef[cf]));
+            for (int i = lane + SL * TL; i < nslot; i += TL)
+                fd[cf * 8 * NM + i] = fx::split(fx::from_double(slot(cf, i), ef[cf]));
+        }
+        __syncwarp(tm);
+        // x-contraction of F, Gx, Gy, R minus the face fluxes lifted onto the
+        // nodes of their faces; a node takes part in at most one x face and one
+        // y face
+        for (int i = lane; i < 4 * ND; i += TL) {
+            const int cf = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
+            const int2* s1 = sy + ((0x1540u >> (4 * cf)) & 15u) * NE + b;
+            const int2* s2 = sy + ((0x3982u >> (4 * cf)) & 15u) * NE + b;
+            fx::Acc s;
+#pragma unroll
+            for (int al = 0; al < NV; ++al) {
+                s.mac(tx.WD[a][al], s1[al * ND1]);
+                s.mac(tx.WB[a][al], s2[al * ND1]);
+            }
+            const int e = cf == 0 ? ex[0] : cf == 1 ? ex[2] : cf == 2 ? ex[3] : ex[1];
+            const int ff = cf == 0 ? ef[0] : cf == 1 ? ef[1] : cf == 2 ? ef[2] : ef[3];
+            long long sf = 0;
+            auto lift = [&](int f, int tn, bool coarse) {
+                fx::Acc q;
+                const int2* v = fd + (cf * 8 + f) * NM;
+                if (!coarse) {
+#pragma unroll
+                    for (int al = 0; al < NM; ++al) q.mac(tx.BmT[tn][al], v[al]);
+                } else {
+#pragma unroll
+                    for (int al = 0; al < NM; ++al) {
+                        q.mac(tx.BmHT[0][tn][al], v[al]);
+                        q.mac(tx.BmHT[1][tn][al], v[4 * NM + al]);
+                    }
+                }
+                sf += q.get();
+            };
+            if (a == 0 || a == ND1 - 1) lift(a == 0 ? 0 : 1, b, a == 0 ? c_f[0] : c_f[1]);
+            if (b == 0 || b == ND1 - 1) lift(b == 0 ? 2 : 3, a, b == 0 ? c_f[2] : c_f[3]);
+            rfield(d, stage, cf, ND)[k * ND + j] =
+                fx::to_double(s.get(), e + tW) - fx::to_double(sf, ff + tx.tBmT);
+        }
+        for (int i = lane; i < 2 * ND; i += TL) { // Lx, Ly
+            const int cl = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
+            fx::Acc s;
+#pragma unroll
+            for (int al = 0; al < NV; ++al) s.mac(tx.WB[a][al], sy[(6 + cl) * NE + al * ND1 + b]);
+            rfield(d, stage, 4 + cl, ND)[k * ND + j] = fx::to_double(s.get(), ex[4] + 2 * tx.tWB);
+        }
+        __syncwarp(tm);
+    }
+}
+
 // 96 registers for the FP64 form; 80 for B = float (six blocks of four
 // warps per SM instead of five; measured 2 % faster despite a few spilled
 // registers, while the FP32-bulk stage update is slower at 80 or 72)
 template <int R, typename Pix, int MODE, typename B>
 __global__ void __maxnreg__(sizeof(B) == 4 ? 80 : 96)
-    k_residual(const __grid_constant__ Dev d, const __grid_constant__ Tables tb_g, int buf,
-               int stage, double c_stage, int want_dt) {
+    k_residual_bulk(const __grid_constant__ Dev d, int buf, int stage, double c_stage, int want_dt) {
     // the basis tables in shared memory: the contractions index them by lane
     // (a different row or column per lane), which the constant cache would
     // serialise (measured: -3 % per launch)
     __shared__ Tables s_tb;
-    {
-        const unsigned* src = (const unsigned*)&tb_g;
-        unsigned* dst = (unsigned*)&s_tb;
-        for (int i = threadIdx.x; i < (int)(sizeof(Tables) / 4); i += blockDim.x) dst[i] = src[i];
-        __syncthreads();
-    }
+    copy_table(s_tb, d.tabs);
     const Tables& tb = s_tb;
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE>;
@@ -849,52 +1344,12 @@ __global__ void __maxnreg__(sizeof(B) == 4 ? 80 : 96)
             for (int al = 0; al < NV; ++al) s += BvB[al][a] * sB[(((2 + cl) * 2 + 1) * NV + al) * ND1 + b];
             rs[(4 + cl) * ND + j] = (double)s;
         }
-        // faces: one (sub)face point per lane; a coarse cell integrates each
-        // 2:1 face over the GLL points of both fine halves
-        double dtl = 0.0;
+        // the face fluxes of this cell, computed once per face point by k_faces
         unsigned fi[4]; // indexed by constants only (registers)
 #pragma unroll
         for (int f = 0; f < 4; ++f) fi[f] = d.finfo ? d.finfo[k * 4 + f] : 0;
-        if (d.fflux) {
-            // the face fluxes of this cell, computed once per face point by k_faces
-            const double* F = d.fflux + k * (32 * NM);
-            for (int i = lane; i < 32 * NM; i += 32) fh[i] = F[i];
-        } else {
-            // the face points of faces 0..3 start at 0, b1, b2, b3 (2 NM points
-            // on a coarse 2:1 face, else NM)
-            auto npts = [&](unsigned inf) { return (((inf & 3) == FI_COARSE) ? 2 : 1) * NM; };
-            const int b1 = npts(fi[0]), b2 = b1 + npts(fi[1]), b3 = b2 + npts(fi[2]),
-                      b4 = b3 + npts(fi[3]);
-            for (int it = lane; it < b4; it += 32) {
-                const int f = (it >= b1) + (it >= b2) + (it >= b3);
-                const int r_ = it - (f == 0 ? 0 : f == 1 ? b1 : f == 2 ? b2 : b3), h = r_ / NM,
-                          al = r_ % NM;
-                const unsigned info = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
-                const bool coarse = (info & 3) == FI_COARSE;
-                B raw[4], pres, lam, out[4];
-                bool own_first, bnd;
-                int64_t nb;
-                face_point<R, Pix, MODE, B>(d, tb, k, su, nullptr, ND, cm, buf, f, h, al, info, hx, hy,
-                                            mem, t, raw, pres, lam, own_first, bnd, nb);
-                if (bnd) {
-#pragma unroll
-                    for (int cf = 0; cf < 4; ++cf) out[cf] = raw[cf];
-                } else {
-                    side_flux<B>(raw, pres, own_first, f, out);
-                }
-                const double L = ((f < 2) ? hy : hx) * (coarse ? 0.5 : 1.0);
-                const double wl = L * tb.wm[al];
-#pragma unroll
-                for (int cf = 0; cf < 4; ++cf)
-                    fh[((cf * 4 + f) * 2 + h) * NM + al] = wl * (double)out[cf];
-                // lambda l / J for the positivity step (l = L, J = hx hy)
-                dtl = fmax(dtl, fmax((double)lam, 1e-12) * ((f < 2) ? ihx : ihy) * (coarse ? 0.5 : 1.0));
-            }
-        }
-        if (want_dt && !d.fflux) {
-            const double m = warp_max(dtl);
-            if (lane == 0) atomic_max_pos(&d.mb[mem].rmax, m);
-        }
+        const double* F = d.fflux + k * (32 * NM);
+        for (int i = lane; i < 32 * NM; i += 32) fh[i] = F[i];
         __syncwarp();
         // lift the face fluxes onto the nodes of each face: one item per field,
         // face and node along it, the x faces (0, 1: node columns a = 0 and
@@ -936,10 +1391,77 @@ __global__ void __maxnreg__(sizeof(B) == 4 ? 80 : 96)
 // with want_dt the wave speed bound of each side (lambda l / J) raises its
 // member's rmax, as the residual does when it integrates the faces itself.
 // One job per lane.
+#ifndef FACE_REGS
+#define FACE_REGS 80
+#endif
+template <int R, typename Pix, int MODE>
+__global__ void __maxnreg__(FACE_REGS)
+    k_faces(const __grid_constant__ Dev d, int buf, double c_stage, int want_dt) {
+    __shared__ FaceTables ft; // its rows are indexed by lane
+    copy_table(ft, &d.tabs->ft);
+    using S = Sz<R>;
+    constexpr int ND = S::ND, NM = S::NM, SL = 32 * NM;
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t n = d.n;
+    for (int64_t j0 = gw * 32; j0 < d.njobs; j0 += nw * 32) { // warp-uniform bounds
+        const int64_t j = j0 + lane;
+        double v = 0.0;
+        int mem = -1;
+        if (j < d.njobs) {
+            const int64_t job = d.fjobs[j];
+            const int64_t k = job >> 8;
+            const int f = (int)(job & 3), h = (int)((job >> 2) & 1), al = (int)((job >> 3) & 31);
+            const unsigned info = d.finfo ? d.finfo[k * 4 + f] : 0;
+            mem = member_of(d, k);
+            const FaceFlux q =
+                face_flux<R, Pix, MODE>(d, ft, k, ufield(d, buf, 0, ND) + k * ND, (size_t)n * ND,
+                                        d.cmask[(size_t)buf * n + k], buf, f, h, al, info, mem, c_stage);
+            // max(lambda, 1e-12), a NaN counting as 1e-12
+            const long long lb = __double_as_longlong(q.lam);
+            const double lam = lb > __double_as_longlong(1e-12) && !nan_bits(q.lam) ? q.lam : 1e-12;
+            // the own side, then the other one (the fine side of a 2:1 face has one
+            // half) with its own weight; extent l_Gamma along the face, 1 / J l_Gamma
+            // across it
+#pragma unroll 1
+            for (int s = 0; s < (q.bnd || q.nb == k ? 1 : 2); ++s) {
+                const int64_t kc = s ? q.nb : k;
+                const int fc = s ? f ^ 1 : f;
+                const unsigned ci = s ? (d.finfo ? d.finfo[kc * 4 + fc] : 0) : info;
+                const int hc = s ? ((info & 3) == FI_FINE ? (int)(info >> 2) : 0) : h;
+                const double sc = (ci & 3) == FI_COARSE ? 0.5 : 1.0;
+                double out[4];
+                side_values(q, fc, s != 0, d.hxhy[2 * kc + (fc < 2 ? 1 : 0)] * sc * ft.wm[al], out);
+                double* F = d.fflux + kc * SL + (fc * 2 + hc) * NM + al;
+#pragma unroll
+                for (int cf = 0; cf < 4; ++cf) F[cf * 8 * NM] = out[cf];
+                if (want_dt) {
+                    const double ih = d.ihxhy ? d.ihxhy[2 * kc + (fc < 2 ? 0 : 1)]
+                                              : 1.0 / d.hxhy[2 * kc + (fc < 2 ? 0 : 1)];
+                    v = fmax(v, lam * ih * sc);
+                }
+            }
+        }
+        if (want_dt) {
+            // one atomic per warp when its jobs share a member, else per job
+            const int m0 = __shfl_sync(0xffffffffu, mem, 0);
+            if (__all_sync(0xffffffffu, mem == m0 || mem < 0)) {
+                const double m = team_max_nonneg(v, 0xffffffffu); // v >= 0, never NaN
+                if (lane == 0 && m0 >= 0) atomic_max_pos(&d.mb[m0].rmax, m);
+            } else if (mem >= 0) {
+                atomic_max_pos(&d.mb[mem].rmax, v);
+            }
+        }
+    }
+}
+
+// the same for the FP32-bulk path, whose fluxes are FP32 (B)
 template <int R, typename Pix, int MODE, typename B>
 __global__ void __maxnreg__(80)
-    k_faces(const __grid_constant__ Dev d, const __grid_constant__ Tables tb, int buf, double c_stage,
-            int want_dt) {
+    k_faces_bulk(const __grid_constant__ Dev d, int buf, double c_stage, int want_dt) {
+    __shared__ FaceTables tb;
+    copy_table(tb, &d.tabs->ft);
     using S = Sz<R>;
     constexpr int ND = S::ND, NM = S::NM, SL = 32 * NM;
     const int lane = threadIdx.x & 31;
@@ -1057,15 +1579,21 @@ __device__ __forceinline__ void mass_scalar_pixels(const Dev& d, const Tables& t
     const OvTab& o = ST::tab(d, k);
     const Pix* t = ST::tile(d, o, k);
     const int np = o.P * o.P;
-    double h = 0.0;
+    // the wet depths as integers, their sum in two parts (exact)
+    const int es = fx::block_exp(max(ST::zmag(d, k), fx::mag(e))) + 1;
+    const long long E = fx::from_double(e, es);
+    long long hi = 0;
+    unsigned long long lo = 0;
     int a = 0;
     for (int i = lane; i < np; i += TL) {
-        const double dd = e + (double)t[i];
-        if (dd > 0.0) {
-            h += dd;
+        const long long D = E + fx_pixel(t[i], es);
+        if (D > 0) {
+            hi += D >> 32;
+            lo += (unsigned)D;
             ++a;
         }
     }
+    const double h = fx::to_double(hi, es + 32) + fx::to_double((long long)lo, es);
     const double w = J / (double)np;
     H = w * team_sum<TL>(h, tm);
     A = w * (double)__reduce_add_sync(tm, a);
@@ -1262,28 +1790,6 @@ struct StageArgs {
     int final_;    // final combination: update time and bookkeeping
 };
 
-template <int R>
-constexpr int stage_union() {
-    // in doubles, one region for what is never live at the same time: the
-    // friction points / the momentum block's point arrays [6 NGP] with its
-    // nodal and tmp pairs (B-typed, sized in doubles); the FP32 solve's float
-    // M, Y (8-byte padded); the FP64 fallback's M [ND ND]
-    using S = Sz<R>;
-    constexpr int mom = 6 * S::NGP + 2 * S::ND + 2 * S::ND1 * S::NG;
-    constexpr int f32 = (S::ND * S::ND + S::ND1 * S::ND1 * S::NM + 1) / 2;
-    constexpr int fb = S::ND * S::ND;
-    constexpr int m = mom > f32 ? mom : f32;
-    return m > fb ? m : fb;
-}
-template <int R>
-constexpr int stage_smem() {
-    using S = Sz<R>;
-    // the FP64 fallback's Y [ND1 ND1 NM] overlays tmp, x, r (see k_stage)
-    static_assert(S::ND1 * S::ND1 * S::NM <= 2 * S::NM * S::NM + 2 * S::ND, "fallback Y");
-    return 4 * S::ND + 5 * S::ND + 3 * S::NMP + 2 * S::NM * S::NM + 2 * S::ND + 4 * S::ND +
-           stage_union<R>();
-}
-
 // Cholesky of the SPD matrix M (ND x ND, row-major, lower part used) on a
 // warp, then M x = b in place by column-oriented forward and back
 // substitution (one reciprocal per column, the updates spread over lanes);
@@ -1405,13 +1911,13 @@ __device__ __forceinline__ void chol_rows(float (&a)[ND], int i, float& rinv, bo
 // Mf (lrow_idx).  The lane's reciprocal pivot 1/L_ii comes back in rinv.
 // Returns false on a non-positive pivot.
 template <int ND1, int NM, int TL>
-__device__ bool mass_factor_rows_f(const Tables& tb, const double* cw, float* Y, float* Mf,
+__device__ bool mass_factor_rows_f(const FxStage& tb, const double* cw, float* Y, float* Mf,
                                    float& rinv, int lane, unsigned tm) {
     constexpr int ND = ND1 * ND1;
     static_assert(ND <= TL, "one row per lane");
     static_assert(NM * NM <= ND * ND, "the weights are staged in Mf");
     float* cwf = Mf; // Mf is written only once the factor is done
-    for (int p = lane; p < NM * NM; p += TL) cwf[p] = (float)cw[p];
+    for (int p = lane; p < NM * NM; p += TL) cwf[p] = f32_of(cw[p]);
     __syncwarp(tm);
     for (int i = lane; i < ND1 * ND1 * NM; i += TL) {
         const int a = i / (ND1 * NM), r_ = i % (ND1 * NM), c = r_ / NM, be = r_ % NM;
@@ -1479,72 +1985,79 @@ __device__ __forceinline__ float chol_subst_rows_f(const float* Mf, float rinv, 
 // tracer matrix of Eq. mass_matrix_concentration, or the masked Jacobian of
 // Eq. mass_matrix) by mixed-precision iterative refinement: H is assembled and
 // factored in FP32, each correction is solved in FP32, and the residual
-// b - H x is formed in FP64 matrix-free by sum factorisation.  The sweeps stop
-// when a correction, or the next one as predicted from the contraction of
-// the last two, is below 1e-15 of x; if that does not happen within 6 sweeps
-// (an ill-conditioned near-dry cell), the FP64 Cholesky decides.  x (FP64, in place of b on
-// return).  Scratch: Mf [ND ND], Yf [ND1 ND1 NM] (float), x, r (ND doubles),
-// q (NMP doubles), tmp (2 NM NM doubles), M, Y, inv (double, fallback).
+// b - H x is formed matrix-free by sum factorisation in block fixed point (60
+// bits of the largest term, on the integer pipe; in FP64 arithmetic the two
+// residuals were a third of the stage update's FP64 instructions), x being
+// held as a fixed-point number too.  The sweeps stop when a correction, or the
+// next one as predicted from the contraction of the last two, is below 1e-15
+// of x; if that does not happen within 6 sweeps (an ill-conditioned near-dry
+// cell), the FP64 Cholesky decides.  x in place of b on return.  Scratch: Mf
+// [ND ND], Yf [ND1 ND1 NM] (float), digit pairs xd [ND], qd [NMP], td [2 NMP],
+// M, Y, inv (double, fallback: Y and inv may overlay xd, qd and td).
 template <int ND1, int NM, int TL = 32>
-__device__ bool solve_mass_mixed(const Tables& tb, const double* cw, double* b, float* Mf,
-                                 float* Yf, double* x, double* r, double* q, double* tmp,
-                                 double* M, double* Y, double* inv, int lane,
-                                 unsigned tm = 0xffffffffu) {
+__device__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const double* cw, double* b,
+                                 float* Mf, float* Yf, int2* xd, int2* qd, int2* td, double* M,
+                                 double* Y, double* inv, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = ND1 * ND1, NMP = NM * NM;
     static_assert(ND <= TL, "one unknown per lane");
+    int2* cwd = td + NM * NM;
+    const double bi = lane < ND ? b[lane] : 0.0;
+    unsigned mc = 0;
+    for (int p = lane; p < NMP; p += TL) mc = max(mc, fx::mag(cw[p]));
+    const int ecw = fx::block_exp(__reduce_max_sync(tm, mc)), eb = team_exp(bi, tm);
     float rinv; // the lane's reciprocal FP32 pivot
-    bool ok = mass_factor_rows_f<ND1, NM, TL>(tb, cw, Yf, Mf, rinv, lane, tm);
+    bool ok = mass_factor_rows_f<ND1, NM, TL>(fs, cw, Yf, Mf, rinv, lane, tm);
+    long long X = 0; // the lane's component of x
+    int ex = fx::EMIN;
     if (ok) {
-        for (int i = lane; i < ND; i += TL) {
-            x[i] = 0.0;
-            r[i] = b[i];
-        }
-        __syncwarp(tm);
+        for (int p = lane; p < NMP; p += TL) cwd[p] = fx::split(fx::from_double(cw[p], ecw));
         ok = false;
-        double dprev = 0.0; // max |correction| of the previous sweep
+        float rv = fx::to_float(fx::from_double(bi, eb), eb);
+        float dprev = 0.0f; // max |correction| / max |x| of the previous sweep
         for (int sweep = 0; sweep < 6; ++sweep) {
             // the lane's component of the correction
-            const float v =
-                chol_subst_rows_f<ND, TL>(Mf, rinv, lane < ND ? (float)r[lane] : 0.0f, lane, tm);
-            // max |correction| and max |x| (a NaN counts as 0, as under fmax),
-            // reduced on their bit patterns
-            float da = 0.0f;
-            double xa = 0.0;
-            if (lane < ND) {
-                x[lane] += (double)v;
-                da = (v == v) ? fabsf(v) : 0.0f;
-                const unsigned long long xb =
-                    (unsigned long long)__double_as_longlong(x[lane]) & 0x7fffffffffffffffull;
-                xa = __longlong_as_double((long long)(xb > 0x7ff0000000000000ull ? 0ull : xb));
-            }
-            const double dmax = (double)team_max_nonneg(da, tm);
-            const double xmax = team_max_nonneg(xa, tm);
+            const float v = chol_subst_rows_f<ND, TL>(Mf, rinv, rv, lane, tm);
+            const float da = lane < ND ? fabsf(v) : 0.0f;
+            const unsigned dbits = __reduce_max_sync(tm, __float_as_uint(da)); // a NaN is the largest
+            const int ev = fx::block_exp_f(dbits);
+            if (sweep == 0) ex = ev;
+            else if (ev > ex) break; // the corrections grow: the fallback
+            X += fx::from_float(v, ex);
+            // max |x| and the ratio of the correction to it, for the stopping test
+            const unsigned xm = __reduce_max_sync(
+                tm, lane < ND ? (unsigned)((unsigned long long)(X < 0 ? -X : X) >> 31) : 0u);
+            if (xm >= 1u << (fx::FB - 30)) break; // x has outgrown its block: the fallback
+            const float dmax = __uint_as_float(dbits);
+            const float dr = dmax / fx::to_float((long long)xm << 31, ex);
             // converged when this correction is below 1e-15 of x, or when the
             // next one is, as predicted from the contraction of the last two
-            // (dmax / dprev, at most 1/2)
-            const bool next_small =
-                sweep > 0 && dmax <= 0.5 * dprev && dmax * dmax <= 1e-15 * xmax * dprev;
-            if (!(dmax <= 1e-15 * xmax) && !(dmax == 0.0) && !next_small) {
-                dprev = dmax;
-                // r = b - H x, H x = B^T (cw * (B x))
-                __syncwarp(tm);
-                tens_interp<ND1, NM, double, TL>(tb.Bm, x, tmp, q, lane, tm);
-                for (int p = lane; p < NMP; p += TL) q[p] *= cw[p];
-                __syncwarp(tm);
-                tens_test<ND1, NM, double, TL>(tb.Bm, q, tmp, r, lane, tm);
-                for (int i = lane; i < ND; i += TL) r[i] = b[i] - r[i];
-                __syncwarp(tm);
-            } else {
+            // (dr / dprev, at most 1/2)
+            const bool next_small = sweep > 0 && dr <= 0.5f * dprev && dr * dr <= 1e-15f * dprev;
+            if (dr <= 1e-15f || dmax == 0.0f || next_small || ex >= fx::POISON_MIN) {
                 ok = true;
                 break;
             }
+            dprev = dr;
+            // r = b - H x, H x = B^T (cw (B x))
+            if (lane < ND) xd[lane] = fx::split(X);
+            __syncwarp(tm);
+            fx_tens<ND1, NM, TL>(fs.Bm, xd, td, lane, tm, [&](int, int p, long long v_) {
+                qd[p] = fx::split(fx::product(fx::split(v_), cwd[p]));
+            });
+            __syncwarp(tm);
+            long long R = 0;
+            fx_tens<NM, ND1, TL>(fs.BmT, qd, td, lane, tm, [&](int, int, long long v_) { R = v_; });
+            const int er = fx::product_exp(ex + 2 * fs.tBm, ecw) + 2 * fs.tBmT, e = max(er, eb);
+            rv = lane < ND ? fx::to_float(fx::from_double(bi, e) - (R >> min(e - er, 63)), e) : 0.0f;
         }
     }
     if (ok) {
-        for (int i = lane; i < ND; i += TL) b[i] = x[i];
+        __syncwarp(tm);
+        if (lane < ND) b[lane] = fx::to_double(X, ex);
         __syncwarp(tm);
         return true;
     }
+    __syncwarp(tm);
     assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
     return chol_solve<ND, TL>(M, b, inv, lane, tm);
 }
@@ -1559,31 +2072,38 @@ __device__ bool solve_mass_mixed(const Tables& tb, const double* cw, double* b, 
 // is kept to FP64 round-off and a constant tracer (b = c s) stays constant up
 // to the rounding of b - c0 s.  A failed FP32 factor falls back to the FP64
 // Cholesky.  b: right-hand side in, C out (FP64).  Scratch: Mf, Yf (float),
-// s (ND doubles), tmp (2 NM NM doubles), M, Y, inv (fallback).  s_known: the
-// continuity target T when the Newton solve ended on its certificate (H is
-// affine between the last two iterates, so H(zeta^(l)) = T up to the
-// rounding of the last update): it stands for s = H 1 = H(zeta^(l)); null:
-// s is integrated from cw.
+// digit pairs td [2 NMP], M, Y, inv (fallback).  known: the Newton solve ended
+// on its certificate (H is affine between the last two iterates, so
+// H(zeta^(l)) = T up to the rounding of the last update) and the continuity
+// target T stands for s = H 1 = H(zeta^(l)); otherwise s is integrated from cw.
 template <int ND1, int NM, int TL>
-__device__ void solve_tracer_bulk(const Tables& tb, const double* cw, double* b, float* Mf,
-                                  float* Yf, double* s, double* tmp, double* M, double* Y,
-                                  double* inv, const double* s_known, int lane, unsigned tm) {
-    constexpr int ND = ND1 * ND1;
+__device__ void solve_tracer_bulk(const Tables& tb, const FxStage& fs, const double* cw, double* b,
+                                  float* Mf, float* Yf, int2* td, double* M, double* Y, double* inv,
+                                  bool known, double T, int lane, unsigned tm) {
+    constexpr int ND = ND1 * ND1, NMP = NM * NM;
     static_assert(ND <= TL, "one unknown per lane");
     float rinv;
-    if (!mass_factor_rows_f<ND1, NM, TL>(tb, cw, Yf, Mf, rinv, lane, tm)) {
+    if (!mass_factor_rows_f<ND1, NM, TL>(fs, cw, Yf, Mf, rinv, lane, tm)) {
         assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
         chol_solve<ND1 * ND1, TL>(M, b, inv, lane, tm);
         return;
     }
-    if (s_known == nullptr) tens_test<ND1, NM, double, TL>(tb.Bm, cw, tmp, s, lane, tm); // s_i = (H 1)_i
-    const double* sv = s_known ? s_known : s;
-    const double bi = lane < ND ? b[lane] : 0.0, si = lane < ND ? sv[lane] : 0.0;
+    if (!known) { // s_i = (H 1)_i
+        unsigned m = 0;
+        for (int p = lane; p < NMP; p += TL) m = max(m, fx::mag(cw[p]));
+        const int e = fx::block_exp(__reduce_max_sync(tm, m));
+        for (int p = lane; p < NMP; p += TL) td[p] = fx::split(fx::from_double(cw[p], e));
+        __syncwarp(tm);
+        fx_tens<NM, ND1, TL>(fs.BmT, td, td + NMP, lane, tm, [&](int, int, long long X) {
+            T = fx::to_double(X, e + 2 * fs.tBmT);
+        });
+    }
+    const double bi = lane < ND ? b[lane] : 0.0, si = lane < ND ? T : 0.0;
     double sb = bi, ss = si;
     team_sum2<TL>(sb, ss, tm);
     const double c0 = ss > 0.0 ? sb / ss : 0.0;
-    const float v = chol_subst_rows_f<ND, TL>(Mf, rinv, (float)(bi - c0 * si), lane, tm);
-    const double xi = lane < ND ? c0 + (double)v : 0.0;
+    const float v = chol_subst_rows_f<ND, TL>(Mf, rinv, f32_of(bi - c0 * si), lane, tm);
+    const double xi = lane < ND ? c0 + f64_any(v) : 0.0;
     const double m = team_sum<TL>(si * xi, tm);
     const double alpha = ss > 0.0 ? (sb - m) / ss : 0.0;
     __syncwarp(tm);
@@ -1591,183 +2111,164 @@ __device__ void solve_tracer_bulk(const Tables& tb, const double* cw, double* b,
     __syncwarp(tm);
 }
 
-// Momentum stage solve of an r_K = r cell in arithmetic T (Eq. algebraic_discharge
-// with the friction-modified mass matrix of Eq. mass_matrix_discharge on the
-// (r+1)^2 Gauss-Legendre points, inverted as S^-1 D^-1 S^-T):
-//   S Q = [D0 q^n + S^-T rq] / D,  D = D0 (1 + add dt gamma),  D0 = J w.
-// gamma (of the previous stage) is formed here from prev (zeta in FP64 for the
-// sub-grid depth, q in T).  Optionally the linearised friction term
-// Llin = -S^T (J w gamma S Q).  Inputs su (v^n, FP64), rq [2][ND] (FP64);
-// outputs Q [2][ND] (FP64) and llin [2][ND] (FP64).
-template <int R, typename Pix, int MODE, typename T, int TL = 32>
-__device__ void momentum_block(const Dev& d, const Tables& tb, int64_t k, double J, double man,
-                               double dt, double add, bool need_gam, bool make_llin, int prev_buf,
-                               const double* su, unsigned cm0, const double* rq, T* w0, T* w1,
-                               T* pts, double* zp, double* tmpd, double* Q, double* llin, int lane,
-                               unsigned tm = 0xffffffffu) {
-    using S = Sz<R>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NG = S::NG, NGP = S::NGP;
-    const auto Bg = tab_or<T>(tb.Bg, tb.BgF);
-    const T(*Bginv)[MXP] = nullptr;
-    if constexpr (sizeof(T) == sizeof(double)) Bginv = (const T(*)[MXP])tb.Bginv;
-    else Bginv = (const T(*)[MXP])tb.BginvF;
-    // w0: [2][ND] nodal pair; w1: [2][ND1 NG] tmp pair; pts: [6][NGP] point
-    // arrays.  The two discharge components are contracted side by side.
-    T* nod = w0;              // [2][ND]
-    T* pg = pts;              // [6][NGP]: 0,1 S^-T rq / point values; 2 gamma; 3,4 q^n; 5 spare
-    T* tmp = w1;
-    T* tmp1 = w1 + ND1 * NG;
-    T* gam = pg + 2 * NGP;
-    const int64_t n = d.n;
-    constexpr bool F64 = sizeof(T) == sizeof(double);
-    // per-cell values in T: for T = float converted once per team (lanes
-    // 0..4), since conversions occupy the FP64 pipe
-    T JT, manT, gT, epsT, adtT;
-    if constexpr (F64) {
-        JT = J;
-        manT = man;
-        gT = d.g;
-        epsT = d.eps;
-        adtT = add * dt;
-    } else {
-        const int q = lane < 5 ? lane : 0;
-        const float f = (float)(q == 0 ? J : q == 1 ? man : q == 2 ? d.g : q == 3 ? d.eps : add * dt);
-        JT = __shfl_sync(tm, f, 0, TL);
-        manT = __shfl_sync(tm, f, 1, TL);
-        gT = __shfl_sync(tm, f, 2, TL);
-        epsT = __shfl_sync(tm, f, 3, TL);
-        adtT = __shfl_sync(tm, f, 4, TL);
-    }
-    // the quadrature weight of momentum point p (T = float: FP32 weights)
-    auto wpt = [&](int p) -> T {
-        if constexpr (F64) return J * tb.wg[p % NG] * tb.wg[p / NG];
-        else return JT * tb.wgF[p % NG] * tb.wgF[p / NG];
-    };
-    if (need_gam) {
-        const unsigned cmp = d.cmask[(size_t)prev_buf * n + k];
-        const double* uz = ufield(d, prev_buf, 0, ND) + k * ND;
-        tens_interp<ND1, NG, double, TL>(tb.Bg, uz, tmpd, zp, lane, tm); // zeta of v^(l-1), FP64
-        if (cmp & 1u)
-            for (int p = lane; p < NGP; p += TL) zp[p] = uz[0];
-        const double* up0 = ufield(d, prev_buf, 1, ND) + k * ND;
-        const double* up1 = ufield(d, prev_buf, 2, ND) + k * ND;
-        for (int i = lane; i < 2 * ND; i += TL) nod[i] = (T)(i < ND ? up0[i] : up1[i - ND]);
-        __syncwarp(tm);
-        tens_interp2<ND1, NG, T, TL>(Bg, nod, nod + ND, tmp, tmp1, pg + 3 * NGP, pg + 4 * NGP, lane, tm);
-        if (cmp & 2u)
-            for (int p = lane; p < NGP; p += TL) pg[3 * NGP + p] = (T)up0[0];
-        if (cmp & 4u)
-            for (int p = lane; p < NGP; p += TL) pg[4 * NGP + p] = (T)up1[0];
-        __syncwarp(tm);
-        for (int p = lane; p < NGP; p += TL) {
-            double V, A;
-            Site<R, Pix, MODE>::VA(d, tb, k, SET_MOM, p % NG, p / NG, zp[p], V, A);
-            gam[p] = gamma_manning<T>(manT, (T)V, pg[3 * NGP + p], pg[4 * NGP + p], gT, epsT);
-        }
-    } else {
-        for (int p = lane; p < NGP; p += TL) gam[p] = T(0);
+__device__ __forceinline__ double bulk_of(double v, double) { return v; }
+__device__ __forceinline__ float bulk_of(double v, float) { return f32_of(v); }
+__device__ __forceinline__ double exact_of(double v) { return v; }
+__device__ __forceinline__ double exact_of(float v) { return f64_any(v); }
+
+// T (N x N) along both directions of NF fields of N x N values, one node per
+// lane (N N <= team width): v[f] is the lane's value in and its result out.
+// FP64 values go through block fixed point (t: the table's exponent), FP32 ones
+// through FP32 sums.  w: 2 NF N N 8-byte words.
+template <int N, int NF>
+__device__ __forceinline__ void square(const int2 (*T)[MXN], int t, double (&v)[NF], int2* w, int lane,
+                                       unsigned tm) {
+    constexpr int NN = N * N;
+    const bool act = lane < NN;
+    const int i = act ? lane : NN - 1, r = i / N, c = i % N;
+    int e[NF];
+    int2* tmp = w + NF * NN;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        e[f] = team_exp(act ? v[f] : 0.0, tm);
+        if (act) w[f * NN + i] = fx::split(fx::from_double(v[f], e[f]));
     }
     __syncwarp(tm);
-    if (F64 && d.qpts != nullptr) { // q^n at the points, from the step start
-        for (int p = lane; p < 2 * NGP; p += TL) pg[3 * NGP + p] = (T)d.qpts[k * 2 * NGP + p];
-    } else {
-        for (int i = lane; i < 2 * ND; i += TL) nod[i] = (T)su[ND + i];
-        __syncwarp(tm);
-        tens_interp2<ND1, NG, T, TL>(Bg, nod, nod + ND, tmp, tmp1, pg + 3 * NGP, pg + 4 * NGP, lane,
-                                     tm);
-        if (cm0 & 2u)
-            for (int p = lane; p < NGP; p += TL) pg[3 * NGP + p] = (T)su[ND];
-        if (cm0 & 4u)
-            for (int p = lane; p < NGP; p += TL) pg[4 * NGP + p] = (T)su[2 * ND];
-    }
-    for (int i = lane; i < 2 * ND; i += TL) nod[i] = (T)rq[i];
-    __syncwarp(tm);
-    kron_apply2<ND1, true, MXP, T, TL>(Bginv, nod, nod + ND, tmp, tmp1, pg, pg + NGP, T(1), lane, tm);
-    for (int p = lane; p < NGP; p += TL) {
-        const T w = wpt(p);
-        const T rD = T(1) / (w * (T(1) + adtT * gam[p]));
-        pg[0 * NGP + p] = (w * pg[3 * NGP + p] + pg[0 * NGP + p]) * rD;
-        pg[1 * NGP + p] = (w * pg[4 * NGP + p] + pg[1 * NGP + p]) * rD;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        fx::Acc s;
+#pragma unroll
+        for (int a = 0; a < N; ++a) s.mac(T[c][a], w[f * NN + r * N + a]);
+        if (act) tmp[f * NN + i] = fx::split(s.get());
     }
     __syncwarp(tm);
-    kron_apply2<ND1, false, MXP, T, TL>(Bginv, pg, pg + NGP, tmp, tmp1, nod, nod + ND, T(1), lane, tm);
-    for (int i = lane; i < 2 * ND; i += TL) Q[i] = (double)nod[i];
-    __syncwarp(tm);
-    if (make_llin) {
-        for (int p = lane; p < NGP; p += TL) {
-            const T w = wpt(p) * gam[p];
-            pg[3 * NGP + p] = -w * pg[p];
-            pg[4 * NGP + p] = -w * pg[NGP + p];
-        }
-        __syncwarp(tm);
-        tens_test2<ND1, NG, T, TL>(Bg, pg + 3 * NGP, pg + 4 * NGP, tmp, tmp1, nod, nod + ND, lane, tm);
-        for (int i = lane; i < 2 * ND; i += TL) llin[i] = (double)nod[i];
-        __syncwarp(tm);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        fx::Acc s;
+#pragma unroll
+        for (int b = 0; b < N; ++b) s.mac(T[r][b], tmp[f * NN + b * N + c]);
+        v[f] = fx::to_double(s.get(), e[f] + 2 * t);
     }
+    __syncwarp(tm);
 }
+template <int N, int NF>
+__device__ __forceinline__ void square(const float (*T)[MXN], int, float (&v)[NF], int2* w, int lane,
+                                       unsigned tm) {
+    constexpr int NN = N * N;
+    const bool act = lane < NN;
+    const int i = act ? lane : NN - 1, r = i / N, c = i % N;
+    float* in = (float*)w;
+    float* tmp = in + NF * NN;
+    if (act) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) in[f * NN + i] = v[f];
+    }
+    __syncwarp(tm);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        float s = 0.0f;
+#pragma unroll
+        for (int a = 0; a < N; ++a) s += T[c][a] * in[f * NN + r * N + a];
+        if (act) tmp[f * NN + i] = s;
+    }
+    __syncwarp(tm);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        float s = 0.0f;
+#pragma unroll
+        for (int b = 0; b < N; ++b) s += T[r][b] * tmp[f * NN + b * N + c];
+        v[f] = s;
+    }
+    __syncwarp(tm);
+}
+// the stage tables of the value type
+__device__ __forceinline__ const int2 (*tab_Bg(const FxStage& s, double))[MXN] { return s.Bg; }
+__device__ __forceinline__ const float (*tab_Bg(const FxStage& s, float))[MXN] { return s.BgF; }
+__device__ __forceinline__ const int2 (*tab_BgT(const FxStage& s, double))[MXN] { return s.BgT; }
+__device__ __forceinline__ const float (*tab_BgT(const FxStage& s, float))[MXN] { return s.BgTF; }
+__device__ __forceinline__ const int2 (*tab_Gi(const FxStage& s, double))[MXN] { return s.Gi; }
+__device__ __forceinline__ const float (*tab_Gi(const FxStage& s, float))[MXN] { return s.GiF; }
+__device__ __forceinline__ const int2 (*tab_GiT(const FxStage& s, double))[MXN] { return s.GiT; }
+__device__ __forceinline__ const float (*tab_GiT(const FxStage& s, float))[MXN] { return s.GiTF; }
+
+// The stage update: one cell per team of 16 lanes, node i and momentum point i
+// on lane i ((r+1)^2 <= 16), mass points i and i + 16.  The FP64 pipe bounds
+// it, so every contraction (the Newton evaluations, the mass inverse, the
+// momentum's S^-T, S^-1 and point values, the tracer's residuals) is block
+// fixed-point on the integer pipe and a lane's nodal values stay in registers;
+// FP64 is left with the right-hand sides, the pointwise physics and the sums
+// that the mass balance needs.  B = float (FP32-bulk): the momentum's point
+// arithmetic and the tracer correction in FP32.
+template <int R>
+struct StageFx {
+    using S = Sz<R>;
+    static constexpr int TL = 16, PP = (S::NMP + TL - 1) / TL;
+    // 8-byte words per team: digit pairs of nodal fields with scratch [6 ND] (the
+    // fallback's Y), mass-point digits with the solve's scratch [2 NMP + NMP],
+    // weights [NMP], right-hand side [ND], then the FP32 solve's M and Y or the
+    // fallback's M
+    static constexpr int W = 6 * S::ND, Q = 3 * S::NMP, CW = S::NMP, BV = S::ND;
+    static constexpr int F32 = (S::ND * S::ND + S::ND1 * S::ND1 * S::NM + 1) / 2;
+    static constexpr int UN = S::ND * S::ND > F32 ? S::ND * S::ND : F32;
+    static constexpr int words = W + Q + CW + BV + UN;
+    static_assert(S::ND <= TL && S::NGP == S::ND, "one node and one momentum point per lane");
+    static_assert(S::ND1 * S::ND1 * S::NM <= W, "fallback Y");
+};
 
 template <int R, typename Pix, int MODE, typename B>
 __global__ void __maxnreg__(96)
     k_stage(const __grid_constant__ Dev d, const __grid_constant__ Tables tb,
             const __grid_constant__ StageArgs sa) {
     using S = Sz<R>;
+    using L = StageFx<R>;
     using ST = Site<R, Pix, MODE>;
     constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
+    constexpr int TL = L::TL, PP = L::PP;
+    constexpr bool F64 = sizeof(B) == sizeof(double);
+    __shared__ FxStage fs;
+    copy_table(fs, &d.tabs->fs);
     extern __shared__ double smem[];
-    // two cells per warp, one per team of 16 lanes (a cell's loops run over 16
-    // nodes and 16 momentum points): "warp" is the team within the block,
-    // "lane" the lane within the team, wpb the teams per block
-    constexpr int TL = 16;
-    const int warp = threadIdx.x / TL, lane = threadIdx.x % TL, wpb = blockDim.x / TL;
+    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
     const unsigned tm = 0xFFFFu << (threadIdx.x & 16); // the team's lanes
-    double* su = smem + warp * stage_smem<R>(); // [4][ND] state v^n
-    double* T = su + 4 * ND;                    // [ND]
-    double* rq = T + ND;                        // [2][ND]
-    double* rc = rq + 2 * ND;                   // [ND]
-    double* z = rc + ND;                        // [ND] Newton iterate
-    double* pe = z + ND;                        // [NMP]
-    double* pV = pe + NMP;                      // [NMP]
-    double* pA = pV + NMP;                      // [NMP]
-    double* tmp = pA + NMP;                     // [2 NM NM]
-    double* xs = tmp + 2 * NM * NM;             // [ND] refinement iterate (also scratch [2 ND]
-    double* rs = xs + ND;                       // [ND] refinement residual   with rs outside a solve)
-    double* o = rs + ND;                        // [4][ND]
-    // the refinement's q [NMP] is pe, idle inside a solve (pe holds the
-    // interpolated iterate only while V and A are evaluated)
-    double* qs = pe;
-    // the last region: friction points pg (the scalar path's; the momentum
-    // block's point arrays on the other path) with the momentum scratch, or
-    // the FP32 solve's arrays, or the FP64 fallback's M.  The momentum block
-    // runs between the two solves; the fallback runs only inside a solve, when
-    // the FP32 arrays are given up, and its Y and pivots take tmp, x, r and q,
-    // which are idle then.
-    double* un = o + 4 * ND;
-    double* pg = un;                            // [6][NGP]
-    double* mw = pg + 6 * NGP;                  // momentum nodal pair [2 ND] (B)
-    double* mt = mw + 2 * ND;                   // momentum tmp pair [2 ND1 NG] (B)
-    float* Mf = (float*)un;                     // [ND ND]
-    float* Yf = Mf + ND * ND;                   // [ND1 ND1 NM]
-    double* M = un;                             // [ND ND] (fallback)
-    double* Y = tmp;                            // [ND1 ND1 NM] (fallback)
-    double* pinv = qs;                          // [ND] (fallback)
+    int2* w = (int2*)(smem + team * L::words); // digit pairs of nodal fields, and scratch
+    int2* qd = w + L::W;                       // [NMP] mass-point digits, then scratch [2 NMP]
+    int2* qt = qd + NMP;
+    double* cw = (double*)(qd + L::Q); // [NMP] weights of a mass-matrix solve
+    double* bv = cw + L::CW;           // [ND] its right-hand side and solution
+    double* un = bv + L::BV;
+    float* Mf = (float*)un;            // [ND ND]
+    float* Yf = Mf + ND * ND;          // [ND1 ND1 NM]
+    double* M = un;                    // [ND ND] (fallback)
     const int64_t n = d.n;
     const double g = d.g, eps = d.eps;
+    const bool act = lane < ND;
+    const int node = act ? lane : 0;
     int its_max = 0;
     int viol = 0, fb = 0, bad = 0;
+    const double dt_all = d.memb ? 0.0 : get_dt(d, 0);
+    const double w2 = fs.wg[node % NG] * fs.wg[node / NG]; // the lane's momentum weight
+    double wm2[PP];                                        // its mass weights
+#pragma unroll
+    for (int j = 0; j < PP; ++j) {
+        const int p = lane + j * TL;
+        wm2[j] = p < NMP ? fs.wm[p % NM] * fs.wm[p / NM] : 0.0;
+    }
+    const float tolf = (float)d.newton_tol;
 
-    for (int64_t k = (int64_t)blockIdx.x * wpb + warp; k < n; k += (int64_t)gridDim.x * wpb) {
-        for (int i = lane; i < 4 * ND; i += TL) su[i] = ufield(d, 0, i / ND, ND)[k * ND + (i % ND)];
+    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
+        const size_t idx = (size_t)k * ND + node;
         const unsigned cm0 = d.cmask[k];
         const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
         const double man = d.manning[k];
         int flag = d.flag[k];
-        const double dt = get_dt(d, member_of(d, k)); // the member's step
+        const double dt = d.memb ? get_dt(d, d.memb[k]) : dt_all; // the member's step
+        const double u0 = ufield(d, 0, 0, ND)[idx];               // zeta^n
         // right-hand sides of Eqs. algebraic_elevation, algebraic_discharge, algebraic_concentration
-        double tsum = 0.0;
-        for (int i = lane; i < ND; i += TL) {
+        const double hn = d.HN[idx], cn0 = d.CN[idx];
+        double T, rq[2], rc, tsum = 0.0;
+        {
             double sf = 0.0, sgx = 0.0, sgy = 0.0, sr = 0.0;
             for (int m = 0; m < sa.nres; ++m) {
-                const size_t idx = (size_t)k * ND + i;
                 const bool lin = sa.use_llin && (m == sa.nres - 1);
                 const double lx = lin ? d.llin[idx] : rfield(d, m, 4, ND)[idx];
                 const double ly = lin ? d.llin[(size_t)n * ND + idx] : rfield(d, m, 5, ND)[idx];
@@ -1776,236 +2277,287 @@ __global__ void __maxnreg__(96)
                 sgy += sa.wa[m] * rfield(d, m, 2, ND)[idx] + sa.wat[m] * ly;
                 sr += sa.wa[m] * rfield(d, m, 3, ND)[idx];
             }
-            T[i] = d.HN[k * ND + i] + dt * sf;
-            tsum += dt * sf;
-            rq[i] = dt * sgx;
-            rq[ND + i] = dt * sgy;
-            rc[i] = d.CN[k * ND + i] + dt * sr;
+            sf *= dt;
+            T = hn + sf;
+            if (act) tsum = sf;
+            rq[0] = dt * sgx;
+            rq[1] = dt * sgy;
+            rc = cn0 + dt * sr;
         }
         const double Tbar = d.HNbar[k] + team_sum<TL>(tsum, tm);
         if (Tbar < 0.0) viol++;
         bool scalar = (flag == 0);
         int its = 0;
-        __syncwarp(tm);
         bool cert = false; // the Newton solve ended on its one-step certificate
+        double z = u0;     // Newton iterate
+        double V[PP], A[PP];
+        // elevations at the lane's mass points of the nodal values v (cst: a constant field)
+        auto mass_points = [&](double v, bool cst, double (&pe)[PP]) {
+            const double v0 = __shfl_sync(tm, v, 0, TL);
+            const int e = team_exp(act ? v : 0.0, tm);
+            if (act) w[lane] = fx::split(fx::from_double(v, e));
+            __syncwarp(tm);
+            fx_tens<ND1, NM, TL>(fs.Bm, w, qt, lane, tm, [&](int it, int, long long X) {
+                pe[it] = cst ? v0 : fx::to_double(X, e + 2 * fs.tBm);
+            });
+            __syncwarp(tm);
+        };
         if (!scalar) {
-            for (int i = lane; i < ND; i += TL) z[i] = su[i];
             bool zc = (cm0 & 1u) != 0;
             bool prev_full = false;
             // every mass point fully wet at zeta^n (known from the step start,
-            // which evaluated H(zeta^n) = HN from the same state by the same
-            // arithmetic): the first Newton step needs no evaluation, since
-            // H(zeta^n) - T = HN - T and M(zeta^n) is the constant mass matrix
+            // which evaluated H(zeta^n) = HN from the same state): the first
+            // Newton step needs no evaluation, since H(zeta^n) - T = HN - T and
+            // M(zeta^n) is the constant mass matrix
             const bool full0 = d.wet0 != nullptr && d.wet0[k] != 0 && d.newton_max > 0;
-            __syncwarp(tm);
             // each pass evaluates V, A at the current iterate; the last pass is
             // the evaluation at the result (for the tracer matrix and the
             // completely-dry test)
             for (int kk = 0;; ++kk) {
-                int ndry = 0, npart = 0;
+                int npart = 0;
+                double o;
                 if (kk == 0 && full0) {
-                    for (int i = lane; i < ND; i += TL) o[i] = d.HN[k * ND + i] - T[i];
+                    o = hn - T;
                 } else {
-                tens_interp<ND1, NM, double, TL>(tb.Bm, z, tmp, pe, lane, tm);
-                for (int p = lane; p < NMP; p += TL) {
-                    if (zc) pe[p] = z[0];
-                    double V, A;
-                    bool full;
-                    ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, pe[p], V, A, full);
-                    pV[p] = J * tb.wm[p % NM] * tb.wm[p / NM] * V;
-                    pA[p] = J * tb.wm[p % NM] * tb.wm[p / NM] * A;
-                    if (zero_bits(A)) ndry++;
-                    else if (!full) npart++;
+                    double pe[PP];
+                    mass_points(z, zc, pe);
+                    bool dry = false, part = false;
+#pragma unroll
+                    for (int j = 0; j < PP; ++j) {
+                        const int p = lane + j * TL;
+                        if (p < NMP) {
+                            bool full;
+                            ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, pe[j], V[j], A[j], full);
+                            if (zero_bits(A[j])) dry = true;
+                            else if (!full) part = true;
+                        }
+                    }
+                    if (__any_sync(tm, dry)) { scalar = true; break; }
+                    npart = __any_sync(tm, part);
+                    // every pixel wet at the previous and at this iterate: H is affine
+                    // on the segment between them and M(previous) is its exact
+                    // Jacobian, so this iterate solves H = T (the fully wet case of
+                    // Sec. 3.4); no verification step is needed
+                    if (kk > 0 && prev_full && npart == 0) {
+                        cert = true;
+                        break;
+                    }
+                    if (kk == d.newton_max) break;
+                    // H_i(zeta_k)
+                    double hv[PP];
+                    unsigned m = 0;
+#pragma unroll
+                    for (int j = 0; j < PP; ++j) {
+                        hv[j] = lane + j * TL < NMP ? J * wm2[j] * V[j] : 0.0;
+                        m = max(m, fx::mag(hv[j]));
+                    }
+                    const int e = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll
+                    for (int j = 0; j < PP; ++j)
+                        if (lane + j * TL < NMP) qd[lane + j * TL] = fx::split(fx::from_double(hv[j], e));
+                    __syncwarp(tm);
+                    double H = 0.0;
+                    fx_tens<NM, ND1, TL>(fs.BmT, qd, qt, lane, tm, [&](int, int, long long X) {
+                        H = fx::to_double(X, e + 2 * fs.tBmT);
+                    });
+                    o = H - T;
+                    __syncwarp(tm);
                 }
-                ndry = __reduce_add_sync(tm, ndry);
-                npart = __reduce_add_sync(tm, npart);
-                if (ndry) { scalar = true; break; }
-                // every pixel wet at the previous and at this iterate: H is affine
-                // on the segment between them and M(previous) is its exact
-                // Jacobian, so this iterate solves H = T (the fully wet case of
-                // Sec. 3.4); no verification step is needed
-                if (kk > 0 && prev_full && npart == 0) {
-                    cert = true;
-                    break;
-                }
-                if (kk == d.newton_max) break;
-                __syncwarp(tm);
-                tens_test<ND1, NM, double, TL>(tb.Bm, pV, tmp, o, lane, tm); // H_i(zeta_k)
-                for (int i = lane; i < ND; i += TL) o[i] -= T[i];
-                }
-                __syncwarp(tm);
+                double dz[1] = {o};
                 if (npart == 0) {
                     // M is the constant mass matrix, inverted by its tensor factors
-                    kron_apply<ND1, false, MXN, double, TL>(tb.M1inv, o, tmp, o + ND, 1.0 / J, lane, tm);
+                    square<ND1, 1>(fs.M1i, fs.tM1i, dz, w, lane, tm);
+                    dz[0] *= d.ihxhy[2 * k] * d.ihxhy[2 * k + 1];
                 } else {
-                    for (int i = lane; i < ND; i += TL) o[ND + i] = o[i];
+                    if (act) bv[lane] = o;
+#pragma unroll
+                    for (int j = 0; j < PP; ++j)
+                        if (lane + j * TL < NMP) cw[lane + j * TL] = J * wm2[j] * A[j];
                     __syncwarp(tm);
-                    if (!solve_mass_mixed<ND1, NM, TL>(tb, pA, o + ND, Mf, Yf, xs, rs, qs,
-                                                       tmp, M, Y, pinv, lane, tm)) {
+                    if (!solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, w, qd, qt, M,
+                                                       (double*)w, (double*)qd, lane, tm)) {
                         scalar = true;
                         break;
                     }
+                    dz[0] = bv[node];
+                    __syncwarp(tm);
                 }
-                double inc = 0.0, scale = 0.0;
-                for (int i = lane; i < ND; i += TL) {
-                    z[i] -= o[ND + i];
-                    inc += fabs(o[ND + i]);
-                    scale += 1.0 + fabs(z[i]) + d.zabs[k];
+                z -= dz[0];
+                // the stopping test in FP32 (sums of magnitudes against 1e-12 of their scale)
+                float inc = 0.0f, scale = 0.0f;
+                if (act) {
+                    inc = f32_of(fabs(dz[0]));
+                    scale = 1.0f + f32_of(fabs(z)) + f32_of(d.zabs[k]);
                 }
-                team_sum2<TL>(inc, scale, tm);
+#pragma unroll
+                for (int s = TL / 2; s > 0; s >>= 1) {
+                    inc += __shfl_xor_sync(tm, inc, s);
+                    scale += __shfl_xor_sync(tm, scale, s);
+                }
                 its++;
                 prev_full = (npart == 0);
-                __syncwarp(tm);
-                {
-                    bool eq = true;
-                    for (int i = lane; i < ND; i += TL) eq = eq && same_bits(z[i], z[0]);
-                    zc = __all_sync(tm, eq);
-                }
-                if (inc <= d.newton_tol * scale) prev_full = false, kk = d.newton_max - 1;
+                const double z0 = __shfl_sync(tm, z, 0, TL);
+                zc = __all_sync(tm, !act || same_bits(z, z0));
+                if (inc <= tolf * scale) prev_full = false, kk = d.newton_max - 1;
             }
             if (scalar) {
                 fb++;
                 flag = 0;
                 if (lane == 0) d.flag[k] = 0;
             }
-            __syncwarp(tm);
         }
-        // friction coefficient of the previous stage on the momentum GL points
-        // (scalar path; the r path forms it inside momentum_block)
-        double* gam = pg + 5 * NGP;
-        const bool need_gam = (sa.add != 0.0 || sa.make_llin) && man != 0.0;
-        if (need_gam && scalar) {
+        // v^(l-1) at the lane's momentum point (a constant field: its value), the
+        // discharges in T; then the friction coefficient there
+        const bool need_gam = (sa.add != 0.0 || sa.make_llin) && !zero_bits(man);
+        auto gamma_prev = [&](auto manT, auto gT, auto epsT) {
+            using T = decltype(manT);
             const unsigned cmp = d.cmask[(size_t)sa.prev_buf * n + k];
-            for (int f = 0; f < 3; ++f) {
-                const double* up = ufield(d, sa.prev_buf, f, ND) + k * ND;
-                if (cmp & (1u << f)) { // a constant field: its value at every point
-                    const double v0 = up[0];
-                    for (int p = lane; p < NGP; p += TL) pg[f * NGP + p] = v0;
-                } else {
-                    for (int i = lane; i < ND; i += TL) o[i] = up[i];
-                    __syncwarp(tm);
-                    tens_interp<ND1, NG, double, TL>(tb.Bg, o, tmp, pg + f * NGP, lane, tm);
-                }
-                __syncwarp(tm);
+            const double z0 = ufield(d, sa.prev_buf, 0, ND)[idx];
+            const T q0 = bulk_of(ufield(d, sa.prev_buf, 1, ND)[idx], T()),
+                    q1 = bulk_of(ufield(d, sa.prev_buf, 2, ND)[idx], T());
+            double zv[1] = {z0}, Vp, Ap;
+            T q[2] = {q0, q1}, gam = T(0);
+            if (!(cmp & 1u)) square<ND1, 1>(fs.Bg, fs.tBg, zv, w, lane, tm);
+            if ((cmp & 6u) != 6u) square<ND1, 2>(tab_Bg(fs, T()), fs.tBg, q, w, lane, tm);
+            if (cmp & 2u) q[0] = q0;
+            if (cmp & 4u) q[1] = q1;
+            if (act) {
+                ST::VA(d, tb, k, SET_MOM, lane % NG, lane / NG, zv[0], Vp, Ap);
+                gam = gamma_manning<T>(manT, bulk_of(Vp, T()), q[0], q[1], gT, epsT);
             }
-            for (int p = lane; p < NGP; p += TL) {
-                double V, A;
-                ST::VA(d, tb, k, SET_MOM, p % NG, p / NG, pg[p], V, A);
-                gam[p] = gamma_manning<double>(man, V, pg[NGP + p], pg[2 * NGP + p], g, eps);
-            }
-        } else {
-            for (int p = lane; p < NGP; p += TL) gam[p] = 0.0;
-        }
-        __syncwarp(tm);
+            return gam;
+        };
+        // v^n's discharges at the momentum point, interpolated
+        auto q_points = [&](auto& v) {
+            using T = std::remove_reference_t<decltype(v[0])>;
+            const T q0 = bulk_of(ufield(d, 0, 1, ND)[idx], T()), q1 = bulk_of(ufield(d, 0, 2, ND)[idx], T());
+            v[0] = q0;
+            v[1] = q1;
+            if ((cm0 & 6u) != 6u) square<ND1, 2>(tab_Bg(fs, T()), fs.tBg, v, w, lane, tm);
+            if (cm0 & 2u) v[0] = q0;
+            if (cm0 & 4u) v[1] = q1;
+        };
+        double oz, oq[2], oc, ll[2];
         if (scalar) {
+            const double gam = need_gam ? gamma_prev(man, g, eps) : 0.0;
             double e;
-            if (cm0 & 1u) e = su[0];
+            if (cm0 & 1u) e = u0;
             else {
-                tens_interp<ND1, NM, double, TL>(tb.Bm, su, tmp, pe, lane, tm);
-                double s = 0.0;
-                for (int p = lane; p < NMP; p += TL) s += tb.wm[p % NM] * tb.wm[p / NM] * pe[p];
+                double pe[PP], s = 0.0;
+                mass_points(u0, false, pe);
+#pragma unroll
+                for (int j = 0; j < PP; ++j)
+                    if (lane + j * TL < NMP) s += wm2[j] * pe[j];
                 e = team_sum<TL>(s, tm);
             }
             its = scalar_newton<R, Pix, MODE, TL>(d, tb, k, J, Tbar, e, lane, tm);
             // momentum: sums of the rows of the friction-modified mass matrix
-            double den = 0.0, num[2] = {0.0, 0.0};
+            double qn[2];
             if (d.qpts) {
-                for (int p = lane; p < 2 * NGP; p += TL) pg[3 * NGP + p] = d.qpts[k * 2 * NGP + p];
-                __syncwarp(tm);
+                qn[0] = d.qpts[k * 2 * NGP + node];
+                qn[1] = d.qpts[k * 2 * NGP + NGP + node];
             } else {
-                for (int f = 0; f < 2; ++f) {
-                    if (cm0 & (2u << f))
-                        for (int p = lane; p < NGP; p += TL) pg[(3 + f) * NGP + p] = su[(1 + f) * ND];
-                    else
-                        tens_interp<ND1, NG, double, TL>(tb.Bg, su + (1 + f) * ND, tmp,
-                                                         pg + (3 + f) * NGP, lane, tm);
-                    __syncwarp(tm);
-                }
+                q_points(qn);
             }
-            for (int p = lane; p < NGP; p += TL) {
-                const double w = J * tb.wg[p % NG] * tb.wg[p / NG];
-                den += w * (1.0 + sa.add * dt * gam[p]);
-                num[0] += w * pg[3 * NGP + p];
-                num[1] += w * pg[4 * NGP + p];
-            }
-            double rs0 = 0.0, rs1 = 0.0, rcs = 0.0;
-            for (int i = lane; i < ND; i += TL) {
-                rs0 += rq[i];
-                rs1 += rq[ND + i];
-                rcs += rc[i] - d.CN[k * ND + i];
+            const double wp = J * w2;
+            double den = 0.0, num[2] = {0.0, 0.0}, rs0 = 0.0, rs1 = 0.0, rcs = 0.0;
+            if (act) {
+                den = wp * (1.0 + sa.add * dt * gam);
+                num[0] = wp * qn[0];
+                num[1] = wp * qn[1];
+                rs0 = rq[0];
+                rs1 = rq[1];
+                rcs = rc - cn0;
             }
             team_sum2<TL>(den, rcs, tm);
             team_sum2<TL>(num[0], rs0, tm);
             team_sum2<TL>(num[1], rs1, tm);
-            const double qxn = (num[0] + rs0) / den;
-            const double qyn = (num[1] + rs1) / den;
+            oz = e;
+            oq[0] = (num[0] + rs0) / den;
+            oq[1] = (num[1] + rs1) / den;
             double Hs, As;
             mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, Hs, As, tm);
-            const bool tr_ok = Hs > 1e-14 * J * d.hlim;
-            const double cn = tr_ok ? (d.CNbar[k] + rcs) / Hs : 0.0;
-            for (int i = lane; i < ND; i += TL) {
-                o[i] = e;
-                o[ND + i] = qxn;
-                o[2 * ND + i] = qyn;
-                o[3 * ND + i] = tr_ok ? cn : su[3 * ND + i];
-            }
-            __syncwarp(tm);
+            oc = Hs > 1e-14 * J * d.hlim ? (d.CNbar[k] + rcs) / Hs : ufield(d, 0, 3, ND)[idx];
             if (sa.make_llin) {
-                for (int p = lane; p < NGP; p += TL) {
-                    const double w = J * tb.wg[p % NG] * tb.wg[p / NG] * gam[p];
-                    pg[3 * NGP + p] = -w * qxn;
-                    pg[4 * NGP + p] = -w * qyn;
-                }
-                __syncwarp(tm);
-                tens_test<ND1, NG, double, TL>(tb.Bg, pg + 3 * NGP, tmp, xs, lane, tm);
-                tens_test<ND1, NG, double, TL>(tb.Bg, pg + 4 * NGP, tmp, rs, lane, tm);
-                for (int i = lane; i < ND; i += TL) {
-                    d.llin[(size_t)k * ND + i] = xs[i];
-                    d.llin[(size_t)n * ND + (size_t)k * ND + i] = xs[ND + i];
-                }
+                ll[0] = -(wp * gam) * oq[0];
+                ll[1] = -(wp * gam) * oq[1];
+                square<ND1, 2>(fs.BgT, fs.tBgT, ll, w, lane, tm);
             }
         } else {
-            // momentum (FP64, or FP32 in the FP32-bulk path)
-            momentum_block<R, Pix, MODE, B, TL>(d, tb, k, J, man, dt, sa.add, need_gam, sa.make_llin != 0,
-                                            sa.prev_buf, su, cm0, rq, (B*)mw, (B*)mt, (B*)pg, pe, tmp,
-                                            o + ND,
-                                            xs, lane, tm);
+            // momentum (Eq. algebraic_discharge with the friction-modified mass
+            // matrix of Eq. mass_matrix_discharge on the (r+1)^2 Gauss-Legendre
+            // points, inverted as S^-1 D^-1 S^-T): S Q = [D0 q^n + S^-T rq] / D,
+            // D = D0 (1 + add dt gamma), D0 = J w, gamma from the previous stage;
+            // optionally the linearised friction term Llin = -S^T (J w gamma S Q)
+            B JB, manB, gB, epsB, adtB;
+            if constexpr (F64) {
+                JB = J; manB = man; gB = g; epsB = eps; adtB = sa.add * dt;
+            } else {
+                JB = f32_of(J); manB = f32_of(man); gB = f32_of(g); epsB = f32_of(eps);
+                adtB = f32_of(sa.add * dt);
+            }
+            const B gam = need_gam ? gamma_prev(manB, gB, epsB) : B(0);
+            B qn[2];
+            if (F64 && d.qpts) { // q^n at the points, from the step start
+                qn[0] = (B)d.qpts[k * 2 * NGP + node];
+                qn[1] = (B)d.qpts[k * 2 * NGP + NGP + node];
+            } else {
+                q_points(qn);
+            }
+            B s[2] = {bulk_of(rq[0], B()), bulk_of(rq[1], B())};
+            square<ND1, 2>(tab_GiT(fs, B()), fs.tGiT, s, w, lane, tm);
+            B wp;
+            if constexpr (F64) wp = J * w2;
+            else wp = JB * fs.wgF[node % NG] * fs.wgF[node / NG];
+            const B rD = B(1) / (wp * (B(1) + adtB * gam));
+            s[0] = (wp * qn[0] + s[0]) * rD;
+            s[1] = (wp * qn[1] + s[1]) * rD;
+            B Q[2] = {s[0], s[1]};
+            square<ND1, 2>(tab_Gi(fs, B()), fs.tGi, Q, w, lane, tm);
             if (sa.make_llin) {
-                for (int i = lane; i < ND; i += TL) {
-                    d.llin[(size_t)k * ND + i] = xs[i];
-                    d.llin[(size_t)n * ND + (size_t)k * ND + i] = xs[ND + i];
-                }
-                __syncwarp(tm);
+                const B wl = wp * gam;
+                B l[2] = {-wl * s[0], -wl * s[1]};
+                square<ND1, 2>(tab_BgT(fs, B()), fs.tBgT, l, w, lane, tm);
+                ll[0] = exact_of(l[0]);
+                ll[1] = exact_of(l[1]);
             }
+            oz = z;
+            oq[0] = exact_of(Q[0]);
+            oq[1] = exact_of(Q[1]);
             // tracer: H(zeta^(l)) C = C~ + dt sum a R with the depth-weighted mass matrix
-            for (int i = lane; i < ND; i += TL) {
-                o[i] = z[i];
-                o[3 * ND + i] = rc[i];
-            }
+            if (act) bv[lane] = rc;
+#pragma unroll
+            for (int j = 0; j < PP; ++j)
+                if (lane + j * TL < NMP) cw[lane + j * TL] = J * wm2[j] * V[j];
             __syncwarp(tm);
-            if constexpr (sizeof(B) == sizeof(float))
-                solve_tracer_bulk<ND1, NM, TL>(tb, pV, o + 3 * ND, Mf, Yf, xs, tmp, M, Y, pinv,
-                                               cert ? T : nullptr, lane, tm);
+            if constexpr (F64)
+                solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, w, qd, qt, M, (double*)w,
+                                              (double*)qd, lane, tm);
             else
-                solve_mass_mixed<ND1, NM, TL>(tb, pV, o + 3 * ND, Mf, Yf, xs, rs, qs, tmp, M,
-                                              Y, pinv, lane, tm);
+                solve_tracer_bulk<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, qt, M, (double*)w,
+                                               (double*)qd, cert, T, lane, tm);
+            oc = bv[node];
+            __syncwarp(tm);
         }
-        __syncwarp(tm);
+        if (sa.make_llin && act) {
+            d.llin[idx] = ll[0];
+            d.llin[(size_t)n * ND + idx] = ll[1];
+        }
         // write v^(l) and its constant-field mask
+        const double ov[4] = {oz, oq[0], oq[1], oc};
         unsigned cmo = 0;
-        for (int f = 0; f < 4; ++f) {
-            bool eq = true;
-            for (int i = lane; i < ND; i += TL) eq = eq && same_bits(o[f * ND + i], o[f * ND]);
-            if (__all_sync(tm, eq)) cmo |= (1u << f);
-        }
         bool fin = true;
-        for (int i = lane; i < 4 * ND; i += TL) {
-            const double v = o[i];
-            fin = fin && finite_bits(v);
-            ufield(d, sa.out_buf, i / ND, ND)[k * ND + (i % ND)] = v;
-            if (d.uF) ufieldF(d, sa.out_buf, i / ND, ND)[k * ND + (i % ND)] = (float)v;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const double v0 = __shfl_sync(tm, ov[f], 0, TL);
+            if (__all_sync(tm, !act || same_bits(ov[f], v0))) cmo |= 1u << f;
+            fin = fin && finite_bits(ov[f]);
+            if (act) {
+                ufield(d, sa.out_buf, f, ND)[idx] = ov[f];
+                if (d.uF) ufieldF(d, sa.out_buf, f, ND)[idx] = f32_of(ov[f]);
+            }
         }
-        if (!__all_sync(tm, fin)) bad = 1;
+        if (!__all_sync(tm, fin || !act)) bad = 1;
         if (lane == 0) d.cmask[(size_t)sa.out_buf * n + k] = (uint8_t)cmo;
         its_max = max(its_max, its);
         __syncwarp(tm);
