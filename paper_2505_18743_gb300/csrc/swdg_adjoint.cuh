@@ -821,13 +821,13 @@ __global__ void __maxnreg__(128)
             }
             allfull = __all_sync(tm, allfull);
             __syncwarp(tm);
-            // the forward's mixed-precision solve (FP32 factor, refinement to 1e-15,
-            // FP64 Cholesky fallback); its FP32 arrays overlay M and Y, its digit
-            // pairs take x, pw and tmp (all idle here)
+            // the forward's mixed-precision solve (FP32 inverse, refinement to 1e-15,
+            // FP64 Cholesky fallback); its FP32 scratch overlays M, its digit pairs
+            // take x, pw and tmp (all idle here)
             for (int i = lane; i < ND; i += TL) rcb[i] = vb[3 * ND + i];
             __syncwarp(tm);
-            solve_mass_mixed<ND1, NM, TL>(tb, tb.fs, pV, rcb, (float*)M, (float*)Y, (int2*)x, (int2*)pw,
-                                          (int2*)tmp, M, Y, inv, lane, tm);
+            solve_mass_mixed<ND1, NM, TL>(tb, tb.fs, pV, rcb, (float*)M, (int2*)x, (int2*)pw, (int2*)tmp, M,
+                                          Y, inv, lane, tm);
             // dH_c/dzeta: zeta_bar(p) -= J w A rcb(p) c(p); the same for delta
             tens_interp<ND1, NM, double, TL>(tb.Bm, rcb, tmp, pw, lane, tm);
             for (int p = lane; p < NMP; p += TL) {

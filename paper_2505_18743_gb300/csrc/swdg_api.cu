@@ -333,6 +333,18 @@ static void build_fx_tables(int R, Tables& tb) {
     memcpy(y.wm, tb.wm, sizeof y.wm);
     memcpy(y.wg, tb.wg, sizeof y.wg);
     memcpy(y.BmF, tb.BmF, sizeof y.BmF);
+    for (int a = 0; a < n1; ++a)
+        for (int q = 0; q < n1; ++q) y.wn[a] += tb.wg[q] * tb.Bg[q][a];
+    double nrm[MXN];
+    for (int a = 0; a < n1; ++a) {
+        double t = 0.0;
+        for (int q = 0; q < nm; ++q) t += tb.Bm[q][a] * tb.Bm[q][a];
+        nrm[a] = 1.0 / std::sqrt(t);
+        y.sc[a] = (float)nrm[a];
+        for (int c = 0; c <= a; ++c)
+            for (int q = 0; q < nm; ++q)
+                y.BB[a * (a + 1) / 2 + c][q] = (float)(tb.Bm[q][a] * tb.Bm[q][c] * nrm[a] * nrm[c]);
+    }
     memcpy(y.wgF, tb.wgF, sizeof y.wgF);
     memcpy(tb.ft.Bm, tb.Bm, sizeof tb.Bm);
     memcpy(tb.ft.BmH, tb.BmH, sizeof tb.BmH);
@@ -733,11 +745,13 @@ static int grid_for(int64_t n, int wpb = WPB) {
 }
 
 // default shapes: WPB warps per block, one block per WPB cells (grid-stride
-// beyond 152 x 64 blocks); the stage update (two cells per warp) 2 warps per
-// block, which its shared memory per cell favours
+// beyond 152 x 64 blocks); the stage update (two cells per warp) at r <= 2 with
+// 2 warps per block: there the cells' costs differ most (pixel sums, Newton
+// steps) and a small block retires sooner (lagoon, r = 2: 394 us with 2 warps,
+// 447 with 4; beach, r = 3: 607 and 580)
 static void default_shapes(swdg_ctx* c) {
     for (int i = 0; i < KK_N; ++i) c->shp[i] = Shape{grid_for(c->n), WPB};
-    c->shp[KK_STAGE] = Shape{grid_for(c->n, 4), 2};
+    if (c->R <= 2) c->shp[KK_STAGE] = Shape{grid_for(c->n, 4), 2};
     c->tuned = false;
 }
 

@@ -85,9 +85,13 @@ struct FxStage {
     int2 Bg[MXN][MXN], BgT[MXN][MXN]; // nodal -> momentum points, its transpose
     int2 Gi[MXN][MXN], GiT[MXN][MXN]; // inverse of Bg, its transpose
     int2 M1i[MXN][MXN];               // inverse 1D mass matrix
-    double wm[MXP], wg[MXP];
+    double wm[MXP], wg[MXP], wn[MXN]; // wn: the nodes' weights in the momentum rule
     float BmF[MXP][MXN], wgF[MXP];
     float BgF[MXN][MXN], BgTF[MXN][MXN], GiF[MXN][MXN], GiTF[MXN][MXN];
+    // the mass matrices' FP32 assembly: node scales 1 / |B_a| (2-norm over the
+    // mass points, per direction) and products of the scaled basis, [pair][point]
+    // with pair (a, c), c <= a, at a (a + 1) / 2 + c
+    float sc[MXN], BB[MXN * (MXN + 1) / 2][MXP];
     int tBm, tBmT, tBg, tBgT, tGi, tGiT, tM1i, pad_;
 };
 
@@ -242,6 +246,16 @@ __device__ __forceinline__ void team_sum2(double& a, double& b, unsigned tm) {
     a = hi ? w : v;
     b = hi ? v : w;
 }
+// maximum over the team of an order-preserving key (okey)
+template <int TL>
+__device__ __forceinline__ long long team_max_key(long long v, unsigned tm) {
+#pragma unroll
+    for (int o = TL / 2; o > 0; o >>= 1) {
+        const long long w = __shfl_xor_sync(tm, v, o);
+        v = w > v ? w : v;
+    }
+    return v;
+}
 // maxima of non-negative values (no NaN) over the team's lanes tm by their bit
 // patterns, which order like the values: integer reductions, off the FP64 pipe
 __device__ __forceinline__ float team_max_nonneg(float v, unsigned tm) {
@@ -275,6 +289,9 @@ __device__ __forceinline__ bool zero_bits(double v) {
 __device__ __forceinline__ long long okey(double v) {
     const long long b = __double_as_longlong(v);
     return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double of_okey(long long b) {
+    return __longlong_as_double(b ^ ((b >> 63) & 0x7fffffffffffffffll));
 }
 // the key of -z for a threshold -z, with -0 taken as +0, so that
 // okey(eta) > nkey_neg(z) is exactly eta > -z for every eta that is not NaN

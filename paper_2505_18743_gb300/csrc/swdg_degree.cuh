@@ -18,7 +18,7 @@ struct Launchers {
         if constexpr (F64) return k_residual<R, Pix, MODE>;
         else return k_residual_bulk<R, Pix, MODE, B>;
     }
-    static constexpr size_t begin_b = sizeof(double) * begin_smem<R>();
+    static constexpr size_t begin_b = 2 * sizeof(double) * BeginFx<R>::words; // two cells per warp
     // k_stage runs two cells per warp (a team of 16 lanes each)
     static constexpr size_t stage_b = 2 * sizeof(double) * StageFx<R>::words;
     static constexpr size_t diag_b = sizeof(double) * (2 * S::ND + 2 * S::NMP + 2 * S::NM * S::NM);
@@ -51,13 +51,15 @@ struct Launchers {
             k_faces_bulk<R, Pix, MODE, B><<<(int)blocks, 256, 0, st>>>(d, buf, c_stage, want_dt);
     }
     static void step_begin(const Dev& d, const Tables& tb, int do_switch, Shape s, cudaStream_t st) {
-        k_step_begin<R, Pix, MODE><<<s.grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, tb, do_switch);
+        const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
+        k_step_begin<R, Pix, MODE><<<grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, do_switch);
     }
     static void stage(const Dev& d, const Tables& tb, const StageArgs& sa, Shape s, cudaStream_t st) {
         // two cells per warp: no more blocks than 2 wpb cells each
         const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
-        k_stage<R, Pix, MODE, B><<<grid, 32 * s.wpb, stage_b * s.wpb, st>>>(d, tb, sa);
+        k_stage<R, Pix, MODE, B><<<grid, 32 * s.wpb, stage_b * s.wpb, st>>>(d, sa);
     }
     static void masks(const Dev& d, int buf, Shape s, cudaStream_t st) {
         k_masks<R><<<s.grid, 32 * s.wpb, 0, st>>>(d, buf);

@@ -101,17 +101,16 @@ __host__ __device__ __forceinline__ long long join(int2 d) {
 
 // exact sum of table x value products, without lo x lo
 struct Acc {
-    long long a1, a2;
+    long long a1, a2, a3; // a3 apart from a2: two chains of dependent additions
     // a2 starts at half a unit of the final shift (round to nearest)
-    __host__ __device__ __forceinline__ Acc() : a1(0), a2(1ll << (FB - LB - 1)) {}
+    __host__ __device__ __forceinline__ Acc() : a1(0), a2(1ll << (FB - LB - 1)), a3(0) {}
     __host__ __device__ __forceinline__ void mac(int2 t, int2 v) {
         a1 += (long long)t.x * v.x;
         a2 += (long long)t.x * v.y;
-        a2 += (long long)t.y * v.x;
+        a3 += (long long)t.y * v.x;
     }
-    // X of the sum: (a1 2^(2 LB) + a2 2^LB) 2^-FB
-    __host__ __device__ __forceinline__ long long get() const {
-        return (a1 << (2 * LB - FB)) + (a2 >> (FB - LB));
+    __host__ __device__ __forceinline__ long long get() const { // X: (a1 2^(2 LB) + (a2 + a3) 2^LB) 2^-FB
+        return (a1 << (2 * LB - FB)) + ((a2 + a3) >> (FB - LB));
     }
 };
 static_assert(2 * LB >= FB, "scale of a1");

@@ -748,10 +748,7 @@ struct ResFx {
 };
 
 template <int R, typename Pix, int MODE>
-#ifndef RES_REGS
-#define RES_REGS 80
-#endif
-__global__ void __maxnreg__(RES_REGS)
+__global__ void __maxnreg__(64)
     k_residual(const __grid_constant__ Dev d, int buf, int stage, double c_stage, int want_dt) {
     // the tables in shared memory: the contractions index them by lane, which
     // the constant cache would serialise
@@ -1391,11 +1388,8 @@ __global__ void __maxnreg__(sizeof(B) == 4 ? 80 : 96)
 // with want_dt the wave speed bound of each side (lambda l / J) raises its
 // member's rmax, as the residual does when it integrates the faces itself.
 // One job per lane.
-#ifndef FACE_REGS
-#define FACE_REGS 80
-#endif
 template <int R, typename Pix, int MODE>
-__global__ void __maxnreg__(FACE_REGS)
+__global__ void __maxnreg__(72)
     k_faces(const __grid_constant__ Dev d, int buf, double c_stage, int want_dt) {
     __shared__ FaceTables ft; // its rows are indexed by lane
     copy_table(ft, &d.tabs->ft);
@@ -1626,154 +1620,6 @@ __device__ int scalar_newton(const Dev& d, const Tables& tb, int64_t k, double J
 }
 
 // ---------------------------------------------------------------------------
-// step start: degree switch (Eq. criteria_p) with mass-exact remap, then
-// H_i(zeta^n), C~_i^n (Eqs. depth_rhs, concentration_rhs) and their sums
-// ---------------------------------------------------------------------------
-template <int R>
-constexpr int begin_smem() {
-    using S = Sz<R>;
-    return 4 * S::ND + 4 * S::NMP + 2 * S::NM * S::NM + 3 * S::NGP + 2 * S::ND;
-}
-
-template <int R, typename Pix, int MODE>
-__global__ void __launch_bounds__(32 * MAXWPB)
-    k_step_begin(const __grid_constant__ Dev d, const __grid_constant__ Tables tb, int do_switch) {
-    using S = Sz<R>;
-    using ST = Site<R, Pix, MODE>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
-    extern __shared__ double smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    double* su = smem + warp * begin_smem<R>();
-    double* pe = su + 4 * ND;    // [NMP] zeta at mass points
-    double* pc = pe + NMP;       // [NMP] c at mass points
-    double* pV = pc + NMP;       // [NMP]
-    double* px = pV + NMP;       // [NMP] scratch products
-    double* tmp = px + NMP;      // [2 NM NM]
-    double* pg = tmp + 2 * NM * NM; // [3][NGP]
-    double* out = pg + 3 * NGP;  // [2][ND]
-    const int64_t n = d.n;
-    if (blockIdx.x == 0) {
-        for (int i = threadIdx.x; i < d.nmemb; i += blockDim.x) d.mb[i].rmax = 0ull;
-        if (threadIdx.x == 0) d.sc->maxits = 0;
-    }
-    for (int64_t k = (int64_t)blockIdx.x * wpb + warp; k < n; k += (int64_t)gridDim.x * wpb) {
-        for (int i = lane; i < 4 * ND; i += 32) su[i] = ufield(d, 0, i / ND, ND)[k * ND + (i % ND)];
-        unsigned cm = d.cmask[k];
-        const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
-        __syncwarp();
-        // zeta and c at the mass points
-        tens_interp<ND1, NM>(tb.Bm, su, tmp, pe, lane);
-        tens_interp<ND1, NM>(tb.Bm, su + 3 * ND, tmp, pc, lane);
-        bool allfull = true;
-        for (int p = lane; p < NMP; p += 32) {
-            if (cm & 1u) pe[p] = su[0];
-            if (cm & 8u) pc[p] = su[3 * ND];
-            double V, A;
-            bool full;
-            ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, pe[p], V, A, full);
-            pV[p] = V;
-            allfull = allfull && full && !zero_bits(A);
-        }
-        allfull = __all_sync(0xffffffffu, allfull);
-        __syncwarp();
-        // r_K = 0 where the smallest wet depth of the mass points is at most
-        // h_lim (a NaN depth never counts, as under fmin)
-        bool low = false;
-        for (int p = lane; p < NMP; p += 32) low = low || pV[p] <= d.hlim;
-        const int flag = (do_switch && __any_sync(0xffffffffu, low)) ? 0 : R;
-        if (flag == 0) {
-            // remap to r_K = 0: mass-exact zeta, GL means of q, tracer-mass-exact c
-            double m = 0.0, tr = 0.0;
-            for (int p = lane; p < NMP; p += 32) {
-                const double w = J * tb.wm[p % NM] * tb.wm[p / NM];
-                m += w * pV[p];
-                tr += w * pV[p] * pc[p];
-            }
-            team_sum2<32>(m, tr, 0xffffffffu);
-            for (int f = 0; f < 3; ++f) {
-                tens_interp<ND1, NG>(tb.Bg, su + (1 + f) * ND, tmp, pg + f * NGP, lane);
-            }
-            double mq[3] = {0.0, 0.0, 0.0};
-            for (int p = lane; p < NGP; p += 32) {
-                const double w = tb.wg[p % NG] * tb.wg[p / NG];
-                for (int f = 0; f < 3; ++f) {
-                    const double v = (cm & (2u << f)) ? su[(1 + f) * ND] : pg[f * NGP + p];
-                    mq[f] += w * v;
-                }
-            }
-            team_sum2<32>(mq[0], mq[1], 0xffffffffu);
-            mq[2] = warp_sum(mq[2]);
-            const double cnew = (m > 1e-14 * J * d.hlim) ? tr / m : mq[2];
-            double emax = -INFINITY;
-            for (int p = lane; p < NMP; p += 32) emax = fmax(emax, pe[p]);
-            emax = warp_max(emax);
-            __syncwarp();
-            if (!(cm & 8u))
-                for (int i = lane; i < ND; i += 32) su[3 * ND + i] = cnew;
-            if (!(cm & 2u))
-                for (int i = lane; i < ND; i += 32) su[ND + i] = mq[0];
-            if (!(cm & 4u))
-                for (int i = lane; i < ND; i += 32) su[2 * ND + i] = mq[1];
-            if (!(cm & 1u)) {
-                double e;
-                if (m <= 0.0) e = -d.zmax[k];
-                else {
-                    e = emax;
-                    scalar_newton<R, Pix, MODE>(d, tb, k, J, m, e, lane);
-                }
-                for (int i = lane; i < ND; i += 32) su[i] = e;
-            }
-            __syncwarp();
-            for (int i = lane; i < 4 * ND; i += 32) {
-                ufield(d, 0, i / ND, ND)[k * ND + (i % ND)] = su[i];
-                if (d.uF) ufieldF(d, 0, i / ND, ND)[k * ND + (i % ND)] = (float)su[i];
-            }
-            cm = 15u;
-            for (int p = lane; p < NMP; p += 32) {
-                pe[p] = su[0];
-                pc[p] = su[3 * ND];
-                double V, A;
-                ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, pe[p], V, A);
-                pV[p] = V;
-            }
-            __syncwarp();
-        }
-        // H_i(zeta^n), C~_i^n and their sums
-        double hb = 0.0, cb = 0.0;
-        for (int p = lane; p < NMP; p += 32) {
-            const double w = J * tb.wm[p % NM] * tb.wm[p / NM];
-            hb += w * pV[p];
-            cb += w * pV[p] * pc[p];
-            px[p] = w * pV[p];
-            pc[p] = px[p] * pc[p]; // c is not needed beyond C~
-        }
-        team_sum2<32>(hb, cb, 0xffffffffu);
-        __syncwarp();
-        tens_test2<ND1, NM>(tb.Bm, px, pc, tmp, tmp + NM * NM, out, out + ND, lane);
-        for (int i = lane; i < ND; i += 32) {
-            d.HN[k * ND + i] = out[i];
-            d.CN[k * ND + i] = out[ND + i];
-        }
-        // the discharges of v^n at the momentum points, the same for every
-        // stage of the step (the stage update reads them rather than
-        // interpolating v^n again; same sums, same constant fields)
-        if (d.qpts) {
-            tens_interp2<ND1, NG>(tb.Bg, su + ND, su + 2 * ND, tmp, tmp + NM * NM, pg, pg + NGP, lane);
-            for (int p = lane; p < 2 * NGP; p += 32)
-                d.qpts[k * 2 * NGP + p] = (cm & (2u << (p / NGP))) ? su[(1 + p / NGP) * ND] : pg[p];
-        }
-        if (lane == 0) {
-            d.HNbar[k] = hb;
-            d.CNbar[k] = cb;
-            d.flag[k] = (uint8_t)flag;
-            d.cmask[k] = (uint8_t)cm;
-            if (d.wet0) d.wet0[k] = (uint8_t)(flag != 0 && allfull);
-        }
-        __syncwarp();
-    }
-}
-
-// ---------------------------------------------------------------------------
 // stage update for one cell: continuity Newton (Eq. newton, Eq. mass_matrix),
 // momentum with the friction-modified mass matrix (Eq. mass_matrix_discharge)
 // inverted as S^-1 D^-1 S^-T (Sec. 3.3), tracer with the depth-weighted mass
@@ -1981,42 +1827,138 @@ __device__ __forceinline__ float chol_subst_rows_f(const float* Mf, float rinv, 
     return bv;
 }
 
+// FP32 inverse of H' = S B^T diag(cw') B S, one row per lane in a[] (ND <= TL):
+// cw' = cw 2^-(ecw - 1022) <= 1 (given as FP32) and S scales the columns of B to
+// norm 1, so the diagonal and every pivot of the elimination is at most 1.
+// Gauss-Jordan in place: step J broadcasts row J through shared memory; with
+// p = 1 / pivot, row i != J loses a_iJ p times it and row J is multiplied by p,
+// written as r_l - (1 - p) r_l, which does not cancel since p >= 1.  The
+// columns rotate by one per step, so that the pivot column is always a[0] and
+// one loop body serves all steps (the unrolled Cholesky with its two
+// substitutions per correction, which this replaces, was three times the
+// instructions, and fetching them stalled the kernel).  buf: 16-byte aligned,
+// 2 NDP + NMP + PR NM floats (NDP = ND rounded up to 4, PR = ND1 (ND1 + 1) / 2).
+// Returns false on a non-positive pivot.
+template <int N>
+__device__ __forceinline__ void read_row(const float* b, float (&r)[N]) {
+#pragma unroll
+    for (int l = 0; l < N; l += 4) {
+        const float4 v = *(const float4*)(b + l);
+        r[l] = v.x;
+        r[l + 1] = v.y;
+        r[l + 2] = v.z;
+        r[l + 3] = v.w;
+    }
+}
+template <int ND1, int NM, int TL>
+__device__ __forceinline__ bool mass_inverse_f(const FxStage& fs, float* buf, float (&a)[ND1 * ND1],
+                                               int lane, unsigned tm) {
+    constexpr int ND = ND1 * ND1, NDP = (ND + 3) / 4 * 4, PR = ND1 * (ND1 + 1) / 2;
+    static_assert(ND <= TL, "one row per lane");
+    const float* cwf = buf + 2 * NDP;  // [NMP], written by the caller
+    float* Y = buf + 2 * NDP + NM * NM; // [PR][NM]: contracted over the points of a row
+    __syncwarp(tm);
+#pragma unroll 1
+    for (int i = lane; i < PR * NM; i += TL) {
+        const int pr = i / NM, be = i % NM;
+        float s = 0.0f;
+#pragma unroll
+        for (int al = 0; al < NM; ++al) s += cwf[al + NM * be] * fs.BB[pr][al];
+        Y[i] = s;
+    }
+    __syncwarp(tm);
+    const int row = lane < ND ? lane : 0, ar = row % ND1, br = row / ND1;
+    auto pair = [](int x, int y) { return x > y ? x * (x + 1) / 2 + y : y * (y + 1) / 2 + x; };
+#pragma unroll
+    for (int t = 0; t < ND; ++t) a[t] = 0.0f;
+#pragma unroll
+    for (int be = 0; be < NM; ++be) {
+        float y[ND1], q[ND1];
+#pragma unroll
+        for (int c = 0; c < ND1; ++c) {
+            y[c] = Y[pair(ar, c) * NM + be];
+            q[c] = fs.BB[pair(br, c)][be];
+        }
+#pragma unroll
+        for (int t = 0; t < ND; ++t) a[t] += y[t % ND1] * q[t / ND1];
+    }
+    bool ok = true;
+#pragma unroll 1
+    for (int J = 0; J < ND; ++J) {
+        float* rb = buf + (J & 1) * NDP;
+        if (lane == J) {
+#pragma unroll
+            for (int l = 0; l < NDP; l += 4)
+                *(float4*)(rb + l) = make_float4(a[l], l + 1 < ND ? a[l + 1] : 0.0f,
+                                                 l + 2 < ND ? a[l + 2] : 0.0f,
+                                                 l + 3 < ND ? a[l + 3] : 0.0f);
+        }
+        __syncwarp(tm);
+        float r[NDP];
+        read_row<NDP>(rb, r);
+        ok = ok && r[0] > 0.0f;
+        const float p = __fdividef(1.0f, r[0]);
+        const float f = lane == J ? 1.0f - p : a[0] * p;
+#pragma unroll
+        for (int l = 1; l < ND; ++l) a[l - 1] = fmaf(-f, r[l], a[l]);
+        a[ND - 1] = lane == J ? p : -f;
+    }
+    __syncwarp(tm);
+    return ok;
+}
+
 // Solve H x = b for the depth-weighted mass matrix H = B^T diag(cw) B (the
 // tracer matrix of Eq. mass_matrix_concentration, or the masked Jacobian of
 // Eq. mass_matrix) by mixed-precision iterative refinement: H is assembled and
-// factored in FP32, each correction is solved in FP32, and the residual
-// b - H x is formed matrix-free by sum factorisation in block fixed point (60
-// bits of the largest term, on the integer pipe; in FP64 arithmetic the two
-// residuals were a third of the stage update's FP64 instructions), x being
-// held as a fixed-point number too.  The sweeps stop when a correction, or the
-// next one as predicted from the contraction of the last two, is below 1e-15
-// of x; if that does not happen within 6 sweeps (an ill-conditioned near-dry
-// cell), the FP64 Cholesky decides.  x in place of b on return.  Scratch: Mf
-// [ND ND], Yf [ND1 ND1 NM] (float), digit pairs xd [ND], qd [NMP], td [2 NMP],
-// M, Y, inv (double, fallback: Y and inv may overlay xd, qd and td).
+// inverted in FP32, each correction is one FP32 product with the inverse, and
+// the residual b - H x is formed matrix-free by sum factorisation in block fixed
+// point (60 bits of the largest term, on the integer pipe; in FP64 arithmetic
+// the two residuals were a third of the stage update's FP64 instructions), x
+// being held as a fixed-point number too.  The sweeps stop when a correction, or
+// the next one as predicted from the contraction of the last two, is below
+// 1e-15 of x; if that does not happen within 6 sweeps (an ill-conditioned
+// near-dry cell), the FP64 Cholesky decides.  x in place of b on return.
+// Scratch: buf (mass_inverse_f's, and 2 floats to align it), digit pairs xd [ND], qd [NMP], td [2 NMP], M,
+// Y, inv (double, fallback: M may overlay buf, Y and inv xd, qd and td).
 template <int ND1, int NM, int TL = 32>
 __device__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const double* cw, double* b,
-                                 float* Mf, float* Yf, int2* xd, int2* qd, int2* td, double* M,
-                                 double* Y, double* inv, int lane, unsigned tm = 0xffffffffu) {
-    constexpr int ND = ND1 * ND1, NMP = NM * NM;
-    static_assert(ND <= TL, "one unknown per lane");
+                                 float* buf, int2* xd, int2* qd, int2* td, double* M, double* Y,
+                                 double* inv, int lane, unsigned tm = 0xffffffffu) {
+    constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4;
+    buf = (float*)(((uintptr_t)buf + 15) & ~(uintptr_t)15);
     int2* cwd = td + NM * NM;
     const double bi = lane < ND ? b[lane] : 0.0;
     unsigned mc = 0;
     for (int p = lane; p < NMP; p += TL) mc = max(mc, fx::mag(cw[p]));
     const int ecw = fx::block_exp(__reduce_max_sync(tm, mc)), eb = team_exp(bi, tm);
-    float rinv; // the lane's reciprocal FP32 pivot
-    bool ok = mass_factor_rows_f<ND1, NM, TL>(fs, cw, Yf, Mf, rinv, lane, tm);
+    for (int p = lane; p < NMP; p += TL) {
+        const int2 c = fx::split(fx::from_double(cw[p], ecw));
+        cwd[p] = c;
+        buf[2 * NDP + p] = (float)c.x * (1.0f / (float)(1 << (fx::FB - fx::LB)));
+    }
+    float a[ND]; // the lane's row of the inverse
+    // the inverse's scales: H = 2^(ecw - 1022) S^-1 H' S^-1
+    const int se = 127 - (ecw - 1022);
+    bool ok = mass_inverse_f<ND1, NM, TL>(fs, buf, a, lane, tm) && se > 0 && se < 255;
     long long X = 0; // the lane's component of x
     int ex = fx::EMIN;
     if (ok) {
-        for (int p = lane; p < NMP; p += TL) cwd[p] = fx::split(fx::from_double(cw[p], ecw));
         ok = false;
+        const float si = lane < ND ? fs.sc[lane % ND1] * fs.sc[lane / ND1] : 0.0f;
+        const float so = si * __uint_as_float((unsigned)se << 23);
         float rv = fx::to_float(fx::from_double(bi, eb), eb);
         float dprev = 0.0f; // max |correction| / max |x| of the previous sweep
+#pragma unroll 1
         for (int sweep = 0; sweep < 6; ++sweep) {
             // the lane's component of the correction
-            const float v = chol_subst_rows_f<ND, TL>(Mf, rinv, rv, lane, tm);
+            float* rb = buf + (sweep & 1) * NDP;
+            if (lane < ND) rb[lane] = rv * si;
+            __syncwarp(tm);
+            float r[NDP], v = 0.0f;
+            read_row<NDP>(rb, r);
+#pragma unroll
+            for (int j = 0; j < ND; ++j) v += a[j] * r[j];
+            v *= so;
             const float da = lane < ND ? fabsf(v) : 0.0f;
             const unsigned dbits = __reduce_max_sync(tm, __float_as_uint(da)); // a NaN is the largest
             const int ev = fx::block_exp_f(dbits);
@@ -2051,13 +1993,12 @@ __device__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const doub
             rv = lane < ND ? fx::to_float(fx::from_double(bi, e) - (R >> min(e - er, 63)), e) : 0.0f;
         }
     }
+    __syncwarp(tm);
     if (ok) {
-        __syncwarp(tm);
         if (lane < ND) b[lane] = fx::to_double(X, ex);
         __syncwarp(tm);
         return true;
     }
-    __syncwarp(tm);
     assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
     return chol_solve<ND, TL>(M, b, inv, lane, tm);
 }
@@ -2191,6 +2132,191 @@ __device__ __forceinline__ const float (*tab_Gi(const FxStage& s, float))[MXN] {
 __device__ __forceinline__ const int2 (*tab_GiT(const FxStage& s, double))[MXN] { return s.GiT; }
 __device__ __forceinline__ const float (*tab_GiT(const FxStage& s, float))[MXN] { return s.GiTF; }
 
+// ---------------------------------------------------------------------------
+// step start: degree switch (Eq. criteria_p) with mass-exact remap, then
+// H_i(zeta^n), C~_i^n (Eqs. depth_rhs, concentration_rhs) and their sums
+// ---------------------------------------------------------------------------
+// One cell per team of 16 lanes, node i on lane i, mass points i and i + 16, as
+// in the stage update; the contractions in block fixed point.
+template <int R>
+struct BeginFx {
+    using S = Sz<R>;
+    static constexpr int TL = 16, PP = (S::NMP + TL - 1) / TL;
+    // 8-byte words per team: digit pairs of nodal fields with scratch [4 ND], of
+    // two mass-point fields [2 NMP], scratch [NMP]
+    static constexpr int W = 4 * S::ND, words = W + 3 * S::NMP;
+    static_assert(S::ND <= TL && S::ND1 * S::NM <= S::NMP, "one node per lane");
+};
+
+template <int R, typename Pix, int MODE>
+__global__ void __maxnreg__(64)
+    k_step_begin(const __grid_constant__ Dev d, int do_switch) {
+    using S = Sz<R>;
+    using L = BeginFx<R>;
+    using ST = Site<R, Pix, MODE>;
+    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
+    constexpr int TL = L::TL, PP = L::PP;
+    __shared__ FxStage fs;
+    copy_table(fs, &d.tabs->fs);
+    const Tables& tb = *d.tabs;
+    extern __shared__ double smem[];
+    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
+    const unsigned tm = 0xFFFFu << (threadIdx.x & 16);
+    int2* w = (int2*)(smem + team * L::words);
+    int2* qd = w + L::W; // [2][NMP]
+    int2* qt = qd + 2 * NMP;
+    const int64_t n = d.n;
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i < d.nmemb; i += blockDim.x) d.mb[i].rmax = 0ull;
+        if (threadIdx.x == 0) d.sc->maxits = 0;
+    }
+    const bool act = lane < ND;
+    const int node = act ? lane : 0;
+    const double wn = act ? fs.wn[node % ND1] * fs.wn[node / ND1] : 0.0;
+    double wm2[PP];
+#pragma unroll
+    for (int j = 0; j < PP; ++j) {
+        const int p = lane + j * TL;
+        wm2[j] = p < NMP ? fs.wm[p % NM] * fs.wm[p / NM] : 0.0;
+    }
+    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
+        const size_t idx = (size_t)k * ND + node;
+        double u[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) u[f] = ufield(d, 0, f, ND)[idx];
+        unsigned cm = d.cmask[k];
+        const double J = d.hxhy[2 * k] * d.hxhy[2 * k + 1];
+        // zeta and c at the lane's mass points
+        double pe[PP], pc[PP], V[PP];
+        {
+            const int ez = team_exp(act ? u[0] : 0.0, tm), ec = team_exp(act ? u[3] : 0.0, tm);
+            if (act) {
+                w[lane] = fx::split(fx::from_double(u[0], ez));
+                w[ND + lane] = fx::split(fx::from_double(u[3], ec));
+            }
+            const double z0 = __shfl_sync(tm, u[0], 0, TL), c0 = __shfl_sync(tm, u[3], 0, TL);
+            __syncwarp(tm);
+            fx_tens<ND1, NM, TL>(fs.Bm, w, qt, lane, tm, [&](int it, int, long long X) {
+                pe[it] = (cm & 1u) ? z0 : fx::to_double(X, ez + 2 * fs.tBm);
+            });
+            fx_tens<ND1, NM, TL>(fs.Bm, w + ND, qd, lane, tm, [&](int it, int, long long X) {
+                pc[it] = (cm & 8u) ? c0 : fx::to_double(X, ec + 2 * fs.tBm);
+            });
+        }
+        bool allfull = true, low = false;
+#pragma unroll
+        for (int j = 0; j < PP; ++j) {
+            const int p = lane + j * TL;
+            V[j] = 0.0;
+            if (p < NMP) {
+                double A;
+                bool full;
+                ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, pe[j], V[j], A, full);
+                allfull = allfull && full && !zero_bits(A);
+                // r_K = 0 where the smallest wet depth of the mass points is at most
+                // h_lim (a NaN depth never counts, as under fmin)
+                low = low || V[j] <= d.hlim;
+            }
+        }
+        allfull = __all_sync(tm, allfull);
+        low = __any_sync(tm, low);
+        const int flag = (do_switch && low) ? 0 : R;
+        if (flag == 0) {
+            // remap to r_K = 0: mass-exact zeta, GL means of q, tracer-mass-exact c
+            double m = 0.0, tr = 0.0;
+            long long ek = (long long)0x8000000000000000ull;
+#pragma unroll
+            for (int j = 0; j < PP; ++j) {
+                if (lane + j * TL >= NMP) continue;
+                const double wv = J * wm2[j] * V[j];
+                m += wv;
+                tr += wv * pc[j];
+                if (!nan_bits(pe[j])) ek = okey(pe[j]) > ek ? okey(pe[j]) : ek;
+            }
+            team_sum2<TL>(m, tr, tm);
+            double mq[3] = {wn * u[1], wn * u[2], wn * u[3]};
+            team_sum2<TL>(mq[0], mq[1], tm);
+            mq[2] = team_sum<TL>(mq[2], tm);
+            const double cnew = (m > 1e-14 * J * d.hlim) ? tr / m : mq[2];
+            ek = team_max_key<TL>(ek, tm);
+            if (!(cm & 8u)) u[3] = cnew;
+            if (!(cm & 2u)) u[1] = mq[0];
+            if (!(cm & 4u)) u[2] = mq[1];
+            if (!(cm & 1u)) {
+                double e = ek == (long long)0x8000000000000000ull ? -INFINITY : of_okey(ek);
+                if (m <= 0.0) e = -d.zmax[k];
+                else scalar_newton<R, Pix, MODE, TL>(d, tb, k, J, m, e, lane, tm);
+                u[0] = e;
+            }
+            if (act) {
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    ufield(d, 0, f, ND)[idx] = u[f];
+                    if (d.uF) ufieldF(d, 0, f, ND)[idx] = f32_of(u[f]);
+                }
+            }
+            cm = 15u;
+            const double z0 = __shfl_sync(tm, u[0], 0, TL), c0 = __shfl_sync(tm, u[3], 0, TL);
+#pragma unroll
+            for (int j = 0; j < PP; ++j) {
+                const int p = lane + j * TL;
+                pc[j] = c0;
+                double A;
+                if (p < NMP) ST::VA(d, tb, k, SET_MASS, p % NM, p / NM, z0, V[j], A);
+            }
+        }
+        // H_i(zeta^n), C~_i^n and their sums
+        double hb = 0.0, cb = 0.0, hv[PP];
+        unsigned mh = 0, mc = 0;
+#pragma unroll
+        for (int j = 0; j < PP; ++j) {
+            hv[j] = J * wm2[j] * V[j];
+            if (lane + j * TL >= NMP) { hv[j] = 0.0; pc[j] = 0.0; }
+            pc[j] *= hv[j]; // c is not needed beyond C~
+            hb += hv[j];
+            cb += pc[j];
+            mh = max(mh, fx::mag(hv[j]));
+            mc = max(mc, fx::mag(pc[j]));
+        }
+        team_sum2<TL>(hb, cb, tm);
+        const int eh = fx::block_exp(__reduce_max_sync(tm, mh)), ec = fx::block_exp(__reduce_max_sync(tm, mc));
+        __syncwarp(tm);
+#pragma unroll
+        for (int j = 0; j < PP; ++j) {
+            if (lane + j * TL >= NMP) continue;
+            qd[lane + j * TL] = fx::split(fx::from_double(hv[j], eh));
+            qd[NMP + lane + j * TL] = fx::split(fx::from_double(pc[j], ec));
+        }
+        __syncwarp(tm);
+        fx_tens<NM, ND1, TL>(fs.BmT, qd, qt, lane, tm, [&](int, int i, long long X) {
+            d.HN[k * ND + i] = fx::to_double(X, eh + 2 * fs.tBmT);
+        });
+        __syncwarp(tm);
+        fx_tens<NM, ND1, TL>(fs.BmT, qd + NMP, qt, lane, tm, [&](int, int i, long long X) {
+            d.CN[k * ND + i] = fx::to_double(X, ec + 2 * fs.tBmT);
+        });
+        // the discharges of v^n at the momentum points, the same for every
+        // stage of the step (the stage update reads them rather than
+        // interpolating v^n again)
+        if (d.qpts) {
+            double q[2] = {u[1], u[2]};
+            if ((cm & 6u) != 6u) square<ND1, 2>(fs.Bg, fs.tBg, q, w, lane, tm);
+            if (act) {
+                d.qpts[k * 2 * NGP + lane] = (cm & 2u) ? u[1] : q[0];
+                d.qpts[k * 2 * NGP + NGP + lane] = (cm & 4u) ? u[2] : q[1];
+            }
+        }
+        if (lane == 0) {
+            d.HNbar[k] = hb;
+            d.CNbar[k] = cb;
+            d.flag[k] = (uint8_t)flag;
+            d.cmask[k] = (uint8_t)cm;
+            if (d.wet0) d.wet0[k] = (uint8_t)(flag != 0 && allfull);
+        }
+        __syncwarp(tm);
+    }
+}
+
 // The stage update: one cell per team of 16 lanes, node i and momentum point i
 // on lane i ((r+1)^2 <= 16), mass points i and i + 16.  The FP64 pipe bounds
 // it, so every contraction (the Newton evaluations, the mass inverse, the
@@ -2213,12 +2339,13 @@ struct StageFx {
     static constexpr int words = W + Q + CW + BV + UN;
     static_assert(S::ND <= TL && S::NGP == S::ND, "one node and one momentum point per lane");
     static_assert(S::ND1 * S::ND1 * S::NM <= W, "fallback Y");
+    static_assert(2 + 2 * ((S::ND + 3) / 4 * 4) + S::NMP + S::ND1 * (S::ND1 + 1) / 2 * S::NM <= 2 * UN,
+                  "the FP32 inverse's scratch");
 };
 
 template <int R, typename Pix, int MODE, typename B>
-__global__ void __maxnreg__(96)
-    k_stage(const __grid_constant__ Dev d, const __grid_constant__ Tables tb,
-            const __grid_constant__ StageArgs sa) {
+__global__ void __maxnreg__(R == 1 ? 128 : 96)
+    k_stage(const __grid_constant__ Dev d, const __grid_constant__ StageArgs sa) {
     using S = Sz<R>;
     using L = StageFx<R>;
     using ST = Site<R, Pix, MODE>;
@@ -2227,6 +2354,7 @@ __global__ void __maxnreg__(96)
     constexpr bool F64 = sizeof(B) == sizeof(double);
     __shared__ FxStage fs;
     copy_table(fs, &d.tabs->fs);
+    const Tables& tb = *d.tabs;
     extern __shared__ double smem[];
     const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
     const unsigned tm = 0xFFFFu << (threadIdx.x & 16); // the team's lanes
@@ -2236,7 +2364,7 @@ __global__ void __maxnreg__(96)
     double* cw = (double*)(qd + L::Q); // [NMP] weights of a mass-matrix solve
     double* bv = cw + L::CW;           // [ND] its right-hand side and solution
     double* un = bv + L::BV;
-    float* Mf = (float*)un;            // [ND ND]
+    float* Mf = (float*)un;            // [ND ND] (FP32-bulk tracer), or the FP32 inverse's scratch
     float* Yf = Mf + ND * ND;          // [ND1 ND1 NM]
     double* M = un;                    // [ND ND] (fallback)
     const int64_t n = d.n;
@@ -2374,8 +2502,8 @@ __global__ void __maxnreg__(96)
                     for (int j = 0; j < PP; ++j)
                         if (lane + j * TL < NMP) cw[lane + j * TL] = J * wm2[j] * A[j];
                     __syncwarp(tm);
-                    if (!solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, w, qd, qt, M,
-                                                       (double*)w, (double*)qd, lane, tm)) {
+                    if (!solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, w, qd, qt, M, (double*)w,
+                                                       (double*)qd, lane, tm)) {
                         scalar = true;
                         break;
                     }
@@ -2531,8 +2659,8 @@ __global__ void __maxnreg__(96)
                 if (lane + j * TL < NMP) cw[lane + j * TL] = J * wm2[j] * V[j];
             __syncwarp(tm);
             if constexpr (F64)
-                solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, w, qd, qt, M, (double*)w,
-                                              (double*)qd, lane, tm);
+                solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, w, qd, qt, M, (double*)w, (double*)qd,
+                                              lane, tm);
             else
                 solve_tracer_bulk<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, qt, M, (double*)w,
                                                (double*)qd, cert, T, lane, tm);
