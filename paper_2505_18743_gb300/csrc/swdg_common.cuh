@@ -370,35 +370,28 @@ __device__ __forceinline__ double f64_of(float v) {
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// x^(-1/3) of a positive double: an FP32 reciprocal-cube-root seed refined by
-// two Newton-Raphson steps for z^-3 = x in FP64, z <- z + z (1 - x z^3) / 3
-// (quadratic convergence, no division: ~1e-7 -> ~1e-14 -> rounding).  Values
-// outside the FP32 seed's comfortable range take 1 / cbrt(x).
+// x^(-1/3) of a positive double: an FP32 reciprocal-cube-root seed (~2^-22)
+// refined by one third-order (Halley) step for z^-3 = x in FP64,
+// z (1 + e/3 + 2/9 e^2), e = 1 - x z^3 (no division).  Values outside the FP32
+// seed's comfortable range take 1 / cbrt(x).
+__device__ __noinline__ inline double inv_cbrt_any(double x) { return 1.0 / cbrt(x); }
+__device__ __noinline__ inline double sqrt_any(double x) { return sqrt(x); }
 __device__ __forceinline__ double inv_cbrt(double x) {
-    if (!f32_range(x)) return 1.0 / cbrt(x);
-    double z = f64_of(rcbrtf(f32_trunc(x)));
-    constexpr double third = 1.0 / 3.0;
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const double e = fma(-x, z * z * z, 1.0);
-        z = fma(z * third, e, z);
-    }
-    return z;
+    if (!f32_range(x)) return inv_cbrt_any(x);
+    const double z = f64_of(rcbrtf(f32_trunc(x)));
+    const double e = fma(-x, z * z * z, 1.0);
+    return fma(fma(e, 2.0 / 9.0, 1.0 / 3.0), z * e, z);
 }
 
-// sqrt(x), x >= 0, in six FP64 instructions (CUDA's takes nine): Goldschmidt's
-// coupled iteration for sqrt(x) and 1 / (2 sqrt(x)) from an FP32 seed, then one
-// Newton correction of the root (within 1 ulp).  Values outside the FP32
-// seed's comfortable range, 0 and NaN among them, take sqrt itself.
+// sqrt(x), x >= 0, in five FP64 instructions (CUDA's takes nine): the same kind
+// of step from an FP32 seed y of x^(-1/2), x y (1 + e/2 + 3/8 e^2),
+// e = 1 - x y^2 (within 1 ulp).  Values outside the FP32 seed's comfortable
+// range, 0 and NaN among them, take sqrt itself.
 __device__ __forceinline__ double sqrt_fast(double x) {
-    if (!f32_range(x)) return sqrt(x);
+    if (!f32_range(x)) return zero_bits(x) ? 0.0 : sqrt_any(x);
     const double y = f64_of(rsqrtf(f32_trunc(x)));
-    double s = x * y;
-    double h = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y)); // y / 2
-    const double r = fma(-s, h, 0.5);
-    s = fma(s, r, s);
-    h = fma(h, r, h);
-    return fma(fma(-s, s, x), h, s);
+    const double t = x * y, e = fma(-t, y, 1.0);
+    return fma(t * e, fma(e, 0.375, 0.5), t);
 }
 
 // 1/h and sqrt(g h) of a wet depth (h >= eps) from one root y = h^(-1/2): an
@@ -445,30 +438,40 @@ __device__ __forceinline__ T gamma_manning(T n, T h, T qx, T qy, T g, T eps) {
     }
 }
 
-// the velocity factor and the Manning coefficient of one point together: on
-// the wet branch (h >= eps, where h_des = h) both come from one root, in FP64
-// z = h^(-1/3) with 1/h = z^3 and h^(-7/3) = z^7 (1/h by division where
-// there is no friction), otherwise from 1/h with h^(-7/3) = (1/h)^2
-// cbrt(1/h); below eps as vel_factor and gamma_manning
+// the velocity factor of one point and, with friction, |q| h_des^(-7/3) (the
+// Manning coefficient without g n^2), in FP64
+// (h < eps, or no friction: rare, not inlined)
+struct VelGam {
+    double fv, gm;
+};
+__device__ __noinline__ inline VelGam vel_friction_any(double h, double qx, double qy, bool friction,
+                                                       double eps) {
+    if (h >= eps) return {1.0 / h, 0.0};
+    return {vel_factor<double>(h, eps), friction ? gamma_manning<double>(1.0, h, qx, qy, 1.0, eps) : 0.0};
+}
+__device__ __forceinline__ void vel_friction(double h, double qx, double qy, bool friction, double eps,
+                                             double& fv, double& gm) {
+    // h >= eps on the bit patterns (h is not negative, eps > 0; a NaN depth stays
+    // on this branch), off the FP64 pipe
+    if (friction && __double_as_longlong(h) >= __double_as_longlong(eps)) {
+        // 1/h = z^3 from z = h^(-1/3) (a few ulp from the rounded quotient, no
+        // FP64 division); h^(-7/3) = z^7
+        const double z = inv_cbrt(h), rh = z * z * z;
+        fv = rh;
+        gm = sqrt_fast(qx * qx + qy * qy) * (rh * rh) * z;
+    } else {
+        const VelGam r = vel_friction_any(h, qx, qy, friction, eps);
+        fv = r.fv;
+        gm = r.gm;
+    }
+}
+
+// the velocity factor and the Manning coefficient of one point together (the
+// FP32-bulk path): on the wet branch (h >= eps, where h_des = h) both come from
+// 1/h with h^(-7/3) = (1/h)^2 cbrt(1/h); below eps as vel_factor and
+// gamma_manning
 template <typename T>
 __device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& fv, T& gam) {
-    if constexpr (std::is_same<T, double>::value) {
-        // h >= eps on the bit patterns (h is not negative, eps > 0; a NaN depth
-        // stays on this branch), off the FP64 pipe
-        if (__double_as_longlong(h) >= __double_as_longlong(eps)) {
-            if (zero_bits(n)) {
-                fv = 1.0 / h;
-                gam = 0.0;
-            } else {
-                // with friction, 1/h = z^3 from z = h^(-1/3) (a few ulp from the
-                // rounded quotient, no FP64 division); gamma ~ z^7
-                const double z = inv_cbrt(h), rh = z * z * z;
-                fv = rh;
-                gam = g * n * n * sqrt_fast(qx * qx + qy * qy) * (rh * rh) * z;
-            }
-            return;
-        }
-    }
     if (h >= eps && h > T(0)) {
         const T rh = T(1) / h;
         fv = rh;

@@ -20,7 +20,8 @@ struct Launchers {
     }
     static constexpr size_t begin_b = 2 * sizeof(double) * BeginFx<R>::words; // two cells per warp
     // k_stage runs two cells per warp (a team of 16 lanes each)
-    static constexpr size_t stage_b = 2 * sizeof(double) * StageFx<R>::words;
+    static constexpr size_t stage_b =
+        2 * sizeof(double) * StageFx<R>::words(sizeof(B) != sizeof(double));
     static constexpr size_t diag_b = sizeof(double) * (2 * S::ND + 2 * S::NMP + 2 * S::NM * S::NM);
     static constexpr size_t vjp_b = sizeof(double) * vjp_smem<R>();
     static constexpr size_t svjp_b = 2 * sizeof(double) * stage_vjp_smem<R>(); // two cells per warp
@@ -34,8 +35,12 @@ struct Launchers {
             // 32 / TL cells per warp: no more blocks than their cells
             const int cpb = s.wpb * 32 / ResFx<R>::TL;
             const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
-            k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage, c_stage,
-                                                                              want_dt);
+            if (MODE == 0 && !d.fflux)
+                k_residual<R, Pix, 0, true><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage,
+                                                                                     c_stage, want_dt);
+            else
+                k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage, c_stage,
+                                                                                  want_dt);
         } else {
             k_residual_bulk<R, Pix, MODE, B><<<s.grid, 32 * s.wpb, res_b * s.wpb, st>>>(
                 d, buf, stage, c_stage, want_dt);
@@ -104,6 +109,8 @@ struct Launchers {
                                     (int)(per_warp * MAXWPB)) == cudaSuccess;
     }
     static bool prepare() {
+        if constexpr (F64)
+            if (!opt_in(k_residual<R, Pix, 0, true>, res_b)) return false;
         return opt_in(residual_kernel(), res_b) &&
                opt_in(k_step_begin<R, Pix, MODE>, begin_b) &&
                opt_in(k_stage<R, Pix, MODE, B>, stage_b) &&

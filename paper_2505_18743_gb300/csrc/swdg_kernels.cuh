@@ -726,10 +726,12 @@ __device__ __forceinline__ void side_flux(const B raw[4], B pres, bool own_first
 // integer pipe too.  A team of TL lanes takes a cell, one volume point per
 // lane: 32 lanes at r = 3 (25 points), 16 at r = 2 (16 points), 8 at r = 1
 // (4 points), so that the FP64 instructions of the points serve 1, 2 or 4
-// cells at once.  The per-point values carry the geometric factors of their
-// test integral (h_y for d/dxi, h_x for d/deta, J for values), the test tables
-// the quadrature weights, so the parts of one residual component share a block
-// exponent and are summed as integers.
+// cells at once.  The products of the point values (fluxes, pressure, friction,
+// tracer) are formed from digit pairs as well: the factors convert instead of
+// the products, four values a point instead of twelve, and the FP64
+// instructions of a cell fall from 60 to 30.  The test tables carry the
+// quadrature weights; the geometric factors h_y of d/dxi and h_x of d/deta enter
+// after the integration.
 template <int R>
 struct ResFx {
     using S = Sz<R>;
@@ -740,15 +742,20 @@ struct ResFx {
     // 8-byte words per team, two regions: nodal digits and x-contractions, then
     // the y-test sums; point values, then the face values (with the nodal values
     // where the faces are integrated inline)
-    static constexpr int UD = 4 * S::ND, TX = 6 * NE, XP = 12 * S::NVP, SY = 10 * NE,
+    static constexpr int UD = 4 * S::ND, TX = 6 * NE, XP = 11 * S::NVP, SY = 11 * NE,
                          FD = 32 * S::NM;
     static constexpr int RA = UD + TX > SY ? UD + TX : SY, RB = XP > FD + UD ? XP : FD + UD;
-    static constexpr int words = RA + RB + 4;
+    static constexpr int words = RA + RB + 12; // and 4 nodal values, 16 block exponents
     static_assert(S::NVP <= TL && S::ND <= SUB, "one point per lane");
 };
 
-template <int R, typename Pix, int MODE>
-__global__ void __maxnreg__(64)
+#ifndef RES_REGS
+#define RES_REGS 64
+#endif
+// INL: the cell integrates its faces itself (the allocation-free entry, which has
+// no slot buffer); a kernel of its own, so that the other's code stays small
+template <int R, typename Pix, int MODE, bool INL = false>
+__global__ void __maxnreg__(RES_REGS)
     k_residual(const __grid_constant__ Dev d, int buf, int stage, double c_stage, int want_dt) {
     // the tables in shared memory: the contractions index them by lane, which
     // the constant cache would serialise
@@ -766,10 +773,11 @@ __global__ void __maxnreg__(64)
         TL == 32 ? 0xffffffffu : ((1u << (TL & 31)) - 1u) << (threadIdx.x & 31 & ~(TL - 1));
     int2* ud = (int2*)(smem + team * L::words); // [4][ND]
     int2* sx = ud + L::UD;                      // [6][ND1][NV]: zeta (Bv, Dv), qx, qy, c (Bv), c (Dv)
-    int2* sy = ud;                              // [10][NV][ND1]
-    int2* xp = ud + L::RA;                      // [12][NVP]
+    int2* sy = ud;                              // [11][NV][ND1]
+    int2* xp = ud + L::RA;                      // [11][NVP]
     int2* fd = xp;                              // [4 fields][2 halves][4 faces][NM]
     double* c0 = (double*)(xp + L::RB);         // [4] first nodal value of each field
+    int* es = (int*)(c0 + 4); // block exponents: fields 0..3, faces 4..7, xi-parts 8..11, eta-parts 12..15
     double* fh = (double*)fd;                   // the face values before their conversion
     double* su = fh + L::FD;                    // [4][ND] (inline faces only)
     const double g = d.g, eps = d.eps;
@@ -782,21 +790,20 @@ __global__ void __maxnreg__(64)
     for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
         const unsigned cm = d.cmask[(size_t)buf * n + k];
         const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1];
-        int eu[4]; // block exponents of the nodal fields
-#pragma unroll
+#pragma unroll 1
         for (int ps = 0; ps < 4 / L::FPP; ++ps) {
             const int sub = lane / L::SUB, f = ps * L::FPP + sub, node = lane % L::SUB;
             const double v = node < ND ? ufield(d, buf, f, ND)[k * ND + node] : 0.0;
-            int e = 0;
+            unsigned m = fx::mag(v);
 #pragma unroll
-            for (int s = 0; s < L::FPP; ++s) {
-                const int eb = fx::block_exp(__reduce_max_sync(tm, sub == s ? fx::mag(v) : 0u));
-                eu[ps * L::FPP + s] = eb;
-                e = sub == s ? eb : e;
-            }
+            for (int o = 1; o < L::SUB; o <<= 1) m = max(m, __shfl_xor_sync(tm, m, o));
+            const int e = fx::block_exp(m);
             if (node < ND) {
                 ud[f * ND + node] = fx::split(fx::from_double(v, e));
-                if (node == 0) c0[f] = v;
+                if (node == 0) {
+                    c0[f] = v;
+                    es[f] = e;
+                }
             }
         }
         unsigned fi[4]; // indexed by constants only (registers)
@@ -809,6 +816,7 @@ __global__ void __maxnreg__(64)
         // x-contractions: zeta (value, d/dxi), qx, qy, c, and c's d/dxi for the
         // tracer numerical diffusion (Eq. numdiff)
         const double nu = d.nu_c ? d.nu_c[k] : 0.0;
+#pragma unroll 1
         for (int i = lane; i < (nu != 0.0 ? 6 : 5) * NE; i += TL) {
             const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
             const int2* T = (f == 1 || f == 5) ? tx.Dv[al] : tx.Bv[al];
@@ -819,10 +827,13 @@ __global__ void __maxnreg__(64)
             sx[i] = fx::split(s.get());
         }
         __syncwarp(tm);
-        // y-contraction and pointwise physics, one volume point per lane
-        int ex[5]; // block exponents of F, R, Gx, Gy, L
+        // y-contraction and pointwise physics, one volume point per lane.  Only the
+        // depth's powers, |q| and the velocities are formed in FP64; the products
+        // are products of digit pairs, with the exponents below
+        const double man = d.manning[k];
+        int eL[2]; // exponents of Lx, Ly
         {
-            double X[12];
+            long long Z, ZX, ZY, QX, QY, C;
             {
                 fx::Acc az, azx, azy, aqx, aqy, ac;
 #pragma unroll
@@ -836,102 +847,134 @@ __global__ void __maxnreg__(64)
                     aqy.mac(Tb, s[3 * NE]);
                     ac.mac(Tb, s[4 * NE]);
                 }
-                // a constant field is that constant exactly
-                const double z = (cm & 1u) ? c0[0] : fx::to_double(az.get(), eu[0] + tBB);
-                const double zx = (cm & 1u) ? 0.0 : fx::to_double(azx.get(), eu[0] + tBD);
-                const double zy = (cm & 1u) ? 0.0 : fx::to_double(azy.get(), eu[0] + tBD);
-                const double qx = (cm & 2u) ? c0[1] : fx::to_double(aqx.get(), eu[1] + tBB);
-                const double qy = (cm & 4u) ? c0[2] : fx::to_double(aqy.get(), eu[2] + tBB);
-                const double c = (cm & 8u) ? c0[3] : fx::to_double(ac.get(), eu[3] + tBB);
-                double h = 0.0, A;
-                if (pt) ST::VA(d, tb, k, SET_VOL, pal, pbe, z, h, A);
-                double fv, gam;
-                vel_gamma<double>(d.manning[k], h, qx, qy, g, eps, fv, gam);
-                const double ux = fv * qx, uy = fv * qy;
-                X[0] = hy * qx;
-                X[1] = hx * qy;
-                X[2] = c * X[0];
-                X[3] = c * X[1];
-                if (nu != 0.0 && !(cm & 8u)) {
-                    // -nu h grad c . grad psi: the reference derivatives of c at the point
-                    fx::Acc acx, acy;
-#pragma unroll
-                    for (int b = 0; b < ND1; ++b) {
-                        acx.mac(tx.Bv[pbe][b], sx[(5 * ND1 + b) * NV + pal]);
-                        acy.mac(tx.Dv[pbe][b], sx[(4 * ND1 + b) * NV + pal]);
-                    }
-                    X[2] -= nu * h * fx::to_double(acx.get(), eu[3] + tBD) * (hy / hx);
-                    X[3] -= nu * h * fx::to_double(acy.get(), eu[3] + tBD) * (hx / hy);
-                }
-                const double gh = g * h, gJ = gam * (hx * hy);
-                X[4] = X[0] * ux; // Gx: h_y qx ux, h_x qx uy (= qy ux), -J g h zeta_x
-                X[5] = X[1] * ux;
-                X[6] = -(gh * hy) * zx;
-                X[7] = X[0] * uy; // Gy
-                X[8] = X[1] * uy;
-                X[9] = -(gh * hx) * zy;
-                X[10] = -gJ * qx; // Lx, Ly
-                X[11] = -gJ * qy;
+                Z = az.get();
+                ZX = azx.get();
+                ZY = azy.get();
+                QX = aqx.get();
+                QY = aqy.get();
+                C = ac.get();
             }
-            unsigned m[5];
-            m[0] = max(fx::mag(X[0]), fx::mag(X[1]));
-            m[1] = max(fx::mag(X[2]), fx::mag(X[3]));
-            m[2] = max(max(fx::mag(X[4]), fx::mag(X[5])), fx::mag(X[6]));
-            m[3] = max(max(fx::mag(X[7]), fx::mag(X[8])), fx::mag(X[9]));
-            m[4] = max(fx::mag(X[10]), fx::mag(X[11]));
+            const int eu0 = es[0], eu3 = es[3];
+            int eD = eu0 + tBD;
+            const int eX = es[1] + tBB, eY = es[2] + tBB, eC = eu3 + tBB;
+            // a constant field is that constant exactly
+            if (cm & 1u) ZX = ZY = 0;
+            {
+                // the gradient is far below the bound its table allows: its block moves
+                // up to the places that are free
+                const unsigned m = __reduce_max_sync(tm, pt ? max(fx::high(ZX), fx::high(ZY)) : 0u);
+                const int s = fx::clz64((unsigned long long)m << 32 | 0xffffffffu) - (63 - fx::FB);
+                ZX <<= s;
+                ZY <<= s;
+                eD -= s;
+            }
+            if (cm & 2u) QX = fx::from_double(c0[1], eX);
+            if (cm & 4u) QY = fx::from_double(c0[2], eY);
+            if (cm & 8u) C = fx::from_double(c0[3], eC);
+            const double z = (cm & 1u) ? c0[0] : fx::to_double(Z, eu0 + tBB);
+            const double qx = fx::to_double(QX, eX), qy = fx::to_double(QY, eY);
+            double h = 0.0, A;
+            if (pt) ST::VA(d, tb, k, SET_VOL, pal, pbe, z, h, A);
+            double fv, gm;
+            vel_friction(h, qx, qy, !zero_bits(man), eps, fv, gm);
+            const double ux = fv * qx, uy = fv * qy, gh = -g * h;
+            auto block = [&](unsigned m) { return fx::block_exp(__reduce_max_sync(tm, pt ? m : 0u)); };
+            const int eU = block(max(fx::mag(ux), fx::mag(uy))), eH = block(fx::mag(gh)),
+                      eM = block(fx::mag(gm));
+            const int2 dqx = fx::split(QX), dqy = fx::split(QY), dc = fx::split(C);
+            const int2 dux = fx::split(fx::from_double(ux, eU)), duy = fx::split(fx::from_double(uy, eU));
+            const int2 dgh = fx::split(fx::from_double(gh, eH)), dgm = fx::split(fx::from_double(gm, eM));
+            // exponents of the products; -g h grad zeta joins the xi-part of Gx and
+            // the eta-part of Gy
+            const int eXU = fx::product_exp(eX, eU), eYU = fx::product_exp(eY, eU),
+                      eHZ = fx::product_exp(eH, eD);
+            const int eGx = max(eXU, eHZ), eGy = max(eYU, eHZ);
+            int eRx = fx::product_exp(eC, eX), eRy = fx::product_exp(eC, eY);
+            eL[0] = fx::product_exp(eM, eX);
+            eL[1] = fx::product_exp(eM, eY);
+            long long RX = fx::product(dc, dqx), RY = fx::product(dc, dqy);
+            if (nu != 0.0 && !(cm & 8u)) {
+                // -nu h grad c . grad psi: the reference derivatives of c at the point
+                fx::Acc acx, acy;
 #pragma unroll
-            for (int j = 0; j < 5; ++j) ex[j] = fx::block_exp(__reduce_max_sync(tm, pt ? m[j] : 0u));
+                for (int b = 0; b < ND1; ++b) {
+                    acx.mac(tx.Bv[pbe][b], sx[(5 * ND1 + b) * NV + pal]);
+                    acy.mac(tx.Dv[pbe][b], sx[(4 * ND1 + b) * NV + pal]);
+                }
+                const double rx = fx::to_double(RX, eRx) - nu * h * fx::to_double(acx.get(), eu3 + tBD) / hx;
+                const double ry = fx::to_double(RY, eRy) - nu * h * fx::to_double(acy.get(), eu3 + tBD) / hy;
+                eRx = eRy = block(max(fx::mag(rx), fx::mag(ry)));
+                RX = fx::from_double(rx, eRx);
+                RY = fx::from_double(ry, eRx);
+            }
+            if (lane == 0) { // of F, Gx, Gy, R
+                es[8] = eX;
+                es[9] = eGx;
+                es[10] = eYU;
+                es[11] = eRx;
+                es[12] = eY;
+                es[13] = eYU;
+                es[14] = eGy;
+                es[15] = eRy;
+            }
             if (pt) {
-#pragma unroll
-                for (int j = 0; j < 12; ++j)
-                    xp[j * NVP + pl] = fx::split(
-                        fx::from_double(X[j], ex[j < 2 ? 0 : j < 4 ? 1 : j < 7 ? 2 : j < 10 ? 3 : 4]));
+                int2* o = xp + pl;
+                o[0 * NVP] = dqx;
+                o[1 * NVP] = dqy;
+                o[2 * NVP] = fx::split(RX);
+                o[3 * NVP] = fx::split(RY);
+                o[4 * NVP] = fx::split(fx::product(dqx, dux) >> min(eGx - eXU, 63));
+                const long long yu = fx::product(dqy, dux); // = qx uy
+                o[5 * NVP] = fx::split(yu);
+                o[6 * NVP] = fx::split(fx::product(dqy, duy) >> min(eGy - eYU, 63));
+                o[7 * NVP] = fx::split(fx::product(dgh, fx::split(ZX)) >> min(eGx - eHZ, 63));
+                o[8 * NVP] = fx::split(fx::product(dgh, fx::split(ZY)) >> min(eGy - eHZ, 63));
+                o[9 * NVP] = fx::split(fx::product(dgm, dqx));
+                o[10 * NVP] = fx::split(fx::product(dgm, dqy));
             }
         }
         __syncwarp(tm);
-        // the face fluxes of k_faces, loaded here (the first halves) so that the
-        // y-contraction hides the latency; slot i = (half, face, point), 0 where a
-        // face has no second half
+        // the face fluxes of k_faces; where no face of the cell has a second half they
+        // are loaded here, so that the y-contraction hides the latency
         constexpr int SL = (4 * NM + TL - 1) / TL;
-        auto slot = [&](int cf, int i) -> double {
-            const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
-            const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
-            if (i >= nslot || !own) return 0.0;
-            return d.fflux ? d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al]
-                           : fh[cf * 8 * NM + i];
-        };
+        const bool conforming = nslot == 4 * NM;
         double fv[SL][4];
-        if (d.fflux) {
+        if (!INL && conforming) {
 #pragma unroll
-            for (int j = 0; j < SL; ++j)
+            for (int j = 0; j < SL; ++j) {
+                const int i = lane + j * TL;
+                const double* F = d.fflux + k * (32 * NM) + (i / NM) * 2 * NM + i % NM;
 #pragma unroll
-                for (int cf = 0; cf < 4; ++cf) fv[j][cf] = slot(cf, lane + j * TL);
+                for (int cf = 0; cf < 4; ++cf) fv[j][cf] = i < 4 * NM ? F[cf * 8 * NM] : 0.0;
+            }
         }
-        // test integration, y-contraction: jobs 0, 1 the x-parts of F and R, 2, 3
-        // their y-parts, 4, 5 the x-parts of Gx and Gy, 6, 7 Lx and Ly; then 8, 9
-        // the y- and value parts of Gx and Gy
-        for (int i = lane; i < 8 * NE; i += TL) {
+        // test integration, y-contraction: jobs 0..3 the xi-parts of F, R, Gx, Gy
+        // (wv Bv), 4, 5 Lx, Ly, 6..8 the eta-parts of F, R, Gx (wv Dv), 9 the value
+        // part of Gx; then 10 the eta- and value parts of Gy
+#pragma unroll 1
+        for (int i = lane; i < 10 * NE; i += TL) {
             const int job = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-            const int2* T = (job == 2 || job == 3) ? tx.WD[b] : tx.WB[b];
-            const int2* X = xp + ((0xBA743120u >> (4 * job)) & 15u) * NVP + al;
+            const int2* T = job < 6 ? tx.WB[b] : job < 9 ? tx.WD[b] : tx.WDB[b];
+            const int2* X = xp + (int)((0x7531A95420ull >> (4 * job)) & 15u) * NVP + al;
             fx::Acc s;
 #pragma unroll
             for (int be = 0; be < NV; ++be) s.mac(T[be], X[NV * be]);
             sy[i] = fx::split(s.get());
         }
-        for (int i = lane; i < 2 * NE; i += TL) {
-            const int cg = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-            const int2* X = xp + (5 + 3 * cg) * NVP + al;
+#pragma unroll 1
+        for (int i = lane; i < NE; i += TL) {
+            const int al = i / ND1, b = i % ND1;
+            const int2* X = xp + 6 * NVP + al;
             fx::Acc s;
 #pragma unroll
             for (int be = 0; be < NV; ++be) {
                 s.mac(tx.WD[b][be], X[NV * be]);
-                s.mac(tx.WDB[b][be], X[NVP + NV * be]);
+                s.mac(tx.WDB[b][be], X[2 * NVP + NV * be]);
             }
-            sy[8 * NE + i] = fx::split(s.get());
+            sy[10 * NE + i] = fx::split(s.get());
         }
         __syncwarp(tm);
-        if (!d.fflux) {
+        if constexpr (INL) {
             // the allocation-free entry: the cell's faces here, one (sub)face
             // point per lane; the face points of faces 0..3 start at 0, b1, b2,
             // b3 (2 NM points on a coarse 2:1 face, else NM)
@@ -966,41 +1009,64 @@ __global__ void __maxnreg__(64)
             }
             __syncwarp(tm);
         }
-        // the face fluxes (of k_faces, or from above) to digits, field by field
-        int ef[4];
+        // the face fluxes to digits, field by field: slot i = (half, face, point)
+        if (!INL && conforming) {
 #pragma unroll
-        for (int cf = 0; cf < 4; ++cf) {
-            unsigned m = 0;
+            for (int cf = 0; cf < 4; ++cf) {
+                unsigned m = 0;
 #pragma unroll
-            for (int j = 0; j < SL; ++j) {
-                if (!d.fflux) fv[j][cf] = slot(cf, lane + j * TL);
-                m = max(m, fx::mag(fv[j][cf]));
+                for (int j = 0; j < SL; ++j) m = max(m, fx::mag(fv[j][cf]));
+                const int e = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll
+                for (int j = 0; j < SL; ++j)
+                    if (lane + j * TL < 4 * NM)
+                        fd[cf * 8 * NM + lane + j * TL] = fx::split(fx::from_double(fv[j][cf], e));
+                if (lane == 0) es[4 + cf] = e;
             }
-            for (int i = lane + SL * TL; i < nslot; i += TL) m = max(m, fx::mag(slot(cf, i)));
-            ef[cf] = fx::block_exp(__reduce_max_sync(tm, m));
-#pragma unroll
-            for (int j = 0; j < SL; ++j)
-                if (lane + j * TL < nslot)
-                    fd[cf * 8 * NM + lane + j * TL] = fx::split(fx::from_double(fv[j][cf], ef[cf]));
-            for (int i = lane + SL * TL; i < nslot; i += TL)
-                fd[cf * 8 * NM + i] = fx::split(fx::from_double(slot(cf, i), ef[cf]));
+        } else {
+            auto slot = [&](int cf, int i) -> double { // 0 where a face has no second half
+                const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
+                const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
+                if (!own) return 0.0;
+                return INL ? fh[cf * 8 * NM + i] : d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al];
+            };
+#pragma unroll 1
+            for (int cf = 0; cf < 4; ++cf) {
+                unsigned m = 0;
+#pragma unroll 1
+                for (int i = lane; i < nslot; i += TL) m = max(m, fx::mag(slot(cf, i)));
+                const int e = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll 1
+                for (int i = lane; i < nslot; i += TL)
+                    fd[cf * 8 * NM + i] = fx::split(fx::from_double(slot(cf, i), e));
+                if (lane == 0) es[4 + cf] = e;
+            }
         }
         __syncwarp(tm);
-        // x-contraction of F, Gx, Gy, R minus the face fluxes lifted onto the
-        // nodes of their faces; a node takes part in at most one x face and one
-        // y face
+        // x-contraction of F, Gx, Gy, R, the xi-parts times h_y and the eta-parts
+        // times h_x, minus the face fluxes lifted onto the nodes of their faces (a
+        // node takes part in at most one x face and one y face)
+        const int eh = fx::block_exp(max(fx::mag(hx), fx::mag(hy)));
+        const int2 dhx = fx::split(fx::from_double(hx, eh)), dhy = fx::split(fx::from_double(hy, eh));
+#pragma unroll 1
         for (int i = lane; i < 4 * ND; i += TL) {
             const int cf = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            const int2* s1 = sy + ((0x1540u >> (4 * cf)) & 15u) * NE + b;
-            const int2* s2 = sy + ((0x3982u >> (4 * cf)) & 15u) * NE + b;
-            fx::Acc s;
+            const int2* s1 = sy + ((0x1320u >> (4 * cf)) & 15u) * NE + b;
+            const int2* s2 = sy + ((0x7A86u >> (4 * cf)) & 15u) * NE + b;
+            fx::Acc sa, sb;
 #pragma unroll
             for (int al = 0; al < NV; ++al) {
-                s.mac(tx.WD[a][al], s1[al * ND1]);
-                s.mac(tx.WB[a][al], s2[al * ND1]);
+                sa.mac(tx.WD[a][al], s1[al * ND1]);
+                sb.mac(tx.WB[a][al], s2[al * ND1]);
             }
-            const int e = cf == 0 ? ex[0] : cf == 1 ? ex[2] : cf == 2 ? ex[3] : ex[1];
-            const int ff = cf == 0 ? ef[0] : cf == 1 ? ef[1] : cf == 2 ? ef[2] : ef[3];
+            if (cf == 1) {
+#pragma unroll
+                for (int al = 0; al < NV; ++al) sa.mac(tx.WB[a][al], sy[9 * NE + al * ND1 + b]);
+            }
+            const int e1 = es[8 + cf], e2 = es[12 + cf], ff = es[4 + cf];
+            const int em = max(e1, e2);
+            const long long vol = (fx::product(fx::split(sa.get()), dhy) >> min(em - e1, 63)) +
+                                  (fx::product(fx::split(sb.get()), dhx) >> min(em - e2, 63));
             long long sf = 0;
             auto lift = [&](int f, int tn, bool coarse) {
                 fx::Acc q;
@@ -1020,14 +1086,17 @@ __global__ void __maxnreg__(64)
             if (a == 0 || a == ND1 - 1) lift(a == 0 ? 0 : 1, b, a == 0 ? c_f[0] : c_f[1]);
             if (b == 0 || b == ND1 - 1) lift(b == 0 ? 2 : 3, a, b == 0 ? c_f[2] : c_f[3]);
             rfield(d, stage, cf, ND)[k * ND + j] =
-                fx::to_double(s.get(), e + tW) - fx::to_double(sf, ff + tx.tBmT);
+                fx::to_double(vol, fx::product_exp(em + tW, eh)) - fx::to_double(sf, ff + tx.tBmT);
         }
+        const double kJ = -(g * man * man) * (hx * hy);
+#pragma unroll 1
         for (int i = lane; i < 2 * ND; i += TL) { // Lx, Ly
             const int cl = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
             fx::Acc s;
 #pragma unroll
-            for (int al = 0; al < NV; ++al) s.mac(tx.WB[a][al], sy[(6 + cl) * NE + al * ND1 + b]);
-            rfield(d, stage, 4 + cl, ND)[k * ND + j] = fx::to_double(s.get(), ex[4] + 2 * tx.tWB);
+            for (int al = 0; al < NV; ++al) s.mac(tx.WB[a][al], sy[(4 + cl) * NE + al * ND1 + b]);
+            rfield(d, stage, 4 + cl, ND)[k * ND + j] =
+                kJ * fx::to_double(s.get(), (cl ? eL[1] : eL[0]) + 2 * tx.tWB);
         }
         __syncwarp(tm);
     }
@@ -1594,7 +1663,7 @@ __device__ __forceinline__ void mass_scalar_pixels(const Dev& d, const Tables& t
 }
 
 template <int R, typename Pix, int MODE, int TL = 32>
-__device__ int scalar_newton(const Dev& d, const Tables& tb, int64_t k, double J, double target,
+__device__ __noinline__ int scalar_newton(const Dev& d, const Tables& tb, int64_t k, double J, double target,
                              double& e, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = Sz<R>::ND;
     double H, A;
@@ -1636,52 +1705,53 @@ struct StageArgs {
     int final_;    // final combination: update time and bookkeeping
 };
 
-// Cholesky of the SPD matrix M (ND x ND, row-major, lower part used) on a
-// warp, then M x = b in place by column-oriented forward and back
+// Cholesky of the SPD matrix M (ND x ND, lower part packed by rows) on a team, then M x = b in place by column-oriented forward and back
 // substitution (one reciprocal per column, the updates spread over lanes);
 // returns false on a non-positive pivot
+__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; } // j <= i
 template <int ND, int TL = 32>
-__device__ bool chol_solve(double* M, double* b, double* inv, int lane, unsigned tm = 0xffffffffu) {
+__device__ __noinline__ bool chol_solve(double* M, double* b, double* inv, int lane, unsigned tm = 0xffffffffu) {
     for (int j = 0; j < ND; ++j) {
         __syncwarp(tm);
-        const double djj = M[j * ND + j];
+        const double djj = M[tri(j, j)];
         if (!(djj > 0.0)) return false;
         const double ljj = sqrt(djj);
         const double r = 1.0 / ljj;
         __syncwarp(tm);
-        for (int i = j + 1 + lane; i < ND; i += TL) M[i * ND + j] *= r;
+        for (int i = j + 1 + lane; i < ND; i += TL) M[tri(i, j)] *= r;
         if (lane == 0) {
-            M[j * ND + j] = ljj;
+            M[tri(j, j)] = ljj;
             inv[j] = r;
         }
         __syncwarp(tm);
         const int m = ND - j - 1;
         for (int idx = lane; idx < m * m; idx += TL) {
             const int i = j + 1 + idx / m, l = j + 1 + idx % m;
-            if (l <= i) M[i * ND + l] -= M[i * ND + j] * M[l * ND + j];
+            if (l <= i) M[tri(i, l)] -= M[tri(i, j)] * M[tri(l, j)];
         }
     }
     __syncwarp(tm);
     for (int j = 0; j < ND; ++j) { // L y = b
         const double yj = b[j] * inv[j];
         __syncwarp(tm);
-        for (int i = j + 1 + lane; i < ND; i += TL) b[i] -= M[i * ND + j] * yj;
+        for (int i = j + 1 + lane; i < ND; i += TL) b[i] -= M[tri(i, j)] * yj;
         if (lane == 0) b[j] = yj;
         __syncwarp(tm);
     }
     for (int j = ND - 1; j >= 0; --j) { // L^T x = y
         const double xj = b[j] * inv[j];
         __syncwarp(tm);
-        for (int i = lane; i < j; i += TL) b[i] -= M[j * ND + i] * xj;
+        for (int i = lane; i < j; i += TL) b[i] -= M[tri(j, i)] * xj;
         if (lane == 0) b[j] = xj;
         __syncwarp(tm);
     }
     return true;
 }
 
-// M_(a,b),(c,d) = sum_{al,be} c_{al,be} Bm[al][a] Bm[al][c] Bm[be][b] Bm[be][d]
+// M_(a,b),(c,d) = sum_{al,be} c_{al,be} Bm[al][a] Bm[al][c] Bm[be][b] Bm[be][d],
+// the lower part packed by rows (rarely reached: not inlined)
 template <int ND1, int NM, int TL = 32>
-__device__ __forceinline__ void assemble_mass(const Tables& tb, const double* cw, double* Y,
+__device__ __noinline__ void assemble_mass(const Tables& tb, const double* cw, double* Y,
                                               double* M, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = ND1 * ND1;
     for (int i = lane; i < ND1 * ND1 * NM; i += TL) {
@@ -1694,12 +1764,13 @@ __device__ __forceinline__ void assemble_mass(const Tables& tb, const double* cw
     __syncwarp(tm);
     for (int i = lane; i < ND * ND; i += TL) {
         const int r_ = i / ND, s_ = i % ND;
+        if (s_ > r_) continue;
         const int a = r_ % ND1, b = r_ / ND1, c = s_ % ND1, dd = s_ / ND1;
         double s = 0.0;
 #pragma unroll
         for (int be = 0; be < NM; ++be)
             s += Y[(a * ND1 + c) * NM + be] * tb.Bm[be][b] * tb.Bm[be][dd];
-        M[i] = s;
+        M[tri(r_, s_)] = s;
     }
     __syncwarp(tm);
 }
@@ -1921,7 +1992,7 @@ __device__ __forceinline__ bool mass_inverse_f(const FxStage& fs, float* buf, fl
 // Scratch: buf (mass_inverse_f's, and 2 floats to align it), digit pairs xd [ND], qd [NMP], td [2 NMP], M,
 // Y, inv (double, fallback: M may overlay buf, Y and inv xd, qd and td).
 template <int ND1, int NM, int TL = 32>
-__device__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const double* cw, double* b,
+__device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const double* cw, double* b,
                                  float* buf, int2* xd, int2* qd, int2* td, double* M, double* Y,
                                  double* inv, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4;
@@ -2018,7 +2089,7 @@ __device__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const doub
 // H(zeta^(l)) = T up to the rounding of the last update) and the continuity
 // target T stands for s = H 1 = H(zeta^(l)); otherwise s is integrated from cw.
 template <int ND1, int NM, int TL>
-__device__ void solve_tracer_bulk(const Tables& tb, const FxStage& fs, const double* cw, double* b,
+__device__ __noinline__ void solve_tracer_bulk(const Tables& tb, const FxStage& fs, const double* cw, double* b,
                                   float* Mf, float* Yf, int2* td, double* M, double* Y, double* inv,
                                   bool known, double T, int lane, unsigned tm) {
     constexpr int ND = ND1 * ND1, NMP = NM * NM;
@@ -2121,6 +2192,37 @@ __device__ __forceinline__ void square(const float (*T)[MXN], int, float (&v)[NF
         v[f] = s;
     }
     __syncwarp(tm);
+}
+// one or two fields, not inlined: the stage update calls them in five places, and
+// its hot code has to fit the instruction cache (32 KB)
+struct Two {
+    double a, b;
+};
+template <int N>
+__device__ __noinline__ Two square_two(const int2 (*T)[MXN], int t, double a, double b, int2* w, int lane,
+                                       unsigned tm) {
+    double v[2] = {a, b};
+    square<N, 2>(T, t, v, w, lane, tm);
+    return {v[0], v[1]};
+}
+template <int N>
+__device__ __noinline__ double square_one(const int2 (*T)[MXN], int t, double a, int2* w, int lane,
+                                          unsigned tm) {
+    double v[1] = {a};
+    square<N, 1>(T, t, v, w, lane, tm);
+    return v[0];
+}
+template <int N>
+__device__ __forceinline__ void square2(const int2 (*T)[MXN], int t, double (&v)[2], int2* w, int lane,
+                                        unsigned tm) {
+    const Two r = square_two<N>(T, t, v[0], v[1], w, lane, tm);
+    v[0] = r.a;
+    v[1] = r.b;
+}
+template <int N>
+__device__ __forceinline__ void square2(const float (*T)[MXN], int t, float (&v)[2], int2* w, int lane,
+                                        unsigned tm) {
+    square<N, 2>(T, t, v, w, lane, tm);
 }
 // the stage tables of the value type
 __device__ __forceinline__ const int2 (*tab_Bg(const FxStage& s, double))[MXN] { return s.Bg; }
@@ -2300,7 +2402,7 @@ __global__ void __maxnreg__(64)
         // interpolating v^n again)
         if (d.qpts) {
             double q[2] = {u[1], u[2]};
-            if ((cm & 6u) != 6u) square<ND1, 2>(fs.Bg, fs.tBg, q, w, lane, tm);
+            if ((cm & 6u) != 6u) square2<ND1>(fs.Bg, fs.tBg, q, w, lane, tm);
             if (act) {
                 d.qpts[k * 2 * NGP + lane] = (cm & 2u) ? u[1] : q[0];
                 d.qpts[k * 2 * NGP + NGP + lane] = (cm & 4u) ? u[2] : q[1];
@@ -2335,16 +2437,23 @@ struct StageFx {
     // fallback's M
     static constexpr int W = 6 * S::ND, Q = 3 * S::NMP, CW = S::NMP, BV = S::ND;
     static constexpr int F32 = (S::ND * S::ND + S::ND1 * S::ND1 * S::NM + 1) / 2;
-    static constexpr int UN = S::ND * S::ND > F32 ? S::ND * S::ND : F32;
-    static constexpr int words = W + Q + CW + BV + UN;
+    // the fallback's matrix; the FP32 inverse's scratch; the FP32-bulk tracer's M, Y
+    static constexpr int TRI = S::ND * (S::ND + 1) / 2;
+    static constexpr int INV =
+        (2 + 2 * ((S::ND + 3) / 4 * 4) + S::NMP + S::ND1 * (S::ND1 + 1) / 2 * S::NM + 1) / 2;
+    static constexpr int un(bool bulk) {
+        return bulk && F32 > TRI && F32 > INV ? F32 : TRI > INV ? TRI : INV;
+    }
+    static constexpr int words(bool bulk) { return W + Q + CW + BV + un(bulk); }
     static_assert(S::ND <= TL && S::NGP == S::ND, "one node and one momentum point per lane");
     static_assert(S::ND1 * S::ND1 * S::NM <= W, "fallback Y");
-    static_assert(2 + 2 * ((S::ND + 3) / 4 * 4) + S::NMP + S::ND1 * (S::ND1 + 1) / 2 * S::NM <= 2 * UN,
-                  "the FP32 inverse's scratch");
 };
 
+#ifndef STAGE_REGS
+#define STAGE_REGS 72
+#endif
 template <int R, typename Pix, int MODE, typename B>
-__global__ void __maxnreg__(R == 1 ? 128 : 96)
+__global__ void __maxnreg__(STAGE_REGS)
     k_stage(const __grid_constant__ Dev d, const __grid_constant__ StageArgs sa) {
     using S = Sz<R>;
     using L = StageFx<R>;
@@ -2358,7 +2467,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
     extern __shared__ double smem[];
     const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
     const unsigned tm = 0xFFFFu << (threadIdx.x & 16); // the team's lanes
-    int2* w = (int2*)(smem + team * L::words); // digit pairs of nodal fields, and scratch
+    int2* w = (int2*)(smem + team * L::words(!F64)); // digit pairs of nodal fields, and scratch
     int2* qd = w + L::W;                       // [NMP] mass-point digits, then scratch [2 NMP]
     int2* qt = qd + NMP;
     double* cw = (double*)(qd + L::Q); // [NMP] weights of a mass-matrix solve
@@ -2366,7 +2475,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
     double* un = bv + L::BV;
     float* Mf = (float*)un;            // [ND ND] (FP32-bulk tracer), or the FP32 inverse's scratch
     float* Yf = Mf + ND * ND;          // [ND1 ND1 NM]
-    double* M = un;                    // [ND ND] (fallback)
+    double* M = un;                    // the fallback's matrix, packed
     const int64_t n = d.n;
     const double g = d.g, eps = d.eps;
     const bool act = lane < ND;
@@ -2494,7 +2603,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
                 double dz[1] = {o};
                 if (npart == 0) {
                     // M is the constant mass matrix, inverted by its tensor factors
-                    square<ND1, 1>(fs.M1i, fs.tM1i, dz, w, lane, tm);
+                    dz[0] = square_one<ND1>(fs.M1i, fs.tM1i, dz[0], w, lane, tm);
                     dz[0] *= d.ihxhy[2 * k] * d.ihxhy[2 * k + 1];
                 } else {
                     if (act) bv[lane] = o;
@@ -2545,8 +2654,8 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
                     q1 = bulk_of(ufield(d, sa.prev_buf, 2, ND)[idx], T());
             double zv[1] = {z0}, Vp, Ap;
             T q[2] = {q0, q1}, gam = T(0);
-            if (!(cmp & 1u)) square<ND1, 1>(fs.Bg, fs.tBg, zv, w, lane, tm);
-            if ((cmp & 6u) != 6u) square<ND1, 2>(tab_Bg(fs, T()), fs.tBg, q, w, lane, tm);
+            if (!(cmp & 1u)) zv[0] = square_one<ND1>(fs.Bg, fs.tBg, zv[0], w, lane, tm);
+            if ((cmp & 6u) != 6u) square2<ND1>(tab_Bg(fs, T()), fs.tBg, q, w, lane, tm);
             if (cmp & 2u) q[0] = q0;
             if (cmp & 4u) q[1] = q1;
             if (act) {
@@ -2561,7 +2670,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
             const T q0 = bulk_of(ufield(d, 0, 1, ND)[idx], T()), q1 = bulk_of(ufield(d, 0, 2, ND)[idx], T());
             v[0] = q0;
             v[1] = q1;
-            if ((cm0 & 6u) != 6u) square<ND1, 2>(tab_Bg(fs, T()), fs.tBg, v, w, lane, tm);
+            if ((cm0 & 6u) != 6u) square2<ND1>(tab_Bg(fs, T()), fs.tBg, v, w, lane, tm);
             if (cm0 & 2u) v[0] = q0;
             if (cm0 & 4u) v[1] = q1;
         };
@@ -2609,7 +2718,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
             if (sa.make_llin) {
                 ll[0] = -(wp * gam) * oq[0];
                 ll[1] = -(wp * gam) * oq[1];
-                square<ND1, 2>(fs.BgT, fs.tBgT, ll, w, lane, tm);
+                square2<ND1>(fs.BgT, fs.tBgT, ll, w, lane, tm);
             }
         } else {
             // momentum (Eq. algebraic_discharge with the friction-modified mass
@@ -2633,7 +2742,7 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
                 q_points(qn);
             }
             B s[2] = {bulk_of(rq[0], B()), bulk_of(rq[1], B())};
-            square<ND1, 2>(tab_GiT(fs, B()), fs.tGiT, s, w, lane, tm);
+            square2<ND1>(tab_GiT(fs, B()), fs.tGiT, s, w, lane, tm);
             B wp;
             if constexpr (F64) wp = J * w2;
             else wp = JB * fs.wgF[node % NG] * fs.wgF[node / NG];
@@ -2641,11 +2750,11 @@ __global__ void __maxnreg__(R == 1 ? 128 : 96)
             s[0] = (wp * qn[0] + s[0]) * rD;
             s[1] = (wp * qn[1] + s[1]) * rD;
             B Q[2] = {s[0], s[1]};
-            square<ND1, 2>(tab_Gi(fs, B()), fs.tGi, Q, w, lane, tm);
+            square2<ND1>(tab_Gi(fs, B()), fs.tGi, Q, w, lane, tm);
             if (sa.make_llin) {
                 const B wl = wp * gam;
                 B l[2] = {-wl * s[0], -wl * s[1]};
-                square<ND1, 2>(tab_BgT(fs, B()), fs.tBgT, l, w, lane, tm);
+                square2<ND1>(tab_BgT(fs, B()), fs.tBgT, l, w, lane, tm);
                 ll[0] = exact_of(l[0]);
                 ll[1] = exact_of(l[1]);
             }
