@@ -3,16 +3,15 @@
 // the Manning coefficient n_K and a bathymetry offset delta_K per cell (every
 // depth of cell K shifted by delta_K), at delta = 0.
 //
-// Gather form, one warp per cell, no atomics: a cell's cotangent collects
+// Gather form, one team of lanes per cell, no atomics: a cell's cotangent collects
 // every residual entry that depends on its own data -- its volume terms, and
 // on each of its (sub)face points both its own face term and its
 // neighbour's (the neighbour's residual cotangent is read there).  The linear
 // parts are the transposes of the forward contractions (interpolation <->
 // test integration, trace <-> lift); the pointwise parts (velocity, friction,
-// reconstruction, Rusanov flux) are differentiated by forward-mode dual
-// numbers through the same templates the forward residual runs, every input
-// direction of a point carried in one evaluation.  The sub-grid operator enters through V and its exact
-// derivative A = dV/d(eta) = dV/d(delta).
+// reconstruction, Rusanov flux) are differentiated in reverse by hand.  The
+// sub-grid operator enters through V and its exact derivative
+// A = dV/d(eta) = dV/d(delta).
 //
 // Derivative conventions at the kinks: max(x, 0) -> [x > 0] (Eq. mask); the
 // reconstruction's min follows its first argument at ties, the first argument
@@ -25,168 +24,6 @@
 #include "swdg_kernels.cuh"
 
 namespace swdg {
-namespace ad {
-
-// value and one directional derivative
-struct D1 {
-    double v, d;
-    __device__ __forceinline__ D1() : v(0.0), d(0.0) {}
-    __device__ __forceinline__ D1(double x) : v(x), d(0.0) {}
-    __device__ __forceinline__ D1(double x, double dx) : v(x), d(dx) {}
-};
-__device__ __forceinline__ D1 operator+(D1 a, D1 b) { return D1(a.v + b.v, a.d + b.d); }
-__device__ __forceinline__ D1 operator-(D1 a, D1 b) { return D1(a.v - b.v, a.d - b.d); }
-__device__ __forceinline__ D1 operator-(D1 a) { return D1(-a.v, -a.d); }
-__device__ __forceinline__ D1 operator*(D1 a, D1 b) { return D1(a.v * b.v, a.d * b.v + a.v * b.d); }
-// a / b through one reciprocal of b (the value is a.v (1/b.v), within an ulp
-// of the forward's quotient; only derivatives are taken from dual values)
-__device__ __forceinline__ D1 operator/(D1 a, D1 b) {
-    const double ib = 1.0 / b.v;
-    const double q = a.v * ib;
-    return D1(q, (a.d - q * b.d) * ib);
-}
-__device__ __forceinline__ D1& operator+=(D1& a, D1 b) { return a = a + b; }
-__device__ __forceinline__ D1& operator*=(D1& a, D1 b) { return a = a * b; }
-__device__ __forceinline__ bool operator<(D1 a, D1 b) { return a.v < b.v; }
-__device__ __forceinline__ bool operator<=(D1 a, D1 b) { return a.v <= b.v; }
-__device__ __forceinline__ bool operator>(D1 a, D1 b) { return a.v > b.v; }
-__device__ __forceinline__ bool operator>=(D1 a, D1 b) { return a.v >= b.v; }
-__device__ __forceinline__ bool operator==(D1 a, D1 b) { return a.v == b.v; }
-__device__ __forceinline__ D1 sqrt(D1 a) {
-    const double s = ::sqrt(a.v);
-    return D1(s, a.v > 0.0 ? 0.5 * a.d / s : 0.0);
-}
-__device__ __forceinline__ D1 cbrt(D1 a) {
-    const double s = ::cbrt(a.v);
-    return D1(s, a.v != 0.0 ? a.d / (3.0 * s * s) : 0.0);
-}
-__device__ __forceinline__ D1 fabs(D1 a) {
-    return D1(::fabs(a.v), a.v > 0.0 ? a.d : (a.v < 0.0 ? -a.d : 0.0));
-}
-__device__ __forceinline__ D1 fmax(D1 a, D1 b) { return a.v >= b.v ? a : b; }
-// the wave-speed bound: the symmetric subgradient at an exact tie
-__device__ __forceinline__ D1 wave_speed_max(D1 a, D1 b) {
-    return a.v > b.v ? a : (a.v < b.v ? b : D1(a.v, 0.5 * (a.d + b.d)));
-}
-__device__ __forceinline__ D1 fmin(D1 a, D1 b) { return a.v <= b.v ? a : b; }
-
-// value and W directional derivatives (all directions in one evaluation)
-template <int W>
-struct DN {
-    double v, d[W];
-    __device__ __forceinline__ DN() : v(0.0) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) d[i] = 0.0;
-    }
-    __device__ __forceinline__ DN(double x) : v(x) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) d[i] = 0.0;
-    }
-    // x with unit derivative along direction dir (none when dir is outside [0, W))
-    __device__ __forceinline__ static DN seed(double x, int dir) {
-        DN r(x);
-#pragma unroll
-        for (int i = 0; i < W; ++i) r.d[i] = (i == dir) ? 1.0 : 0.0;
-        return r;
-    }
-    // derivative v along direction dir, if dir is one of this value's
-    __device__ __forceinline__ void set(int dir, double v) {
-#pragma unroll
-        for (int i = 0; i < W; ++i)
-            if (i == dir) d[i] = v;
-    }
-};
-template <int W>
-__device__ __forceinline__ DN<W> operator+(const DN<W>& a, const DN<W>& b) {
-    DN<W> r;
-    r.v = a.v + b.v;
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = a.d[i] + b.d[i];
-    return r;
-}
-template <int W>
-__device__ __forceinline__ DN<W> operator-(const DN<W>& a, const DN<W>& b) {
-    DN<W> r;
-    r.v = a.v - b.v;
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = a.d[i] - b.d[i];
-    return r;
-}
-template <int W>
-__device__ __forceinline__ DN<W> operator-(const DN<W>& a) {
-    DN<W> r;
-    r.v = -a.v;
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = -a.d[i];
-    return r;
-}
-template <int W>
-__device__ __forceinline__ DN<W> operator*(const DN<W>& a, const DN<W>& b) {
-    DN<W> r;
-    r.v = a.v * b.v;
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = a.d[i] * b.v + a.v * b.d[i];
-    return r;
-}
-// a / b through one reciprocal of b, as for D1
-template <int W>
-__device__ __forceinline__ DN<W> operator/(const DN<W>& a, const DN<W>& b) {
-    DN<W> r;
-    const double ib = 1.0 / b.v;
-    r.v = a.v * ib;
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
-    return r;
-}
-template <int W>
-__device__ __forceinline__ DN<W>& operator+=(DN<W>& a, const DN<W>& b) { return a = a + b; }
-template <int W>
-__device__ __forceinline__ bool operator<(const DN<W>& a, const DN<W>& b) { return a.v < b.v; }
-template <int W>
-__device__ __forceinline__ bool operator<=(const DN<W>& a, const DN<W>& b) { return a.v <= b.v; }
-template <int W>
-__device__ __forceinline__ bool operator>(const DN<W>& a, const DN<W>& b) { return a.v > b.v; }
-template <int W>
-__device__ __forceinline__ bool operator>=(const DN<W>& a, const DN<W>& b) { return a.v >= b.v; }
-template <int W>
-__device__ __forceinline__ bool operator==(const DN<W>& a, const DN<W>& b) { return a.v == b.v; }
-template <int W>
-__device__ __forceinline__ DN<W> scale_d(double v, const DN<W>& a, double f) {
-    DN<W> r(v);
-#pragma unroll
-    for (int i = 0; i < W; ++i) r.d[i] = a.d[i] * f;
-    return r;
-}
-template <int W>
-__device__ __forceinline__ DN<W> sqrt(const DN<W>& a) {
-    const double s = ::sqrt(a.v);
-    return scale_d(s, a, a.v > 0.0 ? 0.5 / s : 0.0);
-}
-template <int W>
-__device__ __forceinline__ DN<W> cbrt(const DN<W>& a) {
-    const double s = ::cbrt(a.v);
-    return scale_d(s, a, a.v != 0.0 ? 1.0 / (3.0 * s * s) : 0.0);
-}
-template <int W>
-__device__ __forceinline__ DN<W> fabs(const DN<W>& a) {
-    return scale_d(::fabs(a.v), a, a.v > 0.0 ? 1.0 : (a.v < 0.0 ? -1.0 : 0.0));
-}
-template <int W>
-__device__ __forceinline__ DN<W> fmax(const DN<W>& a, const DN<W>& b) { return a.v >= b.v ? a : b; }
-template <int W>
-__device__ __forceinline__ DN<W> wave_speed_max(const DN<W>& a, const DN<W>& b) {
-    // selects only (no branch over the whole value): a, b, or at a tie the mean
-    const bool gt = a.v > b.v, lt = a.v < b.v;
-    DN<W> m;
-    m.v = gt ? a.v : b.v;
-#pragma unroll
-    for (int i = 0; i < W; ++i) m.d[i] = gt ? a.d[i] : (lt ? b.d[i] : 0.5 * (a.d[i] + b.d[i]));
-    return m;
-}
-template <int W>
-__device__ __forceinline__ DN<W> fmin(const DN<W>& a, const DN<W>& b) { return a.v <= b.v ? a : b; }
-
-} // namespace ad
 
 template <int R>
 constexpr int vjp_smem() {
@@ -199,23 +36,53 @@ constexpr int vjp_smem() {
            12 * S::ND1 * S::NV + 8 * S::NVP + 32 * S::NM + 3 * S::NV * S::ND1 + S::ND1 * S::NV;
 }
 
-// the face fluxes of one face point seen from side A (outward normal n_A):
-// {F, Gx, Gy, R} of side A's residual including its pressure term
-template <typename T, bool DC = false>
-__device__ __forceinline__ void side_flux(T qxA, T qyA, T cA, T hA, T hsA, T qxB, T qyB, T cB,
-                                          T hB, T hsB, double nx, double ny, double g, double eps,
-                                          T out[4], T* dc = nullptr) {
-    T pres, lam;
-    rusanov<T, DC>(qxA, qyA, cA, hA, hsA, qxB, qyB, cB, hB, hsB, hsA - hsB, T(nx), T(ny), T(g),
-                   T(eps), out, pres, lam, dc);
-    out[1] = out[1] - pres * T(nx);
-    out[2] = out[2] - pres * T(ny);
+// Depth derivatives of the velocity factor and of the Manning coefficient:
+// with h_des the desingularised depth (h where h >= eps), f = 1 / h_des and
+// gamma ~ h_des^(-7/3), f' = -f l and gamma' = -7/3 gamma l, l = h_des' / h_des
+// (1 / h where h >= eps); all 0 on dry points.
+__device__ __forceinline__ double log_hdes_slope(double h, double eps) {
+    if (h >= eps) return 1.0 / h;
+    if (h <= 0.0) return 0.0;
+    const double h2 = h * h, e2 = eps * eps;
+    return 2.0 * h2 * h / (e2 * e2 + h2 * h2) - 1.0 / h;
 }
+// one side of a face for the reverse pass, in the face's frame (swdg_kernels.cuh,
+// face_flux): depth h, reconstructed depth hs, discharges, concentration, then
+// the velocity factor f, the wave speed w, the velocities v (axis), u
+struct VjpSide {
+    double h, hs, qn, qt, c, f, w, v, u;
+    __device__ __forceinline__ void form(const Dev& d) {
+        vel_wave(h, d.g, d.sg, d.eps, f, w);
+        v = f * qn;
+        u = f * qt;
+    }
+    // cotangents of the mass flux pieces: d(h* v), d(h* u) given as qb, rb, the
+    // cotangent lb of |v| + w, and the direct ones of v (vb0); adds to those of
+    // qn, qt, h
+    __device__ __forceinline__ void back(const Dev& d, double qb, double rb, double lb, double vb0,
+                                         double& qnb, double& qtb, double& hb) const {
+        const double vb = vb0 + qb * hs + (v > 0.0 ? lb : v < 0.0 ? -lb : 0.0), ub = rb * hs;
+        qnb = f * vb;
+        qtb = f * ub;
+        const double fb = qn * vb + qt * ub;
+        // f' = -f l, w' = g / (2 w)
+        hb = -fb * f * log_hdes_slope(h, d.eps) + (h > 0.0 ? lb * 0.5 * d.g / w : 0.0);
+    }
+};
 
-// register cap: 160 keeps 12 warps resident per SM at r <= 2 (no spills at
-// r = 2); r = 3 carries all six directions per lane and keeps more
+// The residual's discrete adjoint: gather form, one cell per team of TL lanes (32
+// at r = 3, else 16: 16 volume and 16 conforming face points at r = 2), no
+// atomics.  The pointwise physics is differentiated in reverse by hand: about 60
+// FP64 instructions a volume point and 110 a face point, where forward-mode
+// duals over the inputs (their products with constants included) took some 400
+// per half-warp.  Measured on 128 x 128 cells, r = 2: 1.26 -> 0.33 ms a launch (FP64
+// pipe; 96 registers, 128 and 168: 0.35).
+template <int R>
+struct VjpTeam {
+    static constexpr int TL = R == 3 ? 32 : 16;
+};
 template <int R, typename Pix, int MODE>
-__global__ void __maxnreg__(R == 3 ? 232 : 160)
+__global__ void __maxnreg__(96)
     k_residual_vjp(const __grid_constant__ Dev d,
                    const double* __restrict__ u, const uint8_t* __restrict__ cmask,
                    const double* __restrict__ rbar, double* __restrict__ ubar,
@@ -227,9 +94,11 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE>;
     constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP, NM = S::NM;
+    constexpr int TL = VjpTeam<R>::TL;
     extern __shared__ double smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    double* su = smem + warp * vjp_smem<R>();
+    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
+    const unsigned tm_ = TL == 32 ? 0xffffffffu : 0xFFFFu << (threadIdx.x & 16); // the team's lanes
+    double* su = smem + team * vjp_smem<R>();
     double* rb = su + 4 * ND;          // [6][ND] F, Gx, Gy, R, Lx, Ly bars of the cell
     double* tz = rb + 6 * ND;          // [2][ND1][NV] zeta: x-value, x-derivative
     double* tq = tz + 2 * ND1 * NV;    // [3][ND1][NV] qx, qy, c: x-value
@@ -242,17 +111,17 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
     const int64_t n = d.n;
     const size_t fs = (size_t)n * ND;  // field stride of the state and cotangent arrays
 
-    for (int64_t k = (int64_t)blockIdx.x * wpb + warp; k < n; k += (int64_t)gridDim.x * wpb) {
-        for (int i = lane; i < 4 * ND; i += 32) su[i] = u[(i / ND) * fs + k * ND + (i % ND)];
-        for (int i = lane; i < 6 * ND; i += 32) rb[i] = rbar[(i / ND) * fs + k * ND + (i % ND)];
+    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
+        for (int i = lane; i < 4 * ND; i += TL) su[i] = u[(i / ND) * fs + k * ND + (i % ND)];
+        for (int i = lane; i < 6 * ND; i += TL) rb[i] = rbar[(i / ND) * fs + k * ND + (i % ND)];
         const unsigned cm = cmask[k];
         const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
-        const double ihx = 1.0 / hx, ihy = 1.0 / hy;
+        const double ihx = d.ihxhy[2 * k], ihy = d.ihxhy[2 * k + 1];
         const double man = d.manning[k];
         const double nu = d.nu_c ? d.nu_c[k] : 0.0;
-        __syncwarp();
+        __syncwarp(tm_);
         if (nu != 0.0)
-            for (int i = lane; i < ND1 * NV; i += 32) {
+            for (int i = lane; i < ND1 * NV; i += TL) {
                 const int b = i / NV, al = i % NV;
                 double s = 0.0;
 #pragma unroll
@@ -261,21 +130,21 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
             }
         // x-contractions of the state (values at points) and of the cotangents
         // (value and d/dxi: the transposed test functions)
-        for (int i = lane; i < 2 * ND1 * NV; i += 32) {
+        for (int i = lane; i < 2 * ND1 * NV; i += TL) {
             const int f = i / (ND1 * NV), r_ = i % (ND1 * NV), b = r_ / NV, al = r_ % NV;
             double s = 0.0;
 #pragma unroll
             for (int a = 0; a < ND1; ++a) s += (f ? tb.Dv[al][a] : tb.Bv[al][a]) * su[ND1 * b + a];
             tz[i] = s;
         }
-        for (int i = lane; i < 3 * ND1 * NV; i += 32) {
+        for (int i = lane; i < 3 * ND1 * NV; i += TL) {
             const int f = i / (ND1 * NV), r_ = i % (ND1 * NV), b = r_ / NV, al = r_ % NV;
             double s = 0.0;
 #pragma unroll
             for (int a = 0; a < ND1; ++a) s += tb.Bv[al][a] * su[(1 + f) * ND + ND1 * b + a];
             tq[i] = s;
         }
-        for (int i = lane; i < 12 * ND1 * NV; i += 32) {
+        for (int i = lane; i < 12 * ND1 * NV; i += TL) {
             const int fd = i / (ND1 * NV), r_ = i % (ND1 * NV), b = r_ / NV, al = r_ % NV;
             const int fl = fd >> 1, der = fd & 1;
             double s = 0.0;
@@ -284,24 +153,10 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                 s += (der ? tb.Dv[al][a] : tb.Bv[al][a]) * rb[fl * ND + ND1 * b + a];
             tc[i] = s;
         }
-        __syncwarp();
-        // volume points: one per lane.  Of the 8 input directions of a point
-        // (z, z_xi, z_eta, qx, qy, c, delta, n) the dual numbers carry the first
-        // six: z and delta enter only through h = V(z + delta), so their
-        // derivatives are equal, and n only through gamma, which is
-        // proportional to n^2 (d gamma / dn = 2 gamma / n).  When the points
-        // fit in half a warp the two halves take the same point, each with
-        // three of the six directions (lane + 16 hands its three to lane), so
-        // the dual arithmetic runs on all 32 lanes
-        constexpr bool VSPLIT = NVP <= 16;
-        constexpr int VW = VSPLIT ? 3 : 6;         // directions per lane
-        const int vb0 = VSPLIT ? (lane >> 4) * VW : 0; // first direction of this lane
-        constexpr int VSTEP = VSPLIT ? 16 : 32;
+        __syncwarp(tm_);
+        // volume points: one per lane
         double dsum = 0.0, nsum = 0.0;
-        for (int p0 = 0; p0 < NVP; p0 += VSTEP) {
-            const int pl = p0 + (VSPLIT ? (lane & 15) : lane);
-            const bool pv = pl < NVP;    // a lane past the last point computes point 0, unused
-            const int p = pv ? pl : 0;
+        for (int p = lane; p < NVP; p += TL) {
             const int al = p % NV, be = p / NV;
             double z = 0.0, zxd = 0.0, zyd = 0.0, qx = 0.0, qy = 0.0, c = 0.0;
             // cotangent interpolations: [field][0: (Bv x, Bv y), 1: (Dv x, Bv y), 2: (Bv x, Dv y)]
@@ -339,42 +194,32 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                                    cb[1][1], cb[1][2], cb[1][0],               // Gx x, y, v
                                    cb[2][1], cb[2][2], cb[2][0],               // Gy x, y, v
                                    cb[4][0], cb[5][0]};                        // Lx, Ly
-            double xb[8];
+            // reverse pass: the cotangents of the outputs with their weights, then of
+            // the velocities, of the friction coefficient, and of the inputs
+            double xb[8]; // z, z_xi, z_eta, qx, qy, c, delta, n
             {
-                // dual directions: 0 z, 1 z_xi, 2 z_eta, 3 qx, 4 qy, 5 c
-                // (this lane: vb0 .. vb0 + VW - 1); 6 delta = 0 and 7 n follow
-                using DV = ad::DN<VW>;
-                const DV zx = DV::seed(zxd, 1 - vb0) * DV(ihx);
-                const DV zy = DV::seed(zyd, 2 - vb0) * DV(ihy);
-                const DV vqx = DV::seed(qx, 3 - vb0), vqy = DV::seed(qy, 4 - vb0);
-                const DV vc = DV::seed(c, 5 - vb0);
-                DV h(V);
-                h.set(0 - vb0, A);
-                const DV nn(man);
-                const DV fv = vel_factor<DV>(h, DV(eps));
-                const DV ux = fv * vqx, uy = fv * vqy;
-                const DV gam = gamma_manning<DV>(nn, h, vqx, vqy, DV(g), DV(eps));
-                const DV W(w), wx(w * ihx), wy(w * ihy), gg(g);
-                const DV X[12] = {wx * vqx, wy * vqy, wx * vc * vqx, wy * vc * vqy,
-                                  wx * vqx * ux, wy * vqx * uy, -(W * gg * h * zx),
-                                  wx * vqy * ux, wy * vqy * uy, -(W * gg * h * zy),
-                                  -(W * gam * vqx), -(W * gam * vqy)};
-#pragma unroll
-                for (int dir = 0; dir < VW; ++dir) {
-                    double s_ = 0.0;
-#pragma unroll
-                    for (int o = 0; o < 12; ++o) s_ += Xb[o] * X[o].d[dir];
-                    xb[dir] = s_;
-                }
-                if constexpr (VSPLIT) {
-#pragma unroll
-                    for (int dir = 0; dir < VW; ++dir)
-                        xb[VW + dir] = __shfl_down_sync(0xffffffffu, xb[dir], 16);
-                }
+                const double fv = vel_factor<double>(V, eps);
+                const double gam = gamma_manning<double>(man, V, qx, qy, g, eps);
+                const double ux = fv * qx, uy = fv * qy;
+                const double wx = w * ihx, wy = w * ihy;
+                const double a4 = wx * Xb[4], a5 = wy * Xb[5], a7 = wx * Xb[7], a8 = wy * Xb[8];
+                const double b6 = -(w * g) * Xb[6], b9 = -(w * g) * Xb[9];
+                const double l0 = -w * Xb[10], l1 = -w * Xb[11];
+                const double uxb = a4 * qx + a7 * qy, uyb = a5 * qx + a8 * qy;
+                const double gb = l0 * qx + l1 * qy; // of gamma
+                const double q2 = qx * qx + qy * qy, gq = q2 > 0.0 ? gb * gam / q2 : 0.0;
+                const double cx = wx * Xb[2], cy = wy * Xb[3];
+                const double fb = qx * uxb + qy * uyb;
+                const double hb = b6 * (zxd * ihx) + b9 * (zyd * ihy) -
+                                  (fb * fv + (7.0 / 3.0) * gb * gam) * log_hdes_slope(V, eps);
+                xb[0] = A * hb;
+                xb[1] = b6 * V * ihx;
+                xb[2] = b9 * V * ihy;
+                xb[3] = wx * Xb[0] + cx * c + a4 * ux + a5 * uy + fv * uxb + l0 * gam + gq * qx;
+                xb[4] = wy * Xb[1] + cy * c + a7 * ux + a8 * uy + fv * uyb + l1 * gam + gq * qy;
+                xb[5] = cx * qx + cy * qy;
                 xb[6] = xb[0]; // delta: as z, through h = V(z + delta)
-                // n: X_10 = -w gamma qx, X_11 = -w gamma qy with gamma ~ n^2
-                const double dgdn = man != 0.0 ? 2.0 * gam.v / man : 0.0;
-                xb[7] = -(Xb[10] * w * dgdn * qx + Xb[11] * w * dgdn * qy);
+                xb[7] = man != 0.0 ? 2.0 * gb * gam / man : 0.0; // gamma ~ n^2
             }
             // tracer numerical diffusion (Eq. numdiff): X_2 -= w nu h c_xi / hx^2,
             // X_3 -= w nu h c_eta / hy^2 (linear in grad c; h = V(z + delta))
@@ -393,15 +238,13 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                 xb[0] += A * xh;
                 xb[6] += A * xh;
             }
-            if (pv && (!VSPLIT || lane < 16)) {
-                for (int q = 0; q < 6; ++q) xv[q * NVP + p] = xb[q];
-                xv[6 * NVP + p] = xcx;
-                xv[7 * NVP + p] = xcy;
-                dsum += xb[6];
-                nsum += xb[7];
-            }
+            for (int q = 0; q < 6; ++q) xv[q * NVP + p] = xb[q];
+            xv[6 * NVP + p] = xcx;
+            xv[7 * NVP + p] = xcy;
+            dsum += xb[6];
+            nsum += xb[7];
         }
-        __syncwarp();
+        __syncwarp(tm_);
         // faces: one (sub)face point per lane, as the forward
         unsigned fi[4]; // indexed by constants only (registers)
 #pragma unroll
@@ -411,28 +254,15 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
         auto npts = [&](unsigned inf) { return (((inf & 3) == FI_COARSE) ? 2 : 1) * NM; };
         const int b1 = npts(fi[0]), b2 = b1 + npts(fi[1]), b3 = b2 + npts(fi[2]),
                   b4 = b3 + npts(fi[3]);
-        // the own side's directions at a face point: zeta, qx, qy and delta
-        // are carried by dual numbers; the tracer flux is linear in the
-        // concentrations, so the c direction is its partial derivative dc
-        // (from the same flux evaluation).  As for the volume points: with at
-        // most 16 face points per conforming cell the two halves share a
-        // point, directions 0-1 and 2-3
-        constexpr bool FSPLIT = 4 * NM <= 16;
-        constexpr int FW = FSPLIT ? 2 : 4;
-        const int fb0 = FSPLIT ? (lane >> 4) * FW : 0;
-        constexpr int FSTEP = FSPLIT ? 16 : 32;
-        for (int it0 = 0; it0 < b4; it0 += FSTEP) {
-            const int il = it0 + (FSPLIT ? (lane & 15) : lane);
-            const bool iv = il < b4; // a lane past the last point computes point 0, unused
-            const int it = iv ? il : 0;
+        for (int it = lane; it < b4; it += TL) {
             const int f = (it >= b1) + (it >= b2) + (it >= b3);
             const int r_ = it - (f == 0 ? 0 : f == 1 ? b1 : f == 2 ? b2 : b3), h = r_ / NM,
                       al = r_ % NM;
             const unsigned info = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
             const bool coarse = (info & 3) == FI_COARSE, fine = (info & 3) == FI_FINE;
             const int half = (int)(info >> 2);
-            const double nx = (f == 0) ? -1.0 : (f == 1) ? 1.0 : 0.0;
-            const double ny = (f == 2) ? -1.0 : (f == 3) ? 1.0 : 0.0;
+            const int ax = f >> 1;
+            const double sg = (f & 1) ? 1.0 : -1.0; // the outward normal along the axis
             const double L = ((f < 2) ? hy : hx) * (coarse ? 0.5 : 1.0);
             const double wl = L * tb.wm[al];
             const double(*Bown)[MXN] = coarse ? tb.BmH[h] : tb.Bm;
@@ -450,12 +280,23 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
             const int32_t s0 = d.nbr[k * 8 + f * 2];
             double hm, Am;
             own_VA(tm[0], hm, Am);
-            double xb[5], xl[FW], xc = 0.0; // xc: the c direction
-            if (s0 >= 0) {
+            // the own side (as side A of the flux) and the other: the neighbour, a
+            // mirrored state or the tide over the own operator.  Both fluxes follow
+            // from one: F_own = raw - pres n, F_nb = -raw - pres n
+            VjpSide so, sp;
+            so.h = hm;
+            so.qn = ax ? tm[2] : tm[1];
+            so.qt = ax ? tm[1] : tm[2];
+            so.c = tm[3];
+            double yp[4] = {0.0, 0.0, 0.0, 0.0};
+            double Ao = Am, Az = Am, Ap = 0.0; // d h*own / d delta, / d zeta; d h*other / d delta
+            const bool bnd = s0 < 0;
+            bool tide = false;
+            if (!bnd) {
                 const int64_t nb = coarse ? (int64_t)(h ? d.nbr[k * 8 + f * 2 + 1] : s0) : (int64_t)s0;
                 const int fo = f ^ 1;
                 const double(*Bnb)[MXN] = fine ? tb.BmH[half] : tb.Bm;
-                double tp[4], yp[4];
+                double tp[4];
                 face_trace<ND1>(u + nb * ND, fs, cmask[nb], fo, Bnb, al, tp);
                 face_trace<ND1>(rbar + nb * ND, fs, 0u, fo, Bnb, al, yp);
 #pragma unroll
@@ -466,125 +307,79 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                     if (fine) ST::VA_half(d, nb, fo, half, al, eta, V, A);
                     else ST::VA(d, tb, nb, SET_MASS, ja, jb, eta, V, A);
                 };
-                double hp, Ap, Vnm, Anm, Vop, Aop;
-                nb_VA(tp[0], hp, Ap);
+                double hp, Ax, Vnm, Anm, Vop, Aop;
+                nb_VA(tp[0], hp, Ax);
                 nb_VA(tm[0], Vnm, Anm);
                 own_VA(tp[0], Vop, Aop);
-                {
-                    // dual directions of the own side: 0 zeta, 1 qx, 2 qy, 3 delta
-                    // (this lane: fb0 .. fb0 + FW - 1)
-                    using DF = ad::DN<FW>;
-                    const DF qxm = DF::seed(tm[1], 1 - fb0), qym = DF::seed(tm[2], 2 - fb0);
-                    const DF cmv(tm[3]);
-                    DF hmD(hm), vnmD(Vnm), vopD(Vop);
-                    hmD.set(0 - fb0, Am);   // own operator at own zeta
-                    hmD.set(3 - fb0, Am);
-                    vnmD.set(0 - fb0, Anm); // neighbour's operator at own zeta
-                    vopD.set(3 - fb0, Aop); // own operator at neighbour's zeta
-                    const DF hpD(hp);
-                    const DF hsm = ad::fmin(hmD, vnmD), hsp = ad::fmin(hpD, vopD);
-                    const DF qxp(tp[1]), qyp(tp[2]), cpv(tp[3]);
-                    // the face is evaluated once, the lower cell index as side A
-                    // (as the forward does); the flux of each side follows from it:
-                    // F_side = s raw - pres n_A (momentum), s = +1 for side A, -1 for B
-                    // (one call with the sides selected, so the warp does not split)
-                    const bool own_low = k < nb;
-                    const DF aqx = own_low ? qxm : qxp, aqy = own_low ? qym : qyp;
-                    const DF ac = own_low ? cmv : cpv, ah = own_low ? hmD : hpD;
-                    const DF ahs = own_low ? hsm : hsp;
-                    const DF bqx = own_low ? qxp : qxm, bqy = own_low ? qyp : qym;
-                    const DF bc = own_low ? cpv : cmv, bh = own_low ? hpD : hmD;
-                    const DF bhs = own_low ? hsp : hsm;
-                    const double nAx = own_low ? nx : -nx, nAy = own_low ? ny : -ny;
-                    DF raw[4], pres, lam, dcs[2];
-                    rusanov<DF, true>(aqx, aqy, ac, ah, ahs, bqx, bqy, bc, bh, bhs, ahs - bhs,
-                                      DF(nAx), DF(nAy), DF(g), DF(eps), raw, pres, lam, dcs);
-                    const DF pnx = pres * DF(nAx), pny = pres * DF(nAy);
-                    const DF so(own_low ? 1.0 : -1.0), sn(own_low ? -1.0 : 1.0);
-                    DF oo[4], on[4]; // own side's flux, the neighbour's (its own normal)
-                    oo[0] = so * raw[0];
-                    oo[1] = so * raw[1] - pnx;
-                    oo[2] = so * raw[2] - pny;
-                    oo[3] = so * raw[3];
-                    on[0] = sn * raw[0];
-                    on[1] = sn * raw[1] - pnx;
-                    on[2] = sn * raw[2] - pny;
-                    on[3] = sn * raw[3];
-#pragma unroll
-                    for (int dir = 0; dir < FW; ++dir) {
-                        double s_ = 0.0;
-#pragma unroll
-                        for (int cf = 0; cf < 4; ++cf) s_ += ym[cf] * oo[cf].d[dir] + yp[cf] * on[cf].d[dir];
-                        xl[dir] = s_;
-                    }
-                    // c of the own side: only the tracer flux, R_own = so raw3,
-                    // R_nb = sn raw3
-                    xc = (ym[3] * so.v + yp[3] * sn.v) * (own_low ? dcs[0].v : dcs[1].v);
-                }
+                // h*own = min(V_own(zeta_own), V_nb(zeta_own)): the own operator at ties;
+                // h*other = min(V_nb(zeta_nb), V_own(zeta_nb)): the neighbour's
+                so.hs = hm <= Vnm ? hm : Vnm;
+                Ao = hm <= Vnm ? Am : 0.0;
+                Az = hm <= Vnm ? Am : Anm;
+                sp.h = hp;
+                sp.hs = hp <= Vop ? hp : Vop;
+                Ap = hp <= Vop ? 0.0 : Aop;
+                sp.qn = ax ? tp[2] : tp[1];
+                sp.qt = ax ? tp[1] : tp[2];
+                sp.c = tp[3];
             } else {
                 const int tag = -1 - s0;
                 const int mem = member_of(d, k);
-                const double t = d.mb[mem].t;
-                const bool tide = d.mbc ? d.mbc[mem].kind[tag] == 1 : d.bc_kind[tag] == 1;
-                double zt = 0.0, Vt = 0.0, At = 0.0;
+                tide = d.mbc ? d.mbc[mem].kind[tag] == 1 : d.bc_kind[tag] == 1;
+                so.hs = hm;
+                sp = so;
                 if (tide) {
                     const double amp = d.mbc ? d.mbc[mem].amp[tag] : d.bc_amp[tag];
                     const double per = d.mbc ? d.mbc[mem].per[tag] : d.bc_per[tag];
                     const double ph = d.mbc ? d.mbc[mem].ph[tag] : d.bc_ph[tag];
-                    zt = amp * sin(2.0 * M_PI * t / per + ph);
-                    own_VA(zt, Vt, At);
-                }
-                {
-                    using DF = ad::DN<FW>;
-                    const DF qxm = DF::seed(tm[1], 1 - fb0), qym = DF::seed(tm[2], 2 - fb0);
-                    const DF cmv(tm[3]);
-                    DF hmD(hm);
-                    hmD.set(0 - fb0, Am);
-                    hmD.set(3 - fb0, Am);
-                    DF qxp = qxm, qyp = qym, hpD = hmD;
-                    if (tide) {
-                        hpD = DF(Vt); // ghost elevation fixed, same operator
-                        hpD.set(3 - fb0, At);
-                    } else {
-                        const DF qn = qxm * DF(nx) + qym * DF(ny);
-                        qxp = qxm - DF(2.0) * qn * DF(nx);
-                        qyp = qym - DF(2.0) * qn * DF(ny);
-                    }
-                    DF oo[4], dcs[2];
-                    side_flux<DF, true>(qxm, qym, cmv, hmD, hmD, qxp, qyp, cmv, hpD, hpD, nx, ny, g,
-                                        eps, oo, dcs);
-#pragma unroll
-                    for (int dir = 0; dir < FW; ++dir) {
-                        double s_ = 0.0;
-#pragma unroll
-                        for (int cf = 0; cf < 4; ++cf) s_ += ym[cf] * oo[cf].d[dir];
-                        xl[dir] = s_;
-                    }
-                    // the ghost carries the own concentration: both partials
-                    xc = ym[3] * (dcs[0].v + dcs[1].v);
+                    double At;
+                    own_VA(amp * sin(2.0 * M_PI * d.mb[mem].t / per + ph), sp.h, At);
+                    sp.hs = sp.h;
+                    Ap = At;
+                } else {
+                    sp.qn = -so.qn;
+                    Ap = Am;
                 }
             }
-            // all lanes (the branches have joined): gather the five directions
-            // xb = {zeta, qx, qy, c, delta}
-            if constexpr (FSPLIT) {
-                xb[0] = xl[0];
-                xb[1] = xl[1];
-                xb[2] = __shfl_down_sync(0xffffffffu, xl[0], 16);
-                xb[4] = __shfl_down_sync(0xffffffffu, xl[1], 16);
-            } else {
-                xb[0] = xl[0];
-                xb[1] = xl[1];
-                xb[2] = xl[2];
-                xb[4] = xl[3];
+            so.form(d);
+            sp.form(d);
+            const double lA = ::fabs(so.v) + so.w, lB = ::fabs(sp.v) + sp.w;
+            const double hl = 0.5 * ::fmax(lA, lB), hs = 0.5 * sg;
+            const double qA = so.hs * so.v, qB = sp.hs * sp.v, rA = so.hs * so.u, rB = sp.hs * sp.u;
+            // cotangents of raw (F, axis, tangential, R) and of the pressure scalar
+            const double yma = ax ? ym[2] : ym[1], ymt = ax ? ym[1] : ym[2];
+            const double ypa = ax ? yp[2] : yp[1], ypt = ax ? yp[1] : yp[2];
+            const double Fb = ym[0] - yp[0], Gb = yma - ypa, Tb = ymt - ypt, Rb = ym[3] - yp[3];
+            const double pb = -(yma + ypa) * (0.5 * g * sg);
+            const double lb = 0.5 * (Fb * (so.hs - sp.hs) + Gb * (qA - qB) + Tb * (rA - rB) +
+                                     Rb * (so.hs * so.c - sp.hs * sp.c));
+            // the wave-speed bound: the symmetric subgradient at an exact tie
+            const double lAb = lA > lB ? lb : lA < lB ? 0.0 : 0.5 * lb;
+            const double qAb = hs * (Fb + Gb * so.v + Rb * so.c) + hl * Gb, rAb = Tb * (hs * so.v + hl);
+            const double qBb = hs * (Fb + Gb * sp.v + Rb * sp.c) - hl * Gb, rBb = Tb * (hs * sp.v - hl);
+            const double hAb = qAb * so.v + rAb * so.u + hl * (Fb + Rb * so.c) + pb * so.hs; // of h*own
+            const double hBb = qBb * sp.v + rBb * sp.u - hl * (Fb + Rb * sp.c) - pb * sp.hs; // of h*other
+            double qnb, qtb, hb;
+            so.back(d, qAb, rAb, lAb, hs * (Gb * qA + Tb * rA), qnb, qtb, hb);
+            double cb_ = Rb * (hs * qA + hl * so.hs);
+            double zb = hb * Am + hAb * Az, db = hb * Am + hAb * Ao + hBb * Ap;
+            if (bnd) { // the other side depends on the own state as well
+                double qnB, qtB, hB;
+                sp.back(d, qBb, rBb, lb - lAb, hs * (Gb * qB + Tb * rB), qnB, qtB, hB);
+                qnb += tide ? qnB : -qnB;
+                qtb += qtB;
+                cb_ += Rb * (hs * qB - hl * sp.hs);
+                db += hB * Ap;
+                if (!tide) zb += (hB + hBb) * Am;
             }
-            xb[3] = xc;
-            if (iv && (!FSPLIT || lane < 16)) {
-#pragma unroll
-                for (int cf = 0; cf < 4; ++cf) xf[((cf * 4 + f) * 2 + h) * NM + al] = xb[cf];
-                dsum += xb[4];
-            }
+            const int q = ((f * 2 + h) * NM) + al;
+            xf[q] = zb;
+            xf[8 * NM + q] = ax ? qtb : qnb;
+            xf[16 * NM + q] = ax ? qnb : qtb;
+            xf[24 * NM + q] = cb_;
+            dsum += db;
         }
-        __syncwarp();
+        __syncwarp(tm_);
         // transposed interpolation of the volume-point cotangents, every field
         // in one uniform pass per direction.  y: segments of NV ND1 jobs --
         // 0 zeta (Bv z + Dv z_eta), 1 zeta (Bv z_xi), 2 qx, 3 qy (Bv), 4 c
@@ -596,7 +391,7 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
             constexpr int NY = NV * ND1;
             double* ty = tc; // [6][NV][ND1]
             const int nseg = nu != 0.0 ? 6 : 5;
-            for (int i = lane; i < nseg * NY; i += 32) {
+            for (int i = lane; i < nseg * NY; i += TL) {
                 const int seg = i / NY, r_ = i % NY, al = r_ / ND1, b = r_ % ND1;
                 const int src1 = seg == 0 ? 0 : seg == 1 ? 1 : seg == 5 ? 6 : seg + 1;
                 const double* x1 = xv + src1 * NVP + al;
@@ -608,9 +403,9 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                     s_ += tb.Bv[be][b] * x1[NV * be] + m2 * (tb.Dv[be][b] * x2[NV * be]);
                 ty[i] = s_;
             }
-            __syncwarp();
+            __syncwarp(tm_);
             double* uacc = xv; // [4][ND]: the point cotangents are consumed by now
-            for (int i = lane; i < 4 * ND; i += 32) {
+            for (int i = lane; i < 4 * ND; i += TL) {
                 const int fl = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
                 // (without diffusion the c_xi segment is not formed: t2 = t1, times 0)
                 const int sa = fl == 0 ? 0 : fl + 1, sb = fl == 0 ? 1 : (nu != 0.0 ? 5 : sa);
@@ -629,10 +424,10 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
         // a = 0, ND1 - 1) and then the y faces (rows b = 0, ND1 - 1), one item
         // per field, face and node along it, as in the forward residual
         double* uacc = xv;
-        __syncwarp();
+        __syncwarp(tm_);
 #pragma unroll
         for (int pass = 0; pass < 2; ++pass) {
-            for (int i = lane; i < 4 * 2 * ND1; i += 32) {
+            for (int i = lane; i < 4 * 2 * ND1; i += TL) {
                 const int cf = i / (2 * ND1), r_ = i % (2 * ND1), f = 2 * pass + r_ / ND1;
                 const int tn = r_ % ND1; // node index along the face
                 const unsigned inf = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
@@ -648,19 +443,20 @@ __global__ void __maxnreg__(R == 3 ? 232 : 160)
                 }
                 uacc[cf * ND + face_node<ND1>(f, tn)] += s;
             }
-            __syncwarp();
+            __syncwarp(tm_);
         }
-        for (int i = lane; i < 4 * ND; i += 32) {
+        for (int i = lane; i < 4 * ND; i += TL) {
             const int cf = i / ND, j = i % ND;
             if (accumulate) ubar[cf * fs + k * ND + j] += uacc[i];
             else ubar[cf * fs + k * ND + j] = uacc[i];
         }
-        const double ds = warp_sum(dsum), ns = warp_sum(nsum);
+        team_sum2<TL>(dsum, nsum, tm_);
+        const double ds = dsum, ns = nsum;
         if (lane == 0) {
             dbar[k] = accumulate ? dbar[k] + ds : ds;
             nbar[k] = accumulate ? nbar[k] + ns : ns;
         }
-        __syncwarp();
+        __syncwarp(tm_);
     }
 }
 
@@ -971,16 +767,15 @@ __global__ void __maxnreg__(128)
                 double V, A;
                 ST::VA(d, tb, k, SET_MOM, p % NG, p / NG, g3[p], V, A);
                 const double qx = g3[NGP + p], qy = g3[2 * NGP + p], gbp = gb[p];
-                // directions: 0 h, 1 qx, 2 qy, 3 n
-                using DG = ad::DN<4>;
-                const DG r = gamma_manning<DG>(DG::seed(man, 3), DG::seed(V, 0), DG::seed(qx, 1),
-                                               DG::seed(qy, 2), DG(g), DG(eps));
-                const double* dg = r.d;
-                g3[p] = gbp * dg[0] * A;
-                g3[NGP + p] = gbp * dg[1];
-                g3[2 * NGP + p] = gbp * dg[2];
-                dsum += gbp * dg[0] * A;
-                nsum += gbp * dg[3];
+                // gamma ~ n^2 |q| h_des^(-7/3)
+                const double gg = gbp * gamma_manning<double>(man, V, qx, qy, g, eps);
+                const double q2 = qx * qx + qy * qy, iq = q2 > 0.0 ? gg / q2 : 0.0;
+                const double gh = -(7.0 / 3.0) * gg * log_hdes_slope(V, eps) * A;
+                g3[p] = gh;
+                g3[NGP + p] = iq * qx;
+                g3[2 * NGP + p] = iq * qy;
+                dsum += gh;
+                nsum += 2.0 * gg / man;
             }
             __syncwarp(tm);
             for (int f = 0; f < 3; ++f) {

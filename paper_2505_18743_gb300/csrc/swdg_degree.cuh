@@ -23,7 +23,7 @@ struct Launchers {
     static constexpr size_t stage_b =
         2 * sizeof(double) * StageFx<R>::words(sizeof(B) != sizeof(double));
     static constexpr size_t diag_b = sizeof(double) * (2 * S::ND + 2 * S::NMP + 2 * S::NM * S::NM);
-    static constexpr size_t vjp_b = sizeof(double) * vjp_smem<R>();
+    static constexpr size_t vjp_b = sizeof(double) * vjp_smem<R>() * (32 / VjpTeam<R>::TL); // per warp
     static constexpr size_t svjp_b = 2 * sizeof(double) * stage_vjp_smem<R>(); // two cells per warp
     static constexpr size_t bvjp_b = sizeof(double) * begin_vjp_smem<R>();
     static constexpr size_t ind_b = sizeof(double) * indicator_smem<R>();
@@ -83,7 +83,9 @@ struct Launchers {
     static void residual_vjp(const Dev& d, const Tables& tb, const double* u, const uint8_t* cm,
                              const double* rbar, double* ubar, double* nbar, double* dbar,
                              int accumulate, Shape s, cudaStream_t st) {
-        k_residual_vjp<R, Pix, MODE><<<s.grid, 32 * s.wpb, vjp_b * s.wpb, st>>>(
+        const int cpb = s.wpb * 32 / VjpTeam<R>::TL;
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
+        k_residual_vjp<R, Pix, MODE><<<grid, 32 * s.wpb, vjp_b * s.wpb, st>>>(
             d, u, cm, rbar, ubar, nbar, dbar, accumulate);
     }
     static void stage_vjp(const Dev& d, const Tables& tb, const StageVjpArgs& a, Shape s,

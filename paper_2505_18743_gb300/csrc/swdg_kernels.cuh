@@ -346,32 +346,22 @@ __device__ __forceinline__ void face_trace(const double* u, size_t fstride, unsi
     }
 }
 
-// The wave-speed bound's maximum (Eq. lxf_parameter).  For plain arithmetic
-// types it is fmax; the adjoint's dual types overload it (found by
-// argument-dependent lookup) with the symmetric subgradient at exact ties.
-template <typename T>
-__device__ __forceinline__ T wave_speed_max(T a, T b) {
-    return fmax(a, b);
-}
-
 // Rusanov flux with hydrostatic reconstruction at one face point, seen from
 // side A with outward normal (nx, ny) (Eqs. lxf_parameter, velocity,
 // hydro_rec_vars, mass_rhs, discharge_rhs, r_concentration).  hA = V_A(zeta_A),
 // hsA = min(V_A(zeta_A), V_B(zeta_A)).  out = {F, Gx_cons, Gy_cons, R}; the
 // non-conservative pressure scalar g {{h*}} (h*A - h*B)/2 is returned apart.
-// DC (the adjoint): dc = {dR/dcA, dR/dcB}, the tracer flux's partial
-// derivatives in the two concentrations (it is linear in each).
-template <typename T, bool DC = false>
+template <typename T>
 __device__ __forceinline__ void rusanov(T qxA, T qyA, T cA, T hA, T hsA, T qxB, T qyB, T cB, T hB,
                                         T hsB, T dhAB, T nx, T ny, T g, T eps, T out[4], T& pres,
-                                        T& lam, T* dc = nullptr) {
+                                        T& lam) {
     // dhAB = h*A - h*B, formed in FP64 by the caller (the well-balanced part of
     // the reconstruction); the tracer jump h*A cA - h*B cB = dhAB cA + h*B (cA - cB)
     const T half = T(0.5);
     T fA = vel_factor<T>(hA, eps), fB = vel_factor<T>(hB, eps);
     T uAx = fA * qxA, uAy = fA * qyA, uBx = fB * qxB, uBy = fB * qyB;
     T unA = uAx * nx + uAy * ny, unB = uBx * nx + uBy * ny;
-    T l = wave_speed_max(fabs(unA) + sqrt(g * hA), fabs(unB) + sqrt(g * hB));
+    T l = fmax(fabs(unA) + sqrt(g * hA), fabs(unB) + sqrt(g * hB));
     T qsAx = hsA * uAx, qsAy = hsA * uAy, qsBx = hsB * uBx, qsBy = hsB * uBy;
     out[0] = half * ((qsAx + qsBx) * nx + (qsAy + qsBy) * ny) + half * l * dhAB;
     out[1] = half * (qsAx * unA + qsBx * unB) + half * l * (qsAx - qsBx);
@@ -380,11 +370,6 @@ __device__ __forceinline__ void rusanov(T qxA, T qyA, T cA, T hA, T hsA, T qxB, 
              half * l * (dhAB * cA + hsB * (cA - cB));
     pres = g * half * (hsA + hsB) * half * dhAB;
     lam = l;
-    if constexpr (DC) {
-        // R = 1/2 (qs_A cA + qs_B cB).n + l/2 (h*A cA - h*B cB)
-        dc[0] = half * (qsAx * nx + qsAy * ny) + half * l * hsA;
-        dc[1] = half * (qsBx * nx + qsBy * ny) - half * l * hsB;
-    }
 }
 
 __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double v) {
