@@ -330,6 +330,16 @@ static void build_fx_tables(int R, Tables& tb) {
     y.tGi = put(&tb.Bginv[0][0], MXP, false, n1, n1, &y.Gi[0][0], MXN);
     y.tGiT = put(&tb.Bginv[0][0], MXP, true, n1, n1, &y.GiT[0][0], MXN);
     y.tM1i = put(&tb.M1inv[0][0], MXN, false, n1, n1, &y.M1i[0][0], MXN);
+    BulkTables& z = tb.fb;
+    z.tBv = put(&tb.Bv[0][0], MXN, false, nv, n1, &z.Bv[0][0], MXN);
+    z.tBvT = put(&tb.Bv[0][0], MXN, true, n1, nv, &z.BvT[0][0], MXP);
+    z.tDvT = put(&tb.Dv[0][0], MXN, true, n1, nv, &z.DvT[0][0], MXP);
+    memcpy(z.BmT, x.BmT, sizeof z.BmT);
+    memcpy(z.BmHT, x.BmHT, sizeof z.BmHT);
+    z.tBmT = x.tBmT;
+    memcpy(z.BvF, tb.BvF, sizeof z.BvF);
+    memcpy(z.DvF, tb.DvF, sizeof z.DvF);
+    memcpy(z.wvF, tb.wvF, sizeof z.wvF);
     memcpy(y.wm, tb.wm, sizeof y.wm);
     memcpy(y.wg, tb.wg, sizeof y.wg);
     memcpy(y.BmF, tb.BmF, sizeof y.BmF);

@@ -102,6 +102,16 @@ struct FaceTables {
     float BmF[MXP][MXN], BmHF[2][MXP][MXN];
 };
 
+// what the FP32-bulk residual takes: digit pairs of the elevation's interpolation
+// and of the test integrals of F and R (the transposes, without weights), the
+// face test tables of FxTables, and the FP32 basis
+struct BulkTables {
+    int2 Bv[MXP][MXN], BvT[MXN][MXP], DvT[MXN][MXP];
+    int2 BmT[MXN][MXP], BmHT[2][MXN][MXP];
+    float BvF[MXP][MXN], DvF[MXP][MXN], wvF[MXP];
+    int tBv, tBvT, tDvT, tBmT;
+};
+
 struct Tables {
     double Bv[MXP][MXN], Dv[MXP][MXN], wv[MXP]; // nodal -> volume GL (value, d/dxi)
     double Bm[MXP][MXN], wm[MXP];               // nodal -> mass / face GLL
@@ -119,6 +129,7 @@ struct Tables {
     FxTables fx;
     FxStage fs;
     FaceTables ft;
+    BulkTables fb;
 };
 
 // clock of one ensemble member (a plain context is an ensemble of one)

@@ -13,10 +13,10 @@ struct Launchers {
     using S = Sz<R>;
     static constexpr bool F64 = sizeof(B) == sizeof(double);
     static constexpr size_t res_b =
-        sizeof(double) * (F64 ? ResFx<R>::words * (32 / ResFx<R>::TL) : res_smem<R, B>()); // per warp
+        sizeof(double) * (F64 ? ResFx<R>::words : ResBulk<R>::words) * (32 / ResFx<R>::TL); // per warp
     static auto residual_kernel() {
         if constexpr (F64) return k_residual<R, Pix, MODE>;
-        else return k_residual_bulk<R, Pix, MODE, B>;
+        else return k_residual_bulk<R, Pix, MODE>;
     }
     static constexpr size_t begin_b = 2 * sizeof(double) * BeginFx<R>::words; // two cells per warp
     // k_stage runs two cells per warp (a team of 16 lanes each)
@@ -31,10 +31,10 @@ struct Launchers {
 
     static void residual(const Dev& d, const Tables& tb, int buf, int stage, double c_stage,
                          int want_dt, Shape s, cudaStream_t st) {
+        // 32 / TL cells per warp: no more blocks than their cells
+        const int cpb = s.wpb * 32 / ResFx<R>::TL;
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
         if constexpr (F64) {
-            // 32 / TL cells per warp: no more blocks than their cells
-            const int cpb = s.wpb * 32 / ResFx<R>::TL;
-            const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
             if (MODE == 0 && !d.fflux)
                 k_residual<R, Pix, 0, true><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage,
                                                                                      c_stage, want_dt);
@@ -42,8 +42,7 @@ struct Launchers {
                 k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage, c_stage,
                                                                                   want_dt);
         } else {
-            k_residual_bulk<R, Pix, MODE, B><<<s.grid, 32 * s.wpb, res_b * s.wpb, st>>>(
-                d, buf, stage, c_stage, want_dt);
+            k_residual_bulk<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage);
         }
     }
     static void faces(const Dev& d, const Tables& tb, int buf, double c_stage, int want_dt,

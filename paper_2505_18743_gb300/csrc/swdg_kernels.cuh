@@ -382,20 +382,6 @@ __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double 
 // r+2 Gauss-Lobatto points per face (Eqs. mass_rhs, discharge_rhs,
 // discharge_rhs_implicit, r_concentration)
 // ---------------------------------------------------------------------------
-template <int R, typename B>
-constexpr int res_smem() {
-    // in doubles: su [4 ND], tz [2 ND1 NV], Xd [4 NVP], sd [4 NV ND1], fh [32 NM], rs [6 ND],
-    // tc [2 ND1 NV] (tracer diffusion), then B-typed: suB [4 ND], tB [3 ND1 NV] (B = double;
-    // [5 ND1 NV] for B = float, with the elevation's two x-contractions), XB [8 NVP],
-    // sB [8 NV ND1]
-    using S = Sz<R>;
-    constexpr int nd = 4 * S::ND + 2 * S::ND1 * S::NV + 4 * S::NVP + 4 * S::NV * S::ND1 +
-                       32 * S::NM + 6 * S::ND + 2 * S::ND1 * S::NV;
-    constexpr int ntb = sizeof(B) == sizeof(double) ? 3 : 5;
-    constexpr int nb = 4 * S::ND + ntb * S::ND1 * S::NV + 8 * S::NVP + 8 * S::NV * S::ND1;
-    return nd + (nb * (int)sizeof(B) + 7) / 8;
-}
-
 // traces of zeta (FP64) and of qx, qy, c (type B) at face point al of face f;
 // u32 (B = float, nullable): the FP32 copy of u, same layout and stride
 template <int ND1, typename B>
@@ -734,6 +720,78 @@ struct ResFx {
     static_assert(S::NVP <= TL && S::ND <= SUB, "one point per lane");
 };
 
+// the face fluxes of a conforming cell F [4 fields][4 faces][2 halves][NM], slots
+// i = (face, point) spread over the team's lanes
+template <int NM, int TL>
+__device__ __forceinline__ void face_load(const double* F, double (&fv)[(4 * NM + TL - 1) / TL][4],
+                                          int lane) {
+#pragma unroll
+    for (int j = 0; j < (4 * NM + TL - 1) / TL; ++j) {
+        const int i = lane + j * TL;
+        const double* Fi = F + (i / NM) * 2 * NM + i % NM;
+#pragma unroll
+        for (int cf = 0; cf < 4; ++cf) fv[j][cf] = i < 4 * NM ? Fi[cf * 8 * NM] : 0.0;
+    }
+}
+// ... to digits, field by field: fd [4 fields][2 halves][4 faces][NM], block exponents es
+template <int NM, int TL>
+__device__ __forceinline__ void face_digits(const double (&fv)[(4 * NM + TL - 1) / TL][4], int2* fd,
+                                            int* es, int lane, unsigned tm) {
+    constexpr int SL = (4 * NM + TL - 1) / TL;
+#pragma unroll
+    for (int cf = 0; cf < 4; ++cf) {
+        unsigned m = 0;
+#pragma unroll
+        for (int j = 0; j < SL; ++j) m = max(m, fx::mag(fv[j][cf]));
+        const int e = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll
+        for (int j = 0; j < SL; ++j)
+            if (lane + j * TL < 4 * NM)
+                fd[cf * 8 * NM + lane + j * TL] = fx::split(fx::from_double(fv[j][cf], e));
+        if (lane == 0) es[cf] = e;
+    }
+}
+// the same where faces have second halves (or were integrated inline): slot(cf, i),
+// i = (half, face, point) < nslot
+template <int NM, int TL, typename F>
+__device__ __forceinline__ void face_digits_any(F slot, int nslot, int2* fd, int* es, int lane, unsigned tm) {
+#pragma unroll 1
+    for (int cf = 0; cf < 4; ++cf) {
+        unsigned m = 0;
+#pragma unroll 1
+        for (int i = lane; i < nslot; i += TL) m = max(m, fx::mag(slot(cf, i)));
+        const int e = fx::block_exp(__reduce_max_sync(tm, m));
+#pragma unroll 1
+        for (int i = lane; i < nslot; i += TL) fd[cf * 8 * NM + i] = fx::split(fx::from_double(slot(cf, i), e));
+        if (lane == 0) es[cf] = e;
+    }
+}
+// one field's face fluxes lifted onto node (a, b) (a node takes part in at most one
+// x face and one y face)
+template <int ND1, int NM, typename T>
+__device__ __forceinline__ long long face_lift(const T& tx, const int2* fd, int a, int b,
+                                               const bool (&c_f)[4]) {
+    long long sf = 0;
+    auto lift = [&](int f, int tn, bool coarse) {
+        fx::Acc q;
+        const int2* v = fd + f * NM;
+        if (!coarse) {
+#pragma unroll
+            for (int al = 0; al < NM; ++al) q.mac(tx.BmT[tn][al], v[al]);
+        } else {
+#pragma unroll
+            for (int al = 0; al < NM; ++al) {
+                q.mac(tx.BmHT[0][tn][al], v[al]);
+                q.mac(tx.BmHT[1][tn][al], v[4 * NM + al]);
+            }
+        }
+        sf += q.get();
+    };
+    if (a == 0 || a == ND1 - 1) lift(a == 0 ? 0 : 1, b, a == 0 ? c_f[0] : c_f[1]);
+    if (b == 0 || b == ND1 - 1) lift(b == 0 ? 2 : 3, a, b == 0 ? c_f[2] : c_f[3]);
+    return sf;
+}
+
 #ifndef RES_REGS
 #define RES_REGS 64
 #endif
@@ -921,18 +979,9 @@ __global__ void __maxnreg__(RES_REGS)
         __syncwarp(tm);
         // the face fluxes of k_faces; where no face of the cell has a second half they
         // are loaded here, so that the y-contraction hides the latency
-        constexpr int SL = (4 * NM + TL - 1) / TL;
         const bool conforming = nslot == 4 * NM;
-        double fv[SL][4];
-        if (!INL && conforming) {
-#pragma unroll
-            for (int j = 0; j < SL; ++j) {
-                const int i = lane + j * TL;
-                const double* F = d.fflux + k * (32 * NM) + (i / NM) * 2 * NM + i % NM;
-#pragma unroll
-                for (int cf = 0; cf < 4; ++cf) fv[j][cf] = i < 4 * NM ? F[cf * 8 * NM] : 0.0;
-            }
-        }
+        double fv[(4 * NM + TL - 1) / TL][4];
+        if (!INL && conforming) face_load<NM, TL>(d.fflux + k * (32 * NM), fv, lane);
         // test integration, y-contraction: jobs 0..3 the xi-parts of F, R, Gx, Gy
         // (wv Bv), 4, 5 Lx, Ly, 6..8 the eta-parts of F, R, Gx (wv Dv), 9 the value
         // part of Gx; then 10 the eta- and value parts of Gy
@@ -994,38 +1043,15 @@ __global__ void __maxnreg__(RES_REGS)
             }
             __syncwarp(tm);
         }
-        // the face fluxes to digits, field by field: slot i = (half, face, point)
         if (!INL && conforming) {
-#pragma unroll
-            for (int cf = 0; cf < 4; ++cf) {
-                unsigned m = 0;
-#pragma unroll
-                for (int j = 0; j < SL; ++j) m = max(m, fx::mag(fv[j][cf]));
-                const int e = fx::block_exp(__reduce_max_sync(tm, m));
-#pragma unroll
-                for (int j = 0; j < SL; ++j)
-                    if (lane + j * TL < 4 * NM)
-                        fd[cf * 8 * NM + lane + j * TL] = fx::split(fx::from_double(fv[j][cf], e));
-                if (lane == 0) es[4 + cf] = e;
-            }
+            face_digits<NM, TL>(fv, fd, es + 4, lane, tm);
         } else {
-            auto slot = [&](int cf, int i) -> double { // 0 where a face has no second half
+            face_digits_any<NM, TL>([&](int cf, int i) -> double { // 0 where a face has no second half
                 const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
                 const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
                 if (!own) return 0.0;
                 return INL ? fh[cf * 8 * NM + i] : d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al];
-            };
-#pragma unroll 1
-            for (int cf = 0; cf < 4; ++cf) {
-                unsigned m = 0;
-#pragma unroll 1
-                for (int i = lane; i < nslot; i += TL) m = max(m, fx::mag(slot(cf, i)));
-                const int e = fx::block_exp(__reduce_max_sync(tm, m));
-#pragma unroll 1
-                for (int i = lane; i < nslot; i += TL)
-                    fd[cf * 8 * NM + i] = fx::split(fx::from_double(slot(cf, i), e));
-                if (lane == 0) es[4 + cf] = e;
-            }
+            }, nslot, fd, es + 4, lane, tm);
         }
         __syncwarp(tm);
         // x-contraction of F, Gx, Gy, R, the xi-parts times h_y and the eta-parts
@@ -1052,24 +1078,7 @@ __global__ void __maxnreg__(RES_REGS)
             const int em = max(e1, e2);
             const long long vol = (fx::product(fx::split(sa.get()), dhy) >> min(em - e1, 63)) +
                                   (fx::product(fx::split(sb.get()), dhx) >> min(em - e2, 63));
-            long long sf = 0;
-            auto lift = [&](int f, int tn, bool coarse) {
-                fx::Acc q;
-                const int2* v = fd + (cf * 8 + f) * NM;
-                if (!coarse) {
-#pragma unroll
-                    for (int al = 0; al < NM; ++al) q.mac(tx.BmT[tn][al], v[al]);
-                } else {
-#pragma unroll
-                    for (int al = 0; al < NM; ++al) {
-                        q.mac(tx.BmHT[0][tn][al], v[al]);
-                        q.mac(tx.BmHT[1][tn][al], v[4 * NM + al]);
-                    }
-                }
-                sf += q.get();
-            };
-            if (a == 0 || a == ND1 - 1) lift(a == 0 ? 0 : 1, b, a == 0 ? c_f[0] : c_f[1]);
-            if (b == 0 || b == ND1 - 1) lift(b == 0 ? 2 : 3, a, b == 0 ? c_f[2] : c_f[3]);
+            const long long sf = face_lift<ND1, NM>(tx, fd + cf * 8 * NM, a, b, c_f);
             rfield(d, stage, cf, ND)[k * ND + j] =
                 fx::to_double(vol, fx::product_exp(em + tW, eh)) - fx::to_double(sf, ff + tx.tBmT);
         }
@@ -1087,349 +1096,271 @@ __global__ void __maxnreg__(RES_REGS)
     }
 }
 
-// 96 registers for the FP64 form; 80 for B = float (six blocks of four
-// warps per SM instead of five; measured 2 % faster despite a few spilled
-// registers, while the FP32-bulk stage update is slower at 80 or 72)
-template <int R, typename Pix, int MODE, typename B>
-__global__ void __maxnreg__(sizeof(B) == 4 ? 80 : 96)
-    k_residual_bulk(const __grid_constant__ Dev d, int buf, int stage, double c_stage, int want_dt) {
-    // the basis tables in shared memory: the contractions index them by lane
-    // (a different row or column per lane), which the constant cache would
-    // serialise (measured: -3 % per launch)
-    __shared__ Tables s_tb;
-    copy_table(s_tb, d.tabs);
-    const Tables& tb = s_tb;
+// The FP32-bulk residual: the momentum and the pointwise physics in FP32, the
+// elevation's value, the sub-grid depth, F and R beyond FP32 (block fixed point,
+// as in k_residual; the point values of F and R are FP32 products).  The same
+// teams; the FP64 pipe keeps the conversions and the final differences (it took
+// 69 instructions a cell, and bounded the kernel, while the sums of zeta, F, R
+// and the face lifts ran there).  Measured per launch: r = 2, 172,000 cells 580 ->
+// 282 us; r = 3, 65,536 cells 310 -> 188 us (80 registers: 305, 201).
+template <int R>
+struct ResBulk {
     using S = Sz<R>;
+    static constexpr int NE = ResFx<R>::NE;
+    // 8-byte words per team: y-test sums [4 NE] digits, [6 NE] floats; digits of zeta
+    // and c [ND] each with x-contractions [3 NE], point values of F and R [4 NVP],
+    // floats: nodal [4 ND], x-contractions [5 NE], point values [8 NVP]; the face
+    // values overlay the second part
+    static constexpr int A = 4 * NE + 3 * NE;
+    static constexpr int B1 = 2 * S::ND + 3 * NE + 4 * S::NVP + (4 * S::ND + 5 * NE + 8 * S::NVP + 1) / 2;
+    static constexpr int B = B1 > 32 * S::NM ? B1 : 32 * S::NM;
+    static constexpr int words = A + B + 2; // and the faces' block exponents
+};
+template <int R, typename Pix, int MODE>
+__global__ void __maxnreg__(64)
+    k_residual_bulk(const __grid_constant__ Dev d, int buf, int stage) {
+    __shared__ BulkTables tx;
+    copy_table(tx, &d.tabs->fb);
+    const Tables& tb = *d.tabs;
+    using S = Sz<R>;
+    using L = ResBulk<R>;
     using ST = Site<R, Pix, MODE>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP, NM = S::NM;
+    constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP, NM = S::NM, NE = L::NE;
+    constexpr int TL = ResFx<R>::TL;
     extern __shared__ double smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    double* su = smem + warp * res_smem<R, B>();
-    double* tz = su + 4 * ND;           // [2][ND1][NV] x-contractions of zeta: value, d/dxi
-    double* Xd = tz + 2 * ND1 * NV;     // [4][NVP]: F_x, F_y, R_x, R_y
-    double* sd = Xd + 4 * NVP;          // [4][NV][ND1]
-    double* fh = sd + 4 * NV * ND1;     // [4 fields][4 faces][2 halves][NM]
-    double* rs = fh + 32 * NM;          // [6][ND]
-    double* tc = rs + 6 * ND;           // [2][ND1][NV] x-contractions of c (value, d/dxi), FP64
-    constexpr bool F64 = sizeof(B) == sizeof(double);
-    B* suB = F64 ? (B*)su : (B*)(tc + 2 * ND1 * NV); // [4][ND] (the FP64 state itself when B = double)
-    // [3][ND1][NV]: qx, qy, c; B = float: [5][ND1][NV], then zeta (value, d/dxi)
-    B* tB = (B*)(tc + 2 * ND1 * NV) + 4 * ND;
-    B* XB = tB + (F64 ? 3 : 5) * ND1 * NV; // [8][NVP]: Gx (x, y, v), Gy (x, y, v), Lx, Ly
-    B* sB = XB + 8 * NVP;               // [8][NV][ND1]
-    const auto BvB = tab_or<B>(tb.Bv, tb.BvF);
-    const auto DvB = tab_or<B>(tb.Dv, tb.DvF);
-    const auto BmB = tab_or<B>(tb.Bm, tb.BmF);
-    const double g = d.g, eps = d.eps;
-    const B gB = (B)g, epsB = (B)eps;
+    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
+    const unsigned tm =
+        TL == 32 ? 0xffffffffu : ((1u << (TL & 31)) - 1u) << (threadIdx.x & 31 & ~(TL - 1));
+    int2* sd = (int2*)(smem + team * L::words); // [4][NV][ND1]: F (xi, eta), R (xi, eta)
+    float* sB = (float*)(sd + 4 * NE);          // [6][NV][ND1]: Gx, Gy xi; Lx, Ly; Gx, Gy eta + value
+    int2* zd = sd + L::A;                       // [ND]
+    int2* cd = zd + ND;                         // [ND] (tracer diffusion only)
+    int2* sx = cd + ND;                         // [3][ND1][NV]: zeta (Bv); c (Bv, Dv), diffusion only
+    int2* Xd = sx + 3 * NE;                     // [4][NVP]: F (x, y), R (x, y)
+    float* suB = (float*)(Xd + 4 * NVP);        // [4][ND]
+    float* tB = suB + 4 * ND;                   // [5][ND1][NV]: qx, qy, c, zeta (Bv), zeta (Dv)
+    float* XB = tB + 5 * NE;                    // [8][NVP]: Gx (x, y, v), Gy (x, y, v), Lx, Ly
+    int2* fd = zd;                              // [4 fields][2 halves][4 faces][NM]
+    int* es = (int*)(zd + L::B);                // [4] the faces' block exponents
+    const double eps = d.eps;
+    const float gB = (float)d.g, epsB = (float)eps;
     const int64_t n = d.n;
+    const bool pt = lane < NVP;
 
-    for (int64_t k = (int64_t)blockIdx.x * wpb + warp; k < n; k += (int64_t)gridDim.x * wpb) {
-        if constexpr (F64) {
-            for (int i = lane; i < 4 * ND; i += 32) su[i] = ufield(d, buf, i / ND, ND)[k * ND + (i % ND)];
-        } else {
-            // B = float: all four fields in FP32 (the elevation enters FP32
-            // arithmetic only through its gradient), from the FP32 copy of the
-            // state where the context keeps one; in FP64 the elevation, and the
-            // other fields only where something still reads them in FP64 (the
-            // tracer diffusion, the inline face integration)
-            const bool all64 = !d.uF || !d.fflux || (d.nu_c && d.nu_c[k] != 0.0);
-            for (int i = lane; i < 4 * ND; i += 32) {
-                const bool z64 = i < ND || all64;
-                const double v = z64 ? ufield(d, buf, i / ND, ND)[k * ND + (i % ND)] : 0.0;
-                su[i] = v;
-                suB[i] = d.uF ? ufieldF(d, buf, i / ND, ND)[k * ND + (i % ND)] : (B)v;
-            }
-        }
+    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
         const unsigned cm = d.cmask[(size_t)buf * n + k];
         const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
         const double ihx = d.ihxhy ? d.ihxhy[2 * k] : 1.0 / hx;
         const double ihy = d.ihxhy ? d.ihxhy[2 * k + 1] : 1.0 / hy;
-        B manB, JB, ihxB, ihyB;
-        if constexpr (F64) {
-            manB = d.manning[k];
-            JB = J;
-            ihxB = ihx;
-            ihyB = ihy;
-        } else {
-            // the four per-cell values converted once per warp (lanes 0..3),
-            // since conversions occupy the FP64 pipe
+        const double nu = d.nu_c ? d.nu_c[k] : 0.0;
+        // all four fields in FP32 (the elevation enters FP32 arithmetic only through
+        // its gradient), from the FP32 copy of the state where the context keeps one
+        const double zn = lane < ND ? ufield(d, buf, 0, ND)[k * ND + lane] : 0.0;
+#pragma unroll 1
+        for (int i = lane; i < 4 * ND; i += TL)
+            suB[i] = d.uF ? ufieldF(d, buf, i / ND, ND)[k * ND + (i % ND)]
+                          : (float)ufield(d, buf, i / ND, ND)[k * ND + (i % ND)];
+        unsigned fi[4]; // indexed by constants only (registers)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) fi[f] = d.finfo ? d.finfo[k * 4 + f] : 0;
+        const bool c_f[4] = {(fi[0] & 3) == FI_COARSE, (fi[1] & 3) == FI_COARSE,
+                             (fi[2] & 3) == FI_COARSE, (fi[3] & 3) == FI_COARSE};
+        const int nslot = (c_f[0] || c_f[1] || c_f[2] || c_f[3]) ? 8 * NM : 4 * NM;
+        float manB, JB, ihxB, ihyB;
+        {
+            // the four per-cell values converted once (lanes 0..3)
             const int q = lane & 3;
             const float f = (float)(q == 0 ? d.manning[k] : q == 1 ? J : q == 2 ? ihx : ihy);
-            manB = __shfl_sync(0xffffffffu, f, 0);
-            JB = __shfl_sync(0xffffffffu, f, 1);
-            ihxB = __shfl_sync(0xffffffffu, f, 2);
-            ihyB = __shfl_sync(0xffffffffu, f, 3);
+            manB = __shfl_sync(tm, f, 0, TL);
+            JB = __shfl_sync(tm, f, 1, TL);
+            ihxB = __shfl_sync(tm, f, 2, TL);
+            ihyB = __shfl_sync(tm, f, 3, TL);
         }
-        // the member's stage time t^n + c_l dt (boundary data)
-        const int mem = member_of(d, k);
-        const double t = (c_stage == 0.0) ? d.mb[mem].t : d.mb[mem].t + c_stage * get_dt(d, mem);
-        __syncwarp();
-        // x-contractions: zeta (value, d/dxi) in FP64, qx, qy, c in B
-        if constexpr (F64) {
-            // one job list over the five contractions, the table selected
-            // per job (no branch inside a warp): jobs 0..1 zeta value and
-            // d/dxi into tz, jobs 2..4 qx, qy, c into tB (B = double here)
-            constexpr int NE = ND1 * NV;
-            for (int i = lane; i < 5 * NE; i += 32) {
-                const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
-                const double(*Tb)[MXN] = f == 1 ? tb.Dv : tb.Bv;
-                const double* u = su + (f < 2 ? 0 : f - 1) * ND + ND1 * b;
-                double s = 0.0;
-#pragma unroll
-                for (int a = 0; a < ND1; ++a) s += Tb[al][a] * u[a];
-                if (f < 2) tz[i] = s;
-                else tB[i - 2 * NE] = s;
-            }
-        } else {
-            // the elevation's value in FP64 (the sub-grid depth); in B: qx, qy,
-            // c, and the elevation's value and d/dxi for its gradient
-            for (int i = lane; i < ND1 * NV; i += 32) {
-                const int b = i / NV, al = i % NV;
-                double s = 0.0;
-#pragma unroll
-                for (int a = 0; a < ND1; ++a) s += tb.Bv[al][a] * su[ND1 * b + a];
-                tz[i] = s;
-            }
-            for (int i = lane; i < 5 * ND1 * NV; i += 32) {
-                const int f = i / (ND1 * NV), r_ = i % (ND1 * NV), b = r_ / NV, al = r_ % NV;
-                const B* u = suB + (f < 3 ? 1 + f : 0) * ND + ND1 * b;
-                const B(*Tb)[MXN] = f == 4 ? DvB : BvB;
-                B s = B(0);
-#pragma unroll
-                for (int a = 0; a < ND1; ++a) s += Tb[al][a] * u[a];
-                tB[i] = s;
-            }
+        const int ez = team_exp(zn, tm);
+        const double z0 = __shfl_sync(tm, zn, 0, TL);
+        if (lane < ND) zd[lane] = fx::split(fx::from_double(zn, ez));
+        int ec = 0;
+        if (nu != 0.0) { // tracer numerical diffusion (Eq. numdiff): grad c from the FP64 state
+            const double cn = lane < ND ? ufield(d, buf, 3, ND)[k * ND + lane] : 0.0;
+            ec = team_exp(cn, tm);
+            if (lane < ND) cd[lane] = fx::split(fx::from_double(cn, ec));
         }
-        // tracer numerical diffusion (Eq. numdiff): grad c in FP64
-        const double nu = d.nu_c ? d.nu_c[k] : 0.0;
-        if (nu != 0.0) {
-            for (int i = lane; i < 2 * ND1 * NV; i += 32) {
-                const int f = i / (ND1 * NV), r_ = i % (ND1 * NV), b = r_ / NV, al = r_ % NV;
-                double s = 0.0;
+        __syncwarp(tm);
+        // x-contractions: the elevation's value (the sub-grid depth) in fixed point; in
+        // FP32 qx, qy, c, and the elevation's value and d/dxi for its gradient
+#pragma unroll 1
+        for (int i = lane; i < (nu != 0.0 ? 3 : 1) * NE; i += TL) {
+            const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
+            const int2* T = f == 2 ? tb.fx.Dv[al] : tx.Bv[al];
+            const int2* u = (f ? cd : zd) + ND1 * b;
+            fx::Acc s;
 #pragma unroll
-                for (int a = 0; a < ND1; ++a)
-                    s += (f ? tb.Dv[al][a] : tb.Bv[al][a]) * su[3 * ND + ND1 * b + a];
-                tc[i] = s;
-            }
+            for (int a = 0; a < ND1; ++a) s.mac(T[a], u[a]);
+            sx[i] = fx::split(s.get());
         }
-        __syncwarp();
-        // y-contraction and pointwise physics, one volume point per lane
-        for (int p = lane; p < NVP; p += 32) {
-            const int al = p % NV, be = p / NV;
-            double z = 0.0;
-            B qx = B(0), qy = B(0), c = B(0), zx, zy;
-            if constexpr (F64) {
-                double zxd = 0.0, zyd = 0.0;
+#pragma unroll 1
+        for (int i = lane; i < 5 * NE; i += TL) {
+            const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
+            const float* u = suB + (f < 3 ? 1 + f : 0) * ND + ND1 * b;
+            const float(*Tb)[MXN] = f == 4 ? tx.DvF : tx.BvF;
+            float s = 0.0f;
 #pragma unroll
-                for (int b = 0; b < ND1; ++b) {
-                    z += tb.Bv[be][b] * tz[b * NV + al];
-                    zxd += tb.Bv[be][b] * tz[(ND1 + b) * NV + al];
-                    zyd += tb.Dv[be][b] * tz[b * NV + al];
-                }
-                if (cm & 1u) { z = su[0]; zxd = 0.0; zyd = 0.0; }
-                zx = zxd * ihx;
-                zy = zyd * ihy;
-            } else {
-                // the gradient of the elevation in FP32 (it enters only the
-                // FP32 pressure term g h grad zeta)
-                B zxd = B(0), zyd = B(0);
-#pragma unroll
-                for (int b = 0; b < ND1; ++b) {
-                    z += tb.Bv[be][b] * tz[b * NV + al];
-                    zxd += BvB[be][b] * tB[(4 * ND1 + b) * NV + al];
-                    zyd += DvB[be][b] * tB[(3 * ND1 + b) * NV + al];
-                }
-                if (cm & 1u) { z = su[0]; zxd = B(0); zyd = B(0); }
-                zx = zxd * ihxB;
-                zy = zyd * ihyB;
-            }
+            for (int a = 0; a < ND1; ++a) s += Tb[al][a] * u[a];
+            tB[i] = s;
+        }
+        __syncwarp(tm);
+        // y-contraction and pointwise physics, one volume point per lane (idle lanes
+        // take point 0 and store nothing)
+        int eF, eR; // block exponents of the point values of F, R
+        {
+            const int p = pt ? lane : 0, al = p % NV, be = p / NV;
+            float qx = 0.0f, qy = 0.0f, c = 0.0f, zxd = 0.0f, zyd = 0.0f;
+            fx::Acc az;
 #pragma unroll
             for (int b = 0; b < ND1; ++b) {
-                const B Bb = BvB[be][b];
+                az.mac(tx.Bv[be][b], sx[b * NV + al]);
+                const float Bb = tx.BvF[be][b];
+                zxd += Bb * tB[(4 * ND1 + b) * NV + al];
+                zyd += tx.DvF[be][b] * tB[(3 * ND1 + b) * NV + al];
                 qx += Bb * tB[(0 * ND1 + b) * NV + al];
                 qy += Bb * tB[(1 * ND1 + b) * NV + al];
                 c += Bb * tB[(2 * ND1 + b) * NV + al];
             }
+            double z = fx::to_double(az.get(), ez + 2 * tx.tBv);
+            if (cm & 1u) { z = z0; zxd = 0.0f; zyd = 0.0f; }
+            const float zx = zxd * ihxB, zy = zyd * ihyB;
             if (cm & 2u) qx = suB[ND];
             if (cm & 4u) qy = suB[2 * ND];
             if (cm & 8u) c = suB[3 * ND];
-            double h, A;
-            ST::VA(d, tb, k, SET_VOL, al, be, z, h, A);
-            const B hB = (B)h;
-            B fv, gam;
-            vel_gamma<B>(manB, hB, qx, qy, gB, epsB, fv, gam);
-            const B ux = fv * qx, uy = fv * qy;
-            const double w = J * tb.wv[al] * tb.wv[be];
-            B wB, wx, wy;
-            if constexpr (F64) {
-                wB = w;
-                wx = w * ihx;
-                wy = w * ihy;
-            } else { // the weights of the FP32 terms in FP32 (no conversions per point)
-                wB = JB * tb.wvF[al] * tb.wvF[be];
-                wx = wB * ihxB;
-                wy = wB * ihyB;
-            }
-            Xd[0 * NVP + p] = (double)(wx * qx);
-            Xd[1 * NVP + p] = (double)(wy * qy);
-            Xd[2 * NVP + p] = (double)(wx * c * qx);
-            Xd[3 * NVP + p] = (double)(wy * c * qy);
+            double h = 0.0, A;
+            if (pt) ST::VA(d, tb, k, SET_VOL, al, be, z, h, A);
+            const float hB = (float)h;
+            float fv, gam;
+            vel_gamma<float>(manB, hB, qx, qy, gB, epsB, fv, gam);
+            const float ux = fv * qx, uy = fv * qy;
+            // the weights of the FP32 terms in FP32 (no conversions per point)
+            const float wB = JB * tx.wvF[al] * tx.wvF[be], wx = wB * ihxB, wy = wB * ihyB;
+            const float Fx = wx * qx, Fy = wy * qy, Rx = wx * c * qx, Ry = wy * c * qy;
+            auto mag = [](float v) { return __float_as_uint(v) & 0x7fffffffu; };
+            eF = fx::block_exp_f(__reduce_max_sync(tm, pt ? max(mag(Fx), mag(Fy)) : 0u));
+            long long RX, RY;
             if (nu != 0.0 && !(cm & 8u)) {
                 // -nu h grad c . grad psi: the reference derivatives of c at the point
-                double cxd = 0.0, cyd = 0.0;
+                fx::Acc acx, acy;
 #pragma unroll
                 for (int b = 0; b < ND1; ++b) {
-                    cxd += tb.Bv[be][b] * tc[(ND1 + b) * NV + al];
-                    cyd += tb.Dv[be][b] * tc[b * NV + al];
+                    acx.mac(tx.Bv[be][b], sx[(2 * ND1 + b) * NV + al]);
+                    acy.mac(tb.fx.Dv[be][b], sx[(ND1 + b) * NV + al]);
                 }
-                Xd[2 * NVP + p] -= w * nu * h * cxd * ihx * ihx;
-                Xd[3 * NVP + p] -= w * nu * h * cyd * ihy * ihy;
+                const int e = ec + tx.tBv + tb.fx.tDv;
+                const double wn = J * tb.wv[al] * tb.wv[be] * nu * h;
+                const double rx = (double)Rx - wn * fx::to_double(acx.get(), e) * ihx * ihx;
+                const double ry = (double)Ry - wn * fx::to_double(acy.get(), e) * ihy * ihy;
+                eR = fx::block_exp(__reduce_max_sync(tm, pt ? max(fx::mag(rx), fx::mag(ry)) : 0u));
+                RX = fx::from_double(rx, eR);
+                RY = fx::from_double(ry, eR);
+            } else {
+                eR = fx::block_exp_f(__reduce_max_sync(tm, pt ? max(mag(Rx), mag(Ry)) : 0u));
+                RX = fx::from_float(Rx, eR);
+                RY = fx::from_float(Ry, eR);
             }
-            XB[0 * NVP + p] = wx * qx * ux;
-            XB[1 * NVP + p] = wy * qx * uy;
-            XB[2 * NVP + p] = -wB * gB * hB * zx;
-            XB[3 * NVP + p] = wx * qy * ux;
-            XB[4 * NVP + p] = wy * qy * uy;
-            XB[5 * NVP + p] = -wB * gB * hB * zy;
-            XB[6 * NVP + p] = -wB * gam * qx;
-            XB[7 * NVP + p] = -wB * gam * qy;
+            if (pt) {
+                Xd[0 * NVP + p] = fx::split(fx::from_float(Fx, eF));
+                Xd[1 * NVP + p] = fx::split(fx::from_float(Fy, eF));
+                Xd[2 * NVP + p] = fx::split(RX);
+                Xd[3 * NVP + p] = fx::split(RY);
+                XB[0 * NVP + p] = wx * qx * ux;
+                XB[1 * NVP + p] = wy * qx * uy;
+                XB[2 * NVP + p] = -wB * gB * hB * zx;
+                XB[3 * NVP + p] = wx * qy * ux;
+                XB[4 * NVP + p] = wy * qy * uy;
+                XB[5 * NVP + p] = -wB * gB * hB * zy;
+                XB[6 * NVP + p] = -wB * gam * qx;
+                XB[7 * NVP + p] = -wB * gam * qy;
+            }
         }
-        __syncwarp();
-        // test integration, y-contraction.  FP64: F (x, y), R (x, y); B: Gx, Gy
-        // (x; y + v), Lx, Ly (v)
-        if constexpr (F64) {
-            // every single 5-term sum is one job, so the lanes stay busy: jobs
-            // 0,1 F/R x-part (Bv), 2,3 F/R y-part (Dv), 4,5 Gx/Gy x-part (Bv),
-            // 6,7 Lx/Ly (Bv), NV ND1 entries each; then the Gx/Gy y + v parts
-            constexpr int NE = NV * ND1;
-            for (int i = lane; i < 8 * NE; i += 32) {
-                const int job = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-                const int c2 = job & 1, kind = job >> 1;
-                const double(*Tb)[MXN] = kind == 1 ? tb.Dv : tb.Bv;
-                const double* X = kind == 0   ? Xd + (2 * c2) * NVP
-                                  : kind == 1 ? Xd + (2 * c2 + 1) * NVP
-                                  : kind == 2 ? (const double*)XB + 3 * c2 * NVP
-                                              : (const double*)XB + (6 + c2) * NVP;
-                double* out = kind == 0   ? sd + ((c2 * 2 + 0) * NV + al) * ND1 + b
-                              : kind == 1 ? sd + ((c2 * 2 + 1) * NV + al) * ND1 + b
-                              : kind == 2 ? (double*)sB + ((c2 * 2 + 0) * NV + al) * ND1 + b
-                                          : (double*)sB + (((2 + c2) * 2 + 1) * NV + al) * ND1 + b;
-                double acc = 0.0;
+        __syncwarp(tm);
+        // the face fluxes of k_faces_bulk, loaded here so that the y-contraction hides
+        // the latency
+        const bool conforming = nslot == 4 * NM;
+        double fv[(4 * NM + TL - 1) / TL][4];
+        if (conforming) face_load<NM, TL>(d.fflux + k * (32 * NM), fv, lane);
+        // test integration, y-contraction: F (x, y), R (x, y); in FP32 Gx, Gy (x), Lx, Ly
+        // (value), then Gx, Gy (y + value)
+#pragma unroll 1
+        for (int i = lane; i < 4 * NE; i += TL) {
+            const int job = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
+            const int2* T = (job & 1) ? tx.DvT[b] : tx.BvT[b];
+            const int2* X = Xd + job * NVP + al;
+            const float* Xg = XB + ((0x7630u >> (4 * job)) & 15u) * NVP + al;
+            fx::Acc s;
+            float sx_ = 0.0f;
 #pragma unroll
-                for (int be = 0; be < NV; ++be) acc += Tb[be][b] * X[al + NV * be];
-                *out = acc;
+            for (int be = 0; be < NV; ++be) {
+                s.mac(T[be], X[NV * be]);
+                sx_ += tx.BvF[be][b] * Xg[NV * be];
             }
-            for (int i = lane; i < 2 * NE; i += 32) {
-                const int cg = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-                const B* Xg = XB + 3 * cg * NVP;
-                B so = B(0);
+            sd[i] = fx::split(s.get());
+            sB[i] = sx_;
+        }
+#pragma unroll 1
+        for (int i = lane; i < 2 * NE; i += TL) {
+            const int cg = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
+            const float* Xg = XB + 3 * cg * NVP;
+            float so = 0.0f;
 #pragma unroll
-                for (int be = 0; be < NV; ++be) {
-                    const int p = al + NV * be;
-                    so += DvB[be][b] * Xg[NVP + p] + BvB[be][b] * Xg[2 * NVP + p];
-                }
-                sB[((cg * 2 + 1) * NV + al) * ND1 + b] = so;
+            for (int be = 0; be < NV; ++be) {
+                const int p = al + NV * be;
+                so += tx.DvF[be][b] * Xg[NVP + p] + tx.BvF[be][b] * Xg[2 * NVP + p];
             }
+            sB[4 * NE + i] = so;
+        }
+        __syncwarp(tm);
+        if (conforming) {
+            face_digits<NM, TL>(fv, fd, es, lane, tm);
         } else {
-            for (int i = lane; i < 2 * NV * ND1; i += 32) {
-                const int cf = i / (NV * ND1), r_ = i % (NV * ND1), al = r_ / ND1, b = r_ % ND1;
-                double sx = 0.0, so = 0.0;
+            face_digits_any<NM, TL>([&](int cf, int i) -> double { // 0 where a face has no second half
+                const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
+                const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
+                return own ? d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al] : 0.0;
+            }, nslot, fd, es, lane, tm);
+        }
+        __syncwarp(tm);
+        // x-contraction: F and R, then Gx and Gy, minus the face fluxes
+#pragma unroll 1
+        for (int i = lane; i < 4 * ND; i += TL) {
+            const int q = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
+            const int cf = (0x2130 >> (4 * q)) & 15;
+            double v;
+            if (q < 2) {
+                const int2* s1 = sd + 2 * q * NE + b;
+                fx::Acc s;
 #pragma unroll
-                for (int be = 0; be < NV; ++be) {
-                    const int p = al + NV * be;
-                    sx += tb.Bv[be][b] * Xd[(2 * cf) * NVP + p];
-                    so += tb.Dv[be][b] * Xd[(2 * cf + 1) * NVP + p];
+                for (int al = 0; al < NV; ++al) {
+                    s.mac(tx.DvT[a][al], s1[al * ND1]);
+                    s.mac(tx.BvT[a][al], s1[NE + al * ND1]);
                 }
-                sd[((cf * 2 + 0) * NV + al) * ND1 + b] = sx;
-                sd[((cf * 2 + 1) * NV + al) * ND1 + b] = so;
+                v = fx::to_double(s.get(), (q ? eR : eF) + tx.tBvT + tx.tDvT);
+            } else {
+                const float* s1 = sB + (q - 2) * NE + b;
+                float s = 0.0f;
+#pragma unroll
+                for (int al = 0; al < NV; ++al)
+                    s += tx.DvF[al][a] * s1[al * ND1] + tx.BvF[al][a] * s1[4 * NE + al * ND1];
+                v = f64_any(s);
             }
-            // Gx, Gy: grad-x part, and grad-y + value parts
-            for (int i = lane; i < 2 * NV * ND1; i += 32) {
-                const int cg = i / (NV * ND1), r_ = i % (NV * ND1), al = r_ / ND1, b = r_ % ND1;
-                const B* Xg = XB + 3 * cg * NVP;
-                B sx = B(0), so = B(0);
-#pragma unroll
-                for (int be = 0; be < NV; ++be) {
-                    const int p = al + NV * be;
-                    sx += BvB[be][b] * Xg[p];
-                    so += DvB[be][b] * Xg[NVP + p] + BvB[be][b] * Xg[2 * NVP + p];
-                }
-                sB[((cg * 2 + 0) * NV + al) * ND1 + b] = sx;
-                sB[((cg * 2 + 1) * NV + al) * ND1 + b] = so;
-            }
-            // Lx, Ly: value parts only
-            for (int i = lane; i < 2 * NV * ND1; i += 32) {
-                const int cl = i / (NV * ND1), r_ = i % (NV * ND1), al = r_ / ND1, b = r_ % ND1;
-                const B* Xl = XB + (6 + cl) * NVP;
-                B so = B(0);
-#pragma unroll
-                for (int be = 0; be < NV; ++be) so += BvB[be][b] * Xl[al + NV * be];
-                sB[(((2 + cl) * 2 + 1) * NV + al) * ND1 + b] = so;
-            }
+            const long long sf = face_lift<ND1, NM>(tx, fd + cf * 8 * NM, a, b, c_f);
+            rfield(d, stage, cf, ND)[k * ND + j] = v - fx::to_double(sf, es[cf] + tx.tBmT);
         }
-        __syncwarp();
-        // x-contraction into rs = [F, Gx, Gy, R, Lx, Ly]: F and R in FP64
-        for (int i = lane; i < 2 * ND; i += 32) {
-            const int cf = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            double s = 0.0;
-#pragma unroll
-            for (int al = 0; al < NV; ++al)
-                s += tb.Dv[al][a] * sd[((cf * 2 + 0) * NV + al) * ND1 + b] +
-                     tb.Bv[al][a] * sd[((cf * 2 + 1) * NV + al) * ND1 + b];
-            rs[(cf == 0 ? 0 : 3) * ND + j] = s;
-        }
-        for (int i = lane; i < 2 * ND; i += 32) { // Gx, Gy
-            const int cg = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            B s = B(0);
-#pragma unroll
-            for (int al = 0; al < NV; ++al)
-                s += DvB[al][a] * sB[((cg * 2 + 0) * NV + al) * ND1 + b] +
-                     BvB[al][a] * sB[((cg * 2 + 1) * NV + al) * ND1 + b];
-            rs[(1 + cg) * ND + j] = (double)s;
-        }
-        for (int i = lane; i < 2 * ND; i += 32) { // Lx, Ly
+#pragma unroll 1
+        for (int i = lane; i < 2 * ND; i += TL) { // Lx, Ly
             const int cl = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            B s = B(0);
+            float s = 0.0f;
 #pragma unroll
-            for (int al = 0; al < NV; ++al) s += BvB[al][a] * sB[(((2 + cl) * 2 + 1) * NV + al) * ND1 + b];
-            rs[(4 + cl) * ND + j] = (double)s;
+            for (int al = 0; al < NV; ++al) s += tx.BvF[al][a] * sB[(2 + cl) * NE + al * ND1 + b];
+            rfield(d, stage, 4 + cl, ND)[k * ND + j] = f64_any(s);
         }
-        // the face fluxes of this cell, computed once per face point by k_faces
-        unsigned fi[4]; // indexed by constants only (registers)
-#pragma unroll
-        for (int f = 0; f < 4; ++f) fi[f] = d.finfo ? d.finfo[k * 4 + f] : 0;
-        const double* F = d.fflux + k * (32 * NM);
-        for (int i = lane; i < 32 * NM; i += 32) fh[i] = F[i];
-        __syncwarp();
-        // lift the face fluxes onto the nodes of each face: one item per field,
-        // face and node along it, the x faces (0, 1: node columns a = 0 and
-        // ND1 - 1) in one pass and the y faces (2, 3: rows b = 0 and ND1 - 1) in
-        // the next, so that the items of a pass touch distinct nodes and every
-        // lane does the same work
-#pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int i = lane; i < 4 * 2 * ND1; i += 32) {
-                const int cf = i / (2 * ND1), r_ = i % (2 * ND1), f = 2 * pass + r_ / ND1;
-                const int tn = r_ % ND1; // node index along the face
-                const unsigned inf = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
-                const double* fp = fh + (cf * 4 + f) * 2 * NM;
-                double s = 0.0;
-                if ((inf & 3) == FI_COARSE) {
-#pragma unroll
-                    for (int al = 0; al < NM; ++al)
-                        s += tb.BmH[0][al][tn] * fp[al] + tb.BmH[1][al][tn] * fp[NM + al];
-                } else {
-#pragma unroll
-                    for (int al = 0; al < NM; ++al) s += tb.Bm[al][tn] * fp[al];
-                }
-                rs[cf * ND + face_node<ND1>(f, tn)] -= s;
-            }
-            __syncwarp();
-        }
-        for (int i = lane; i < 6 * ND; i += 32)
-            rfield(d, stage, i / ND, ND)[k * ND + (i % ND)] = rs[i];
-        __syncwarp();
+        __syncwarp(tm);
     }
 }
 
@@ -1770,119 +1701,6 @@ __device__ __forceinline__ int lrow_idx(int i, int t) {
     else return i * ND + t;
 }
 
-// The steps of a Cholesky factorisation with row i of the matrix in the
-// lane's registers a (lower part used).  Step J takes the pivot from lane J,
-// scales column J and updates the columns l > J with L_lJ from lane l.  The
-// steps are expanded from index sequences, so that every index into a is a
-// constant and the row stays in registers.  After a non-positive pivot the
-// steps go on (no branch) and ok is false.
-template <int ND, int TL, int J, int L>
-__device__ __forceinline__ void chol_row_update(float (&a)[ND], int i, unsigned tm) {
-    constexpr int l = J + 1 + L;
-    const float llj = __shfl_sync(tm, a[J], l, TL); // L_lJ
-    if (l <= i) a[l] -= a[J] * llj;
-}
-template <int ND, int TL, int J, int... L>
-__device__ __forceinline__ void chol_row_step(float (&a)[ND], int i, float& rinv, bool& ok,
-                                              unsigned tm, std::integer_sequence<int, L...>) {
-    const float djj = __shfl_sync(tm, a[J], J, TL); // the same on every lane of the team
-    ok = ok && djj > 0.0f;
-    const float ljj = sqrtf(djj);
-    const float r = 1.0f / ljj;
-    if (i == J) {
-        a[J] = ljj;
-        rinv = r;
-    } else if (i > J) {
-        a[J] *= r;
-    }
-    (chol_row_update<ND, TL, J, L>(a, i, tm), ...);
-}
-template <int ND, int TL, int... J>
-__device__ __forceinline__ void chol_rows(float (&a)[ND], int i, float& rinv, bool& ok, unsigned tm,
-                                          std::integer_sequence<int, J...>) {
-    (chol_row_step<ND, TL, J>(a, i, rinv, ok, tm, std::make_integer_sequence<int, ND - J - 1>{}),
-     ...);
-}
-
-// FP32 copy of M_(a,b),(c,d) = sum c_{al,be} Bm[al][a] Bm[al][c] Bm[be][b] Bm[be][d],
-// assembled and Cholesky-factored with one row per lane (ND <= TL).  The
-// weights cw are converted once (conversions run on the FP64 pipe: converting
-// inside the sums would cost one per term); lane i forms the lower part of
-// row i of M from the FP32 basis table, the factor's column updates take the
-// pivot column from the other lanes by shuffles, and L is stored by rows in
-// Mf (lrow_idx).  The lane's reciprocal pivot 1/L_ii comes back in rinv.
-// Returns false on a non-positive pivot.
-template <int ND1, int NM, int TL>
-__device__ bool mass_factor_rows_f(const FxStage& tb, const double* cw, float* Y, float* Mf,
-                                   float& rinv, int lane, unsigned tm) {
-    constexpr int ND = ND1 * ND1;
-    static_assert(ND <= TL, "one row per lane");
-    static_assert(NM * NM <= ND * ND, "the weights are staged in Mf");
-    float* cwf = Mf; // Mf is written only once the factor is done
-    for (int p = lane; p < NM * NM; p += TL) cwf[p] = f32_of(cw[p]);
-    __syncwarp(tm);
-    for (int i = lane; i < ND1 * ND1 * NM; i += TL) {
-        const int a = i / (ND1 * NM), r_ = i % (ND1 * NM), c = r_ / NM, be = r_ % NM;
-        float s = 0.0f;
-#pragma unroll
-        for (int al = 0; al < NM; ++al) s += cwf[al + NM * be] * tb.BmF[al][a] * tb.BmF[al][c];
-        Y[i] = s;
-    }
-    __syncwarp(tm);
-    // lanes past the last row repeat it and store nothing
-    const int i = lane < ND ? lane : ND - 1;
-    const int ar = i % ND1, br = i / ND1;
-    float bb[NM];
-#pragma unroll
-    for (int be = 0; be < NM; ++be) bb[be] = tb.BmF[be][br];
-    float a[ND];
-#pragma unroll
-    for (int t = 0; t < ND; ++t) {
-        float s = 0.0f;
-#pragma unroll
-        for (int be = 0; be < NM; ++be)
-            s += Y[(ar * ND1 + t % ND1) * NM + be] * bb[be] * tb.BmF[be][t / ND1];
-        a[t] = s;
-    }
-    bool ok = true;
-    rinv = 0.0f;
-    chol_rows<ND, TL>(a, i, rinv, ok, tm, std::make_integer_sequence<int, ND>{});
-    if (ok && lane < ND) {
-#pragma unroll
-        for (int t = 0; t < ND; ++t)
-            if (t <= i) Mf[lrow_idx<ND>(i, t)] = a[t];
-    }
-    __syncwarp(tm);
-    return ok;
-}
-
-// (L L^T)^-1 b in FP32 with the factor of mass_factor_rows_f: lane i brings
-// b_i and gets x_i; the solved component of each step is passed by a
-// shuffle (forward, then backward substitution, column by column).
-template <int ND, int TL>
-__device__ __forceinline__ float chol_subst_rows_f(const float* Mf, float rinv, float bv, int lane,
-                                                   unsigned tm) {
-    const int i = lane < ND ? lane : ND - 1;
-    float lr[ND];
-#pragma unroll
-    for (int j = 0; j < ND; ++j) lr[j] = j < i ? Mf[lrow_idx<ND>(i, j)] : 0.0f; // row i of L
-#pragma unroll
-    for (int j = 0; j < ND; ++j) { // L y = b
-        const float yj = __shfl_sync(tm, bv * rinv, j, TL);
-        if (i == j) bv = yj;
-        else if (i > j) bv -= lr[j] * yj;
-    }
-#pragma unroll
-    for (int j = 0; j < ND; ++j) lr[j] = j > i ? Mf[lrow_idx<ND>(j, i)] : 0.0f; // column i of L
-#pragma unroll
-    for (int j = ND - 1; j >= 0; --j) { // L^T x = y
-        const float xj = __shfl_sync(tm, bv * rinv, j, TL);
-        if (i == j) bv = xj;
-        else if (i < j) bv -= lr[j] * xj;
-    }
-    return bv;
-}
-
 // FP32 inverse of H' = S B^T diag(cw') B S, one row per lane in a[] (ND <= TL):
 // cw' = cw 2^-(ecw - 1022) <= 1 (given as FP32) and S scales the columns of B to
 // norm 1, so the diagonal and every pivot of the elimination is at most 1.
@@ -2064,27 +1882,34 @@ __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& f
 // C = c0 + delta, where c0 = sum_i b_i / sum_i s_i is the cell's mean
 // concentration (s = H 1, the row sums of H, i.e. H_i(zeta^(l)) of the
 // continuity equation, in FP64), delta = H^-1 (b - c0 s) is solved once in
-// FP32 (FP32 factor of mass_factor_rows_f), and a constant correction makes
+// FP32, and a constant correction makes
 // sum_i (H C)_i = sum_i s_i C_i equal sum_i b_i in FP64, so the tracer mass
 // is kept to FP64 round-off and a constant tracer (b = c s) stays constant up
 // to the rounding of b - c0 s.  A failed FP32 factor falls back to the FP64
-// Cholesky.  b: right-hand side in, C out (FP64).  Scratch: Mf, Yf (float),
-// digit pairs td [2 NMP], M, Y, inv (fallback).  known: the Newton solve ended
-// on its certificate (H is affine between the last two iterates, so
-// H(zeta^(l)) = T up to the rounding of the last update) and the continuity
-// target T stands for s = H 1 = H(zeta^(l)); otherwise s is integrated from cw.
+// Cholesky.  b: right-hand side in, C out (FP64).  Scratch: Mf [ND ND], Yf [ND1
+// ND1 NM] (float), digit pairs td [2 NMP], M, Y, inv (fallback).  known: the
+// Newton solve ended on its certificate (H is affine between the last two
+// iterates, so H(zeta^(l)) = T up to the rounding of the last update) and the
+// continuity target T stands for s = H 1 = H(zeta^(l)); otherwise s is
+// integrated from cw.
+//
+// The factor is a Cholesky with one row per lane in registers (lanes past the
+// last row repeat it).  Step J takes the pivot from lane J, and column J goes to
+// the other lanes through shared memory, shifted by J + 1; the row's columns
+// move down by one per step, so that the pivot column is always a[0] and one
+// loop body serves every step; entries above the diagonal or past the last
+// column are computed and never used.  The forward substitution goes along.
+// Unrolled with one shuffle per entry, this solve was 20 KB of code, which has
+// to share the 32 KB instruction cache with the rest of the stage update (a stage of
+// 65,536 cells, r = 3: 497 -> 468 us).
 template <int ND1, int NM, int TL>
 __device__ __noinline__ void solve_tracer_bulk(const Tables& tb, const FxStage& fs, const double* cw, double* b,
                                   float* Mf, float* Yf, int2* td, double* M, double* Y, double* inv,
                                   bool known, double T, int lane, unsigned tm) {
-    constexpr int ND = ND1 * ND1, NMP = NM * NM;
-    static_assert(ND <= TL, "one unknown per lane");
-    float rinv;
-    if (!mass_factor_rows_f<ND1, NM, TL>(fs, cw, Yf, Mf, rinv, lane, tm)) {
-        assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
-        chol_solve<ND1 * ND1, TL>(M, b, inv, lane, tm);
-        return;
-    }
+    constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4;
+    static_assert(ND <= TL, "one row per lane");
+    static_assert(NMP <= ND * ND, "the weights are staged in Mf");
+    static_assert(2 * NDP + 2 <= ND1 * ND1 * NM, "the columns overlay Yf");
     if (!known) { // s_i = (H 1)_i
         unsigned m = 0;
         for (int p = lane; p < NMP; p += TL) m = max(m, fx::mag(cw[p]));
@@ -2099,8 +1924,70 @@ __device__ __noinline__ void solve_tracer_bulk(const Tables& tb, const FxStage& 
     double sb = bi, ss = si;
     team_sum2<TL>(sb, ss, tm);
     const double c0 = ss > 0.0 ? sb / ss : 0.0;
-    const float v = chol_subst_rows_f<ND, TL>(Mf, rinv, f32_of(bi - c0 * si), lane, tm);
-    const double xi = lane < ND ? c0 + f64_any(v) : 0.0;
+    // the matrix, contracted over the points of a row, then over the rows
+    for (int p = lane; p < NMP; p += TL) Mf[p] = f32_of(cw[p]);
+    __syncwarp(tm);
+#pragma unroll 1
+    for (int i = lane; i < ND1 * ND1 * NM; i += TL) {
+        const int a = i / (ND1 * NM), r_ = i % (ND1 * NM), c = r_ / NM, be = r_ % NM;
+        float s = 0.0f;
+#pragma unroll
+        for (int al = 0; al < NM; ++al) s += Mf[al + NM * be] * fs.BmF[al][a] * fs.BmF[al][c];
+        Yf[i] = s;
+    }
+    __syncwarp(tm);
+    const int i = lane < ND ? lane : ND - 1, ar = i % ND1, br = i / ND1;
+    float a[ND];
+#pragma unroll
+    for (int t = 0; t < ND; ++t) a[t] = 0.0f;
+#pragma unroll
+    for (int be = 0; be < NM; ++be) {
+        const float bb = fs.BmF[be][br];
+        float y[ND1];
+#pragma unroll
+        for (int c = 0; c < ND1; ++c) y[c] = Yf[(ar * ND1 + c) * NM + be] * bb;
+#pragma unroll
+        for (int t = 0; t < ND; ++t) a[t] += y[t % ND1] * fs.BmF[be][t / ND1];
+    }
+    float bv = f32_of(bi - c0 * si), rinv = 0.0f;
+    float* cb = (float*)(((size_t)Yf + 15) & ~(size_t)15); // two columns, in turn
+    bool ok = true;
+    __syncwarp(tm);
+#pragma unroll 1
+    for (int J = 0; J < ND; ++J) {
+        float* col = cb + (J & 1) * NDP;
+        const float djj = __shfl_sync(tm, a[0], J, TL); // the same on every lane of the team
+        ok = ok && djj > 0.0f;
+        const float r = 1.0f / sqrtf(djj);
+        const float yj = __shfl_sync(tm, bv * r, J, TL);
+        float lj = 0.0f;
+        if (i == J) {
+            rinv = r;
+            bv = yj;
+        } else if (i > J) {
+            lj = a[0] * r;
+            bv -= lj * yj;
+            col[i - J - 1] = lj;
+            Mf[lrow_idx<ND>(i, J)] = lj;
+        }
+        __syncwarp(tm);
+        float cl[NDP];
+        read_row<NDP>(col, cl);
+#pragma unroll
+        for (int l = 0; l < ND - 1; ++l) a[l] = a[l + 1] - lj * cl[l];
+    }
+    if (!ok) {
+        assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
+        chol_solve<ND, TL>(M, b, inv, lane, tm);
+        return;
+    }
+#pragma unroll 1
+    for (int j = ND - 1; j >= 0; --j) { // L^T x = y
+        const float xj = __shfl_sync(tm, bv * rinv, j, TL);
+        if (i == j) bv = xj;
+        else if (i < j) bv -= Mf[lrow_idx<ND>(j, i)] * xj;
+    }
+    const double xi = lane < ND ? c0 + f64_any(bv) : 0.0;
     const double m = team_sum<TL>(si * xi, tm);
     const double alpha = ss > 0.0 ? (sb - m) / ss : 0.0;
     __syncwarp(tm);
@@ -2110,6 +1997,13 @@ __device__ __noinline__ void solve_tracer_bulk(const Tables& tb, const FxStage& 
 
 __device__ __forceinline__ double bulk_of(double v, double) { return v; }
 __device__ __forceinline__ float bulk_of(double v, float) { return f32_of(v); }
+// a nodal value, FP32 ones from the FP32 copy of the state where there is one
+template <typename T, int ND>
+__device__ __forceinline__ T nodal(const Dev& d, int buf, int f, size_t idx) {
+    if constexpr (sizeof(T) == 4)
+        if (d.uF) return ufieldF(d, buf, f, ND)[idx];
+    return bulk_of(ufield(d, buf, f, ND)[idx], T());
+}
 __device__ __forceinline__ double exact_of(double v) { return v; }
 __device__ __forceinline__ double exact_of(float v) { return f64_any(v); }
 
@@ -2635,8 +2529,7 @@ __global__ void __maxnreg__(STAGE_REGS)
             using T = decltype(manT);
             const unsigned cmp = d.cmask[(size_t)sa.prev_buf * n + k];
             const double z0 = ufield(d, sa.prev_buf, 0, ND)[idx];
-            const T q0 = bulk_of(ufield(d, sa.prev_buf, 1, ND)[idx], T()),
-                    q1 = bulk_of(ufield(d, sa.prev_buf, 2, ND)[idx], T());
+            const T q0 = nodal<T, ND>(d, sa.prev_buf, 1, idx), q1 = nodal<T, ND>(d, sa.prev_buf, 2, idx);
             double zv[1] = {z0}, Vp, Ap;
             T q[2] = {q0, q1}, gam = T(0);
             if (!(cmp & 1u)) zv[0] = square_one<ND1>(fs.Bg, fs.tBg, zv[0], w, lane, tm);
@@ -2652,7 +2545,7 @@ __global__ void __maxnreg__(STAGE_REGS)
         // v^n's discharges at the momentum point, interpolated
         auto q_points = [&](auto& v) {
             using T = std::remove_reference_t<decltype(v[0])>;
-            const T q0 = bulk_of(ufield(d, 0, 1, ND)[idx], T()), q1 = bulk_of(ufield(d, 0, 2, ND)[idx], T());
+            const T q0 = nodal<T, ND>(d, 0, 1, idx), q1 = nodal<T, ND>(d, 0, 2, idx);
             v[0] = q0;
             v[1] = q1;
             if ((cm0 & 6u) != 6u) square2<ND1>(tab_Bg(fs, T()), fs.tBg, v, w, lane, tm);
