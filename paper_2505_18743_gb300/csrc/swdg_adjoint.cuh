@@ -712,8 +712,8 @@ __global__ void __maxnreg__(128)
                 qs[0] += team_sum<TL>(s0, tm);
                 qs[1] += team_sum<TL>(s1, tm);
             }
-            double Hs, As;
-            mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, Hs, As, tm);
+            const Mass ms = mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, tm);
+            const double Hs = ms.H, As = ms.A;
             // tracer: c = (CNbar + dt sum a sum_i R_i) / Hbar(e), or c^n in a dry cell
             if (Hs > 1e-14 * J * d.hlim) {
                 const double rsb = cs / Hs, Hsb = -cs * cl / Hs;
@@ -931,8 +931,7 @@ __global__ void __maxnreg__(96)
             __syncwarp();
             // zeta~ = e with Hbar(e, delta) = m(zeta^n, delta); dry: e = -max(z_b + delta)
             if (m > 0.0) {
-                double Hs, As;
-                mass_scalar_pixels<R, Pix, MODE>(d, tb, k, J, a.un[k * ND], lane, Hs, As);
+                const double As = mass_scalar_pixels<R, Pix, MODE>(d, tb, k, J, a.un[k * ND], lane).A;
                 if (As > 0.0) mb += ez / As;
             }
             if (lane == 0) dsum -= ez;

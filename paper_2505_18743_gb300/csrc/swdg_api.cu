@@ -755,13 +755,14 @@ static int grid_for(int64_t n, int wpb = WPB) {
 }
 
 // default shapes: WPB warps per block, one block per WPB cells (grid-stride
-// beyond 152 x 64 blocks); the stage update (two cells per warp) at r <= 2 with
-// 2 warps per block: there the cells' costs differ most (pixel sums, Newton
-// steps) and a small block retires sooner (lagoon, r = 2: 394 us with 2 warps,
-// 447 with 4; beach, r = 3: 607 and 580)
+// beyond 152 x 64 blocks); the stage update (two cells per warp) with one block
+// per 2 WPB cells without a limit: its cells' costs differ most (pixel sums,
+// Newton steps), and with several passes per block the slowest sequence of cells
+// decides (ensemble of 172,000 cells, r = 2: 915 us a stage with 9728 blocks, 886
+// with one pass)
 static void default_shapes(swdg_ctx* c) {
     for (int i = 0; i < KK_N; ++i) c->shp[i] = Shape{grid_for(c->n), WPB};
-    if (c->R <= 2) c->shp[KK_STAGE] = Shape{grid_for(c->n, 4), 2};
+    c->shp[KK_STAGE].grid = (int)std::max<int64_t>(1, (c->n + 2 * WPB - 1) / (2 * WPB));
     c->tuned = false;
 }
 

@@ -521,7 +521,9 @@ __device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab
         return {wet ? eta : 0.0, wet ? 1.0 : 0.0, wet};
     }
     if (zmag == 0) {
+#pragma unroll 1
         for (int j = 0; j < cy; ++j)
+#pragma unroll 1
             for (int i = 0; i < cx; ++i)
                 zmag = max(zmag, fx::mag((double)tile[(loy + j) * P + lox + i]));
     }
@@ -532,16 +534,19 @@ __device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab
 #pragma unroll 1
     for (int j = 0; j < cy; ++j) {
         const Pix* row = tile + (loy + j) * P + lox;
-        long long T = 0, first = 0, last = 0; // sums over the row, its first and last pixel
-        int c = 0, cf = 0, cl = 0;
-        for (int i = 0; i < cx; ++i) {
+        // the row's sum, its first and its last pixel (0 where it has only one)
+        const long long D0 = E + fx_pixel(row[0], es);
+        const int cf = D0 > 0;
+        const long long first = cf ? D0 : 0;
+        long long T = first, last = 0;
+        int c = cf, cl = 0;
+#pragma unroll 2
+        for (int i = 1; i < cx; ++i) {
             const long long D = E + fx_pixel(row[i], es);
-            const int w = D > 0;
-            const long long Dp = w ? D : 0;
-            T += Dp;
-            c += w;
-            if (i == 0) { first = Dp; cf = w; }
-            if (i == cx - 1 && i > 0) { last = Dp; cl = w; }
+            cl = D > 0;
+            last = cl ? D : 0;
+            T += last;
+            c += cl;
         }
         wet += c;
         const int2 f0 = ov->ed[setx][ia][0], f1 = ov->ed[setx][ia][1], f2 = ov->ed[setx][ia][2];

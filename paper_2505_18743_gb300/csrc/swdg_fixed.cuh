@@ -29,7 +29,8 @@
 // by two row bounds (hi Tlo and lo Thi are below 2^59 each).
 //
 // A block that holds an infinity or a NaN takes the exponent POISON; every
-// value converted back from it is NaN.  Blocks below 2^-958 count as zero.
+// value converted back from it is NaN.  Blocks below 2^-958 keep the exponent of
+// that size: they lose places, and values below 2^-1018 are zero.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -183,7 +184,7 @@ __host__ __device__ __forceinline__ long long from_float(float v, int eb) {
     int d = eb - (ef + 896);
     d = ef == 0 ? 63 : (d < 63 ? d : 63);
     const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (FB - 24);
-    const long long X = (long long)(m >> d);
+    const long long X = (long long)((m + ((1ull << d) >> 1)) >> d); // to nearest
     return (int)b < 0 ? -X : X;
 }
 __host__ __device__ __forceinline__ float to_float(long long X, int eb) {
