@@ -360,11 +360,13 @@ int swdg_amr_adapt(swdg_ctx* ctx, const double* eta, int kind, double theta_r, d
 int swdg_amr_leaves(const swdg_ctx* ctx, int32_t* lij);
 
 /* ---- launch shapes (the paper has no counterpart) ----
- * Each kernel kind runs one warp per cell, grid-stride over all cells: kind
+ * Each kernel kind gives a cell to a warp or to a part of one, grid-stride over
+ * all cells: kind
  * SWDG_KIND_BEGIN (degree switch and H, C~), SWDG_KIND_RESIDUAL,
  * SWDG_KIND_STAGE (stage update and final combination), SWDG_KIND_AUX (masks,
  * diagnostics).  A shape is (grid blocks, warps per block 1..8); the default
- * is 4 warps per block and one block per 4 cells (at most 9728 blocks).
+ * is 4 warps per block and one block per 4 cells (at most 9728 blocks; the stage
+ * update one per 8 cells, without a limit).
  * Shapes change speed only: every cell's arithmetic is the same, so results
  * are bitwise identical under any shape. */
 #define SWDG_KIND_BEGIN 0
@@ -396,9 +398,8 @@ int swdg_autotune(swdg_ctx* ctx, int repeats, double* report);
 int swdg_probe_fma(int dtype, double* tflops, double* ms);
 
 /* Test helper (the paper has no counterpart): the kernels' own root of the
- * Manning term, z = h^(-1/3) (an FP32 reciprocal cube root refined by two
- * Newton-Raphson steps for z^-3 = h in FP64; 1 / cbrt(h) outside the FP32
- * range), and z^3, the 1/h the residual takes at wet points with friction,
+ * Manning term, z = h^(-1/3) (an FP32 reciprocal cube root refined by one
+ * Halley step for z^-3 = h in FP64; 1 / cbrt(h) outside the FP32 range), and z^3, the 1/h the residual takes at wet points with friction,
  * evaluated on the device for n host values h [n] > 0 into z [n] and
  * rcp [n] (host).  1 <= n <= 2^24.  Allocates 24 n bytes of device memory for
  * the duration of the call.  Returns SWDG_EINVAL for bad sizes or pointers,
@@ -411,8 +412,8 @@ int swdg_probe_roots(const double* h, int64_t n, double* z, double* rcp);
  * already reserved every byte of the device).  It evaluates exactly what
  * swdg_residual evaluates, plus the CFL step of swdg_cfl_dt, without a
  * context: the caller passes every input and output as device buffers, and
- * the only scratch (the step scalars, the pixel-overlap table and one
- * constant-field byte per cell, about 1.01 MiB in all) lives in a fixed array
+ * the only scratch (the step scalars, the pixel-overlap and basis tables and one
+ * constant-field byte per cell, about 1.02 MiB in all) lives in a fixed array
  * inside the library, held on each GPU where the library's device code is
  * loaded until the process exits.  It calls no cudaMalloc/cudaFree.  CUDA
  * loads device code lazily by default: the array and this degree's kernels

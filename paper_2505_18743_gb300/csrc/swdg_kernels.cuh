@@ -2,12 +2,12 @@
 // path (arXiv 2505.18743): residual (Sec. 3.2), degree switch (Eq.
 // criteria_p), stage update (Sec. 3.1) and auxiliary reductions.
 //
-// Mapping: one warp per cell, a launch-time number of warps per block (1..8,
-// chosen by the autotuner), grid-stride over cells; one launch covers every
-// member of an ensemble.
-// Each warp stages its cell in shared memory and evaluates the tensor-product
-// operators by sum factorisation (1D contractions), one quadrature point,
-// degree of freedom or face point per lane.
+// Mapping: one cell per team of 8, 16 or 32 lanes, a launch-time number of warps
+// per block (1..8), grid-stride over cells; one launch covers every member of an
+// ensemble.  Each team stages its cell in shared memory and evaluates the
+// tensor-product operators by sum factorisation (1D contractions, in block fixed
+// point), one quadrature point or degree of freedom per lane; the face points
+// are one per lane over the whole mesh (k_faces).
 #pragma once
 #include "swdg_common.cuh"
 
