@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(32 * MAXWPB)
     k_indicator(const __grid_constant__ Dev d, const __grid_constant__ Tables tb, int kind,
                 double* eta) {
     using S = Sz<R>;
-    using ST = Site<R, Pix, MODE>;
+    using ST = Site<R, Pix, MODE, false>;
     constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP;
     extern __shared__ double smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;

@@ -330,19 +330,8 @@ static void build_fx_tables(int R, Tables& tb) {
     y.tGi = put(&tb.Bginv[0][0], MXP, false, n1, n1, &y.Gi[0][0], MXN);
     y.tGiT = put(&tb.Bginv[0][0], MXP, true, n1, n1, &y.GiT[0][0], MXN);
     y.tM1i = put(&tb.M1inv[0][0], MXN, false, n1, n1, &y.M1i[0][0], MXN);
-    BulkTables& z = tb.fb;
-    z.tBv = put(&tb.Bv[0][0], MXN, false, nv, n1, &z.Bv[0][0], MXN);
-    z.tBvT = put(&tb.Bv[0][0], MXN, true, n1, nv, &z.BvT[0][0], MXP);
-    z.tDvT = put(&tb.Dv[0][0], MXN, true, n1, nv, &z.DvT[0][0], MXP);
-    memcpy(z.BmT, x.BmT, sizeof z.BmT);
-    memcpy(z.BmHT, x.BmHT, sizeof z.BmHT);
-    z.tBmT = x.tBmT;
-    memcpy(z.BvF, tb.BvF, sizeof z.BvF);
-    memcpy(z.DvF, tb.DvF, sizeof z.DvF);
-    memcpy(z.wvF, tb.wvF, sizeof z.wvF);
     memcpy(y.wm, tb.wm, sizeof y.wm);
     memcpy(y.wg, tb.wg, sizeof y.wg);
-    memcpy(y.BmF, tb.BmF, sizeof y.BmF);
     for (int a = 0; a < n1; ++a)
         for (int q = 0; q < n1; ++q) y.wn[a] += tb.wg[q] * tb.Bg[q][a];
     double nrm[MXN];
@@ -355,17 +344,11 @@ static void build_fx_tables(int R, Tables& tb) {
             for (int q = 0; q < nm; ++q)
                 y.BB[a * (a + 1) / 2 + c][q] = (float)(tb.Bm[q][a] * tb.Bm[q][c] * nrm[a] * nrm[c]);
     }
-    memcpy(y.wgF, tb.wgF, sizeof y.wgF);
     memcpy(tb.ft.Bm, tb.Bm, sizeof tb.Bm);
     memcpy(tb.ft.BmH, tb.BmH, sizeof tb.BmH);
     memcpy(tb.ft.wm, tb.wm, sizeof tb.wm);
     memcpy(tb.ft.BmF, tb.BmF, sizeof tb.BmF);
     memcpy(tb.ft.BmHF, tb.BmHF, sizeof tb.BmHF);
-    for (int a = 0; a < n1; ++a)
-        for (int q = 0; q < n1; ++q) {
-            y.BgF[q][a] = y.BgTF[a][q] = tb.BgF[q][a];
-            y.GiF[a][q] = y.GiTF[q][a] = tb.BginvF[a][q];
-        }
 }
 
 static bool build_tables(int R, Tables& tb) {

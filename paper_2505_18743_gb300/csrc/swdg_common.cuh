@@ -86,8 +86,6 @@ struct FxStage {
     int2 Gi[MXN][MXN], GiT[MXN][MXN]; // inverse of Bg, its transpose
     int2 M1i[MXN][MXN];               // inverse 1D mass matrix
     double wm[MXP], wg[MXP], wn[MXN]; // wn: the nodes' weights in the momentum rule
-    float BmF[MXP][MXN], wgF[MXP];
-    float BgF[MXN][MXN], BgTF[MXN][MXN], GiF[MXN][MXN], GiTF[MXN][MXN];
     // the mass matrices' FP32 assembly: node scales 1 / |B_a| (2-norm over the
     // mass points, per direction) and products of the scaled basis, [pair][point]
     // with pair (a, c), c <= a, at a (a + 1) / 2 + c
@@ -102,34 +100,25 @@ struct FaceTables {
     float BmF[MXP][MXN], BmHF[2][MXP][MXN];
 };
 
-// what the FP32-bulk residual takes: digit pairs of the elevation's interpolation
-// and of the test integrals of F and R (the transposes, without weights), the
-// face test tables of FxTables, and the FP32 basis
-struct BulkTables {
-    int2 Bv[MXP][MXN], BvT[MXN][MXP], DvT[MXN][MXP];
-    int2 BmT[MXN][MXP], BmHT[2][MXN][MXP];
-    float BvF[MXP][MXN], DvF[MXP][MXN], wvF[MXP];
-    int tBv, tBvT, tDvT, tBmT;
-};
-
-struct Tables {
+// the basis tables in FP64, and the FP32 copies of the FP32-bulk kernels
+struct BaseTables {
     double Bv[MXP][MXN], Dv[MXP][MXN], wv[MXP]; // nodal -> volume GL (value, d/dxi)
     double Bm[MXP][MXN], wm[MXP];               // nodal -> mass / face GLL
     double Bg[MXP][MXN], wg[MXP];               // nodal -> momentum GL (square)
     double Bginv[MXN][MXP];                     // inverse of Bg
     double M1inv[MXN][MXN];                     // inverse of the 1D GLL mass matrix
     double BmH[2][MXP][MXN];                    // nodal -> fine-face GLL points of half h
-    // FP32 copies for the FP32-bulk kernels
     float BvF[MXP][MXN], DvF[MXP][MXN], BmF[MXP][MXN], BmHF[2][MXP][MXN], BgF[MXP][MXN];
     float BginvF[MXN][MXP];
     float wvF[MXP];                             // volume GL weights (FP32-bulk residual)
     float wgF[MXP];                             // momentum GL weights (FP32-bulk stage update)
     double xs[MXN];                             // support nodes on [0, 1]
     double xq[3][MXP];                          // nodes of the three point sets on [0, 1]
+};
+struct Tables : BaseTables {
     FxTables fx;
     FxStage fs;
     FaceTables ft;
-    BulkTables fb;
 };
 
 // clock of one ensemble member (a plain context is an ensemble of one)
@@ -356,9 +345,8 @@ __device__ __forceinline__ float f32_trunc(double x) {
     const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
     return __uint_as_float(((h - 0x38000000u) << 3) | (l >> 29));
 }
-// the nearest FP32 value of any double (ties to even, as a conversion rounds)
-// and the double of any FP32 value, the same way; outside the FP32 normal
-// range by conversion
+// the nearest FP32 value of any double (ties to even, as a conversion rounds), the
+// same way; outside the FP32 normal range by conversion
 __device__ __forceinline__ float f32_of(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned h = (unsigned)(b >> 32) & 0x7fffffffu;
@@ -368,13 +356,6 @@ __device__ __forceinline__ float f32_of(double x) {
         return __uint_as_float((m - 0xc0000000u) | ((unsigned)(b >> 32) & 0x80000000u));
     }
     return b << 1 ? (float)x : 0.0f;
-}
-__device__ __forceinline__ double f64_any(float v) {
-    const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xffu;
-    if (e - 1u < 254u)
-        return __hiloint2double((int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)),
-                                (int)(b << 29));
-    return b << 1 ? (double)v : 0.0;
 }
 __device__ __forceinline__ double f64_of(float v) {
     const unsigned b = __float_as_uint(v);
@@ -564,6 +545,35 @@ __device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab
     }
     const bool full = wet == cx * cy;
     return {fx::to_double(v.get(), es), full ? 1.0 : wet ? fx::to_double(a.get(), 1028) : 0.0, full};
+}
+
+// the same sums in FP64
+template <typename Pix>
+__device__ __forceinline__ SubV subgrid_f64(const Pix* __restrict__ tile, const OvTab& ov, int setx,
+                                            int ia, int sety, int ib, double eta) {
+    const int P = ov.P;
+    const int lox = ov.lo[setx][ia], cx = ov.cnt[setx][ia];
+    const int loy = ov.lo[sety][ib], cy = ov.cnt[sety][ib];
+    double v = 0.0, a = 0.0;
+    bool f = true;
+    for (int j = 0; j < cy; ++j) {
+        const Pix* row = tile + (size_t)(loy + j) * P + lox;
+        double vr = 0.0, ar = 0.0;
+        for (int i = 0; i < cx; ++i) {
+            double dd = eta + (double)row[i];
+            if (dd > 0.0) {
+                double fx = ov.frac[setx][ia][i];
+                vr += fx * dd;
+                ar += fx;
+            } else {
+                f = false;
+            }
+        }
+        double fy = ov.frac[sety][ib][j];
+        v += fy * vr;
+        a += fy * ar;
+    }
+    return {v, a, f};
 }
 
 __device__ __forceinline__ void subgrid_P(double z, double eta, double& V, double& A) {

@@ -2,6 +2,7 @@
 // swdg_r{1,2,3}.cu with SWDG_DEGREE defined).
 #pragma once
 #include "swdg_adjoint.cuh"
+#include "swdg_bulk.cuh"
 #include "swdg_amr.cuh"
 #include "swdg_kernels.cuh"
 #include "swdg_launch.h"
@@ -12,16 +13,26 @@ template <int R, typename Pix, int MODE, typename B>
 struct Launchers {
     using S = Sz<R>;
     static constexpr bool F64 = sizeof(B) == sizeof(double);
+    // shared memory per warp; the step start gives a cell 16 lanes (FP32-bulk: 32), the
+    // stage update 16
     static constexpr size_t res_b =
-        sizeof(double) * (F64 ? ResFx<R>::words : ResBulk<R>::words) * (32 / ResFx<R>::TL); // per warp
+        sizeof(double) * (F64 ? ResFx<R>::words : bulk::Res<R>::words) * (32 / ResFx<R>::TL);
+    static constexpr int begin_cells = F64 ? 2 : 1;
+    static constexpr size_t begin_b = sizeof(double) * (F64 ? 2 * BeginFx<R>::words : bulk::begin_smem<R>());
+    static constexpr size_t stage_b =
+        2 * sizeof(double) * (F64 ? StageFx<R>::words : bulk::stage_smem<R>());
     static auto residual_kernel() {
         if constexpr (F64) return k_residual<R, Pix, MODE>;
-        else return k_residual_bulk<R, Pix, MODE>;
+        else return bulk::k_residual<R, Pix, MODE>;
     }
-    static constexpr size_t begin_b = 2 * sizeof(double) * BeginFx<R>::words; // two cells per warp
-    // k_stage runs two cells per warp (a team of 16 lanes each)
-    static constexpr size_t stage_b =
-        2 * sizeof(double) * StageFx<R>::words(sizeof(B) != sizeof(double));
+    static auto begin_kernel() {
+        if constexpr (F64) return k_step_begin<R, Pix, MODE>;
+        else return bulk::k_step_begin<R, Pix, MODE>;
+    }
+    static auto stage_kernel() {
+        if constexpr (F64) return k_stage<R, Pix, MODE>;
+        else return bulk::k_stage<R, Pix, MODE>;
+    }
     static constexpr size_t diag_b = sizeof(double) * (2 * S::ND + 2 * S::NMP + 2 * S::NM * S::NM);
     static constexpr size_t vjp_b = sizeof(double) * vjp_smem<R>() * (32 / VjpTeam<R>::TL); // per warp
     static constexpr size_t svjp_b = 2 * sizeof(double) * stage_vjp_smem<R>(); // two cells per warp
@@ -42,7 +53,7 @@ struct Launchers {
                 k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage, c_stage,
                                                                                   want_dt);
         } else {
-            k_residual_bulk<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage);
+            bulk::k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage);
         }
     }
     static void faces(const Dev& d, const Tables& tb, int buf, double c_stage, int want_dt,
@@ -55,18 +66,24 @@ struct Launchers {
         if constexpr (F64)
             k_faces<R, Pix, MODE><<<(int)blocks, 128, 0, st>>>(d, buf, c_stage, want_dt);
         else
-            k_faces_bulk<R, Pix, MODE, B><<<(int)blocks, 128, 0, st>>>(d, buf, c_stage, want_dt);
+            bulk::k_faces<R, Pix, MODE><<<(int)blocks, 128, 0, st>>>(d, buf, c_stage, want_dt);
     }
     static void step_begin(const Dev& d, const Tables& tb, int do_switch, Shape s, cudaStream_t st) {
-        const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
-        k_step_begin<R, Pix, MODE><<<grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, do_switch);
+        const int cpb = begin_cells * s.wpb;
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
+        if constexpr (F64)
+            k_step_begin<R, Pix, MODE><<<grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, do_switch);
+        else
+            bulk::k_step_begin<R, Pix, MODE><<<grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, do_switch);
     }
     static void stage(const Dev& d, const Tables& tb, const StageArgs& sa, Shape s, cudaStream_t st) {
         // two cells per warp: no more blocks than 2 wpb cells each
         const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
-        k_stage<R, Pix, MODE, B><<<grid, 32 * s.wpb, stage_b * s.wpb, st>>>(d, sa);
+        if constexpr (F64)
+            k_stage<R, Pix, MODE><<<grid, 32 * s.wpb, stage_b * s.wpb, st>>>(d, sa);
+        else
+            bulk::k_stage<R, Pix, MODE><<<grid, 32 * s.wpb, stage_b * s.wpb, st>>>(d, sa);
     }
     static void masks(const Dev& d, int buf, Shape s, cudaStream_t st) {
         k_masks<R><<<s.grid, 32 * s.wpb, 0, st>>>(d, buf);
@@ -116,8 +133,8 @@ struct Launchers {
         if constexpr (F64)
             if (!opt_in(k_residual<R, Pix, 0, true>, res_b)) return false;
         return opt_in(residual_kernel(), res_b) &&
-               opt_in(k_step_begin<R, Pix, MODE>, begin_b) &&
-               opt_in(k_stage<R, Pix, MODE, B>, stage_b) &&
+               opt_in(begin_kernel(), begin_b) &&
+               opt_in(stage_kernel(), stage_b) &&
                opt_in(k_cell_diag<R, Pix, MODE>, diag_b) &&
                opt_in(k_residual_vjp<R, Pix, MODE>, vjp_b) &&
                opt_in(k_stage_vjp<R, Pix, MODE>, svjp_b) &&
@@ -134,9 +151,9 @@ struct Launchers {
     static int occupancy(int kind, int wpb) {
         if (wpb < 1 || wpb > MAXWPB) return 0;
         switch (kind) {
-        case KK_BEGIN: return occ(k_step_begin<R, Pix, MODE>, wpb, begin_b);
+        case KK_BEGIN: return occ(begin_kernel(), wpb, begin_b);
         case KK_RESIDUAL: return occ(residual_kernel(), wpb, res_b);
-        case KK_STAGE: return occ(k_stage<R, Pix, MODE, B>, wpb, stage_b);
+        case KK_STAGE: return occ(stage_kernel(), wpb, stage_b);
         default: return occ(k_cell_diag<R, Pix, MODE>, wpb, diag_b);
         }
     }

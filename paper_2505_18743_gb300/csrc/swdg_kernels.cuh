@@ -125,9 +125,17 @@ __device__ __forceinline__ int team_exp(double v, unsigned tm) {
 // ---------------------------------------------------------------------------
 // bathymetry sampling sites
 // ---------------------------------------------------------------------------
-template <int R, typename Pix, int MODE>
+// FX: partly wet sub-cells sum their pixels in fixed point (subgrid_S), else in FP64
+// (subgrid_f64: the FP32-bulk path, the diagnostics and the refinement indicator)
+template <int R, typename Pix, int MODE, bool FX = true>
 struct Site {
     using S = Sz<R>;
+    static __device__ __forceinline__ SubV pixels(const Dev& d, int64_t k, int setx, int ia, int sety,
+                                                  int ib, double eta) {
+        const OvTab& o = tab(d, k);
+        if constexpr (FX) return subgrid_S<Pix>(tile(d, o, k), &o, setx, ia, sety, ib, eta, zmag(d, k));
+        else return subgrid_f64<Pix>(tile(d, o, k), o, setx, ia, sety, ib, eta);
+    }
     static __device__ __forceinline__ int offset(int set) {
         return set == SET_VOL ? 0 : (set == SET_MASS ? S::NVP : S::NVP + S::NMP);
     }
@@ -194,8 +202,7 @@ struct Site {
                     if (shortcut_b(eta, (double)b.x, (double)b.y, zbar, V, A, full)) return;
                 }
             }
-            const OvTab& o = tab(d, k);
-            const SubV r = subgrid_S<Pix>(tile(d, o, k), &o, set, ia, set, ib, eta, zmag(d, k));
+            const SubV r = pixels(d, k, set, ia, set, ib, eta);
             V = r.V;
             A = r.A;
             full = r.full;
@@ -218,10 +225,9 @@ struct Site {
         if (MODE == 0) {
             bool full;
             if (shortcut(d, k, eta, zh, V, A, full)) return;
-            const OvTab& o = tab(d, k);
             const int m = (f == 0 || f == 2) ? 0 : S::NM - 1, t = h * S::NM + al;
-            const SubV r = subgrid_S<Pix>(tile(d, o, k), &o, f < 2 ? SET_MASS : SET_HALF, f < 2 ? m : t,
-                                          f < 2 ? SET_HALF : SET_MASS, f < 2 ? t : m, eta, zmag(d, k));
+            const SubV r = pixels(d, k, f < 2 ? SET_MASS : SET_HALF, f < 2 ? m : t,
+                                  f < 2 ? SET_HALF : SET_MASS, f < 2 ? t : m, eta);
             V = r.V;
             A = r.A;
         } else {
@@ -266,32 +272,6 @@ __device__ __forceinline__ void face_trace(const double* u, size_t fstride, unsi
     }
 }
 
-// Rusanov flux with hydrostatic reconstruction at one face point, seen from
-// side A with outward normal (nx, ny) (Eqs. lxf_parameter, velocity,
-// hydro_rec_vars, mass_rhs, discharge_rhs, r_concentration).  hA = V_A(zeta_A),
-// hsA = min(V_A(zeta_A), V_B(zeta_A)).  out = {F, Gx_cons, Gy_cons, R}; the
-// non-conservative pressure scalar g {{h*}} (h*A - h*B)/2 is returned apart.
-template <typename T>
-__device__ __forceinline__ void rusanov(T qxA, T qyA, T cA, T hA, T hsA, T qxB, T qyB, T cB, T hB,
-                                        T hsB, T dhAB, T nx, T ny, T g, T eps, T out[4], T& pres,
-                                        T& lam) {
-    // dhAB = h*A - h*B, formed in FP64 by the caller (the well-balanced part of
-    // the reconstruction); the tracer jump h*A cA - h*B cB = dhAB cA + h*B (cA - cB)
-    const T half = T(0.5);
-    T fA = vel_factor<T>(hA, eps), fB = vel_factor<T>(hB, eps);
-    T uAx = fA * qxA, uAy = fA * qyA, uBx = fB * qxB, uBy = fB * qyB;
-    T unA = uAx * nx + uAy * ny, unB = uBx * nx + uBy * ny;
-    T l = fmax(fabs(unA) + sqrt(g * hA), fabs(unB) + sqrt(g * hB));
-    T qsAx = hsA * uAx, qsAy = hsA * uAy, qsBx = hsB * uBx, qsBy = hsB * uBy;
-    out[0] = half * ((qsAx + qsBx) * nx + (qsAy + qsBy) * ny) + half * l * dhAB;
-    out[1] = half * (qsAx * unA + qsBx * unB) + half * l * (qsAx - qsBx);
-    out[2] = half * (qsAy * unA + qsBy * unB) + half * l * (qsAy - qsBy);
-    out[3] = half * ((qsAx * cA + qsBx * cB) * nx + (qsAy * cA + qsBy * cB) * ny) +
-             half * l * (dhAB * cA + hsB * (cA - cB));
-    pres = g * half * (hsA + hsB) * half * dhAB;
-    lam = l;
-}
-
 __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double v) {
     // non-negative doubles order like their bit patterns
     atomicMax(addr, (unsigned long long)__double_as_longlong(v));
@@ -302,157 +282,9 @@ __device__ __forceinline__ void atomic_max_pos(unsigned long long* addr, double 
 // r+2 Gauss-Lobatto points per face (Eqs. mass_rhs, discharge_rhs,
 // discharge_rhs_implicit, r_concentration)
 // ---------------------------------------------------------------------------
-// traces of zeta (FP64) and of qx, qy, c (type B) at face point al of face f;
-// u32 (B = float, nullable): the FP32 copy of u, same layout and stride
-template <int ND1, typename B>
-__device__ __forceinline__ void face_trace_mixed(const double* u, const float* u32, size_t fstride,
-                                                 unsigned cm, int f, const double (*Bd)[MXN],
-                                                 const B (*Bb)[MXN], int al, double& z, B t[3]) {
-    if (cm & 1u) z = u[0];
-    else {
-        double s = 0.0;
-#pragma unroll
-        for (int j = 0; j < ND1; ++j) s += Bd[al][j] * u[face_node<ND1>(f, j)];
-        z = s;
-    }
-#pragma unroll
-    for (int fl = 1; fl < 4; ++fl) {
-        const double* uf = u + fl * fstride;
-        if constexpr (sizeof(B) == sizeof(float)) {
-            if (u32 != nullptr) { // the same values as (float)uf[.], without conversions
-                const float* vf = u32 + fl * fstride;
-                if (cm & (1u << fl)) {
-                    t[fl - 1] = vf[0];
-                    continue;
-                }
-                B s = B(0);
-#pragma unroll
-                for (int j = 0; j < ND1; ++j) s += Bb[al][j] * vf[face_node<ND1>(f, j)];
-                t[fl - 1] = s;
-                continue;
-            }
-        }
-        if (cm & (1u << fl)) {
-            t[fl - 1] = (B)uf[0];
-            continue;
-        }
-        B s = B(0);
-#pragma unroll
-        for (int j = 0; j < ND1; ++j) s += Bb[al][j] * (B)uf[face_node<ND1>(f, j)];
-        t[fl - 1] = s;
-    }
-}
-
-template <typename B>
-__device__ __forceinline__ const B (*tab_or(const double (*d)[MXN], const float (*f)[MXN]))[MXN] {
-    if constexpr (sizeof(B) == sizeof(double)) return (const B(*)[MXN])d;
-    else return (const B(*)[MXN])f;
-}
-
-// B = double: the plain FP64 method.  B = float (FP32-bulk): elevation,
-// sub-grid integrals, hydrostatic reconstruction and the continuity and
-// tracer test integrals stay FP64 (so mass, tracer mass and c = 1 are kept to
-// FP64 round-off and the lake at rest exactly); the momentum, friction and
-// flux arithmetic is FP32.
-// one face point (Sec. 3.2): the Rusanov flux with the hydrostatic
-// reconstruction at GLL point al of half h of face f of cell k, whose state
-// (4 fields, stride ustride) is uk with constant-field mask cm.  An interior
-// point returns the flux of the canonical side order (the lower cell index is
-// side A, so both cells of a face get bit-identical values) in raw, with the
-// pressure term pres, own_first = (k is side A) and the neighbour nb; a
-// boundary point returns k's final flux in raw (bnd = true, nb = -1).  lam is
-// the wave speed bound of the point.
-template <int R, typename Pix, int MODE, typename B>
-__device__ __forceinline__ void face_point(const Dev& d, const FaceTables& tb, int64_t k, const double* uk,
-                                           const float* ukF, size_t ustride, unsigned cm, int buf,
-                                           int f, int h, int al,
-                                           unsigned info, double hx, double hy, int mem, double t,
-                                           B raw[4], B& pres, B& lam, bool& own_first, bool& bnd,
-                                           int64_t& nb_out) {
-    using S = Sz<R>;
-    using ST = Site<R, Pix, MODE>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM;
-    const int64_t n = d.n;
-    const B gB = (B)d.g, epsB = (B)d.eps;
-    const auto BmB = tab_or<B>(tb.Bm, tb.BmF);
-    const bool coarse = (info & 3) == FI_COARSE, fine = (info & 3) == FI_FINE;
-    const int half = (int)(info >> 2);
-    const double nx = (f == 0) ? -1.0 : (f == 1) ? 1.0 : 0.0;
-    const double ny = (f == 2) ? -1.0 : (f == 3) ? 1.0 : 0.0;
-    double zm;
-    B tm[3];
-    face_trace_mixed<ND1, B>(uk, ukF, ustride, cm, f, coarse ? tb.BmH[h] : tb.Bm,
-                             coarse ? tab_or<B>(tb.BmH[h], tb.BmHF[h]) : BmB, al, zm, tm);
-    int ia, ib;
-    face_site_index<NM>(f, al, ia, ib);
-    auto own_V = [&](double eta) {
-        double V, A;
-        if (coarse) ST::VA_half(d, k, f, h, al, eta, V, A);
-        else ST::VA(d, *d.tabs, k, SET_MASS, ia, ib, eta, V, A);
-        return V;
-    };
-    const int32_t s0 = d.nbr[k * 8 + f * 2];
-    const double hm = own_V(zm);
-    double zp, hp, hsm, hsp;
-    B tp[3];
-    if (s0 >= 0) {
-        const int64_t nb = coarse ? (int64_t)(h ? d.nbr[k * 8 + f * 2 + 1] : s0) : (int64_t)s0;
-        const int fo = f ^ 1;
-        face_trace_mixed<ND1, B>(ufield(d, buf, 0, ND) + nb * ND,
-                                 d.uF ? ufieldF(d, buf, 0, ND) + nb * ND : nullptr, (size_t)n * ND,
-                                 d.cmask[(size_t)buf * n + nb], fo, fine ? tb.BmH[half] : tb.Bm,
-                                 fine ? tab_or<B>(tb.BmH[half], tb.BmHF[half]) : BmB, al, zp, tp);
-        int ja, jb;
-        face_site_index<NM>(fo, al, ja, jb);
-        auto nb_V = [&](double eta) {
-            double V, A;
-            if (fine) ST::VA_half(d, nb, fo, half, al, eta, V, A);
-            else ST::VA(d, *d.tabs, nb, SET_MASS, ja, jb, eta, V, A);
-            return V;
-        };
-        hp = nb_V(zp);
-        hsm = fmin(hm, nb_V(zm)); // min(V-(zeta-), V+(zeta-)), FP64
-        hsp = fmin(hp, own_V(zp)); // min(V+(zeta+), V-(zeta+)), FP64
-        own_first = k < nb;
-        if (own_first)
-            rusanov<B>(tm[0], tm[1], tm[2], (B)hm, (B)hsm, tp[0], tp[1], tp[2], (B)hp, (B)hsp,
-                       (B)(hsm - hsp), (B)nx, (B)ny, gB, epsB, raw, pres, lam);
-        else
-            rusanov<B>(tp[0], tp[1], tp[2], (B)hp, (B)hsp, tm[0], tm[1], tm[2], (B)hm, (B)hsm,
-                       (B)(hsp - hsm), (B)(-nx), (B)(-ny), gB, epsB, raw, pres, lam);
-        bnd = false;
-        nb_out = nb;
-    } else {
-        const int tag = -1 - s0;
-        zp = zm;
-        tp[0] = tm[0]; tp[1] = tm[1]; tp[2] = tm[2];
-        const bool tide = d.mbc ? d.mbc[mem].kind[tag] == 1 : d.bc_kind[tag] == 1;
-        if (tide) {
-            const double amp = d.mbc ? d.mbc[mem].amp[tag] : d.bc_amp[tag];
-            const double per = d.mbc ? d.mbc[mem].per[tag] : d.bc_per[tag];
-            const double ph = d.mbc ? d.mbc[mem].ph[tag] : d.bc_ph[tag];
-            zp = amp * sin(2.0 * M_PI * t / per + ph);
-        } else {
-            const B qn = tm[0] * (B)nx + tm[1] * (B)ny;
-            tp[0] = tm[0] - B(2) * qn * (B)nx;
-            tp[1] = tm[1] - B(2) * qn * (B)ny;
-        }
-        hp = own_V(zp); // ghost: same sub-grid operator
-        hsm = hm;
-        hsp = hp;
-        rusanov<B>(tm[0], tm[1], tm[2], (B)hm, (B)hsm, tp[0], tp[1], tp[2], (B)hp, (B)hsp,
-                   (B)(hsm - hsp), (B)nx, (B)ny, gB, epsB, raw, pres, lam);
-        raw[1] -= pres * (B)nx;
-        raw[2] -= pres * (B)ny;
-        own_first = true;
-        bnd = true;
-        nb_out = -1;
-    }
-}
-
-// One face point in FP64 (Sec. 3.2), as face_point below evaluates it for the
-// FP32-bulk path, in the face's own frame: faces are axis-aligned, so the
-// fluxes have an axis and a tangential component, normals are signs (applied to
+// One face point (Sec. 3.2) in FP64: the Rusanov flux with the hydrostatic
+// reconstruction at GLL point al of half h of face f of cell k, in the face's own
+// frame: faces are axis-aligned, so the fluxes have an axis and a tangential component, normals are signs (applied to
 // the sign bit) and one evaluation serves interior and boundary points.  flux =
 // {F, G axis, G tangential, R} outward from side A (the lower cell index), pr
 // the pressure vector's axis component g {{h*}} (h*A - h*B)/2 n_A, lam the wave
@@ -592,22 +424,6 @@ __device__ __forceinline__ void side_values(const FaceFlux& q, int f, bool other
     o[1] = f < 2 ? a : t;
     o[2] = f < 2 ? t : a;
     o[3] = w * flip(q.flux[3], sg);
-}
-
-// the flux of an interior face point as seen from the cell whose face f it
-// is: the canonical flux with the sign of that side, and the pressure vector
-// g {{h*}} (h*A - h*B)/2 n_A, which is the same for both sides
-template <typename B>
-__device__ __forceinline__ void side_flux(const B raw[4], B pres, bool own_first, int f, B out[4]) {
-    const double nx = (f == 0) ? -1.0 : (f == 1) ? 1.0 : 0.0;
-    const double ny = (f == 2) ? -1.0 : (f == 3) ? 1.0 : 0.0;
-    const B sg = own_first ? B(1) : B(-1);
-    const B pnx = own_first ? pres * (B)nx : pres * (B)(-nx);
-    const B pny = own_first ? pres * (B)ny : pres * (B)(-ny);
-    out[0] = raw[0] * sg;
-    out[1] = sg * raw[1] - pnx;
-    out[2] = sg * raw[2] - pny;
-    out[3] = raw[3] * sg;
 }
 
 // The FP64 residual.  What bounds it is the FP64 pipe (one warp instruction
@@ -1013,274 +829,6 @@ __global__ void __maxnreg__(64)
     }
 }
 
-// The FP32-bulk residual: the momentum and the pointwise physics in FP32, the
-// elevation's value, the sub-grid depth, F and R beyond FP32 (block fixed point,
-// as in k_residual; the point values of F and R are FP32 products).  The same
-// teams; the FP64 pipe keeps the conversions and the final differences (it took
-// 69 instructions a cell, and bounded the kernel, while the sums of zeta, F, R
-// and the face lifts ran there).  Measured per launch: r = 2, 172,000 cells 580 ->
-// 282 us; r = 3, 65,536 cells 310 -> 188 us (80 registers: 305, 201).
-template <int R>
-struct ResBulk {
-    using S = Sz<R>;
-    static constexpr int NE = ResFx<R>::NE;
-    // 8-byte words per team: y-test sums [4 NE] digits, [6 NE] floats; digits of zeta
-    // and c [ND] each with x-contractions [3 NE], point values of F and R [4 NVP],
-    // floats: nodal [4 ND], x-contractions [5 NE], point values [8 NVP]; the face
-    // values overlay the second part
-    static constexpr int A = 4 * NE + 3 * NE;
-    static constexpr int B1 = 2 * S::ND + 3 * NE + 4 * S::NVP + (4 * S::ND + 5 * NE + 8 * S::NVP + 1) / 2;
-    static constexpr int B = B1 > 32 * S::NM ? B1 : 32 * S::NM;
-    static constexpr int words = A + B + 2; // and the faces' block exponents
-};
-template <int R, typename Pix, int MODE>
-__global__ void __maxnreg__(64)
-    k_residual_bulk(const __grid_constant__ Dev d, int buf, int stage) {
-    __shared__ BulkTables tx;
-    copy_table(tx, &d.tabs->fb);
-    const Tables& tb = *d.tabs;
-    using S = Sz<R>;
-    using L = ResBulk<R>;
-    using ST = Site<R, Pix, MODE>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NV = S::NV, NVP = S::NVP, NM = S::NM, NE = L::NE;
-    constexpr int TL = ResFx<R>::TL;
-    extern __shared__ double smem[];
-    const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
-    const unsigned tm =
-        TL == 32 ? 0xffffffffu : ((1u << (TL & 31)) - 1u) << (threadIdx.x & 31 & ~(TL - 1));
-    int2* sd = (int2*)(smem + team * L::words); // [4][NV][ND1]: F (xi, eta), R (xi, eta)
-    float* sB = (float*)(sd + 4 * NE);          // [6][NV][ND1]: Gx, Gy xi; Lx, Ly; Gx, Gy eta + value
-    int2* zd = sd + L::A;                       // [ND]
-    int2* cd = zd + ND;                         // [ND] (tracer diffusion only)
-    int2* sx = cd + ND;                         // [3][ND1][NV]: zeta (Bv); c (Bv, Dv), diffusion only
-    int2* Xd = sx + 3 * NE;                     // [4][NVP]: F (x, y), R (x, y)
-    float* suB = (float*)(Xd + 4 * NVP);        // [4][ND]
-    float* tB = suB + 4 * ND;                   // [5][ND1][NV]: qx, qy, c, zeta (Bv), zeta (Dv)
-    float* XB = tB + 5 * NE;                    // [8][NVP]: Gx (x, y, v), Gy (x, y, v), Lx, Ly
-    int2* fd = zd;                              // [4 fields][2 halves][4 faces][NM]
-    int* es = (int*)(zd + L::B);                // [4] the faces' block exponents
-    const double eps = d.eps;
-    const float gB = (float)d.g, epsB = (float)eps;
-    const int64_t n = d.n;
-    const bool pt = lane < NVP;
-
-    for (int64_t k = (int64_t)blockIdx.x * tpb + team; k < n; k += (int64_t)gridDim.x * tpb) {
-        const unsigned cm = d.cmask[(size_t)buf * n + k];
-        const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
-        const double ihx = d.ihxhy ? d.ihxhy[2 * k] : 1.0 / hx;
-        const double ihy = d.ihxhy ? d.ihxhy[2 * k + 1] : 1.0 / hy;
-        const double nu = d.nu_c ? d.nu_c[k] : 0.0;
-        // all four fields in FP32 (the elevation enters FP32 arithmetic only through
-        // its gradient), from the FP32 copy of the state where the context keeps one
-        const double zn = lane < ND ? ufield(d, buf, 0, ND)[k * ND + lane] : 0.0;
-#pragma unroll 1
-        for (int i = lane; i < 4 * ND; i += TL)
-            suB[i] = d.uF ? ufieldF(d, buf, i / ND, ND)[k * ND + (i % ND)]
-                          : (float)ufield(d, buf, i / ND, ND)[k * ND + (i % ND)];
-        unsigned fi[4]; // indexed by constants only (registers)
-#pragma unroll
-        for (int f = 0; f < 4; ++f) fi[f] = d.finfo ? d.finfo[k * 4 + f] : 0;
-        const bool c_f[4] = {(fi[0] & 3) == FI_COARSE, (fi[1] & 3) == FI_COARSE,
-                             (fi[2] & 3) == FI_COARSE, (fi[3] & 3) == FI_COARSE};
-        const int nslot = (c_f[0] || c_f[1] || c_f[2] || c_f[3]) ? 8 * NM : 4 * NM;
-        float manB, JB, ihxB, ihyB;
-        {
-            // the four per-cell values converted once (lanes 0..3)
-            const int q = lane & 3;
-            const float f = (float)(q == 0 ? d.manning[k] : q == 1 ? J : q == 2 ? ihx : ihy);
-            manB = __shfl_sync(tm, f, 0, TL);
-            JB = __shfl_sync(tm, f, 1, TL);
-            ihxB = __shfl_sync(tm, f, 2, TL);
-            ihyB = __shfl_sync(tm, f, 3, TL);
-        }
-        const int ez = team_exp(zn, tm);
-        const double z0 = __shfl_sync(tm, zn, 0, TL);
-        if (lane < ND) zd[lane] = fx::split(fx::from_double(zn, ez));
-        int ec = 0;
-        if (nu != 0.0) { // tracer numerical diffusion (Eq. numdiff): grad c from the FP64 state
-            const double cn = lane < ND ? ufield(d, buf, 3, ND)[k * ND + lane] : 0.0;
-            ec = team_exp(cn, tm);
-            if (lane < ND) cd[lane] = fx::split(fx::from_double(cn, ec));
-        }
-        __syncwarp(tm);
-        // x-contractions: the elevation's value (the sub-grid depth) in fixed point; in
-        // FP32 qx, qy, c, and the elevation's value and d/dxi for its gradient
-#pragma unroll 1
-        for (int i = lane; i < (nu != 0.0 ? 3 : 1) * NE; i += TL) {
-            const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
-            const int2* T = f == 2 ? tb.fx.Dv[al] : tx.Bv[al];
-            const int2* u = (f ? cd : zd) + ND1 * b;
-            fx::Acc s;
-#pragma unroll
-            for (int a = 0; a < ND1; ++a) s.mac(T[a], u[a]);
-            sx[i] = fx::split(s.get());
-        }
-#pragma unroll 1
-        for (int i = lane; i < 5 * NE; i += TL) {
-            const int f = i / NE, r_ = i % NE, b = r_ / NV, al = r_ % NV;
-            const float* u = suB + (f < 3 ? 1 + f : 0) * ND + ND1 * b;
-            const float(*Tb)[MXN] = f == 4 ? tx.DvF : tx.BvF;
-            float s = 0.0f;
-#pragma unroll
-            for (int a = 0; a < ND1; ++a) s += Tb[al][a] * u[a];
-            tB[i] = s;
-        }
-        __syncwarp(tm);
-        // y-contraction and pointwise physics, one volume point per lane (idle lanes
-        // take point 0 and store nothing)
-        int eF, eR; // block exponents of the point values of F, R
-        {
-            const int p = pt ? lane : 0, al = p % NV, be = p / NV;
-            float qx = 0.0f, qy = 0.0f, c = 0.0f, zxd = 0.0f, zyd = 0.0f;
-            fx::Acc az;
-#pragma unroll
-            for (int b = 0; b < ND1; ++b) {
-                az.mac(tx.Bv[be][b], sx[b * NV + al]);
-                const float Bb = tx.BvF[be][b];
-                zxd += Bb * tB[(4 * ND1 + b) * NV + al];
-                zyd += tx.DvF[be][b] * tB[(3 * ND1 + b) * NV + al];
-                qx += Bb * tB[(0 * ND1 + b) * NV + al];
-                qy += Bb * tB[(1 * ND1 + b) * NV + al];
-                c += Bb * tB[(2 * ND1 + b) * NV + al];
-            }
-            double z = fx::to_double(az.get(), ez + 2 * tx.tBv);
-            if (cm & 1u) { z = z0; zxd = 0.0f; zyd = 0.0f; }
-            const float zx = zxd * ihxB, zy = zyd * ihyB;
-            if (cm & 2u) qx = suB[ND];
-            if (cm & 4u) qy = suB[2 * ND];
-            if (cm & 8u) c = suB[3 * ND];
-            double h = 0.0, A;
-            if (pt) ST::VA(d, tb, k, SET_VOL, al, be, z, h, A);
-            const float hB = (float)h;
-            float fv, gam;
-            vel_gamma<float>(manB, hB, qx, qy, gB, epsB, fv, gam);
-            const float ux = fv * qx, uy = fv * qy;
-            // the weights of the FP32 terms in FP32 (no conversions per point)
-            const float wB = JB * tx.wvF[al] * tx.wvF[be], wx = wB * ihxB, wy = wB * ihyB;
-            const float Fx = wx * qx, Fy = wy * qy, Rx = wx * c * qx, Ry = wy * c * qy;
-            auto mag = [](float v) { return __float_as_uint(v) & 0x7fffffffu; };
-            eF = fx::block_exp_f(__reduce_max_sync(tm, pt ? max(mag(Fx), mag(Fy)) : 0u));
-            long long RX, RY;
-            if (nu != 0.0 && !(cm & 8u)) {
-                // -nu h grad c . grad psi: the reference derivatives of c at the point
-                fx::Acc acx, acy;
-#pragma unroll
-                for (int b = 0; b < ND1; ++b) {
-                    acx.mac(tx.Bv[be][b], sx[(2 * ND1 + b) * NV + al]);
-                    acy.mac(tb.fx.Dv[be][b], sx[(ND1 + b) * NV + al]);
-                }
-                const int e = ec + tx.tBv + tb.fx.tDv;
-                const double wn = J * tb.wv[al] * tb.wv[be] * nu * h;
-                const double rx = (double)Rx - wn * fx::to_double(acx.get(), e) * ihx * ihx;
-                const double ry = (double)Ry - wn * fx::to_double(acy.get(), e) * ihy * ihy;
-                eR = fx::block_exp(__reduce_max_sync(tm, pt ? max(fx::mag(rx), fx::mag(ry)) : 0u));
-                RX = fx::from_double(rx, eR);
-                RY = fx::from_double(ry, eR);
-            } else {
-                eR = fx::block_exp_f(__reduce_max_sync(tm, pt ? max(mag(Rx), mag(Ry)) : 0u));
-                RX = fx::from_float(Rx, eR);
-                RY = fx::from_float(Ry, eR);
-            }
-            if (pt) {
-                Xd[0 * NVP + p] = fx::split(fx::from_float(Fx, eF));
-                Xd[1 * NVP + p] = fx::split(fx::from_float(Fy, eF));
-                Xd[2 * NVP + p] = fx::split(RX);
-                Xd[3 * NVP + p] = fx::split(RY);
-                XB[0 * NVP + p] = wx * qx * ux;
-                XB[1 * NVP + p] = wy * qx * uy;
-                XB[2 * NVP + p] = -wB * gB * hB * zx;
-                XB[3 * NVP + p] = wx * qy * ux;
-                XB[4 * NVP + p] = wy * qy * uy;
-                XB[5 * NVP + p] = -wB * gB * hB * zy;
-                XB[6 * NVP + p] = -wB * gam * qx;
-                XB[7 * NVP + p] = -wB * gam * qy;
-            }
-        }
-        __syncwarp(tm);
-        // the face fluxes of k_faces_bulk, loaded here so that the y-contraction hides
-        // the latency
-        const bool conforming = nslot == 4 * NM;
-        double fv[(4 * NM + TL - 1) / TL][4];
-        if (conforming) face_load<NM, TL>(d.fflux + k * (32 * NM), fv, lane);
-        // test integration, y-contraction: F (x, y), R (x, y); in FP32 Gx, Gy (x), Lx, Ly
-        // (value), then Gx, Gy (y + value)
-#pragma unroll 1
-        for (int i = lane; i < 4 * NE; i += TL) {
-            const int job = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-            const int2* T = (job & 1) ? tx.DvT[b] : tx.BvT[b];
-            const int2* X = Xd + job * NVP + al;
-            const float* Xg = XB + ((0x7630u >> (4 * job)) & 15u) * NVP + al;
-            fx::Acc s;
-            float sx_ = 0.0f;
-#pragma unroll
-            for (int be = 0; be < NV; ++be) {
-                s.mac(T[be], X[NV * be]);
-                sx_ += tx.BvF[be][b] * Xg[NV * be];
-            }
-            sd[i] = fx::split(s.get());
-            sB[i] = sx_;
-        }
-#pragma unroll 1
-        for (int i = lane; i < 2 * NE; i += TL) {
-            const int cg = i / NE, r_ = i % NE, al = r_ / ND1, b = r_ % ND1;
-            const float* Xg = XB + 3 * cg * NVP;
-            float so = 0.0f;
-#pragma unroll
-            for (int be = 0; be < NV; ++be) {
-                const int p = al + NV * be;
-                so += tx.DvF[be][b] * Xg[NVP + p] + tx.BvF[be][b] * Xg[2 * NVP + p];
-            }
-            sB[4 * NE + i] = so;
-        }
-        __syncwarp(tm);
-        if (conforming) {
-            face_digits<NM, TL>(fv, fd, es, lane, tm);
-        } else {
-            face_digits_any<NM, TL>([&](int cf, int i) -> double { // 0 where a face has no second half
-                const int h = i / (4 * NM), f = i / NM & 3, al = i % NM;
-                const bool own = h == 0 || (f == 0 ? c_f[0] : f == 1 ? c_f[1] : f == 2 ? c_f[2] : c_f[3]);
-                return own ? d.fflux[k * (32 * NM) + ((cf * 4 + f) * 2 + h) * NM + al] : 0.0;
-            }, nslot, fd, es, lane, tm);
-        }
-        __syncwarp(tm);
-        // x-contraction: F and R, then Gx and Gy, minus the face fluxes
-#pragma unroll 1
-        for (int i = lane; i < 4 * ND; i += TL) {
-            const int q = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            const int cf = (0x2130 >> (4 * q)) & 15;
-            double v;
-            if (q < 2) {
-                const int2* s1 = sd + 2 * q * NE + b;
-                fx::Acc s;
-#pragma unroll
-                for (int al = 0; al < NV; ++al) {
-                    s.mac(tx.DvT[a][al], s1[al * ND1]);
-                    s.mac(tx.BvT[a][al], s1[NE + al * ND1]);
-                }
-                v = fx::to_double(s.get(), (q ? eR : eF) + tx.tBvT + tx.tDvT);
-            } else {
-                const float* s1 = sB + (q - 2) * NE + b;
-                float s = 0.0f;
-#pragma unroll
-                for (int al = 0; al < NV; ++al)
-                    s += tx.DvF[al][a] * s1[al * ND1] + tx.BvF[al][a] * s1[4 * NE + al * ND1];
-                v = f64_any(s);
-            }
-            const long long sf = face_lift<ND1, NM>(tx, fd + cf * 8 * NM, a, b, c_f);
-            rfield(d, stage, cf, ND)[k * ND + j] = v - fx::to_double(sf, es[cf] + tx.tBmT);
-        }
-#pragma unroll 1
-        for (int i = lane; i < 2 * ND; i += TL) { // Lx, Ly
-            const int cl = i / ND, j = i % ND, a = j % ND1, b = j / ND1;
-            float s = 0.0f;
-#pragma unroll
-            for (int al = 0; al < NV; ++al) s += tx.BvF[al][a] * sB[(2 + cl) * NE + al * ND1 + b];
-            rfield(d, stage, 4 + cl, ND)[k * ND + j] = f64_any(s);
-        }
-        __syncwarp(tm);
-    }
-}
-
 // every face point of the mesh once (the residual's face integrals, Sec. 3.2):
 // job j of d.fjobs is cell k = job >> 8 with face f, half h and GLL point al
 // packed as f | h << 2 | al << 3, k the lower cell index of the face (or the
@@ -1337,85 +885,6 @@ __global__ void __maxnreg__(72)
                                               : 1.0 / d.hxhy[2 * kc + (fc < 2 ? 0 : 1)];
                     v = fmax(v, lam * ih * sc);
                 }
-            }
-        }
-        if (want_dt) {
-            // one atomic per warp when its jobs share a member, else per job
-            const int m0 = __shfl_sync(0xffffffffu, mem, 0);
-            if (__all_sync(0xffffffffu, mem == m0 || mem < 0)) {
-                const double m = team_max_nonneg(v, 0xffffffffu); // v >= 0, never NaN
-                if (lane == 0 && m0 >= 0) atomic_max_pos(&d.mb[m0].rmax, m);
-            } else if (mem >= 0) {
-                atomic_max_pos(&d.mb[mem].rmax, v);
-            }
-        }
-    }
-}
-
-// the same for the FP32-bulk path, whose fluxes are FP32 (B)
-template <int R, typename Pix, int MODE, typename B>
-__global__ void __maxnreg__(80)
-    k_faces_bulk(const __grid_constant__ Dev d, int buf, double c_stage, int want_dt) {
-    __shared__ FaceTables tb;
-    copy_table(tb, &d.tabs->ft);
-    using S = Sz<R>;
-    constexpr int ND = S::ND, NM = S::NM, SL = 32 * NM;
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t n = d.n;
-    for (int64_t j0 = gw * 32; j0 < d.njobs; j0 += nw * 32) { // warp-uniform bounds
-        const int64_t j = j0 + lane;
-        double v = 0.0;
-        int mem = -1;
-        if (j < d.njobs) {
-            const int64_t job = d.fjobs[j];
-            const int64_t k = job >> 8;
-            const int f = (int)(job & 3), h = (int)((job >> 2) & 1), al = (int)((job >> 3) & 31);
-            const unsigned info = d.finfo ? d.finfo[k * 4 + f] : 0;
-            const bool coarse = (info & 3) == FI_COARSE;
-            const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1];
-            const double ihx = d.ihxhy ? d.ihxhy[2 * k] : 1.0 / hx;
-            const double ihy = d.ihxhy ? d.ihxhy[2 * k + 1] : 1.0 / hy;
-            mem = member_of(d, k);
-            const double t = (c_stage == 0.0) ? d.mb[mem].t : d.mb[mem].t + c_stage * get_dt(d, mem);
-            B raw[4], pres, lam, out[4];
-            bool own_first, bnd;
-            int64_t nb;
-            face_point<R, Pix, MODE, B>(d, tb, k, ufield(d, buf, 0, ND) + k * ND,
-                                        d.uF ? ufieldF(d, buf, 0, ND) + k * ND : nullptr, (size_t)n * ND,
-                                        d.cmask[(size_t)buf * n + k], buf, f, h, al, info, hx, hy,
-                                        mem, t, raw, pres, lam, own_first, bnd, nb);
-            if (bnd) {
-#pragma unroll
-                for (int cf = 0; cf < 4; ++cf) out[cf] = raw[cf];
-            } else {
-                side_flux<B>(raw, pres, own_first, f, out);
-            }
-            const double L = ((f < 2) ? hy : hx) * (coarse ? 0.5 : 1.0);
-            const double wl = L * tb.wm[al];
-            double* F = d.fflux + k * SL;
-#pragma unroll
-            for (int cf = 0; cf < 4; ++cf) F[((cf * 4 + f) * 2 + h) * NM + al] = wl * (double)out[cf];
-            v = fmax((double)lam, 1e-12) * ((f < 2) ? ihx : ihy) * (coarse ? 0.5 : 1.0);
-            if (!bnd && nb != k) {
-                // the other side: its face fo, its half (the fine side of a 2:1
-                // face has one) and its own weight
-                const int fo = f ^ 1;
-                const unsigned ninfo = d.finfo ? d.finfo[nb * 4 + fo] : 0;
-                const bool ncoarse = (ninfo & 3) == FI_COARSE;
-                const int hn = ((info & 3) == FI_FINE) ? (int)(info >> 2) : 0;
-                const double nhx = d.hxhy[2 * nb], nhy = d.hxhy[2 * nb + 1];
-                const double nihx = d.ihxhy ? d.ihxhy[2 * nb] : 1.0 / nhx;
-                const double nihy = d.ihxhy ? d.ihxhy[2 * nb + 1] : 1.0 / nhy;
-                side_flux<B>(raw, pres, !own_first, fo, out);
-                const double Ln = ((fo < 2) ? nhy : nhx) * (ncoarse ? 0.5 : 1.0);
-                const double wln = Ln * tb.wm[al];
-                double* Fn = d.fflux + nb * SL;
-#pragma unroll
-                for (int cf = 0; cf < 4; ++cf)
-                    Fn[((cf * 4 + fo) * 2 + hn) * NM + al] = wln * (double)out[cf];
-                v = fmax(v, fmax((double)lam, 1e-12) * ((fo < 2) ? nihx : nihy) * (ncoarse ? 0.5 : 1.0));
             }
         }
         if (want_dt) {
@@ -1597,7 +1066,7 @@ __device__ __noinline__ bool chol_solve(double* M, double* b, double* inv, int l
 // M_(a,b),(c,d) = sum_{al,be} c_{al,be} Bm[al][a] Bm[al][c] Bm[be][b] Bm[be][d],
 // the lower part packed by rows (rarely reached: not inlined)
 template <int ND1, int NM, int TL = 32>
-__device__ __noinline__ void assemble_mass(const Tables& tb, const double* cw, double* Y,
+__device__ __noinline__ void assemble_mass(const BaseTables& tb, const double* cw, double* Y,
                                               double* M, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = ND1 * ND1;
 #pragma unroll 1
@@ -1621,16 +1090,6 @@ __device__ __noinline__ void assemble_mass(const Tables& tb, const double* cw, d
         M[tri(r_, s_)] = s;
     }
     __syncwarp(tm);
-}
-
-// Index of element (i, t) of an FP32 factor stored by rows.  For a
-// power-of-two order the column is XOR-swizzled with i / 2, so that a team's
-// lanes reading one element of each row, or of each column, hit distinct
-// shared-memory banks; an odd order needs no swizzle.
-template <int ND>
-__device__ __forceinline__ int lrow_idx(int i, int t) {
-    if constexpr ((ND & (ND - 1)) == 0) return i * ND + (t ^ ((i >> 1) & (ND - 1)));
-    else return i * ND + t;
 }
 
 // FP32 inverse of H' = S B^T diag(cw') B S, one row per lane in a[] (ND <= TL):
@@ -1811,143 +1270,9 @@ __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& f
     return chol_solve<ND, TL>(M, b, inv, lane, tm);
 }
 
-// Tracer stage solve of the FP32-bulk path (Eq. algebraic_concentration,
-// H(zeta^(l)) C = b with the depth-weighted mass matrix H = B^T diag(cw) B):
-// C = c0 + delta, where c0 = sum_i b_i / sum_i s_i is the cell's mean
-// concentration (s = H 1, the row sums of H, i.e. H_i(zeta^(l)) of the
-// continuity equation, in FP64), delta = H^-1 (b - c0 s) is solved once in
-// FP32, and a constant correction makes
-// sum_i (H C)_i = sum_i s_i C_i equal sum_i b_i in FP64, so the tracer mass
-// is kept to FP64 round-off and a constant tracer (b = c s) stays constant up
-// to the rounding of b - c0 s.  A failed FP32 factor falls back to the FP64
-// Cholesky.  b: right-hand side in, C out (FP64).  Scratch: Mf [ND ND], Yf [ND1
-// ND1 NM] (float), digit pairs td [2 NMP], M, Y, inv (fallback).  known: the
-// Newton solve ended on its certificate (H is affine between the last two
-// iterates, so H(zeta^(l)) = T up to the rounding of the last update) and the
-// continuity target T stands for s = H 1 = H(zeta^(l)); otherwise s is
-// integrated from cw.
-//
-// The factor is a Cholesky with one row per lane in registers (lanes past the
-// last row repeat it).  Step J takes the pivot from lane J, and column J goes to
-// the other lanes through shared memory, shifted by J + 1; the row's columns
-// move down by one per step, so that the pivot column is always a[0] and one
-// loop body serves every step; entries above the diagonal or past the last
-// column are computed and never used.  The forward substitution goes along.
-// Unrolled with one shuffle per entry, this solve was 20 KB of code, which has
-// to share the 32 KB instruction cache with the rest of the stage update (a stage of
-// 65,536 cells, r = 3: 497 -> 468 us).
-template <int ND1, int NM, int TL>
-__device__ __noinline__ void solve_tracer_bulk(const Tables& tb, const FxStage& fs, const double* cw, double* b,
-                                  float* Mf, float* Yf, int2* td, double* M, double* Y, double* inv,
-                                  bool known, double T, int lane, unsigned tm) {
-    constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4;
-    static_assert(ND <= TL, "one row per lane");
-    static_assert(NMP <= ND * ND, "the weights are staged in Mf");
-    static_assert(2 * NDP + 2 <= ND1 * ND1 * NM, "the columns overlay Yf");
-    if (!known) { // s_i = (H 1)_i
-        unsigned m = 0;
-#pragma unroll 1
-        for (int p = lane; p < NMP; p += TL) m = max(m, fx::mag(cw[p]));
-        const int e = fx::block_exp(__reduce_max_sync(tm, m));
-#pragma unroll 1
-        for (int p = lane; p < NMP; p += TL) td[p] = fx::split(fx::from_double(cw[p], e));
-        __syncwarp(tm);
-        fx_tens<NM, ND1, TL>(fs.BmT, td, td + NMP, lane, tm, [&](int, int, long long X) {
-            T = fx::to_double(X, e + 2 * fs.tBmT);
-        });
-    }
-    const double bi = lane < ND ? b[lane] : 0.0, si = lane < ND ? T : 0.0;
-    double sb = bi, ss = si;
-    team_sum2<TL>(sb, ss, tm);
-    const double c0 = ss > 0.0 ? sb / ss : 0.0;
-    // the matrix, contracted over the points of a row, then over the rows
-#pragma unroll 1
-    for (int p = lane; p < NMP; p += TL) Mf[p] = f32_of(cw[p]);
-    __syncwarp(tm);
-#pragma unroll 1
-    for (int i = lane; i < ND1 * ND1 * NM; i += TL) {
-        const int a = i / (ND1 * NM), r_ = i % (ND1 * NM), c = r_ / NM, be = r_ % NM;
-        float s = 0.0f;
-#pragma unroll
-        for (int al = 0; al < NM; ++al) s += Mf[al + NM * be] * fs.BmF[al][a] * fs.BmF[al][c];
-        Yf[i] = s;
-    }
-    __syncwarp(tm);
-    const int i = lane < ND ? lane : ND - 1, ar = i % ND1, br = i / ND1;
-    float a[ND];
-#pragma unroll
-    for (int t = 0; t < ND; ++t) a[t] = 0.0f;
-#pragma unroll
-    for (int be = 0; be < NM; ++be) {
-        const float bb = fs.BmF[be][br];
-        float y[ND1];
-#pragma unroll
-        for (int c = 0; c < ND1; ++c) y[c] = Yf[(ar * ND1 + c) * NM + be] * bb;
-#pragma unroll
-        for (int t = 0; t < ND; ++t) a[t] += y[t % ND1] * fs.BmF[be][t / ND1];
-    }
-    float bv = f32_of(bi - c0 * si), rinv = 0.0f;
-    float* cb = (float*)(((size_t)Yf + 15) & ~(size_t)15); // two columns, in turn
-    bool ok = true;
-    __syncwarp(tm);
-#pragma unroll 1
-    for (int J = 0; J < ND; ++J) {
-        float* col = cb + (J & 1) * NDP;
-        const float djj = __shfl_sync(tm, a[0], J, TL); // the same on every lane of the team
-        ok = ok && djj > 0.0f;
-        const float r = 1.0f / sqrtf(djj);
-        const float yj = __shfl_sync(tm, bv * r, J, TL);
-        float lj = 0.0f;
-        if (i == J) {
-            rinv = r;
-            bv = yj;
-        } else if (i > J) {
-            lj = a[0] * r;
-            bv -= lj * yj;
-            col[i - J - 1] = lj;
-            Mf[lrow_idx<ND>(i, J)] = lj;
-        }
-        __syncwarp(tm);
-        float cl[NDP];
-        read_row<NDP>(col, cl);
-#pragma unroll
-        for (int l = 0; l < ND - 1; ++l) a[l] = a[l + 1] - lj * cl[l];
-    }
-    if (!ok) {
-        assemble_mass<ND1, NM, TL>(tb, cw, Y, M, lane, tm);
-        chol_solve<ND, TL>(M, b, inv, lane, tm);
-        return;
-    }
-#pragma unroll 1
-    for (int j = ND - 1; j >= 0; --j) { // L^T x = y
-        const float xj = __shfl_sync(tm, bv * rinv, j, TL);
-        if (i == j) bv = xj;
-        else if (i < j) bv -= Mf[lrow_idx<ND>(j, i)] * xj;
-    }
-    const double xi = lane < ND ? c0 + f64_any(bv) : 0.0;
-    const double m = team_sum<TL>(si * xi, tm);
-    const double alpha = ss > 0.0 ? (sb - m) / ss : 0.0;
-    __syncwarp(tm);
-    if (lane < ND) b[lane] = xi + alpha;
-    __syncwarp(tm);
-}
-
-__device__ __forceinline__ double bulk_of(double v, double) { return v; }
-__device__ __forceinline__ float bulk_of(double v, float) { return f32_of(v); }
-// a nodal value, FP32 ones from the FP32 copy of the state where there is one
-template <typename T, int ND>
-__device__ __forceinline__ T nodal(const Dev& d, int buf, int f, size_t idx) {
-    if constexpr (sizeof(T) == 4)
-        if (d.uF) return ufieldF(d, buf, f, ND)[idx];
-    return bulk_of(ufield(d, buf, f, ND)[idx], T());
-}
-__device__ __forceinline__ double exact_of(double v) { return v; }
-__device__ __forceinline__ double exact_of(float v) { return f64_any(v); }
-
 // T (N x N) along both directions of NF fields of N x N values, one node per
-// lane (N N <= team width): v[f] is the lane's value in and its result out.
-// FP64 values go through block fixed point (t: the table's exponent), FP32 ones
-// through FP32 sums.  w: 2 NF N N 8-byte words.
+// lane (N N <= team width), in block fixed point (t: the table's exponent): v[f] is
+// the lane's value in and its result out.  w: 2 NF N N 8-byte words.
 template <int N, int NF>
 __device__ __forceinline__ void square(const int2 (*T)[MXN], int t, double (&v)[NF], int2* w, int lane,
                                        unsigned tm) {
@@ -1979,36 +1304,6 @@ __device__ __forceinline__ void square(const int2 (*T)[MXN], int t, double (&v)[
     }
     __syncwarp(tm);
 }
-template <int N, int NF>
-__device__ __forceinline__ void square(const float (*T)[MXN], int, float (&v)[NF], int2* w, int lane,
-                                       unsigned tm) {
-    constexpr int NN = N * N;
-    const bool act = lane < NN;
-    const int i = act ? lane : NN - 1, r = i / N, c = i % N;
-    float* in = (float*)w;
-    float* tmp = in + NF * NN;
-    if (act) {
-#pragma unroll
-        for (int f = 0; f < NF; ++f) in[f * NN + i] = v[f];
-    }
-    __syncwarp(tm);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        float s = 0.0f;
-#pragma unroll
-        for (int a = 0; a < N; ++a) s += T[c][a] * in[f * NN + r * N + a];
-        if (act) tmp[f * NN + i] = s;
-    }
-    __syncwarp(tm);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        float s = 0.0f;
-#pragma unroll
-        for (int b = 0; b < N; ++b) s += T[r][b] * tmp[f * NN + b * N + c];
-        v[f] = s;
-    }
-    __syncwarp(tm);
-}
 // one or two fields, not inlined: the stage update calls them in five places, and
 // its hot code has to fit the instruction cache (32 KB)
 struct Two {
@@ -2035,33 +1330,6 @@ __device__ __forceinline__ void square2(const int2 (*T)[MXN], int t, double (&v)
     v[0] = r.a;
     v[1] = r.b;
 }
-struct TwoF {
-    float a, b;
-};
-template <int N>
-__device__ __noinline__ TwoF square_two(const float (*T)[MXN], float a, float b, int2* w, int lane,
-                                        unsigned tm) {
-    float v[2] = {a, b};
-    square<N, 2>(T, 0, v, w, lane, tm);
-    return {v[0], v[1]};
-}
-template <int N>
-__device__ __forceinline__ void square2(const float (*T)[MXN], int, float (&v)[2], int2* w, int lane,
-                                        unsigned tm) {
-    const TwoF r = square_two<N>(T, v[0], v[1], w, lane, tm);
-    v[0] = r.a;
-    v[1] = r.b;
-}
-// the stage tables of the value type
-__device__ __forceinline__ const int2 (*tab_Bg(const FxStage& s, double))[MXN] { return s.Bg; }
-__device__ __forceinline__ const float (*tab_Bg(const FxStage& s, float))[MXN] { return s.BgF; }
-__device__ __forceinline__ const int2 (*tab_BgT(const FxStage& s, double))[MXN] { return s.BgT; }
-__device__ __forceinline__ const float (*tab_BgT(const FxStage& s, float))[MXN] { return s.BgTF; }
-__device__ __forceinline__ const int2 (*tab_Gi(const FxStage& s, double))[MXN] { return s.Gi; }
-__device__ __forceinline__ const float (*tab_Gi(const FxStage& s, float))[MXN] { return s.GiF; }
-__device__ __forceinline__ const int2 (*tab_GiT(const FxStage& s, double))[MXN] { return s.GiT; }
-__device__ __forceinline__ const float (*tab_GiT(const FxStage& s, float))[MXN] { return s.GiTF; }
-
 // ---------------------------------------------------------------------------
 // step start: degree switch (Eq. criteria_p) with mass-exact remap, then
 // H_i(zeta^n), C~_i^n (Eqs. depth_rhs, concentration_rhs) and their sums
@@ -2180,10 +1448,7 @@ __global__ void __maxnreg__(64)
             }
             if (act) {
 #pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    ufield(d, 0, f, ND)[idx] = u[f];
-                    if (d.uF) ufieldF(d, 0, f, ND)[idx] = f32_of(u[f]);
-                }
+                for (int f = 0; f < 4; ++f) ufield(d, 0, f, ND)[idx] = u[f];
             }
             cm = 15u;
             const double z0 = __shfl_sync(tm, u[0], 0, TL), c0 = __shfl_sync(tm, u[3], 0, TL);
@@ -2253,26 +1518,20 @@ __global__ void __maxnreg__(64)
 // momentum's S^-T, S^-1 and point values, the tracer's residuals) is block
 // fixed-point on the integer pipe and a lane's nodal values stay in registers;
 // FP64 is left with the right-hand sides, the pointwise physics and the sums
-// that the mass balance needs.  B = float (FP32-bulk): the momentum's point
-// arithmetic and the tracer correction in FP32.
+// that the mass balance needs.
 template <int R>
 struct StageFx {
     using S = Sz<R>;
     static constexpr int TL = 16, PP = (S::NMP + TL - 1) / TL;
     // 8-byte words per team: digit pairs of nodal fields with scratch [6 ND] (the
     // fallback's Y), mass-point digits with the solve's scratch [2 NMP + NMP],
-    // weights [NMP], right-hand side [ND], then the FP32 solve's M and Y or the
+    // weights [NMP], right-hand side [ND], then the FP32 inverse's scratch or the
     // fallback's M
     static constexpr int W = 6 * S::ND, Q = 3 * S::NMP, CW = S::NMP, BV = S::ND;
-    static constexpr int F32 = (S::ND * S::ND + S::ND1 * S::ND1 * S::NM + 1) / 2;
-    // the fallback's matrix; the FP32 inverse's scratch; the FP32-bulk tracer's M, Y
     static constexpr int TRI = S::ND * (S::ND + 1) / 2;
     static constexpr int INV =
         (2 + 2 * ((S::ND + 3) / 4 * 4) + S::NMP + S::ND1 * (S::ND1 + 1) / 2 * S::NM + 1) / 2;
-    static constexpr int un(bool bulk) {
-        return bulk && F32 > TRI && F32 > INV ? F32 : TRI > INV ? TRI : INV;
-    }
-    static constexpr int words(bool bulk) { return W + Q + CW + BV + un(bulk); }
+    static constexpr int words = W + Q + CW + BV + (TRI > INV ? TRI : INV);
     static_assert(S::ND <= TL && S::NGP == S::ND, "one node and one momentum point per lane");
     static_assert(S::ND1 * S::ND1 * S::NM <= W, "fallback Y");
 };
@@ -2280,30 +1539,44 @@ struct StageFx {
 // the friction coefficient of v^(l-1) at the lane's momentum point (a constant
 // field: its value).  w: the scratch of square.  Not inlined: both paths of the
 // stage update call it.
-template <int R, typename Pix, int MODE, typename T>
-__device__ __noinline__ T stage_gamma(const Dev& d, const FxStage& fs, int buf, int64_t k, T man, int2* w,
-                                      int lane, unsigned tm) {
+template <int R, typename Pix, int MODE>
+__device__ __noinline__ double stage_gamma(const Dev& d, const FxStage& fs, int buf, int64_t k, double man,
+                                           int2* w, int lane, unsigned tm) {
     using S = Sz<R>;
     constexpr int ND1 = S::ND1, ND = S::ND, NG = S::NG;
     const bool act = lane < ND;
     const size_t idx = (size_t)k * ND + (act ? lane : 0);
     const unsigned cmp = d.cmask[(size_t)buf * d.n + k];
-    const T q0 = nodal<T, ND>(d, buf, 1, idx), q1 = nodal<T, ND>(d, buf, 2, idx);
+    const double q0 = ufield(d, buf, 1, ND)[idx], q1 = ufield(d, buf, 2, ND)[idx];
     double z = ufield(d, buf, 0, ND)[idx], V, A;
-    T q[2] = {q0, q1}, gam = T(0);
+    double q[2] = {q0, q1}, gam = 0.0;
     if (!(cmp & 1u)) z = square_one<ND1>(fs.Bg, fs.tBg, z, w, lane, tm);
-    if ((cmp & 6u) != 6u) square2<ND1>(tab_Bg(fs, T()), fs.tBg, q, w, lane, tm);
+    if ((cmp & 6u) != 6u) square2<ND1>(fs.Bg, fs.tBg, q, w, lane, tm);
     if (cmp & 2u) q[0] = q0;
     if (cmp & 4u) q[1] = q1;
     if (act) {
         Site<R, Pix, MODE>::VA(d, *d.tabs, k, SET_MOM, lane % NG, lane / NG, z, V, A);
-        gam = gamma_manning<T>(man, bulk_of(V, T()), q[0], q[1], bulk_of(d.g, T()), bulk_of(d.eps, T()));
+        gam = gamma_manning<double>(man, V, q[0], q[1], d.g, d.eps);
     }
     return gam;
 }
 
+// Position v of a launch -> group of cells: from both ends of the mesh inwards,
+// STAGE_RUN groups from the end, then as many from the start, and so on: the cells
+// that take several times as long (pixel sums, Newton steps) lie at the shore, and
+// shores lie at the edge of a domain rather than in its middle, so the launch does
+// not end on them, at whichever end they are.  A run is about what the chip holds
+// at once: neighbours run at the same time, do much the same and share the
+// instruction cache.  Measured, a stage of the lagoon (r = 2, 44,000 cells, the
+// shore last): 405 us in the mesh's order, 320 so; groups from the two ends in turn
+// 331, 61 stretches of the mesh interleaved 394.
 constexpr unsigned STAGE_RUN = 1024;
-template <int R, typename Pix, int MODE, typename B>
+__device__ __forceinline__ unsigned from_both_ends(unsigned v, unsigned ng) {
+    const unsigned i = v / (2 * STAGE_RUN) * STAGE_RUN + v % STAGE_RUN;
+    return v / STAGE_RUN & 1 ? i : ng - 1 - i;
+}
+
+template <int R, typename Pix, int MODE>
 __global__ void __maxnreg__(72)
     k_stage(const __grid_constant__ Dev d, const __grid_constant__ StageArgs sa) {
     using S = Sz<R>;
@@ -2311,21 +1584,19 @@ __global__ void __maxnreg__(72)
     using ST = Site<R, Pix, MODE>;
     constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
     constexpr int TL = L::TL, PP = L::PP;
-    constexpr bool F64 = sizeof(B) == sizeof(double);
     __shared__ FxStage fs;
     copy_table(fs, &d.tabs->fs);
     const Tables& tb = *d.tabs;
     extern __shared__ double smem[];
     const int team = threadIdx.x / TL, lane = threadIdx.x % TL, tpb = blockDim.x / TL;
     const unsigned tm = 0xFFFFu << (threadIdx.x & 16); // the team's lanes
-    int2* w = (int2*)(smem + team * L::words(!F64)); // digit pairs of nodal fields, and scratch
+    int2* w = (int2*)(smem + team * L::words); // digit pairs of nodal fields, and scratch
     int2* qd = w + L::W;                       // [NMP] mass-point digits, then scratch [2 NMP]
     int2* qt = qd + NMP;
     double* cw = (double*)(qd + L::Q); // [NMP] weights of a mass-matrix solve
     double* bv = cw + L::CW;           // [ND] its right-hand side and solution
     double* un = bv + L::BV;
-    float* Mf = (float*)un;            // [ND ND] (FP32-bulk tracer), or the FP32 inverse's scratch
-    float* Yf = Mf + ND * ND;          // [ND1 ND1 NM]
+    float* Mf = (float*)un;            // the FP32 inverse's scratch
     double* M = un;                    // the fallback's matrix, packed
     const int64_t n = d.n;
     const bool act = lane < ND;
@@ -2342,20 +1613,10 @@ __global__ void __maxnreg__(72)
     }
     const float tolf = (float)d.newton_tol;
 
-#pragma unroll 1
-    // Groups of tpb cells from both ends of the mesh inwards, STAGE_RUN groups from the
-    // end, then as many from the start, and so on: the cells that take several times
-    // as long (pixel sums, Newton steps) lie at the shore, and shores lie at the
-    // edge of a domain rather than in its middle, so the launch does not end on them,
-    // at whichever end they are.  A run is about what the chip holds at once:
-    // neighbours run at the same time, do much the same and share the instruction
-    // cache.  Measured, a stage of the lagoon (r = 2, 44,000 cells, the shore last):
-    // 405 us in the mesh's order, 320 so; groups from the two ends in turn 331,
-    // 61 stretches of the mesh interleaved 394.
     const unsigned ng = (unsigned)((n + tpb - 1) / tpb);
+#pragma unroll 1
     for (unsigned v = blockIdx.x; v < ng; v += gridDim.x) {
-        const unsigned i = v / (2 * STAGE_RUN) * STAGE_RUN + v % STAGE_RUN;
-        const int64_t k = (int64_t)(v / STAGE_RUN & 1 ? i : ng - 1 - i) * tpb + team;
+        const int64_t k = (int64_t)from_both_ends(v, ng) * tpb + team;
         if (k >= n) continue;
         const size_t idx = (size_t)k * ND + node;
         const unsigned cm0 = d.cmask[k];
@@ -2390,7 +1651,6 @@ __global__ void __maxnreg__(72)
         if (Tbar < 0.0) viol++;
         bool scalar = (flag == 0);
         int its = 0;
-        bool cert = false; // the Newton solve ended on its one-step certificate
         double z = u0;     // Newton iterate
         double V[PP], A[PP];
         // elevations at the lane's mass points of the nodal values v (cst: a constant field)
@@ -2441,10 +1701,7 @@ __global__ void __maxnreg__(72)
                     // on the segment between them and M(previous) is its exact
                     // Jacobian, so this iterate solves H = T (the fully wet case of
                     // Sec. 3.4); no verification step is needed
-                    if (kk > 0 && prev_full && npart == 0) {
-                        cert = true;
-                        break;
-                    }
+                    if (kk > 0 && prev_full && npart == 0) break;
                     if (kk == d.newton_max) break;
                     // H_i(zeta_k)
                     double hv[PP];
@@ -2512,22 +1769,27 @@ __global__ void __maxnreg__(72)
         // v^(l-1) at the lane's momentum point (a constant field: its value), the
         // discharges in T; then the friction coefficient there
         const bool need_gam = (sa.add != 0.0 || sa.make_llin) && !zero_bits(man);
-        auto gamma_prev = [&](auto manT) {
-            return stage_gamma<R, Pix, MODE, decltype(manT)>(d, fs, sa.prev_buf, k, manT, w, lane, tm);
-        };
         // v^n's discharges at the momentum point, interpolated
-        auto q_points = [&](auto& v) {
-            using T = std::remove_reference_t<decltype(v[0])>;
-            const T q0 = nodal<T, ND>(d, 0, 1, idx), q1 = nodal<T, ND>(d, 0, 2, idx);
+        auto q_points = [&](double (&v)[2]) {
+            const double q0 = ufield(d, 0, 1, ND)[idx], q1 = ufield(d, 0, 2, ND)[idx];
             v[0] = q0;
             v[1] = q1;
-            if ((cm0 & 6u) != 6u) square2<ND1>(tab_Bg(fs, T()), fs.tBg, v, w, lane, tm);
+            if ((cm0 & 6u) != 6u) square2<ND1>(fs.Bg, fs.tBg, v, w, lane, tm);
             if (cm0 & 2u) v[0] = q0;
             if (cm0 & 4u) v[1] = q1;
         };
         double oz, oq[2], oc, ll[2];
+        const double gam =
+            need_gam ? stage_gamma<R, Pix, MODE>(d, fs, sa.prev_buf, k, man, w, lane, tm) : 0.0;
+        double qn[2]; // q^n at the point, from the step start
+        if (d.qpts) {
+            qn[0] = d.qpts[k * 2 * NGP + node];
+            qn[1] = d.qpts[k * 2 * NGP + NGP + node];
+        } else {
+            q_points(qn);
+        }
+        const double wp = J * w2;
         if (scalar) {
-            const double gam = need_gam ? gamma_prev(man) : 0.0;
             double e;
             if (cm0 & 1u) e = u0;
             else {
@@ -2540,14 +1802,6 @@ __global__ void __maxnreg__(72)
             }
             its = scalar_newton<R, Pix, MODE, TL>(d, tb, k, J, Tbar, e, lane, tm);
             // momentum: sums of the rows of the friction-modified mass matrix
-            double qn[2];
-            if (d.qpts) {
-                qn[0] = d.qpts[k * 2 * NGP + node];
-                qn[1] = d.qpts[k * 2 * NGP + NGP + node];
-            } else {
-                q_points(qn);
-            }
-            const double wp = J * w2;
             double den = 0.0, num[2] = {0.0, 0.0}, rs0 = 0.0, rs1 = 0.0, rcs = 0.0;
             if (act) {
                 den = wp * (1.0 + sa.add * dt * gam);
@@ -2576,47 +1830,29 @@ __global__ void __maxnreg__(72)
             // points, inverted as S^-1 D^-1 S^-T): S Q = [D0 q^n + S^-T rq] / D,
             // D = D0 (1 + add dt gamma), D0 = J w, gamma from the previous stage;
             // optionally the linearised friction term Llin = -S^T (J w gamma S Q)
-            const B JB = bulk_of(J, B()), manB = bulk_of(man, B()), adtB = bulk_of(sa.add * dt, B());
-            const B gam = need_gam ? gamma_prev(manB) : B(0);
-            B qn[2];
-            if (F64 && d.qpts) { // q^n at the points, from the step start
-                qn[0] = (B)d.qpts[k * 2 * NGP + node];
-                qn[1] = (B)d.qpts[k * 2 * NGP + NGP + node];
-            } else {
-                q_points(qn);
-            }
-            B s[2] = {bulk_of(rq[0], B()), bulk_of(rq[1], B())};
-            square2<ND1>(tab_GiT(fs, B()), fs.tGiT, s, w, lane, tm);
-            B wp;
-            if constexpr (F64) wp = J * w2;
-            else wp = JB * fs.wgF[node % NG] * fs.wgF[node / NG];
-            const B rD = B(1) / (wp * (B(1) + adtB * gam));
+            double s[2] = {rq[0], rq[1]};
+            square2<ND1>(fs.GiT, fs.tGiT, s, w, lane, tm);
+            const double rD = 1.0 / (wp * (1.0 + sa.add * dt * gam));
             s[0] = (wp * qn[0] + s[0]) * rD;
             s[1] = (wp * qn[1] + s[1]) * rD;
-            B Q[2] = {s[0], s[1]};
-            square2<ND1>(tab_Gi(fs, B()), fs.tGi, Q, w, lane, tm);
+            oq[0] = s[0];
+            oq[1] = s[1];
+            square2<ND1>(fs.Gi, fs.tGi, oq, w, lane, tm);
             if (sa.make_llin) {
-                const B wl = wp * gam;
-                B l[2] = {-wl * s[0], -wl * s[1]};
-                square2<ND1>(tab_BgT(fs, B()), fs.tBgT, l, w, lane, tm);
-                ll[0] = exact_of(l[0]);
-                ll[1] = exact_of(l[1]);
+                const double wl = wp * gam;
+                ll[0] = -wl * s[0];
+                ll[1] = -wl * s[1];
+                square2<ND1>(fs.BgT, fs.tBgT, ll, w, lane, tm);
             }
             oz = z;
-            oq[0] = exact_of(Q[0]);
-            oq[1] = exact_of(Q[1]);
             // tracer: H(zeta^(l)) C = C~ + dt sum a R with the depth-weighted mass matrix
             if (act) bv[lane] = rc;
 #pragma unroll
             for (int j = 0; j < PP; ++j)
                 if (lane + j * TL < NMP) cw[lane + j * TL] = J * wm2[j] * V[j];
             __syncwarp(tm);
-            if constexpr (F64)
-                solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, w, qd, qt, M, (double*)w, (double*)qd,
-                                              lane, tm);
-            else
-                solve_tracer_bulk<ND1, NM, TL>(tb, fs, cw, bv, Mf, Yf, qt, M, (double*)w,
-                                               (double*)qd, cert, T, lane, tm);
+            solve_mass_mixed<ND1, NM, TL>(tb, fs, cw, bv, Mf, w, qd, qt, M, (double*)w, (double*)qd, lane,
+                                          tm);
             oc = bv[node];
             __syncwarp(tm);
         }
@@ -2633,10 +1869,7 @@ __global__ void __maxnreg__(72)
             const double v0 = __shfl_sync(tm, ov[f], 0, TL);
             if (__all_sync(tm, !act || same_bits(ov[f], v0))) cmo |= 1u << f;
             fin = fin && finite_bits(ov[f]);
-            if (act) {
-                ufield(d, sa.out_buf, f, ND)[idx] = ov[f];
-                if (d.uF) ufieldF(d, sa.out_buf, f, ND)[idx] = f32_of(ov[f]);
-            }
+            if (act) ufield(d, sa.out_buf, f, ND)[idx] = ov[f];
         }
         if (!__all_sync(tm, fin || !act)) bad = 1;
         if (lane == 0) d.cmask[(size_t)sa.out_buf * n + k] = (uint8_t)cmo;
@@ -2710,7 +1943,7 @@ __global__ void __launch_bounds__(32 * MAXWPB)
             const double e = (cm & 1u) ? su[0] : pe[p];
             const double c = (cm & 8u) ? su[ND] : pc[p];
             double V, A;
-            Site<R, Pix, MODE>::VA(d, tb, k, SET_MASS, p % NM, p / NM, e, V, A);
+            Site<R, Pix, MODE, false>::VA(d, tb, k, SET_MASS, p % NM, p / NM, e, V, A);
             const double w = J * tb.wm[p % NM] * tb.wm[p / NM];
             m += w * V;
             tm += w * V * c;
