@@ -293,7 +293,7 @@ static int fx_tables(const double* T, int m, int no, int ni, int ld, int2* out, 
     return t;
 }
 
-static void build_fx_tables(int R, Tables& tb) {
+static bool build_fx_tables(int R, Tables& tb) {
     const int n1 = R + 1, nv = (3 * R) / 2 + 1, nm = R + 2;
     FxTables& x = tb.fx;
     double B[MXP * MXN], D[MXP * MXN], WB[MXP * MXN], WD[MXP * MXN], F[3 * MXP * MXN];
@@ -309,6 +309,11 @@ static void build_fx_tables(int R, Tables& tb) {
     x.tWB = fx_tables(WB, 1, n1, nv, MXP, &x.WB[0][0], 0);
     x.tWD = fx_tables(WD, 1, n1, nv, MXP, &x.WD[0][0], 0);
     fx_tables(WB, 1, n1, nv, MXP, &x.WDB[0][0], 0, x.tWD);
+    for (int a = 0; a < n1; ++a) { // sums of both tables at once: |X| <= 1.75 2^FB < 2^60.9 (r = 1: 1.5)
+        double s = 0.0;
+        for (int q = 0; q < nv; ++q) s += std::fabs(WB[a * nv + q]) + std::fabs(WD[a * nv + q]);
+        if (s > std::ldexp(1.75, x.tWD)) return false;
+    }
     for (int m = 0; m < 3; ++m)
         for (int a = 0; a < n1; ++a)
             for (int q = 0; q < nm; ++q)
@@ -349,6 +354,7 @@ static void build_fx_tables(int R, Tables& tb) {
     memcpy(tb.ft.wm, tb.wm, sizeof tb.wm);
     memcpy(tb.ft.BmF, tb.BmF, sizeof tb.BmF);
     memcpy(tb.ft.BmHF, tb.BmHF, sizeof tb.BmHF);
+    return true;
 }
 
 static bool build_tables(int R, Tables& tb) {
@@ -412,8 +418,7 @@ static bool build_tables(int R, Tables& tb) {
         tb.wvF[q] = (float)tb.wv[q];
         tb.wgF[q] = (float)tb.wg[q];
     }
-    build_fx_tables(R, tb);
-    return true;
+    return build_fx_tables(R, tb);
 }
 
 // overlap tables of the four point sets for P pixels per cell side

@@ -13,8 +13,9 @@
 // |value| < 2^(eb - 1022)).  X = hi 2^LB + lo with lo in [-2^(LB-1), 2^(LB-1)):
 // the digit pair that the multiply-adds take.  Tables are held the same way,
 // T = Tint 2^(tb - FB), where 2^tb bounds every row's sum of |T|, so a
-// contraction of |X| <= 2^FB gives |X| <= 2^FB again, with exponent eb + tb:
-// nothing overflows and no step renormalises.
+// contraction of |X| <= 2^FB gives |X| <= 2^FB again, with exponent eb + tb.
+// A block far below its bound may be moved up within it (headroom).  What is split
+// or multiplied is below 2^60.9 (the digit pair wraps from 2^61 - 2^29 on).
 //
 // Rounding: a conversion rounds at 2^-60 of the block's largest value, a
 // contraction leaves out lo lo (at most a quarter of a unit of 2^-60 per term)
@@ -25,8 +26,9 @@
 // accuracy of a value far below the largest of its block, which the FP64 sum
 // of the block does not have either.
 //
-// Room: the sums hold up to 13 terms of tables whose rows together are bounded
-// by two row bounds (hi Tlo and lo Thi are below 2^59 each).
+// Room: the sums hold up to 13 terms (hi Tlo and lo Thi are below 2^59 each).  Two
+// sums of the residual take a second table at the first one's scale: |X| <= 1.75
+// 2^FB there, which the joint rows are checked for where the tables are built.
 //
 // A block that holds an infinity or a NaN takes the exponent POISON; every
 // value converted back from it is NaN.  Blocks below 2^-958 keep the exponent of
@@ -158,6 +160,12 @@ __host__ __device__ __forceinline__ double to_double(long long X, int eb) {
     if ((unsigned)(eb - 128) >= 1792u) return out_of_range(X, eb);
     const unsigned long long b = dbits((double)X);
     return bitsd(X == 0 ? 0ull : b + ((unsigned long long)(long long)(eb - (FB + 1022)) << 52));
+}
+// how far a block moves up, m = the largest high word of its |X|, for |X| < 2^FB
+// (|X| = 2^FB itself stays)
+__host__ __device__ __forceinline__ int headroom(unsigned m) {
+    const int s = clz64((unsigned long long)m << 32 | 0xffffffffu) - (64 - FB);
+    return s < 0 ? 0 : s;
 }
 // high word of |X|
 __host__ __device__ __forceinline__ unsigned high(long long X) {

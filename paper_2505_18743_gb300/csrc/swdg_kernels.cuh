@@ -639,7 +639,7 @@ __global__ void __maxnreg__(64)
                 // the gradient is far below the bound its table allows: its block moves
                 // up to the places that are free
                 const unsigned m = __reduce_max_sync(tm, pt ? max(fx::high(ZX), fx::high(ZY)) : 0u);
-                const int s = fx::clz64((unsigned long long)m << 32 | 0xffffffffu) - (63 - fx::FB);
+                const int s = fx::headroom(m);
                 ZX <<= s;
                 ZY <<= s;
                 eD -= s;
