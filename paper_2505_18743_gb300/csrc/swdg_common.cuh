@@ -476,78 +476,12 @@ __device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& f
 }
 
 // sub-grid wet depth V and wet area A of sub-cell (ia, ib) of point sets setx,
-// sety (mode S): V = sum_k w_k max(eta + z_k, 0), A = sum_k w_k [eta + z_k > 0].
-// The pixels are summed as integers (swdg_fixed.cuh): in FP64 a pixel costs five
-// instructions of the FP64 pipe (80 clocks per warp), here about 15 of the
-// integer pipe, and the weights enter once per row, since w_k = fy fx with fx
-// equal for all but the first and last pixel of a row.  The block exponent is
-// that of eta and the cell's largest depth (zmag: its high word; 0: found
-// here), with six bits of room for a row's sum: 2^-54 of the larger of the two,
-// half the last place of eta + z.  Not inlined: most cells never get here, and
-// the callers' code stays small.
+// sety (mode S): V = sum_k w_k max(eta + z_k, 0), A = sum_k w_k [eta + z_k > 0]
 struct SubV {
     double V, A;
     bool full;
 };
-__device__ __forceinline__ long long fx_pixel(float z, int e) { return fx::from_float(z, e); }
-__device__ __forceinline__ long long fx_pixel(double z, int e) { return fx::from_double(z, e); }
-template <typename Pix>
-__device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab* __restrict__ ov,
-                                       int setx, int ia, int sety, int ib, double eta, unsigned zmag) {
-    const int P = ov->P;
-    const int lox = ov->lo[setx][ia], cx = ov->cnt[setx][ia];
-    const int loy = ov->lo[sety][ib], cy = ov->cnt[sety][ib];
-    if (fx::mag(eta) >= 0x7ff00000u) { // an infinity or a NaN reads as entirely wet or dry
-        const bool wet = eta > 0.0;
-        return {wet ? eta : 0.0, wet ? 1.0 : 0.0, wet};
-    }
-    if (zmag == 0) {
-#pragma unroll 1
-        for (int j = 0; j < cy; ++j)
-#pragma unroll 1
-            for (int i = 0; i < cx; ++i)
-                zmag = max(zmag, fx::mag((double)tile[(loy + j) * P + lox + i]));
-    }
-    const int es = fx::block_exp(max(zmag, fx::mag(eta))) + 6;
-    const long long E = fx::from_double(eta, es);
-    fx::Acc v, a;
-    int wet = 0;
-#pragma unroll 1
-    for (int j = 0; j < cy; ++j) {
-        const Pix* row = tile + (loy + j) * P + lox;
-        // the row's sum, its first and its last pixel (0 where it has only one)
-        const long long D0 = E + fx_pixel(row[0], es);
-        const int cf = D0 > 0;
-        const long long first = cf ? D0 : 0;
-        long long T = first, last = 0;
-        int c = cf, cl = 0;
-#pragma unroll 2
-        for (int i = 1; i < cx; ++i) {
-            const long long D = E + fx_pixel(row[i], es);
-            cl = D > 0;
-            last = cl ? D : 0;
-            T += last;
-            c += cl;
-        }
-        wet += c;
-        const int2 f0 = ov->ed[setx][ia][0], f1 = ov->ed[setx][ia][1], f2 = ov->ed[setx][ia][2];
-        const int2 fy = ov->ed[sety][ib][j == 0 ? 0 : j == cy - 1 ? 2 : 1];
-        fx::Acc r, q;
-        r.mac(f0, fx::split(first));
-        r.mac(f1, fx::split(T - first - last));
-        r.mac(f2, fx::split(last));
-        v.mac(fy, fx::split(r.get()));
-        constexpr long long ONE = 1ll << (fx::FB - 6); // a count of one, at exponent 1028
-        q.mac(f0, fx::split(cf * ONE));
-        q.mac(f1, fx::split((c - cf - cl) * ONE));
-        q.mac(f2, fx::split(cl * ONE));
-        a.mac(fy, fx::split(q.get()));
-    }
-    const bool full = wet == cx * cy;
-    return {fx::to_double(v.get(), es), full ? 1.0 : wet ? fx::to_double(a.get(), 1028) : 0.0, full};
-}
-
-// the same sums in FP64
+// in FP64
 template <typename Pix>
 __device__ __forceinline__ SubV subgrid_f64(const Pix* __restrict__ tile, const OvTab& ov, int setx,
                                             int ia, int sety, int ib, double eta) {
@@ -574,6 +508,131 @@ __device__ __forceinline__ SubV subgrid_f64(const Pix* __restrict__ tile, const 
         a += fy * ar;
     }
     return {v, a, f};
+}
+
+// a pixel is wet (eta + z > 0, that is z > -eta) exactly: against the largest FP32
+// value up to -eta, or by order-preserving keys; a NaN pixel is dry
+struct WetF {
+    float t;
+    __device__ __forceinline__ WetF(double eta) { t = __double2float_rd(-eta); }
+    __device__ __forceinline__ bool operator()(float z) const { return z > t; }
+};
+struct WetD {
+    unsigned long long t, span; // wet: the key is in (-eta, inf], as one comparison
+    __device__ __forceinline__ WetD(double eta) {
+        t = (unsigned long long)nkey_neg(eta) + 1;
+        span = 0x7ff0000000000001ull - t;
+    }
+    __device__ __forceinline__ bool operator()(double z) const {
+        return (unsigned long long)okey(z) - t < span;
+    }
+};
+template <typename Pix>
+using Wet = std::conditional_t<std::is_same<Pix, float>::value, WetF, WetD>;
+// the larger of two depths (a NaN z: m), and a bound of one in FP32
+__device__ __forceinline__ float deeper(float m, float z) { return z > m ? z : m; }
+__device__ __forceinline__ double deeper(double m, double z) { return okey(z) > okey(m) && !nan_bits(z) ? z : m; }
+__device__ __forceinline__ float bound_f(float z) { return z; }
+__device__ __forceinline__ float bound_f(double z) { return __double2float_ru(z); }
+template <typename Pix>
+__device__ __noinline__ Pix deepest(const Pix* __restrict__ t, int P, int cx, int cy) {
+    Pix m = (Pix)-INFINITY;
+#pragma unroll 1
+    for (int j = 0; j < cy; ++j, t += P)
+#pragma unroll 1
+        for (int i = 0; i < cx; ++i) m = deeper(m, t[i]);
+    return m;
+}
+// a sub-cell with depths past FP32's range (rare: not inlined)
+template <typename Pix>
+__device__ __noinline__ SubV subgrid_inf(const Pix* __restrict__ tile, const OvTab* __restrict__ ov, int setx,
+                                         int ia, int sety, int ib, double eta) {
+    return subgrid_f64<Pix>(tile, *ov, setx, ia, sety, ib, eta);
+}
+__device__ __forceinline__ long long fx_pixel(float z, int e) { return fx::from_float(z, e); }
+__device__ __forceinline__ long long fx_pixel(double z, int e) { return fx::from_double(z, e); }
+
+// The same with the pixels summed as integers (swdg_fixed.cuh): in FP64 a pixel costs
+// five instructions of the FP64 pipe (80 clocks per warp), here about 15 of the
+// integer pipe, and the weights enter once per row, since w_k = fy fx with fx
+// equal for all but the first and last pixel of a row.
+// zhi is a bound of the sub-cell's pixel depths (NaN: found here).  A wet pixel lies
+// between -eta and zhi, so the block exponent is that of the larger of the two, and
+// dry pixels, however high, have no part in it.  With room for the sum of a row
+// (cx <= 2^lg pixels), eta and the wet pixels keep 2^-(58 - lg) of it: exactly what
+// they are where eta + z cancels, and below the rounding of eta + z where it does
+// not.  The rows' sums are then moved up to the bound eta + zhi of a pixel's depth, so
+// that a film of water at a great height, or beside a deep cell, has its own
+// relative accuracy (59 places of cx times that bound).  Not inlined: most cells never
+// get here, and the callers' code stays small.
+template <typename Pix>
+__device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab* __restrict__ ov,
+                                       int setx, int ia, int sety, int ib, double eta, float zhi) {
+    const int P = ov->P;
+    const int lox = ov->lo[setx][ia], cx = ov->cnt[setx][ia];
+    const int loy = ov->lo[sety][ib], cy = ov->cnt[sety][ib];
+    if (fx::mag(eta) >= 0x7ff00000u) { // an infinity or a NaN reads as entirely wet or dry
+        const bool wet = eta > 0.0;
+        return {wet ? eta : 0.0, wet ? 1.0 : 0.0, wet};
+    }
+    const Wet<Pix> is_wet(eta);
+    const int lg = 32 - __clz(cx - 1); // ceil(log2(cx))
+    int es;
+    long long E, D1;
+    // the block of a bound, and the bound of a pixel's depth in it
+    auto block = [&]() {
+        es = max(fx::block_exp(fx::mag(eta)), fx::block_exp_f(__float_as_uint(zhi) & 0x7fffffffu)) + lg + 2;
+        E = fx::from_double(eta, es);
+        D1 = E + fx::from_float(zhi, es);
+    };
+    const bool given = zhi == zhi;
+    if (given) block();
+    // no bound, or (FP64 pixels) one that its rounding to FP32 may leave far above the depths
+    if (!given || (sizeof(Pix) == sizeof(double) && D1 < 1ll << 36)) {
+        const Pix m = deepest<Pix>(tile + loy * P + lox, P, cx, cy);
+        if (!is_wet(m)) return {0.0, 0.0, false};
+        zhi = bound_f(m);
+        block();
+        if (sizeof(Pix) == sizeof(double)) D1 = E + fx_pixel(m, es);
+    }
+    if (fx::fbits(zhi) == 0x7f800000u) return subgrid_inf<Pix>(tile, ov, setx, ia, sety, ib, eta);
+    const int up = D1 > 0 ? fx::clz64((unsigned long long)D1) - (64 - fx::FB) - lg : 0;
+    fx::Acc v, a;
+    int wet = 0;
+#pragma unroll 1
+    for (int j = 0; j < cy; ++j) {
+        const Pix* row = tile + (loy + j) * P + lox;
+        // the row's sum, its first and its last pixel (0 where it has only one)
+        // (a dry pixel's integer means nothing; it is selected out, without a branch)
+        const long long D0 = E + fx_pixel(row[0], es);
+        const int cf = is_wet(row[0]);
+        const long long first = cf ? D0 : 0;
+        long long T = first, last = 0;
+        int c = cf, cl = 0;
+#pragma unroll 2
+        for (int i = 1; i < cx; ++i) {
+            const Pix z = row[i];
+            const long long D = E + fx_pixel(z, es);
+            cl = is_wet(z);
+            last = cl ? D : 0;
+            T += last;
+            c += cl;
+        }
+        wet += c;
+        const int2 f0 = ov->ed[setx][ia][0], f1 = ov->ed[setx][ia][1], f2 = ov->ed[setx][ia][2];
+        const int2 fy = ov->ed[sety][ib][j == 0 ? 0 : j == cy - 1 ? 2 : 1];
+        fx::Acc r;
+        r.mac(f0, fx::split(first << up));
+        r.mac(f1, fx::split((T - first - last) << up));
+        r.mac(f2, fx::split(last << up));
+        v.mac(fy, fx::split(r.get()));
+        // the row's wet width, exactly (at most 1)
+        a.mac(fy, fx::split((cf ? fx::join(f0) : 0) + (cl ? fx::join(f2) : 0) + (c - cf - cl) * fx::join(f1)));
+    }
+    const bool full = wet == cx * cy;
+    const long long X = v.get(); // a wet pixel of less than a place may have rounded below 0
+    return {fx::to_double(X > 0 ? X : 0, es - up),
+            full ? 1.0 : wet ? fx::to_double(a.get(), 1022) : 0.0, full};
 }
 
 __device__ __forceinline__ void subgrid_P(double z, double eta, double& V, double& A) {

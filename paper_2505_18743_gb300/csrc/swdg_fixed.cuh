@@ -22,9 +22,11 @@
 // and rounds the table to 2^-61 of its row bound: together about a unit of
 // 2^-60 of the bound of the result, against 2^-53 of each partial sum in FP64
 // arithmetic (the row bounds of two or four contractions in a row exceed the
-// values by a few bits, so the room is used).  What this gives up is relative
-// accuracy of a value far below the largest of its block, which the FP64 sum
-// of the block does not have either.
+// values by a few bits, so the room is used).  What this gives up is the relative
+// accuracy of a value far below the largest of its block: no loss in a sum that
+// the large value is part of, but one in a sum that leaves it out.  So a block
+// holds only values that meet in the same sums (the pixels' land, which no sum
+// takes, is kept out of theirs).
 //
 // Room: the sums hold up to 13 terms (hi Tlo and lo Thi are below 2^59 each).  Two
 // sums of the residual take a second table at the first one's scale: |X| <= 1.75
@@ -189,8 +191,8 @@ __host__ __device__ __forceinline__ int block_exp_f(unsigned maxbits) {
 __host__ __device__ __forceinline__ long long from_float(float v, int eb) {
     const unsigned b = fbits(v);
     const int ef = (int)(b >> 23) & 0xff;
-    int d = eb - (ef + 896);
-    d = ef == 0 ? 63 : (d < 63 ? d : 63);
+    unsigned d = (unsigned)(eb - (ef + 896));
+    d = ef == 0 ? 63u : (d < 63u ? d : 63u);
     const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (FB - 24);
     const long long X = (long long)((m + ((1ull << d) >> 1)) >> d); // to nearest
     return (int)b < 0 ? -X : X;

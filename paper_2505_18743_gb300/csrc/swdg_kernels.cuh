@@ -130,10 +130,11 @@ __device__ __forceinline__ int team_exp(double v, unsigned tm) {
 template <int R, typename Pix, int MODE, bool FX = true>
 struct Site {
     using S = Sz<R>;
+    // zhi: a bound of the sub-cell's pixel depths (NaN: unknown)
     static __device__ __forceinline__ SubV pixels(const Dev& d, int64_t k, int setx, int ia, int sety,
-                                                  int ib, double eta) {
+                                                  int ib, double eta, float zhi) {
         const OvTab& o = tab(d, k);
-        if constexpr (FX) return subgrid_S<Pix>(tile(d, o, k), &o, setx, ia, sety, ib, eta, zmag(d, k));
+        if constexpr (FX) return subgrid_S<Pix>(tile(d, o, k), &o, setx, ia, sety, ib, eta, zhi);
         else return subgrid_f64<Pix>(tile(d, o, k), o, setx, ia, sety, ib, eta);
     }
     static __device__ __forceinline__ int offset(int set) {
@@ -147,10 +148,6 @@ struct Site {
     }
     static __device__ __forceinline__ const Pix* tile(const Dev& d, const OvTab& o, int64_t k) {
         return (const Pix*)d.tiles + (d.tile_off ? d.tile_off[k] : (int64_t)k * o.P * o.P);
-    }
-    // high word of the cell's largest depth magnitude (0: unknown)
-    static __device__ __forceinline__ unsigned zmag(const Dev& d, int64_t k) {
-        return d.zabs ? fx::mag(d.zabs[k]) : 0u;
     }
     // mode S: a cell entirely wet (eta > -min z_b) gives V = eta + the sub-cell
     // mean depth and A = 1; entirely dry (eta <= -max z_b) gives V = A = 0;
@@ -190,6 +187,7 @@ struct Site {
                                               int ia, int ib, double eta, double& V, double& A,
                                               bool& full) {
         if (MODE == 0) {
+            float zhi = NAN;
             if (d.zmin != nullptr) {
                 const size_t ip = (size_t)k * S::NZP + offset(set) + ia + count(set) * ib;
                 const double zbar = d.zpts[ip];
@@ -200,9 +198,10 @@ struct Site {
                 if (d.zsb != nullptr) {
                     const float2 b = d.zsb[ip];
                     if (shortcut_b(eta, (double)b.x, (double)b.y, zbar, V, A, full)) return;
+                    zhi = b.y;
                 }
             }
-            const SubV r = pixels(d, k, set, ia, set, ib, eta);
+            const SubV r = pixels(d, k, set, ia, set, ib, eta, zhi);
             V = r.V;
             A = r.A;
             full = r.full;
@@ -227,7 +226,7 @@ struct Site {
             if (shortcut(d, k, eta, zh, V, A, full)) return;
             const int m = (f == 0 || f == 2) ? 0 : S::NM - 1, t = h * S::NM + al;
             const SubV r = pixels(d, k, f < 2 ? SET_MASS : SET_HALF, f < 2 ? m : t,
-                                  f < 2 ? SET_HALF : SET_MASS, f < 2 ? t : m, eta);
+                                  f < 2 ? SET_HALF : SET_MASS, f < 2 ? t : m, eta, NAN);
             V = r.V;
             A = r.A;
         } else {
@@ -930,7 +929,9 @@ __device__ __forceinline__ void mass_scalar(const Dev& d, const Tables& tb, int6
 // is split among, and Hbar(e) = J / P^2 sum_k max(e + z_k, 0), Abar = J / P^2
 // #{e + z_k > 0} (equal to mass_scalar up to rounding, with P^2 terms
 // instead of the sub-cells' split pixels).  Cells wholly wet or dry, and mode
-// P, take mass_scalar (its shortcut makes it cheap there).
+// P, take mass_scalar (its shortcut makes it cheap there), as does a cell with an
+// infinite depth.  The wet depths are integers (as in subgrid_S, in the block of e
+// and the deepest pixel) and their sum is exact.
 // Not inlined: the scalar path calls it in three places, and its code shares the
 // instruction cache with the other cells'.
 struct Mass {
@@ -941,7 +942,8 @@ __device__ __noinline__ Mass mass_scalar_pixels(const Dev& d, const Tables& tb, 
                                                 double e, int lane, unsigned tm = 0xffffffffu) {
     using ST = Site<R, Pix, MODE>;
     const bool mixed = MODE == 0 && d.zmin != nullptr && !nan_bits(e) &&
-                       !(okey(e) > nkey_neg(d.zmin[k])) && okey(e) > nkey_neg(d.zmax[k]);
+                       !(okey(e) > nkey_neg(d.zmin[k])) && okey(e) > nkey_neg(d.zmax[k]) &&
+                       finite_bits(d.zmax[k]);
     if (!mixed) {
         Mass m;
         mass_scalar<R, Pix, MODE, TL>(d, tb, k, J, e, lane, m.H, m.A, tm);
@@ -950,20 +952,19 @@ __device__ __noinline__ Mass mass_scalar_pixels(const Dev& d, const Tables& tb, 
     const OvTab& o = ST::tab(d, k);
     const Pix* t = ST::tile(d, o, k);
     const int np = o.P * o.P;
-    // the wet depths as integers, their sum in two parts (exact)
-    const int es = fx::block_exp(max(ST::zmag(d, k), fx::mag(e))) + 1;
+    const int es = fx::block_exp(max(fx::mag(d.zmax[k]), fx::mag(e))) + 1;
     const long long E = fx::from_double(e, es);
+    const Wet<Pix> is_wet(e);
     long long hi = 0;
     unsigned long long lo = 0;
     int a = 0;
 #pragma unroll 1
     for (int i = lane; i < np; i += TL) {
-        const long long D = E + fx_pixel(t[i], es);
-        if (D > 0) {
-            hi += D >> 32;
-            lo += (unsigned)D;
-            ++a;
-        }
+        const Pix z = t[i];
+        const long long D0 = E + fx_pixel(z, es), D = is_wet(z) ? D0 : 0;
+        hi += D >> 32;
+        lo += (unsigned)D;
+        a += is_wet(z);
     }
     const double h = fx::to_double(hi, es + 32) + fx::to_double((long long)lo, es);
     const double w = J / (double)np;
