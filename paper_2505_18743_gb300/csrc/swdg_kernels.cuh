@@ -1178,19 +1178,22 @@ __device__ __forceinline__ bool mass_inverse_f(const FxStage& fs, float* buf, fl
 // Eq. mass_matrix) by mixed-precision iterative refinement: H is assembled and
 // inverted in FP32, each correction is one FP32 product with the inverse, and
 // the residual b - H x is formed matrix-free by sum factorisation in block fixed
-// point (60 bits of the largest term, on the integer pipe; in FP64 arithmetic
-// the two residuals were a third of the stage update's FP64 instructions), x
-// being held as a fixed-point number too.  The sweeps stop when a correction, or
-// the next one as predicted from the contraction of the last two, is below
-// 1e-15 of x; if that does not happen within 6 sweeps (an ill-conditioned
-// near-dry cell), the FP64 Cholesky decides.  x in place of b on return.
+// point (on the integer pipe; in FP64 arithmetic the two residuals were a third of
+// the stage update's FP64 instructions), x being held as a fixed-point number too.
+// The point values B x and cw B x move up to the top of their blocks, so that a
+// residual keeps 57 places of the largest of them.  What goes through FP32 is scaled
+// by the exponents of the blocks, so the magnitudes of b, cw and x do not matter.
+// The sweeps stop when a correction, or the next one as predicted from the
+// contraction of the last two, is below 1e-15 of x; if that does not happen within 6
+// sweeps (an ill-conditioned near-dry cell), if the corrections grow or one is not
+// finite, the FP64 Cholesky decides.  x in place of b on return.
 // Scratch: buf (mass_inverse_f's, and 2 floats to align it), digit pairs xd [ND], qd [NMP], td [2 NMP], M,
 // Y, inv (double, fallback: M may overlay buf, Y and inv xd, qd and td).
 template <int ND1, int NM, int TL = 32>
 __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& fs, const double* cw, double* b,
                                  float* buf, int2* xd, int2* qd, int2* td, double* M, double* Y,
                                  double* inv, int lane, unsigned tm = 0xffffffffu) {
-    constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4;
+    constexpr int ND = ND1 * ND1, NMP = NM * NM, NDP = (ND + 3) / 4 * 4, PP = (NMP + TL - 1) / TL;
     buf = (float*)(((uintptr_t)buf + 15) & ~(uintptr_t)15);
     int2* cwd = td + NM * NM;
     const double bi = lane < ND ? b[lane] : 0.0;
@@ -1200,25 +1203,26 @@ __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& f
     const int ecw = fx::block_exp(__reduce_max_sync(tm, mc)), eb = team_exp(bi, tm);
 #pragma unroll 1
     for (int p = lane; p < NMP; p += TL) {
-        const int2 c = fx::split(fx::from_double(cw[p], ecw));
-        cwd[p] = c;
-        buf[2 * NDP + p] = (float)c.x * (1.0f / (float)(1 << (fx::FB - fx::LB)));
+        const long long c = fx::from_double(cw[p], ecw);
+        cwd[p] = fx::split(c);
+        buf[2 * NDP + p] = fx::to_float(c, 1022); // of cw 2^(1022 - ecw) <= 1
     }
     float a[ND]; // the lane's row of the inverse
-    // the inverse's scales: H = 2^(ecw - 1022) S^-1 H' S^-1
-    const int se = 127 - (ecw - 1022);
-    bool ok = mass_inverse_f<ND1, NM, TL>(fs, buf, a, lane, tm) && se > 0 && se < 255;
+    bool ok = mass_inverse_f<ND1, NM, TL>(fs, buf, a, lane, tm);
     long long X = 0; // the lane's component of x
     int ex = fx::EMIN;
-    if (ok) {
+    if (ok && eb >= fx::POISON_MIN) { // b holds an infinity or a NaN
+        ex = fx::POISON;
+    } else if (ok) {
         ok = false;
         const float si = lane < ND ? fs.sc[lane % ND1] * fs.sc[lane / ND1] : 0.0f;
-        const float so = si * __uint_as_float((unsigned)se << 23);
-        float rv = fx::to_float(fx::from_double(bi, eb), eb);
+        float rv = fx::to_float(fx::from_double(bi, eb), 1022); // the residual, 2^(1022 - er) of it
+        int er = eb;
         float dprev = 0.0f; // max |correction| / max |x| of the previous sweep
 #pragma unroll 1
         for (int sweep = 0; sweep < 6; ++sweep) {
-            // the lane's component of the correction
+            // the lane's component of the correction, 2^(ecw - er) of it:
+            // H = 2^(ecw - 1022) S^-1 H' S^-1
             float* rb = buf + (sweep & 1) * NDP;
             if (lane < ND) rb[lane] = rv * si;
             __syncwarp(tm);
@@ -1226,24 +1230,25 @@ __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& f
             read_row<NDP>(rb, r);
 #pragma unroll
             for (int j = 0; j < ND; ++j) v += a[j] * r[j];
-            v *= so;
+            v *= si;
             const float da = lane < ND ? fabsf(v) : 0.0f;
             const unsigned dbits = __reduce_max_sync(tm, __float_as_uint(da)); // a NaN is the largest
-            const int ev = fx::block_exp_f(dbits);
-            if (sweep == 0) ex = ev;
-            else if (ev > ex) break; // the corrections grow: the fallback
-            X += fx::from_float(v, ex);
+            if (dbits >= 0x7f800000u) break;
+            const int sc = er - ecw, ev = fx::block_exp_f(dbits) + sc;
+            if (sweep == 0) ex = ev + 1; // a place of room for the corrections
+            else if (ev > ex) break;
+            X += fx::from_float(v, ex - sc);
             // max |x| and the ratio of the correction to it, for the stopping test
             const unsigned xm = __reduce_max_sync(
                 tm, lane < ND ? (unsigned)((unsigned long long)(X < 0 ? -X : X) >> 31) : 0u);
-            if (xm >= 1u << (fx::FB - 30)) break; // x has outgrown its block: the fallback
+            if (xm >= 1u << (fx::FB - 31)) break; // x has outgrown its block
             const float dmax = __uint_as_float(dbits);
-            const float dr = dmax / fx::to_float((long long)xm << 31, ex);
+            const float dr = dmax / fx::to_float((long long)xm << 31, ex - sc);
             // converged when this correction is below 1e-15 of x, or when the
             // next one is, as predicted from the contraction of the last two
             // (dr / dprev, at most 1/2)
             const bool next_small = sweep > 0 && dr <= 0.5f * dprev && dr * dr <= 1e-15f * dprev;
-            if (dr <= 1e-15f || dmax == 0.0f || next_small || ex >= fx::POISON_MIN) {
+            if (dr <= 1e-15f || dmax == 0.0f || next_small) {
                 ok = true;
                 break;
             }
@@ -1251,14 +1256,34 @@ __device__ __noinline__ bool solve_mass_mixed(const Tables& tb, const FxStage& f
             // r = b - H x, H x = B^T (cw (B x))
             if (lane < ND) xd[lane] = fx::split(X);
             __syncwarp(tm);
-            fx_tens<ND1, NM, TL>(fs.Bm, xd, td, lane, tm, [&](int, int p, long long v_) {
-                qd[p] = fx::split(fx::product(fx::split(v_), cwd[p]));
+            long long q[PP];
+            unsigned m = 0;
+#pragma unroll
+            for (int i = 0; i < PP; ++i) q[i] = 0;
+            fx_tens<ND1, NM, TL>(fs.Bm, xd, td, lane, tm, [&](int it, int, long long v_) {
+                q[it] = v_;
+                m = max(m, fx::high(v_));
             });
+            const int s1 = fx::headroom(__reduce_max_sync(tm, m));
+            m = 0;
+#pragma unroll
+            for (int i = 0; i < PP; ++i) {
+                const int p = lane + i * TL;
+                if (p < NMP) q[i] = fx::product(fx::split(q[i] << s1), cwd[p]);
+                m = max(m, fx::high(q[i]));
+            }
+            const int s2 = fx::headroom(__reduce_max_sync(tm, m));
+#pragma unroll
+            for (int i = 0; i < PP; ++i) {
+                const int p = lane + i * TL;
+                if (p < NMP) qd[p] = fx::split(q[i] << s2);
+            }
             __syncwarp(tm);
             long long R = 0;
             fx_tens<NM, ND1, TL>(fs.BmT, qd, td, lane, tm, [&](int, int, long long v_) { R = v_; });
-            const int er = fx::product_exp(ex + 2 * fs.tBm, ecw) + 2 * fs.tBmT, e = max(er, eb);
-            rv = lane < ND ? fx::to_float(fx::from_double(bi, e) - (R >> min(e - er, 63)), e) : 0.0f;
+            const int eR = fx::product_exp(ex + 2 * fs.tBm - s1, ecw) - s2 + 2 * fs.tBmT;
+            er = max(eR, eb);
+            rv = lane < ND ? fx::to_float(fx::from_double(bi, er) - (R >> min(er - eR, 63)), 1022) : 0.0f;
         }
     }
     __syncwarp(tm);
