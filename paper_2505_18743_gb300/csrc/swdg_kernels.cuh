@@ -630,22 +630,28 @@ __global__ void __maxnreg__(64)
                 C = ac.get();
             }
             const int eu0 = es[0], eu3 = es[3];
-            int eD = eu0 + tBD;
-            const int eX = es[1] + tBB, eY = es[2] + tBB, eC = eu3 + tBB;
+            int eD = eu0 + tBD, eX = es[1] + tBB, eY = es[2] + tBB, eC = eu3 + tBB;
             // a constant field is that constant exactly
             if (cm & 1u) ZX = ZY = 0;
+            if (cm & 2u) QX = fx::from_double(c0[1], eX);
+            if (cm & 4u) QY = fx::from_double(c0[2], eY);
+            if (cm & 8u) C = fx::from_double(c0[3], eC);
+            // the factors of products move up to the places that are free in their blocks:
+            // the tables' bounds are a few places above the values, and far above the gradient
+            auto up = [&](long long& x, int& e) {
+                const int s = fx::headroom(__reduce_max_sync(tm, pt ? fx::high(x) : 0u));
+                x <<= s;
+                e -= s;
+            };
             {
-                // the gradient is far below the bound its table allows: its block moves
-                // up to the places that are free
-                const unsigned m = __reduce_max_sync(tm, pt ? max(fx::high(ZX), fx::high(ZY)) : 0u);
-                const int s = fx::headroom(m);
+                const int s = fx::headroom(__reduce_max_sync(tm, pt ? max(fx::high(ZX), fx::high(ZY)) : 0u));
                 ZX <<= s;
                 ZY <<= s;
                 eD -= s;
             }
-            if (cm & 2u) QX = fx::from_double(c0[1], eX);
-            if (cm & 4u) QY = fx::from_double(c0[2], eY);
-            if (cm & 8u) C = fx::from_double(c0[3], eC);
+            up(QX, eX);
+            up(QY, eY);
+            up(C, eC);
             const double z = (cm & 1u) ? c0[0] : fx::to_double(Z, eu0 + tBB);
             const double qx = fx::to_double(QX, eX), qy = fx::to_double(QY, eY);
             double h = 0.0, A;
