@@ -33,8 +33,7 @@
 // 2^FB there, which the joint rows are checked for where the tables are built.
 //
 // A block that holds an infinity or a NaN takes the exponent POISON; every
-// value converted back from it is NaN.  Blocks below 2^-958 keep the exponent of
-// that size: they lose places, and values below 2^-1018 are zero.
+// value converted back from it is NaN.  Values below 2^-1018 are zero.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -44,7 +43,7 @@ namespace fx {
 
 constexpr int FB = 60;
 constexpr int LB = 30;
-constexpr int EMIN = 64;       // smallest block exponent: values below it shift out to 0
+constexpr int EMIN = 5;        // smallest block exponent: values below 2^(EMIN - 1023) read as 0
 constexpr int POISON = 4096;   // block exponent of a block with an infinity or a NaN
 constexpr int POISON_MIN = 3072; // any exponent derived from POISON by table exponents is above
 
@@ -145,7 +144,8 @@ __host__ __device__ __forceinline__ int block_exp(unsigned maxmag) {
 __host__ __device__ __forceinline__ long long from_double(double v, int eb) {
     const unsigned long long b = dbits(v);
     const int s = FB + 1022 - eb;
-    if (((int)(b >> 52) & 0x7ff) + s <= 0) return 0; // below the block's last place (or poisoned)
+    const int least = s > 1 - EMIN ? EMIN - 1 : -s; // below the block's last place (or poisoned)
+    if (((int)(b >> 52) & 0x7ff) <= least) return 0;
     return to_int(bitsd(b + ((unsigned long long)(long long)s << 52)));
 }
 // to_double at the ends of the exponent range (rare; not inlined: the callers'
