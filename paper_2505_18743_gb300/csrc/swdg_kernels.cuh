@@ -304,6 +304,11 @@ __device__ __forceinline__ void vel_wave(double h, double g, double sg, double e
         w = h > 0.0 ? sqrt(g * h) : 0.0;
     }
 }
+// a side's wave speed bound as an integer that orders like it; a side whose velocity
+// is NaN leaves the bound to the other one (as under fmax), both give a NaN
+__device__ __forceinline__ long long wave_key(double l, double ut) {
+    return nan_bits(l) || nan_bits(ut) ? -1 : __double_as_longlong(l);
+}
 struct FaceFlux {
     double flux[4], pr, lam;
     bool own_first, bnd;
@@ -402,8 +407,7 @@ __device__ __forceinline__ FaceFlux face_flux(const Dev& d, const FaceTables& ft
     vel_wave(hB, d.g, d.sg, d.eps, fB, wB);
     const double vA = fA * (of ? qnm : qnp), uA = fA * (of ? qtm : qtp);
     const double vB = fB * (of ? qnp : qnm), uB = fB * (of ? qtp : qtm);
-    const double lA = fabs(vA) + wA, lB = fabs(vB) + wB;
-    const double lam = __double_as_longlong(lA) > __double_as_longlong(lB) ? lA : lB;
+    const double lam = __longlong_as_double(max(wave_key(fabs(vA) + wA, uA), wave_key(fabs(vB) + wB, uB)));
     const double hl = 0.5 * lam, dh = hsA - hsB;
     const double qsA = hsA * vA, qsB = hsB * vB, rsA = hsA * uA, rsB = hsB * uB;
     out.flux[0] = fma(hl, dh, flip(0.5 * (qsA + qsB), sA));
