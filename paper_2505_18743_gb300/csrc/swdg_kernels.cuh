@@ -1572,6 +1572,14 @@ struct StageFx {
     static_assert(S::ND1 * S::ND1 * S::NM <= W, "fallback Y");
 };
 
+// Newton's stopping test in FP64 (rare: not inlined)
+template <int TL>
+__device__ __noinline__ bool newton_done(double dz, double z, double zabs, double tol, bool act, unsigned tm) {
+    double inc = act ? fabs(dz) : 0.0, scale = act ? 1.0 + fabs(z) + zabs : 0.0;
+    team_sum2<TL>(inc, scale, tm);
+    return inc <= tol * scale;
+}
+
 // the friction coefficient of v^(l-1) at the lane's momentum point (a constant
 // field: its value).  w: the scratch of square.  Not inlined: both paths of the
 // stage update call it.
@@ -1779,7 +1787,8 @@ __global__ void __maxnreg__(72)
                     __syncwarp(tm);
                 }
                 z -= dz[0];
-                // the stopping test in FP32 (sums of magnitudes against 1e-12 of their scale)
+                // the stopping test, sums of magnitudes against newton_tol of their scale, in
+                // FP32 where that decides it (its error is below 1e-6 of either side)
                 float inc = 0.0f, scale = 0.0f;
                 if (act) {
                     inc = f32_of(fabs(dz[0]));
@@ -1794,7 +1803,11 @@ __global__ void __maxnreg__(72)
                 prev_full = (npart == 0);
                 const double z0 = __shfl_sync(tm, z, 0, TL);
                 zc = __all_sync(tm, !act || same_bits(z, z0));
-                if (inc <= tolf * scale) prev_full = false, kk = d.newton_max - 1;
+                const float lim = tolf * scale;
+                bool done = inc <= lim;
+                if (!(fabsf(inc - lim) > 1e-5f * lim && lim > 1e-30f))
+                    done = newton_done<TL>(dz[0], z, d.zabs[k], d.newton_tol, act, tm);
+                if (done) prev_full = false, kk = d.newton_max - 1;
             }
             if (scalar) {
                 fb++;
