@@ -1479,8 +1479,8 @@ int swdg_residual(swdg_ctx* ctx, double t, double* F, double* Gx, double* Gy, do
     if (!ctx->has_state) return fail(ctx, SWDG_ESTATE, "residual: no state");
     int rc = put_time(ctx, t, -1.0);
     if (rc) return rc;
-    if (ctx->d.fflux) ctx->L.faces(ctx->d, ctx->tb, 0, 0.0, 0, ctx->st);
-    ctx->L.residual(ctx->d, ctx->tb, 0, 0, 0.0, 0, ctx->shp[KK_RESIDUAL], ctx->st);
+    if (ctx->d.fflux) ctx->L.faces(ctx->d, 0, 0.0, 0, ctx->st);
+    ctx->L.residual(ctx->d, 0, 0, 0.0, 0, ctx->shp[KK_RESIDUAL], ctx->st);
     CK(cudaGetLastError());
     double* dst[6] = {F, Gx, Gy, R, Lx, Ly};
     const size_t sz = (size_t)ctx->n * ctx->nd * sizeof(double);
@@ -1499,8 +1499,8 @@ int swdg_cfl_dt(swdg_ctx* ctx, double t, double* dt) {
     int rc = put_clocks(ctx, t, 1);
     if (!rc) rc = put_fixed_dt(ctx, -1.0);
     if (rc) return rc;
-    if (ctx->d.fflux) ctx->L.faces(ctx->d, ctx->tb, 0, 0.0, 1, ctx->st);
-    ctx->L.residual(ctx->d, ctx->tb, 0, 0, 0.0, 1, ctx->shp[KK_RESIDUAL], ctx->st);
+    if (ctx->d.fflux) ctx->L.faces(ctx->d, 0, 0.0, 1, ctx->st);
+    ctx->L.residual(ctx->d, 0, 0, 0.0, 1, ctx->shp[KK_RESIDUAL], ctx->st);
     CK(cudaGetLastError());
     std::vector<Member> mh;
     rc = read_clocks(ctx, mh);
@@ -1557,7 +1557,7 @@ static int enqueue_step(swdg_ctx* ctx, cudaEvent_t (*ev)[2] = nullptr, int rec_s
     };
     keep(0, 0, -1);
     mark(0, 0);
-    ctx->L.step_begin(d, ctx->tb, 1, ctx->shp[KK_BEGIN], ctx->st);
+    ctx->L.step_begin(d, 1, ctx->shp[KK_BEGIN], ctx->st);
     mark(0, 1);
     keep(0, 1, 0);
     keep_flags(0);
@@ -1576,16 +1576,16 @@ static int enqueue_step(swdg_ctx* ctx, cudaEvent_t (*ev)[2] = nullptr, int rec_s
             sa.make_llin = (l == s - 1 && d.at[l][l] != 0.0) ? 1 : 0;
             sa.final_ = 0;
             mark(4 + l, 0);
-            ctx->L.stage(d, ctx->tb, sa, ctx->shp[KK_STAGE], ctx->st);
+            ctx->L.stage(d, sa, ctx->shp[KK_STAGE], ctx->st);
             mark(4 + l, 1);
             keep(l, 1 + l, l);
             keep_flags(l);
         }
         mark(9 + l, 0);
-        if (d.fflux) ctx->L.faces(d, ctx->tb, l, d.c[l], l == 0 ? 1 : 0, ctx->st);
+        if (d.fflux) ctx->L.faces(d, l, d.c[l], l == 0 ? 1 : 0, ctx->st);
         mark(9 + l, 1);
         mark(1 + l, 0);
-        ctx->L.residual(d, ctx->tb, l, l, d.c[l], l == 0 ? 1 : 0, ctx->shp[KK_RESIDUAL], ctx->st);
+        ctx->L.residual(d, l, l, d.c[l], l == 0 ? 1 : 0, ctx->shp[KK_RESIDUAL], ctx->st);
         mark(1 + l, 1);
     }
     StageArgs sa{};
@@ -1601,7 +1601,7 @@ static int enqueue_step(swdg_ctx* ctx, cudaEvent_t (*ev)[2] = nullptr, int rec_s
     sa.make_llin = 0;
     sa.final_ = 1;
     mark(8, 0);
-    ctx->L.stage(d, ctx->tb, sa, ctx->shp[KK_STAGE], ctx->st);
+    ctx->L.stage(d, sa, ctx->shp[KK_STAGE], ctx->st);
     mark(8, 1);
     keep(0, s + 1, s);
     keep_flags(s);
@@ -1703,7 +1703,7 @@ int swdg_step_profile(swdg_ctx* ctx, int n_steps, double dt, double* t_inout, do
 int swdg_degree_switch(swdg_ctx* ctx, uint8_t* flags_out) {
     if (!ctx) return SWDG_EINVAL;
     if (!ctx->has_state) return fail(ctx, SWDG_ESTATE, "degree_switch: no state");
-    ctx->L.step_begin(ctx->d, ctx->tb, 1, ctx->shp[KK_BEGIN], ctx->st);
+    ctx->L.step_begin(ctx->d, 1, ctx->shp[KK_BEGIN], ctx->st);
     CK(cudaGetLastError());
     if (flags_out)
         CK(cudaMemcpyAsync(flags_out, ctx->flag, ctx->n, cudaMemcpyDeviceToHost, ctx->st));
@@ -1844,7 +1844,7 @@ int swdg_residual_vjp(swdg_ctx* ctx, double t, const double* Fb, const double* G
     double* ub = ctx->adj + 6 * f;
     double* nb = ctx->adj + 10 * f;
     double* db = nb + n;
-    ctx->L.residual_vjp(ctx->d, ctx->tb, ctx->U, ctx->cmask, ctx->adj, ub, nb, db, 0,
+    ctx->L.residual_vjp(ctx->d, ctx->U, ctx->cmask, ctx->adj, ub, nb, db, 0,
                         Shape{grid_for(n), WPB}, ctx->st);
     CK(cudaGetLastError());
     double* dst[4] = {zeta_b, qx_b, qy_b, c_b};
@@ -2009,13 +2009,13 @@ int swdg_step_vjp_slot(swdg_ctx* ctx, int slot, const double* zeta_b, const doub
     a.nres = s;
     a.make_llin = 0;
     a.use_llin = imp ? 1 : 0;
-    ctx->L.stage_vjp(d, ctx->tb, a, shp, ctx->st);
+    ctx->L.stage_vjp(d, a, shp, ctx->st);
     CK(cudaGetLastError());
     for (int l = s - 1; l >= 0; --l) {
         // residual of stage l at t^n + c_l dt
         rc = put_clocks(ctx, t0 + d.c[l] * dt, 0);
         if (rc) return rc;
-        ctx->L.residual_vjp(d, ctx->tb, ust(l), cst(l), w.rbar + (size_t)l * 6 * f,
+        ctx->L.residual_vjp(d, ust(l), cst(l), w.rbar + (size_t)l * 6 * f,
                             w.ubs + (size_t)l * 4 * f, w.nbar, w.dbar, 1, shp, ctx->st);
         CK(cudaGetLastError());
         if (l == 0) break;
@@ -2037,7 +2037,7 @@ int swdg_step_vjp_slot(swdg_ctx* ctx, int slot, const double* zeta_b, const doub
         }
         b.add = d.at[l][l];
         b.nres = l;
-        ctx->L.stage_vjp(d, ctx->tb, b, shp, ctx->st);
+        ctx->L.stage_vjp(d, b, shp, ctx->st);
         CK(cudaGetLastError());
     }
     BeginVjpArgs bg{};
@@ -2050,7 +2050,7 @@ int swdg_step_vjp_slot(swdg_ctx* ctx, int slot, const double* zeta_b, const doub
     bg.ubn = w.ubs;
     bg.ubpre = w.ubpre;
     bg.dbar = w.dbar;
-    ctx->L.begin_vjp(d, ctx->tb, bg, shp, ctx->st);
+    ctx->L.begin_vjp(d, bg, shp, ctx->st);
     CK(cudaGetLastError());
     rc = put_clocks(ctx, t0 + dt, 0);
     if (rc) return rc;
@@ -2937,7 +2937,7 @@ extern "C" int swdg_residual_noalloc(const swdg_config* cfg, int64_t n, const do
                             "non-conforming face)");
     const Shape shp{grid_for(n), WPB};
     L.masks(d, 0, shp, st);
-    L.residual(d, tb, 0, 0, 0.0, 1, shp, st);
+    L.residual(d, 0, 0, 0.0, 1, shp, st);
     if (dt_out) k_noalloc_end<<<1, 1, 0, st>>>(sc, cfg->cfl, dt_out);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -131,6 +131,22 @@ __device__ __forceinline__ double gamma_f64(double n, double h, double qx, doubl
     return g * n * n * sqrt(qx * qx + qy * qy) * (z3 * z3 * z);
 }
 
+// the velocity factor and the Manning coefficient of one point together: on the
+// wet branch (h >= eps, where h_des = h) both come from 1/h, with
+// h^(-7/3) = (1/h)^2 cbrt(1/h); below eps as vel_factor and gamma_manning
+__device__ __forceinline__ void vel_gamma(float n, float h, float qx, float qy, float g, float eps, float& fv,
+                                          float& gam) {
+    if (h >= eps && h > 0.0f) {
+        const float rh = 1.0f / h;
+        fv = rh;
+        const float c3 = cbrt(rh); // h^(-1/3)
+        gam = (n == 0.0f) ? 0.0f : g * n * n * sqrt(qx * qx + qy * qy) * (rh * rh) * c3;
+    } else {
+        fv = vel_factor<float>(h, eps);
+        gam = gamma_manning<float>(n, h, qx, qy, g, eps);
+    }
+}
+
 // traces of zeta (FP64) and of qx, qy, c (FP32) at face point al of face f; u32
 // (nullable): the FP32 copy of u, same layout and stride
 template <int ND1>
@@ -458,7 +474,7 @@ __global__ void __maxnreg__(80)
             ST::VA(d, *d.tabs, k, SET_VOL, al, be, z, h, A);
             const float hB = (float)h;
             float fv, gam;
-            vel_gamma<float>(manB, hB, qx, qy, gB, epsB, fv, gam);
+            vel_gamma(manB, hB, qx, qy, gB, epsB, fv, gam);
             const float ux = fv * qx, uy = fv * qy;
             const double w = J * tb.wv[al] * tb.wv[be];
             // the weights of the FP32 terms in FP32 (no conversions per point)

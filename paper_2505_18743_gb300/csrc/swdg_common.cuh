@@ -9,8 +9,9 @@
 //   tiles   [cell][P][P] float32|float64 bathymetry depth (mode S)
 //   zpts    [cell][NV^2 + NM^2 + NG^2] float64: point samples (mode P) or
 //           sub-cell mean depths sum_k w_k z_k (mode S)
-// Small per-degree tables (1D interpolation matrices, quadrature weights,
-// pixel-overlap fractions) travel as a __grid_constant__ kernel parameter.
+// Small per-degree tables (1D interpolation matrices, quadrature weights) lie in
+// device memory (Dev::tabs) and are copied to shared memory by the blocks that
+// index them by lane; rarely run kernels take them as a parameter.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -455,23 +456,6 @@ __device__ __forceinline__ void vel_friction(double h, double qx, double qy, boo
         const VelGam r = vel_friction_any(h, qx, qy, friction, eps);
         fv = r.fv;
         gm = r.gm;
-    }
-}
-
-// the velocity factor and the Manning coefficient of one point together (the
-// FP32-bulk path): on the wet branch (h >= eps, where h_des = h) both come from
-// 1/h with h^(-7/3) = (1/h)^2 cbrt(1/h); below eps as vel_factor and
-// gamma_manning
-template <typename T>
-__device__ __forceinline__ void vel_gamma(T n, T h, T qx, T qy, T g, T eps, T& fv, T& gam) {
-    if (h >= eps && h > T(0)) {
-        const T rh = T(1) / h;
-        fv = rh;
-        const T c3 = cbrt(rh); // h^(-1/3)
-        gam = (n == T(0)) ? T(0) : g * n * n * sqrt(qx * qx + qy * qy) * (rh * rh) * c3;
-    } else {
-        fv = vel_factor<T>(h, eps);
-        gam = gamma_manning<T>(n, h, qx, qy, g, eps);
     }
 }
 

@@ -40,7 +40,7 @@ struct Launchers {
     static constexpr size_t ind_b = sizeof(double) * indicator_smem<R>();
     static constexpr size_t remap_b = sizeof(double) * remap_smem<R>();
 
-    static void residual(const Dev& d, const Tables& tb, int buf, int stage, double c_stage,
+    static void residual(const Dev& d, int buf, int stage, double c_stage,
                          int want_dt, Shape s, cudaStream_t st) {
         // 32 / TL cells per warp: no more blocks than their cells
         const int cpb = s.wpb * 32 / ResFx<R>::TL;
@@ -56,7 +56,7 @@ struct Launchers {
             bulk::k_residual<R, Pix, MODE><<<grid, 32 * s.wpb, res_b * s.wpb, st>>>(d, buf, stage);
         }
     }
-    static void faces(const Dev& d, const Tables& tb, int buf, double c_stage, int want_dt,
+    static void faces(const Dev& d, int buf, double c_stage, int want_dt,
                       cudaStream_t st) {
         if (d.njobs <= 0) return;
         // one point per lane and one pass; 4 warps a block, so that small meshes spread
@@ -68,7 +68,7 @@ struct Launchers {
         else
             bulk::k_faces<R, Pix, MODE><<<(int)blocks, 128, 0, st>>>(d, buf, c_stage, want_dt);
     }
-    static void step_begin(const Dev& d, const Tables& tb, int do_switch, Shape s, cudaStream_t st) {
+    static void step_begin(const Dev& d, int do_switch, Shape s, cudaStream_t st) {
         const int cpb = begin_cells * s.wpb;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, (d.n + cpb - 1) / cpb));
         if constexpr (F64)
@@ -76,7 +76,7 @@ struct Launchers {
         else
             bulk::k_step_begin<R, Pix, MODE><<<grid, 32 * s.wpb, begin_b * s.wpb, st>>>(d, do_switch);
     }
-    static void stage(const Dev& d, const Tables& tb, const StageArgs& sa, Shape s, cudaStream_t st) {
+    static void stage(const Dev& d, const StageArgs& sa, Shape s, cudaStream_t st) {
         // two cells per warp: no more blocks than 2 wpb cells each
         const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
@@ -99,7 +99,7 @@ struct Launchers {
                            const double* gbar, double* zb, const int32_t* cell, cudaStream_t st) {
         k_gauges_vjp<R><<<(ng + 63) / 64, 64, 0, st>>>(d, tb, ng, xy, gbar, zb, cell);
     }
-    static void residual_vjp(const Dev& d, const Tables& tb, const double* u, const uint8_t* cm,
+    static void residual_vjp(const Dev& d, const double* u, const uint8_t* cm,
                              const double* rbar, double* ubar, double* nbar, double* dbar,
                              int accumulate, Shape s, cudaStream_t st) {
         const int cpb = s.wpb * 32 / VjpTeam<R>::TL;
@@ -107,13 +107,13 @@ struct Launchers {
         k_residual_vjp<R, Pix, MODE><<<grid, 32 * s.wpb, vjp_b * s.wpb, st>>>(
             d, u, cm, rbar, ubar, nbar, dbar, accumulate);
     }
-    static void stage_vjp(const Dev& d, const Tables& tb, const StageVjpArgs& a, Shape s,
+    static void stage_vjp(const Dev& d, const StageVjpArgs& a, Shape s,
                           cudaStream_t st) {
         const int64_t need = (d.n + 2 * s.wpb - 1) / (2 * s.wpb);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(s.grid, need));
         k_stage_vjp<R, Pix, MODE><<<grid, 32 * s.wpb, svjp_b * s.wpb, st>>>(d, a);
     }
-    static void begin_vjp(const Dev& d, const Tables& tb, const BeginVjpArgs& a, Shape s,
+    static void begin_vjp(const Dev& d, const BeginVjpArgs& a, Shape s,
                           cudaStream_t st) {
         k_begin_vjp<R, Pix, MODE><<<s.grid, 32 * s.wpb, bvjp_b * s.wpb, st>>>(d, a);
     }

@@ -1388,7 +1388,7 @@ __global__ void __maxnreg__(64)
     using S = Sz<R>;
     using L = BeginFx<R>;
     using ST = Site<R, Pix, MODE>;
-    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
+    constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NGP = S::NGP;
     constexpr int TL = L::TL, PP = L::PP;
     __shared__ FxStage fs;
     copy_table(fs, &d.tabs->fs);

@@ -19,12 +19,11 @@ struct Shape {
 enum { KK_BEGIN = 0, KK_RESIDUAL = 1, KK_STAGE = 2, KK_AUX = 3, KK_N = 4 };
 
 struct Launch {
-    void (*residual)(const Dev&, const Tables&, int buf, int stage, double c_stage, int want_dt,
-                     Shape, cudaStream_t);
+    void (*residual)(const Dev&, int buf, int stage, double c_stage, int want_dt, Shape, cudaStream_t);
     // the face points of the residual, each once, into d.fflux (before residual)
-    void (*faces)(const Dev&, const Tables&, int buf, double c_stage, int want_dt, cudaStream_t);
-    void (*step_begin)(const Dev&, const Tables&, int do_switch, Shape, cudaStream_t);
-    void (*stage)(const Dev&, const Tables&, const StageArgs&, Shape, cudaStream_t);
+    void (*faces)(const Dev&, int buf, double c_stage, int want_dt, cudaStream_t);
+    void (*step_begin)(const Dev&, int do_switch, Shape, cudaStream_t);
+    void (*stage)(const Dev&, const StageArgs&, Shape, cudaStream_t);
     void (*masks)(const Dev&, int buf, Shape, cudaStream_t);
     void (*cell_diag)(const Dev&, const Tables&, double* part, Shape, cudaStream_t);
     // zeta at gauge points (cell: the cell of each point, -1 none; null: search [k0, k1))
@@ -35,12 +34,12 @@ struct Launch {
                        double* zb, const int32_t* cell, cudaStream_t);
     // discrete adjoint of the residual (FP64): rbar [6][n][nd] -> ubar [4][n][nd],
     // nbar [n] (Manning), dbar [n] (bathymetry offset)
-    void (*residual_vjp)(const Dev&, const Tables&, const double* u, const uint8_t* cmask,
+    void (*residual_vjp)(const Dev&, const double* u, const uint8_t* cmask,
                          const double* rbar, double* ubar, double* nbar, double* dbar,
                          int accumulate, Shape, cudaStream_t);
     // adjoints of a stage update / the final combination and of the step start (FP64)
-    void (*stage_vjp)(const Dev&, const Tables&, const StageVjpArgs&, Shape, cudaStream_t);
-    void (*begin_vjp)(const Dev&, const Tables&, const BeginVjpArgs&, Shape, cudaStream_t);
+    void (*stage_vjp)(const Dev&, const StageVjpArgs&, Shape, cudaStream_t);
+    void (*begin_vjp)(const Dev&, const BeginVjpArgs&, Shape, cudaStream_t);
     // refinement indicator (kind 0 |curl u|, 1 |grad c|) and state remap (Sec. 3.4)
     void (*indicator)(const Dev&, const Tables&, int kind, double* eta, Shape, cudaStream_t);
     void (*remap)(const Tables&, const RemapArgs&, Shape, cudaStream_t);
