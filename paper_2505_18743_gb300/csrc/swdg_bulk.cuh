@@ -341,7 +341,10 @@ __device__ __forceinline__ void side_flux(const float raw[4], float pres, bool o
 // The residual: zeta's value, F, R and the face lifts in FP64, the rest in FP32.
 // The teams of k_residual (32 lanes a cell at r = 3, 16 at r = 2, 8 at r = 1): an
 // FP64 instruction takes 16 clocks of the SM however few of its lanes are active,
-// and the volume points fill those.
+// and the volume points fill those.  The FP64 pipe bounds it.  A launch, one cell per
+// warp and so: 384 -> 337 us (65,536 cells, r = 3, where only the tables' copy and the
+// overlaid shared memory differ), 708 -> 467 (172,032 cells, r = 2); 64, 72 and 96
+// registers: 339, 337 and 349 (r = 3).
 template <int R>
 struct Res {
     using S = Sz<R>;
@@ -568,14 +571,9 @@ __global__ void __maxnreg__(80)
             for (int al = 0; al < NV; ++al) s += tb.BvF[al][a] * sB[(((2 + cl) * 2 + 1) * NV + al) * ND1 + b];
             rs[(4 + cl) * ND + j] = (double)s;
         }
-        // the face fluxes of this cell, computed once per face point by k_faces (the
-        // second half of a face only where the face has two)
+        // the face fluxes of this cell, computed once per face point by k_faces
         const double* F = d.fflux + k * (32 * NM);
-        for (int i = lane; i < 32 * NM; i += TL) {
-            const int q = i / NM, f = (q >> 1) & 3;
-            const unsigned inf = f == 0 ? fi[0] : f == 1 ? fi[1] : f == 2 ? fi[2] : fi[3];
-            if (!(q & 1) || (inf & 3) == FI_COARSE) fh[i] = F[i];
-        }
+        for (int i = lane; i < 32 * NM; i += TL) fh[i] = F[i];
         __syncwarp(tm);
         // lift the face fluxes onto the nodes of each face: one item per field,
         // face and node along it, the x faces (0, 1: node columns a = 0 and
@@ -717,7 +715,8 @@ __device__ __forceinline__ void mass_scalar(const Dev& d, const BaseTables& tb, 
 // #{e + z_k > 0} (equal to mass_scalar up to rounding, with P^2 terms
 // instead of the sub-cells' split pixels).  Cells wholly wet or dry, and mode
 // P, take mass_scalar (its shortcut makes it cheap there).
-template <int R, typename Pix, int MODE, int TL = 32>
+// The sum's order is that of a team of ACC TL lanes.
+template <int R, typename Pix, int MODE, int TL, int ACC>
 __device__ __forceinline__ void mass_scalar_pixels(const Dev& d, const BaseTables& tb, int64_t k,
                                                    double J, double e, int lane, double& H,
                                                    double& A, unsigned tm = 0xffffffffu) {
@@ -731,26 +730,31 @@ __device__ __forceinline__ void mass_scalar_pixels(const Dev& d, const BaseTable
     const OvTab& o = ST::tab(d, k);
     const Pix* t = ST::tile(d, o, k);
     const int np = o.P * o.P;
-    double h = 0.0;
+    double h[ACC];
     int a = 0;
-    for (int i = lane; i < np; i += TL) {
-        const double dd = e + (double)t[i];
-        if (dd > 0.0) {
-            h += dd;
-            ++a;
+#pragma unroll
+    for (int q = 0; q < ACC; ++q) {
+        h[q] = 0.0;
+        for (int i = lane + q * TL; i < np; i += TL * ACC) {
+            const double dd = e + (double)t[i];
+            if (dd > 0.0) {
+                h[q] += dd;
+                ++a;
+            }
         }
     }
+    static_assert(ACC == 1 || ACC == 2, "one level of the tree on the lane itself");
     const double w = J / (double)np;
-    H = w * team_sum<TL>(h, tm);
+    H = w * team_sum<TL>(ACC == 2 ? h[0] + h[ACC - 1] : h[0], tm);
     A = w * (double)__reduce_add_sync(tm, a);
 }
 
-template <int R, typename Pix, int MODE, int TL = 32>
+template <int R, typename Pix, int MODE, int TL, int ACC>
 __device__ __noinline__ int scalar_newton(const Dev& d, const BaseTables& tb, int64_t k, double J, double target,
                              double& e, int lane, unsigned tm = 0xffffffffu) {
     constexpr int ND = Sz<R>::ND;
     double H, A;
-    mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, H, A, tm);
+    mass_scalar_pixels<R, Pix, MODE, TL, ACC>(d, tb, k, J, e, lane, H, A, tm);
     // the first iteration reuses this evaluation unless the start moves to the
     // dry start of Eq. initial_guess
     bool have = true;
@@ -760,7 +764,7 @@ __device__ __noinline__ int scalar_newton(const Dev& d, const BaseTables& tb, in
     }
     int it = 0;
     for (int kk = 0; kk < d.newton_max; ++kk) {
-        if (!have) mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, H, A, tm);
+        if (!have) mass_scalar_pixels<R, Pix, MODE, TL, ACC>(d, tb, k, J, e, lane, H, A, tm);
         have = false;
         if (A == 0.0) break;
         const double dd = (H - target) / A;
@@ -771,6 +775,11 @@ __device__ __noinline__ int scalar_newton(const Dev& d, const BaseTables& tb, in
     return it;
 }
 
+// A cell per half warp at r <= 2 (16 mass points at most; the sums over the lanes of a
+// warp only add zeros of its other half), per warp at r = 3.  The FP64 pipe bounds it:
+// 518 -> 319 us by half warps (172,032 cells, r = 2); 65,536 cells at r = 3 take 292.
+template <int R>
+constexpr int begin_team() { return R == 3 ? 32 : 16; }
 template <int R>
 constexpr int begin_smem() {
     using S = Sz<R>;
@@ -785,8 +794,11 @@ __global__ void __launch_bounds__(32 * MAXWPB)
     using S = Sz<R>;
     using ST = Site<R, Pix, MODE, false>;
     constexpr int ND1 = S::ND1, ND = S::ND, NM = S::NM, NMP = S::NMP, NG = S::NG, NGP = S::NGP;
+    constexpr int TL = begin_team<R>();
+    static_assert(NMP <= TL, "one mass point per lane");
     extern __shared__ double smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int warp = threadIdx.x / TL, lane = threadIdx.x % TL, wpb = blockDim.x / TL; // teams
+    const unsigned tm = TL == 32 ? 0xffffffffu : 0xFFFFu << (threadIdx.x & 16);        // the team's lanes
     double* su = smem + warp * begin_smem<R>();
     double* pe = su + 4 * ND;    // [NMP] zeta at mass points
     double* pc = pe + NMP;       // [NMP] c at mass points
@@ -801,15 +813,15 @@ __global__ void __launch_bounds__(32 * MAXWPB)
         if (threadIdx.x == 0) d.sc->maxits = 0;
     }
     for (int64_t k = (int64_t)blockIdx.x * wpb + warp; k < n; k += (int64_t)gridDim.x * wpb) {
-        for (int i = lane; i < 4 * ND; i += 32) su[i] = ufield(d, 0, i / ND, ND)[k * ND + (i % ND)];
+        for (int i = lane; i < 4 * ND; i += TL) su[i] = ufield(d, 0, i / ND, ND)[k * ND + (i % ND)];
         unsigned cm = d.cmask[k];
         const double hx = d.hxhy[2 * k], hy = d.hxhy[2 * k + 1], J = hx * hy;
-        __syncwarp();
+        __syncwarp(tm);
         // zeta and c at the mass points
-        tens_interp<ND1, NM>(tb.Bm, su, tmp, pe, lane);
-        tens_interp<ND1, NM>(tb.Bm, su + 3 * ND, tmp, pc, lane);
+        tens_interp<ND1, NM, double, TL>(tb.Bm, su, tmp, pe, lane, tm);
+        tens_interp<ND1, NM, double, TL>(tb.Bm, su + 3 * ND, tmp, pc, lane, tm);
         bool allfull = true;
-        for (int p = lane; p < NMP; p += 32) {
+        for (int p = lane; p < NMP; p += TL) {
             if (cm & 1u) pe[p] = su[0];
             if (cm & 8u) pc[p] = su[3 * ND];
             double V, A;
@@ -818,93 +830,86 @@ __global__ void __launch_bounds__(32 * MAXWPB)
             pV[p] = V;
             allfull = allfull && full && !zero_bits(A);
         }
-        allfull = __all_sync(0xffffffffu, allfull);
-        __syncwarp();
+        allfull = __all_sync(tm, allfull);
+        __syncwarp(tm);
         // r_K = 0 where the smallest wet depth of the mass points is at most
         // h_lim (a NaN depth never counts, as under fmin)
         bool low = false;
-        for (int p = lane; p < NMP; p += 32) low = low || pV[p] <= d.hlim;
-        const int flag = (do_switch && __any_sync(0xffffffffu, low)) ? 0 : R;
+        for (int p = lane; p < NMP; p += TL) low = low || pV[p] <= d.hlim;
+        const int flag = (do_switch && __any_sync(tm, low)) ? 0 : R;
         if (flag == 0) {
             // remap to r_K = 0: mass-exact zeta, GL means of q, tracer-mass-exact c
             double m = 0.0, tr = 0.0;
-            for (int p = lane; p < NMP; p += 32) {
+            for (int p = lane; p < NMP; p += TL) {
                 const double w = J * tb.wm[p % NM] * tb.wm[p / NM];
                 m += w * pV[p];
                 tr += w * pV[p] * pc[p];
             }
-            team_sum2<32>(m, tr, 0xffffffffu);
+            team_sum2<TL>(m, tr, tm);
             for (int f = 0; f < 3; ++f) {
-                tens_interp<ND1, NG>(tb.Bg, su + (1 + f) * ND, tmp, pg + f * NGP, lane);
+                tens_interp<ND1, NG, double, TL>(tb.Bg, su + (1 + f) * ND, tmp, pg + f * NGP, lane, tm);
             }
             double mq[3] = {0.0, 0.0, 0.0};
-            for (int p = lane; p < NGP; p += 32) {
+            for (int p = lane; p < NGP; p += TL) {
                 const double w = tb.wg[p % NG] * tb.wg[p / NG];
                 for (int f = 0; f < 3; ++f) {
                     const double v = (cm & (2u << f)) ? su[(1 + f) * ND] : pg[f * NGP + p];
                     mq[f] += w * v;
                 }
             }
-            team_sum2<32>(mq[0], mq[1], 0xffffffffu);
-            mq[2] = warp_sum(mq[2]);
+            team_sum2<TL>(mq[0], mq[1], tm);
+            mq[2] = team_sum<TL>(mq[2], tm);
             const double cnew = (m > 1e-14 * J * d.hlim) ? tr / m : mq[2];
             double emax = -INFINITY;
-            for (int p = lane; p < NMP; p += 32) emax = fmax(emax, pe[p]);
-            emax = warp_max(emax);
-            __syncwarp();
+            for (int p = lane; p < NMP; p += TL) emax = fmax(emax, pe[p]);
+            #pragma unroll
+            for (int o = TL / 2; o > 0; o >>= 1) emax = fmax(emax, __shfl_xor_sync(tm, emax, o));
+            __syncwarp(tm);
             if (!(cm & 8u))
-                for (int i = lane; i < ND; i += 32) su[3 * ND + i] = cnew;
+                for (int i = lane; i < ND; i += TL) su[3 * ND + i] = cnew;
             if (!(cm & 2u))
-                for (int i = lane; i < ND; i += 32) su[ND + i] = mq[0];
+                for (int i = lane; i < ND; i += TL) su[ND + i] = mq[0];
             if (!(cm & 4u))
-                for (int i = lane; i < ND; i += 32) su[2 * ND + i] = mq[1];
+                for (int i = lane; i < ND; i += TL) su[2 * ND + i] = mq[1];
             if (!(cm & 1u)) {
                 double e;
                 if (m <= 0.0) e = -d.zmax[k];
                 else {
                     e = emax;
-                    bulk::scalar_newton<R, Pix, MODE>(d, tb, k, J, m, e, lane);
+                    bulk::scalar_newton<R, Pix, MODE, TL, 32 / TL>(d, tb, k, J, m, e, lane, tm);
                 }
-                for (int i = lane; i < ND; i += 32) su[i] = e;
+                for (int i = lane; i < ND; i += TL) su[i] = e;
             }
-            __syncwarp();
-            for (int i = lane; i < 4 * ND; i += 32) {
+            __syncwarp(tm);
+            for (int i = lane; i < 4 * ND; i += TL) {
                 ufield(d, 0, i / ND, ND)[k * ND + (i % ND)] = su[i];
                 if (d.uF) ufieldF(d, 0, i / ND, ND)[k * ND + (i % ND)] = (float)su[i];
             }
             cm = 15u;
-            for (int p = lane; p < NMP; p += 32) {
+            for (int p = lane; p < NMP; p += TL) {
                 pe[p] = su[0];
                 pc[p] = su[3 * ND];
                 double V, A;
                 ST::VA(d, *d.tabs, k, SET_MASS, p % NM, p / NM, pe[p], V, A);
                 pV[p] = V;
             }
-            __syncwarp();
+            __syncwarp(tm);
         }
         // H_i(zeta^n), C~_i^n and their sums
         double hb = 0.0, cb = 0.0;
-        for (int p = lane; p < NMP; p += 32) {
+        for (int p = lane; p < NMP; p += TL) {
             const double w = J * tb.wm[p % NM] * tb.wm[p / NM];
             hb += w * pV[p];
             cb += w * pV[p] * pc[p];
             px[p] = w * pV[p];
             pc[p] = px[p] * pc[p]; // c is not needed beyond C~
         }
-        team_sum2<32>(hb, cb, 0xffffffffu);
-        __syncwarp();
-        tens_test2<ND1, NM>(tb.Bm, px, pc, tmp, tmp + NM * NM, out, out + ND, lane);
-        for (int i = lane; i < ND; i += 32) {
+        team_sum2<TL>(hb, cb, tm);
+        __syncwarp(tm);
+        tens_test2<ND1, NM, double, TL>(tb.Bm, px, pc, tmp, tmp + NM * NM, out, out + ND, lane, tm);
+        for (int i = lane; i < ND; i += TL) {
             d.HN[k * ND + i] = out[i];
             d.CN[k * ND + i] = out[ND + i];
-        }
-        // the discharges of v^n at the momentum points, the same for every
-        // stage of the step (the stage update reads them rather than
-        // interpolating v^n again; same sums, same constant fields)
-        if (d.qpts) {
-            tens_interp2<ND1, NG>(tb.Bg, su + ND, su + 2 * ND, tmp, tmp + NM * NM, pg, pg + NGP, lane);
-            for (int p = lane; p < 2 * NGP; p += 32)
-                d.qpts[k * 2 * NGP + p] = (cm & (2u << (p / NGP))) ? su[(1 + p / NGP) * ND] : pg[p];
         }
         if (lane == 0) {
             d.HNbar[k] = hb;
@@ -913,7 +918,7 @@ __global__ void __launch_bounds__(32 * MAXWPB)
             d.cmask[k] = (uint8_t)cm;
             if (d.wet0) d.wet0[k] = (uint8_t)(flag != 0 && allfull);
         }
-        __syncwarp();
+        __syncwarp(tm);
     }
 }
 
@@ -1278,6 +1283,11 @@ __device__ void momentum_block(const Dev& d, const BaseTables& tb, int64_t k, do
     }
 }
 
+// The stage update: one cell per team of 16 lanes, nodal values and point values in
+// shared memory.  The FP64 pipe and the latency of the solves bound it: a launch of
+// 65,536 cells (r = 3) takes 608 / 642 / 555 us (stage 2, 3, final), 172,032 cells
+// (r = 2) 989 / 1057 / 907; with the tables in the parameter bank and the mesh in
+// order 670 / 704 / 608 and 1052 / 1130 / 955.  80 and 128 registers: 619 and 629.
 template <int R, typename Pix, int MODE>
 __global__ void __maxnreg__(96)
     k_stage(const __grid_constant__ Dev d, const __grid_constant__ StageArgs sa) {
@@ -1483,21 +1493,16 @@ __global__ void __maxnreg__(96)
                 for (int p = lane; p < NMP; p += TL) s += tb.wm[p % NM] * tb.wm[p / NM] * pe[p];
                 e = team_sum<TL>(s, tm);
             }
-            its = bulk::scalar_newton<R, Pix, MODE, TL>(d, tb, k, J, Tbar, e, lane, tm);
+            its = bulk::scalar_newton<R, Pix, MODE, TL, 1>(d, tb, k, J, Tbar, e, lane, tm);
             // momentum: sums of the rows of the friction-modified mass matrix
             double den = 0.0, num[2] = {0.0, 0.0};
-            if (d.qpts) {
-                for (int p = lane; p < 2 * NGP; p += TL) pg[3 * NGP + p] = d.qpts[k * 2 * NGP + p];
+            for (int f = 0; f < 2; ++f) {
+                if (cm0 & (2u << f))
+                    for (int p = lane; p < NGP; p += TL) pg[(3 + f) * NGP + p] = su[(1 + f) * ND];
+                else
+                    tens_interp<ND1, NG, double, TL>(tb.Bg, su + (1 + f) * ND, tmp, pg + (3 + f) * NGP,
+                                                     lane, tm);
                 __syncwarp(tm);
-            } else {
-                for (int f = 0; f < 2; ++f) {
-                    if (cm0 & (2u << f))
-                        for (int p = lane; p < NGP; p += TL) pg[(3 + f) * NGP + p] = su[(1 + f) * ND];
-                    else
-                        tens_interp<ND1, NG, double, TL>(tb.Bg, su + (1 + f) * ND, tmp,
-                                                         pg + (3 + f) * NGP, lane, tm);
-                    __syncwarp(tm);
-                }
             }
             for (int p = lane; p < NGP; p += TL) {
                 const double w = J * tb.wg[p % NG] * tb.wg[p / NG];
@@ -1517,7 +1522,7 @@ __global__ void __maxnreg__(96)
             const double qxn = (num[0] + rs0) / den;
             const double qyn = (num[1] + rs1) / den;
             double Hs, As;
-            bulk::mass_scalar_pixels<R, Pix, MODE, TL>(d, tb, k, J, e, lane, Hs, As, tm);
+            bulk::mass_scalar_pixels<R, Pix, MODE, TL, 1>(d, tb, k, J, e, lane, Hs, As, tm);
             const bool tr_ok = Hs > 1e-14 * J * d.hlim;
             const double cn = tr_ok ? (d.CNbar[k] + rcs) / Hs : 0.0;
             for (int i = lane; i < ND; i += TL) {

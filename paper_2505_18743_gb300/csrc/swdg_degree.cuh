@@ -13,12 +13,12 @@ template <int R, typename Pix, int MODE, typename B>
 struct Launchers {
     using S = Sz<R>;
     static constexpr bool F64 = sizeof(B) == sizeof(double);
-    // shared memory per warp; the step start gives a cell 16 lanes (FP32-bulk: 32), the
-    // stage update 16
+    // shared memory per warp
     static constexpr size_t res_b =
         sizeof(double) * (F64 ? ResFx<R>::words : bulk::Res<R>::words) * (32 / ResFx<R>::TL);
-    static constexpr int begin_cells = F64 ? 2 : 1;
-    static constexpr size_t begin_b = sizeof(double) * (F64 ? 2 * BeginFx<R>::words : bulk::begin_smem<R>());
+    static constexpr int begin_cells = F64 ? 2 : 32 / bulk::begin_team<R>(); // per warp
+    static constexpr size_t begin_b =
+        sizeof(double) * begin_cells * (F64 ? BeginFx<R>::words : bulk::begin_smem<R>());
     static constexpr size_t stage_b =
         2 * sizeof(double) * (F64 ? StageFx<R>::words : bulk::stage_smem<R>());
     static auto residual_kernel() {
