@@ -548,7 +548,9 @@ __device__ __forceinline__ long long fx_pixel(double z, int e) { return fx::from
 // not.  The rows' sums are then moved up to the bound eta + zhi of a pixel's depth, so
 // that a film of water at a great height, or beside a deep cell, has its own
 // relative accuracy (59 places of cx times that bound).  Not inlined: most cells never
-// get here, and the callers' code stays small.
+// get here, and the callers' code stays small.  Measured, a step of the lagoon (r = 2,
+// 8 to 32 pixels a side): 3543 us with FP64 pixel sums, 2104 with integers; without the
+// move up 10 us less, and with a branch around the conversion of a dry pixel 150 more.
 template <typename Pix>
 __device__ __noinline__ SubV subgrid_S(const Pix* __restrict__ tile, const OvTab* __restrict__ ov,
                                        int setx, int ia, int sety, int ib, double eta, float zhi) {
