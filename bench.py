@@ -79,8 +79,8 @@ def load_counters(path=COUNTERS):
     """the ncu counters of one step's launches (profiles/counters_...txt):
     ({precision: {slot: (fp64 flops per cell, fp32 flops per cell, DRAM bytes
     per launch)}}, whether they were taken on the current kernel sources).
-    The kernels here are bound by the FP64 pipe, so the FP64 flops per cell
-    give the roofline's achieved rate."""
+    The FP64 flops per cell give the roofline's achieved rate; what the FP64 path
+    forms on the integer pipe (its contractions and pixel sums) is not in them."""
     table, sha = {}, None
     with open(path) as f:
         for line in f:
@@ -732,8 +732,9 @@ def run_gpu(args, rank, world, local):
     avg_ms = sum(per_launch[k] for k in slots) / len(slots)
     counters, fresh = load_counters()
     table = counters["fp64" if prec == 0 else "fp32bulk"]
-    flops = sum(table[k][0] for k in slots) / len(slots) * wl.mesh.n
-    ach = flops / (avg_ms / 1e3) / 1e12
+    # no rate from counters of other kernels
+    flops = sum(table[k][0] for k in slots) / len(slots) * wl.mesh.n if fresh else None
+    ach = flops / (avg_ms / 1e3) / 1e12 if fresh else None
     pk, src = peaks()
     nres = {"stage_2": 1, "stage_3": 2, "stage_4": 3, "final": STAGES}
     bpc = sum(algorithmic_bytes_per_cell(k, nres=nres.get(k, STAGES)) for k in slots) / len(slots)
@@ -749,7 +750,7 @@ def run_gpu(args, rank, world, local):
         fp64_peak = FP64_PEAK_TFLOPS
         peak_src = "FP64 pipe, nominal 152 SMs x 2.07 GHz x 4 flop/clk (probe unavailable)"
     roof = {"bound": "alu", "kernel": dom_fn, "achieved": ach, "peak": fp64_peak,
-            "unit": "TFLOP/s", "frac": ach / fp64_peak,
+            "unit": "TFLOP/s", "frac": ach / fp64_peak if fresh else None,
             "traffic": (sum(traffic) / len(traffic)) if all(x is not None for x in traffic) else None,
             "peak_source": peak_src,
             "pipe_peaks_measured_tflops": {k: round(v[0], 3) for k, v in pipe.items()},
